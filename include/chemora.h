@@ -313,9 +313,9 @@ int chemora_adjoint_rk4(chemora_system* sys, const double* state0, const double*
  * with a model of idle edge threads and wave quantisation, times the
  * plausible ones on `state` (its ghosts are filled first) and keeps the
  * fastest for this system.  Shapes of the same body perform the same
- * per-point arithmetic; the lane-, shared-memory- and z-queue-sharing bodies
- * form the stencils' differences in another order, so results of different
- * bodies agree to rounding (each within the parity tolerances of the
+ * per-point arithmetic (every shape of a scalar wave gives the same bits); the
+ * lane- and shared-memory-sharing BSSN bodies form the stencils' differences
+ * in another order, so results of different bodies agree to rounding (each within the parity tolerances of the
  * oracle).  *variant and *best_ms (time of a middle RK stage of the winner)
  * may be NULL.  For the order-4 scalar wave it also times whole RK4 steps
  * (on a copy of `state`) with the per-stage kernels and with the
@@ -406,10 +406,10 @@ int chemora_opcount(int kind, int64_t* fp64_instructions, int64_t* flops);
 
 /* Operation counts per interior point of one RHS evaluation by the body the
  * system currently launches (the autotuned launch shape may use a body that
- * shares x-direction work across warp lanes, y differences through shared
- * memory, or z differences through a register queue; the counts then
- * include, per point, that sharing's own work).  Counts as
- * chemora_opcount. */
+ * shares x-direction work across warp lanes or y differences through shared
+ * memory; the counts then include, per point, that sharing's own work).
+ * Counts as chemora_opcount; a stencil evaluated on the integer units counts
+ * its algorithmic flops and no FP64 instruction. */
 int chemora_system_opcount(chemora_system* sys, int64_t* fp64_instructions, int64_t* flops);
 
 /* Measure the device's FP64 fused-multiply-add throughput (flop/s, fma = 2)

@@ -8,8 +8,8 @@
 // 1.5x slower than its best are skipped, the rest are timed with CUDA
 // events on the caller's grid (a middle RK stage, two repetitions after a
 // warm-up) and the fastest is kept by the system.  Shapes of one body
-// perform the same arithmetic; different bodies (direct, lane-, shared-
-// memory- or z-queue-sharing) agree to rounding.
+// perform the same arithmetic; different BSSN bodies (direct, lane- or
+// shared-memory-sharing) agree to rounding.
 #include <math.h>
 
 #include <algorithm>
@@ -34,7 +34,7 @@ static int64_t xy_prologue_flops(int ty) {
 
 static double model_cost(int kind, const Dims& d, const LaunchVariant& v, int sms) {
   // lane-sharing shapes need whole warps of x points
-  if (v.xshare && v.xshare != 8 && d.nx % v.tx != 0) return 1e300;
+  if ((v.xshare == 1 || v.xshare == 2) && d.nx % v.tx != 0) return 1e300;
   const double nbx = ceil((double)d.nx / v.tx), nby = ceil((double)d.ny / v.ty);
   const double blocks = nbx * nby * d.nz;
   const double threads = blocks * v.tx * v.ty;  // launched, including idle edge threads
@@ -46,7 +46,7 @@ static double model_cost(int kind, const Dims& d, const LaunchVariant& v, int sm
   const double waves = blocks / (double)(sms * bps);
   const double quant = waves < 1.0 ? 1.0 / std::max(waves, 1e-9) : ceil(waves) / waves;
   // x-sharing bodies issue about 11 % fewer FP64 instructions per point
-  // (the x/z wave shapes: 24 of 30 FP64 instructions per point)
+  // (the marching wave shapes: fewer loads and integer operations)
   const double work = v.xshare == 2 ? 0.81 : (v.xshare == 1 ? 0.89 : (v.xshare == 4 ? 0.8 : 1.0));
   return work * threads * (waves < 8.0 ? quant : 1.0 + 0.5 / waves);
 }
@@ -113,12 +113,10 @@ int chemora_variant_info(int kind, int variant, int* tx, int* ty, int* min_block
 int chemora_system_opcount(chemora_system* sys, int64_t* fp64_instructions, int64_t* flops) {
   if (!is_handle(sys, H_SYSTEM)) return set_error(CHEMORA_EINVAL, "not a system handle");
   const LaunchVariant* v = variant_info(sys->kind, sys->variant);
-  if (sys->kind == CHEMORA_WAVE && sys->sc.order == 4 && v && v->xshare == 4 &&
-      sys->grid->d.nx % v->tx == 0 && sys->grid->d.g >= 2) {
-    // x-lane / z-queue body plus, per point, the queue's new difference and
-    // its two combinations and the lane-halo difference
-    if (fp64_instructions) *fp64_instructions = CHEMORA_OPS_WAVE_XZ_INSTR + 4;
-    if (flops) *flops = CHEMORA_OPS_WAVE_XZ_FLOPS + 4;
+  if (sys->kind == CHEMORA_WAVE && sys->sc.order == 4) {
+    // the stencil runs on the integer units: one FP64 multiply is left
+    if (fp64_instructions) *fp64_instructions = 1;
+    if (flops) *flops = CHEMORA_OPS_WAVE_FLOPS;
     return CHEMORA_OK;
   }
   const bool xs = v && v->xshare && sys->grid->d.nx % v->tx == 0 && sys->grid->d.g >= 3;

@@ -1,0 +1,97 @@
+// Finite-difference stencils on the integer units.
+//
+// On GB300 an FP64 fma occupies the SM's FP64 pipe for 17-19 cycles per warp
+// (1.7-1.9 fmas per clock per SM, measured), a 32-bit integer operation for
+// 0.4-0.8, on pipes that run beside it (measured: twelve integer operations
+// per fma, or a load, do not slow a saturated fma stream).  A stencil is a
+// sum of values times small integers, so it is evaluated in integers: the
+// values it reads are written as multiples of one power of two, taken from
+// the largest of them (align), added exactly in 64 or 96 bits, and the sum is
+// rounded once to a double (to_double).  With K guard bits every value down
+// to 2^-K of the largest is represented exactly and a smaller one is
+// truncated at 2^(-52-K) of the largest value's power of two, so the result
+// is at least as close to the exact sum as that of a chain of FP64
+// additions.  It depends on the values alone, not on the order of the sum or
+// on the launch shape that evaluates it.
+//
+// A set of values whose largest exponent lies outside [128, 2030] (zeros,
+// numbers near the ends of the FP64 range, Inf, NaN) is left to the caller's
+// FP64 body (in_range).  Compiles for the host too (tests).
+#pragma once
+#include <stdint.h>
+#if !defined(__CUDACC__)
+#include <string.h>
+#endif
+
+namespace chemora {
+namespace fx {
+
+#if defined(__CUDACC__)
+#define CHEMORA_FX __device__ __forceinline__
+CHEMORA_FX unsigned hiword(double v) { return (unsigned)__double2hiint(v); }
+CHEMORA_FX unsigned loword(double v) { return (unsigned)__double2loint(v); }
+CHEMORA_FX double from_bits(unsigned long long b) { return __longlong_as_double((long long)b); }
+// PTX shifts clamp: an amount of 64 or more gives 0
+CHEMORA_FX unsigned long long shr(unsigned long long a, unsigned s) {
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(s));
+  return r;
+}
+CHEMORA_FX unsigned long long shl(unsigned long long a, unsigned s) {
+  unsigned long long r;
+  asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(s));
+  return r;
+}
+CHEMORA_FX int clz64(unsigned long long a) { return __clzll((long long)a); }
+#else
+#define CHEMORA_FX inline
+CHEMORA_FX unsigned long long bits(double v) {
+  unsigned long long b;
+  memcpy(&b, &v, 8);
+  return b;
+}
+CHEMORA_FX unsigned hiword(double v) { return (unsigned)(bits(v) >> 32); }
+CHEMORA_FX unsigned loword(double v) { return (unsigned)bits(v); }
+CHEMORA_FX double from_bits(unsigned long long b) {
+  double v;
+  memcpy(&v, &b, 8);
+  return v;
+}
+CHEMORA_FX unsigned long long shr(unsigned long long a, unsigned s) { return s > 63 ? 0 : a >> s; }
+CHEMORA_FX unsigned long long shl(unsigned long long a, unsigned s) { return s > 63 ? 0 : a << s; }
+CHEMORA_FX int clz64(unsigned long long a) { return a ? __builtin_clzll(a) : 64; }
+#endif
+
+// The exponent field of v, in place (bits 20-30 of the high word).
+CHEMORA_FX unsigned ebits(double v) { return hiword(v) & 0x7ff00000u; }
+CHEMORA_FX unsigned emax(unsigned a, unsigned b) { return a > b ? a : b; }
+constexpr unsigned kExpMin = 128u << 20, kExpMax = 2030u << 20;
+CHEMORA_FX bool in_range(unsigned e) { return e - kExpMin <= kExpMax - kExpMin; }
+
+// v in units of 2^(E - 1075 - K), E the exponent field e of the largest value:
+// |result| < 2^(53 + K).  Zeros and subnormals carry a false leading bit that
+// the shift (at least 128) removes.
+template <int K>
+CHEMORA_FX long long align(double v, unsigned e) {
+  const unsigned h = hiword(v), d = (e - (h & 0x7ff00000u)) >> 20;
+  unsigned long long m = (unsigned long long)((h & 0xfffffu) | 0x100000u) << 32 | loword(v);
+  m = shr(m << K, d);
+  const unsigned long long s = (unsigned long long)(long long)((int)h >> 31);
+  return (long long)((m ^ s) - s);
+}
+
+// v units of 2^(E - 1075 - K) as a double (nearest, ties away from zero).
+template <int K>
+CHEMORA_FX double to_double(long long v, unsigned e) {
+  const unsigned long long s = (unsigned long long)(v >> 63);
+  const unsigned long long a = ((unsigned long long)v ^ s) - s;
+  const int lz = clz64(a);
+  const unsigned long long m = shl(a, (unsigned)lz);
+  unsigned long long r = (m >> 11) + ((m >> 10) & 1);
+  r += (unsigned long long)((e >> 20) + (unsigned)(10 - K) - (unsigned)lz) << 52;
+  r |= s & 0x8000000000000000ull;
+  return a == 0 ? 0.0 : from_bits(r);
+}
+
+}  // namespace fx
+}  // namespace chemora

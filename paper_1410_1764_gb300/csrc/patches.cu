@@ -20,7 +20,7 @@
 #include "internal.h"
 #include "stage.cuh"
 #include "generated/gen_bssn.cuh"
-#include "generated/gen_wave.cuh"
+#include "wave_point.cuh"
 
 struct chemora_batch {
   uint32_t type;
@@ -63,7 +63,7 @@ template <>
 struct BatchBody<2> {
   template <class LD, class OUT>
   __device__ __forceinline__ static void eval(const LD& ld, const Scalars& sc, OUT& out) {
-    chemora_wave_point(ld, sc, out);
+    wave_point(ld, sc, out);
   }
 };
 

@@ -3,7 +3,7 @@
 // are compiled for the autotuner.
 #include "internal.h"
 #include "stage.cuh"
-#include "generated/gen_wave.cuh"
+#include "wave_point.cuh"
 #include "generated/gen_wave_varc.cuh"
 
 namespace chemora {
@@ -17,7 +17,7 @@ __global__ void __launch_bounds__(TX * TY) wave_stage_kernel(Dims d, Scalars sc,
   const int64_t c = (int64_t)(k + d.g) * d.sz + (int64_t)(j + d.g) * d.sy + (i + d.g);
   Loader<2> ld{a.src + c, nullptr, d.sy, d.sz, d.sv};
   StageOutFma out = CHEMORA_STAGE_OUT_FMA(a, c, d.sv, sc);
-  chemora_wave_point(ld, sc, out);
+  wave_point(ld, sc, out);
 }
 
 // Loader of the variable-speed body: state variables 0-1, then the
@@ -45,76 +45,51 @@ __global__ void __launch_bounds__(TX * TY) varc_stage_kernel(Dims d, Scalars sc,
   chemora_varc_point(ld, sc, out);
 }
 
-// 2.5D blocking for the order-4 scalar wave: a warp is 32 consecutive x
-// points of one row (x-direction first differences shared across lanes, as
-// in the BSSN x-sharing body), and each thread marches ZB points along z
-// keeping the z first differences e_m = u(z+m+1) - u(z+m), m = -2..1, of its
-// own column in registers; the generated body (chemora_wave_xz_point) takes
-// 12h^2 D_zz u = 15 (e_0 - e_-1) - (e_1 - e_-2).  Per point: one new z load
-// and three FP64 operations for the queue instead of four loads and seven
-// operations.  Requires nx % TX == 0 (every lane an interior point).
-#include "generated/gen_wave_xz.cuh"
-
-struct XZLoader : XLoader<2> {
-  double qa[1], qb[1];  // e_0 - e_-1 and e_1 - e_-2 of u at the current z
+// 2.5D blocking for the order-4 scalar wave: each thread marches ZB points
+// along z and keeps the five column values its stencil reads in registers, so
+// a point costs one new column load instead of four, and the column's values
+// are taken apart into integers once (the unrolled march reuses them).
+struct ColumnLoader {
+  const double* __restrict__ p;  // centre point of variable 0
+  int64_t sy, sv;
+  double z[5];  // u at z-2 .. z+2
+  __device__ __forceinline__ double operator()(int v, int dx, int dy, int dz) const {
+    if (v == 0 && dx == 0 && dy == 0) return z[dz + 2];
+    return __ldg(p + v * sv + dx + dy * sy);
+  }
 };
 
 template <int TX, int TY, int ZB>
-__global__ void __launch_bounds__(TX * TY) wave_xz_kernel(Dims d, Scalars sc, StageParams a) {
+__global__ void __launch_bounds__(TX * TY) wave_march_kernel(Dims d, Scalars sc, StageParams a) {
   const int i = blockIdx.x * TX + threadIdx.x;
   const int j = blockIdx.y * TY + threadIdx.y;
   const int k0 = blockIdx.z * ZB;
-  if (j >= d.ny) return;  // whole warps (a warp is one row)
-  const double one = sc.k[CHEMORA_K_ONE];
+  if (i >= d.nx || j >= d.ny) return;
   int64_t c = (int64_t)(k0 + d.g) * d.sz + (int64_t)(j + d.g) * d.sy + (i + d.g);
   const double* u = a.src + c;
-  double e[4], ulast;
-  {
-    const double um2 = __ldg(u - 2 * d.sz), um1 = __ldg(u - d.sz), u0 = __ldg(u), u1 = __ldg(u + d.sz);
-    ulast = __ldg(u + 2 * d.sz);
-    e[0] = fma(um2, -one, um1);
-    e[1] = fma(um1, -one, u0);
-    e[2] = fma(u0, -one, u1);
-    e[3] = fma(u1, -one, ulast);
-  }
-  const int lane = threadIdx.x & 31;
-  // x halo of the lane-shared first differences: lanes 1, 2 hold x0-2, x0-1
-  // and lane 3 holds x0+32 (lanes 0 and 4 repeat a neighbour: the radius-2
-  // stencil needs no more, and with 2 ghost layers every read stays in the row)
-  const int xo = lane == 0 ? -2 : (lane < 3 ? -3 : (lane == 3 ? 29 : (lane == 4 ? 28 : 0)));
-#pragma unroll 1
+  ColumnLoader ld;
+  ld.sy = d.sy;
+  ld.sv = d.sv;
+#pragma unroll
+  for (int m = 1; m < 5; ++m) ld.z[m] = __ldg(u + (int64_t)(m - 3) * d.sz);
+#pragma unroll
   for (int kz = 0; kz < ZB; ++kz) {
     if (k0 + kz >= d.nz) break;  // uniform over the block
-    XZLoader ld;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) ld.z[m] = ld.z[m + 1];
     ld.p = a.src + c;
-    ld.sy = d.sy;
-    ld.sz = d.sz;
-    ld.sv = d.sv;
-    ld.xo_dx = xo;
-    ld.xo_d1 = 0;
-    ld.qa[0] = fma(e[1], -one, e[2]);
-    ld.qb[0] = fma(e[0], -one, e[3]);
+    ld.z[4] = __ldg(ld.p + 2 * d.sz);
     StageOutFma out = CHEMORA_STAGE_OUT_FMA(a, c, d.sv, sc);
-    chemora_wave_xz_point(ld, sc, out);
-    if (k0 + kz + 1 < d.nz) {  // advance the queue (u(z+3) is inside the ghost layers only then)
-      const double unew = __ldg(a.src + c + 3 * d.sz);
-      e[0] = e[1];
-      e[1] = e[2];
-      e[2] = e[3];
-      e[3] = fma(ulast, -one, unew);
-      ulast = unew;
-    }
+    wave_point(ld, sc, out);
     c += d.sz;
   }
 }
 
 template <int TX, int TY, int ZB>
-static int launch_wave_xz(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s) {
-  if (d.nx % TX != 0 || d.g < 2)
-    return set_error(CHEMORA_EUNSUPPORTED, "x/z-sharing wave kernel needs nx %% %d == 0", TX);
-  dim3 grid(d.nx / TX, (d.ny + TY - 1) / TY, (d.nz + ZB - 1) / ZB);
-  wave_xz_kernel<TX, TY, ZB><<<grid, dim3(TX, TY), 0, s>>>(d, sc, a);
-  return launched("wave_xz_kernel");
+static int launch_wave_march(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s) {
+  dim3 grid((d.nx + TX - 1) / TX, (d.ny + TY - 1) / TY, (d.nz + ZB - 1) / ZB);
+  wave_march_kernel<TX, TY, ZB><<<grid, dim3(TX, TY), 0, s>>>(d, sc, a);
+  return launched("wave_march_kernel");
 }
 
 // Staged tiles: the block's 32 x 8 tile of u with its 2-point halo, for the
@@ -154,7 +129,7 @@ __global__ void __launch_bounds__(TX * TY) wave_tile_kernel(Dims d, Scalars sc, 
   const int64_t c = (int64_t)(k + d.g) * d.sz + (int64_t)(j + d.g) * d.sy + (i + d.g);
   TileLoader ld{tile + 2 * PLANE + (threadIdx.y + 2) * PX + threadIdx.x + 2, a.src + d.sv + c, PX, PLANE};
   StageOutFma out = CHEMORA_STAGE_OUT_FMA(a, c, d.sv, sc);
-  chemora_wave_point(ld, sc, out);
+  wave_point(ld, sc, out);
 }
 
 template <int TX, int TY>
@@ -182,9 +157,9 @@ const LaunchVariant kWaveVariants[] = {
     {32, 8, 0, launch_wave_variant<32, 8>},  {32, 4, 0, launch_wave_variant<32, 4>},
     {64, 4, 0, launch_wave_variant<64, 4>},  {128, 2, 0, launch_wave_variant<128, 2>},
     {32, 16, 0, launch_wave_variant<32, 16>}, {16, 16, 0, launch_wave_variant<16, 16>},
-    {32, 8, 0, launch_wave_xz<32, 8, 8>, 4},   {32, 8, 0, launch_wave_xz<32, 8, 16>, 4},
-    {32, 4, 0, launch_wave_xz<32, 4, 16>, 4},  {64, 4, 0, launch_wave_xz<64, 4, 32>, 4},
-    {32, 16, 0, launch_wave_xz<32, 16, 8>, 4},
+    {32, 8, 0, launch_wave_march<32, 8, 4>, 4},  {32, 8, 0, launch_wave_march<32, 8, 8>, 4},
+    {32, 4, 0, launch_wave_march<32, 4, 4>, 4},  {64, 4, 0, launch_wave_march<64, 4, 8>, 4},
+    {32, 16, 0, launch_wave_march<32, 16, 8>, 4},
     {32, 8, 0, launch_wave_tile<32, 8>, 8},    {32, 4, 0, launch_wave_tile<32, 4>, 8},
 };
 const int kNumWaveVariants = sizeof(kWaveVariants) / sizeof(kWaveVariants[0]);
@@ -200,7 +175,6 @@ int launch_wave_stage(const Dims& d, const Scalars& sc, const StageParams& a, cu
   if (sc.order != 4) return launch_wave_order_stage(d, sc, a, s, variant);
   if (variant < 0 || variant >= kNumWaveVariants) variant = 0;
   const LaunchVariant& v = kWaveVariants[variant];
-  if (v.xshare == 4 && (d.nx % v.tx != 0 || d.g < 2)) return kWaveVariants[0].launch(d, sc, a, s);
   return v.launch(d, sc, a, s);
 }
 

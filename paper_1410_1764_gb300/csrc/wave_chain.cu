@@ -19,7 +19,7 @@
 #include <vector>
 
 #include "internal.h"
-#include "generated/gen_wave.cuh"
+#include "wave_point.cuh"
 
 namespace chemora {
 
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(128) wave_chain_stage_kernel(Dims d, Scalars s
     out.yn[v] = __ldcg(a.yn + c + v * d.sv);
     if (a.mode >= 2) out.acc[v] = __ldcg(a.acc + c + v * d.sv);
   }
-  chemora_wave_point(ld, sc, out);
+  wave_point(ld, sc, out);
 }
 
 struct ChainGraph {
