@@ -162,17 +162,18 @@ def kernel_source_hash():
 
 
 def _kernel_name(api, fp64_instr, variant, specialised):
-    """The BSSN stage kernel the chosen launch shape runs: the direct body,
-    the x lane-sharing body or the x lane + y shared-memory body (the last
-    carries the prologue in its count); run-time specialised kernels are all
-    named chemora_jit_stage."""
-    if fp64_instr == api.opcount(api.BSSN)[0]:
-        name, body = "bssn_stage_kernel", "direct"
+    """The BSSN stage kernels the chosen launch shape runs: derivative fields
+    and algebra, the x lane-sharing body or the x lane + y shared-memory body
+    (the last carries the prologue in its count); run-time specialised kernels
+    are all named chemora_jit_stage."""
+    if api.variant_info(api.BSSN, variant)[3] == 0:
+        name, body = "bssn_algebra_kernel", "algebra"
     elif api.variant_info(api.BSSN, variant)[3] == 2:
         name, body = "bssn_xystage_kernel", "x/y-sharing"
     else:
         name, body = "bssn_xstage_kernel", "x-sharing"
-    return "chemora_jit_stage (%s body)" % body if specialised else name
+    name = "chemora_jit_stage (%s body)" % body if specialised else name
+    return "bssn_fields_kernel + " + name if body == "algebra" else name
 
 
 def cpu_baseline(n, nsteps=2, nz1=16):

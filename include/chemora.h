@@ -89,8 +89,9 @@ int chemora_grid_layout(const chemora_grid* grid, int64_t* sy, int64_t* sz, int6
 /* A PDE system on a grid (Sec. 3.2.1: the physics description).  kind is
  * CHEMORA_WAVE, CHEMORA_WAVE_VARC, CHEMORA_BSSN or CHEMORA_WAVE1; params may
  * be NULL for the defaults (eps 0.1, eta 2, 1+log, Gamma-driver, order 4);
- * the wave systems read only fd_order.  The grid must outlive the system.  Scratch for RK4 (three states)
- * is allocated on first use.  Errors: EINVAL for a wrong nvars/nghost for the
+ * the wave systems read only fd_order.  The grid must outlive the system.  Scratch for RK4 (three states;
+ * for BSSN also a workspace of derivative fields, 1296 bytes per point of at
+ * most 2^20 points or one xy plane at a time) is allocated on first use.  Errors: EINVAL for a wrong nvars/nghost for the
  * kind or bad params, ENOMEM. */
 int chemora_system_create(chemora_grid* grid, int kind, const chemora_params* params,
                           chemora_system** out);
@@ -118,7 +119,11 @@ int chemora_fill_ghosts_axes(chemora_system* sys, double* state, int axes, void*
 
 /* rhs <- RHS(state) on the interior (Sec. 3.2: the "RHS" calculation).  The
  * ghosts of state must be valid; the ghosts of rhs are left untouched.
- * state and rhs must not overlap. */
+ * state and rhs must not overlap.  A BSSN system takes a workspace of
+ * derivative fields from a pool of its own in stream order (also in
+ * chemora_stage and chemora_constraints), so calls on several streams do not
+ * share one; without a workspace (a stream that is being captured, no memory
+ * left) it runs a slower kernel that agrees to rounding. */
 int chemora_rhs(chemora_system* sys, const double* state, double* rhs, void* stream);
 
 /* nsteps classic RK4 steps of size dt, in place (Sec. 2, time integrator).
@@ -342,8 +347,8 @@ int chemora_variant_count(int kind);
 
 /* Launch shape `variant` of the stage kernel of `kind`: block tx x ty
  * threads, min_blocks resident blocks per SM asked of the compiler (the
- * register cap), and sharing: 0 the direct body (neighbours through the
- * read-only cache), 1 x-direction work shared across warp lanes (needs
+ * register cap), and sharing: 0 one point per thread (BSSN: derivative fields
+ * and algebra in two kernels, tx x ty the algebra kernel's block), 1 x-direction work shared across warp lanes (needs
  * nx % tx == 0 and 3 ghost layers), 2 in addition y-direction differences
  * and z-derivative rows shared through shared memory (any ny), 4 (scalar
  * wave, order 4) x-direction work shared across warp lanes and each thread
@@ -359,7 +364,9 @@ int chemora_system_variant(chemora_system* sys, int set, int* variant, int* tx, 
 /* Run-time specialisation of the stage kernel (Sec. 3.2.3: the run-time
  * library compiles loop kernels once parameter values are known, to cut code
  * and register overhead).  With enable = 1 the library writes a CUDA source
- * that instantiates the body of the system's current launch shape with the
+ * that instantiates the body of the system's current launch shape (for the
+ * shapes of sharing 0, and where a sharing shape does not fit the grid, the
+ * algebra kernel) with the
  * grid extents, ghost width and strides as literals, the scalars 1/(12h),
  * 1/(12h^2), 1/(144h^2), the dissipation scale and the gauge parameters as
  * compile-time constants (exact hexadecimal literals: same arithmetic as the

@@ -12,8 +12,10 @@
 // is computed that a later stage does not read.
 //
 // The boxes are patches of a batched work-list (the persistent stage kernel
-// of patches.cu): one launch per fine RK stage advances every box, over a
-// per-stage patch table whose interiors shrink by r per stage.  For
+// of patches.cu; for BSSN the split kernels of bssn_split.cu): one launch per
+// fine RK stage (BSSN: one field and one algebra launch per chunk) advances
+// every box, over a per-stage patch table whose interiors shrink by r per
+// stage.  For
 // comparison, mode 1 launches the single-grid stage kernel box by box.
 //
 // Prolongation: quintic Lagrange interpolation along each axis (weights
@@ -71,7 +73,11 @@ struct chemora_amr {
   chemora::AmrBox* dev_boxes;
   chemora::PatchDesc* dev_pd;
   chemora::WorkItem* items;
-  unsigned int* counters;  // 8: fine step (2) x stage (4) of a coarse step
+  chemora::FieldPlan plan[4];   // BSSN: the work-list of each fine stage
+  double* work;                 // BSSN: derivative fields (coarse stages and fine chunks)
+  int64_t work_points;
+  int counter_off[5];           // stage s's counters: [counter_off[s-1], counter_off[s])
+  unsigned int* counters;  // fine step (2) x stage (4) [x chunk] of a coarse step
   int* err;
 };
 
@@ -191,6 +197,13 @@ static int nblocks(int64_t n) {
   return (int)(b > 4096 ? 4096 : (b < 1 ? 1 : b));
 }
 
+static FieldWork amr_work(const chemora_amr* A) {
+  FieldWork w;
+  w.w = A->work;
+  w.points = A->work_points;
+  return w;
+}
+
 // Fill every box's buffer from the coarse time levels with weights w.
 static int amr_prolong(chemora_amr* A, const TimeLevels& tl, cudaStream_t s) {
   int64_t nt = 0, n1 = 0, n2 = 0, n3 = 0;
@@ -233,7 +246,7 @@ static int rk4_coarse(chemora_amr* A, double* Y, double dt, double* kn, cudaStre
     StageParams p{};
     p.src = srcs[q]; p.yn = Y; p.acc = acc; p.dst = dsts[q];
     p.c1 = dt / 6.0; p.c2 = c2[q]; p.mode = q + 1;
-    if ((rc = launch_stage(A->kind, d, A->scc, p, s, A->coarse_variant))) return rc;
+    if ((rc = launch_stage(A->kind, d, A->scc, p, s, A->coarse_variant, amr_work(A)))) return rc;
     if (q == 0) {
       CHEMORA_CUDA(cudaMemcpyAsync(kn, acc, n * sizeof(double), cudaMemcpyDeviceToDevice, s));
       if ((rc = fill_ghosts(d, A->nv, kn, s))) return rc;  // read near the box edges
@@ -259,17 +272,20 @@ static int rk4_fine(chemora_amr* A, double dt, int step, cudaStream_t s) {
     StageParams p{};
     p.src = srcs[q]; p.yn = Y; p.acc = acc; p.dst = dsts[q];
     p.c1 = dt / 6.0; p.c2 = c2[q]; p.mode = q + 1;
-    if (A->mode == 0) {
+    unsigned int* counters = A->counters + step * A->counter_off[4] + A->counter_off[q];
+    if (A->mode == 0 && A->kind == CHEMORA_BSSN) {
+      if ((rc = launch_field_plan(A->plan[q], counters, A->err, 0, A->scf, p, A->work, s))) return rc;
+    } else if (A->mode == 0) {
       const int i0 = A->item_off[q], i1 = A->item_off[q + 1];
-      if ((rc = launch_batch_stage(A->nv, A->dev_pd + q * A->nbox, A->nbox, A->items + i0, i1 - i0,
-                                   A->counters + 4 * step + q, A->err, 0, A->scf, p, s)))
+      if ((rc = launch_batch_stage(A->dev_pd + q * A->nbox, A->nbox, A->items + i0, i1 - i0, counters, A->err, 0,
+                                   A->scf, p, s)))
         return rc;
     } else {
       for (int b = 0; b < A->nbox; ++b) {
         const PatchDesc& P = A->stage_pd[q * A->nbox + b];
         StageParams pb = p;
         pb.src += P.offset; pb.yn += P.offset; pb.acc += P.offset; pb.dst += P.offset;
-        if ((rc = launch_stage(A->kind, P.d, A->scf, pb, s))) return rc;
+        if ((rc = launch_stage(A->kind, P.d, A->scf, pb, s, 0, amr_work(A)))) return rc;
       }
     }
   }
@@ -358,13 +374,29 @@ static int create_amr(int kind, const int* nc, int nbox, const int* lo, const in
       P.d = Dims{X.rf[0] - 2 * g, X.rf[1] - 2 * g, X.rf[2] - 2 * g, g, sy, sz, sv};
       P.offset = X.fine_off;
       P.npts = (int64_t)P.d.nx * P.d.ny * P.d.nz;
-      append_items(items, b, P.npts);  // patch index within the stage's table
+      if (kind == CHEMORA_WAVE) append_items(items, b, P.npts);  // patch index within the stage's table
     }
     if (items.size() > (size_t)0x7fffffff) {
       delete A;
       return set_error(CHEMORA_EINVAL, "too many work items");
     }
     A->item_off[q + 1] = (int)items.size();
+  }
+  for (int q = 0; q <= 4; ++q) A->counter_off[q] = q;
+  if (kind == CHEMORA_BSSN) {
+    int rc = CHEMORA_OK;
+    A->work_points = field_work_points(A->dc);
+    for (int q = 0; q < 4 && !rc; ++q) {
+      const std::vector<PatchDesc> table(A->stage_pd.begin() + q * nbox, A->stage_pd.begin() + (q + 1) * nbox);
+      rc = field_plan_create(table, &A->plan[q]);
+      A->work_points = std::max(A->work_points, A->plan[q].points);
+      A->counter_off[q + 1] = A->counter_off[q] + (int)A->plan[q].chunks.size();
+    }
+    if (rc) {
+      for (FieldPlan& P : A->plan) field_plan_free(&P);
+      delete A;
+      return rc;
+    }
   }
   const size_t cs = (size_t)nv * A->dc.sv;
   const size_t total = cs * (1 + 3 + 3) + (size_t)foff * (1 + 3) + (size_t)woff;
@@ -373,15 +405,16 @@ static int create_amr(int kind, const int* nc, int nbox, const int* lo, const in
   if (e == cudaSuccess) e = cudaMemset(buf, 0, total * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&A->dev_boxes, nbox * sizeof(AmrBox));
   if (e == cudaSuccess) e = cudaMalloc(&A->dev_pd, 4 * nbox * sizeof(PatchDesc));
-  if (e == cudaSuccess) e = cudaMalloc(&A->items, items.size() * sizeof(WorkItem));
-  if (e == cudaSuccess) e = cudaMalloc(&A->counters, 8 * sizeof(unsigned int));
+  if (e == cudaSuccess && kind == CHEMORA_WAVE) e = cudaMalloc(&A->items, items.size() * sizeof(WorkItem));
+  if (e == cudaSuccess && kind == CHEMORA_BSSN) e = cudaMalloc(&A->work, field_work_bytes(A->work_points));
+  if (e == cudaSuccess) e = cudaMalloc(&A->counters, 2 * A->counter_off[4] * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMalloc(&A->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(A->err, 0, sizeof(int));
   if (e == cudaSuccess)
     e = cudaMemcpy(A->dev_boxes, A->boxes.data(), nbox * sizeof(AmrBox), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)
     e = cudaMemcpy(A->dev_pd, A->stage_pd.data(), 4 * nbox * sizeof(PatchDesc), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && kind == CHEMORA_WAVE)
     e = cudaMemcpy(A->items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -389,6 +422,8 @@ static int create_amr(int kind, const int* nc, int nbox, const int* lo, const in
     cudaFree(A->dev_boxes);
     cudaFree(A->dev_pd);
     cudaFree(A->items);
+    for (FieldPlan& P : A->plan) field_plan_free(&P);
+    cudaFree(A->work);
     cudaFree(A->counters);
     cudaFree(A->err);
     delete A;
@@ -458,9 +493,9 @@ int chemora_amr_step_mode(chemora_amr* A, double dt, int nsteps, int mode, void*
     if ((rc = rk4_coarse(A, A->coarse, dt, A->kn, s))) return rc;  // also k_n = RHS(y_n)
     StageParams p{};
     p.src = A->coarse; p.dst = A->kn1; p.mode = 0;
-    if ((rc = launch_stage(A->kind, A->dc, A->scc, p, s, A->coarse_variant))) return rc;
+    if ((rc = launch_stage(A->kind, A->dc, A->scc, p, s, A->coarse_variant, amr_work(A)))) return rc;
     if ((rc = fill_ghosts(A->dc, nv, A->kn1, s))) return rc;
-    if (mode == 0) CHEMORA_CUDA(cudaMemsetAsync(A->counters, 0, 8 * sizeof(unsigned int), s));
+    if (mode == 0) CHEMORA_CUDA(cudaMemsetAsync(A->counters, 0, 2 * A->counter_off[4] * sizeof(unsigned int), s));
     for (int m = 0; m < 2; ++m) {
       const double th = 0.5 * m;
       TimeLevels tl;
@@ -501,7 +536,7 @@ int chemora_amr_autotune(chemora_amr* A, int* variant, void* stream) {
   StageParams p{};  // a middle RK stage into the coarse scratch
   p.src = A->coarse; p.yn = A->coarse; p.acc = A->cscratch; p.dst = A->cscratch + cs; p.mode = 2;
   int best = A->coarse_variant;
-  if ((rc = autotune_stage(A->kind, A->dc, A->scc, p, s, &best, nullptr))) return rc;
+  if ((rc = autotune_stage(A->kind, A->dc, A->scc, p, s, &best, nullptr, amr_work(A)))) return rc;
   A->coarse_variant = best;
   if (variant) *variant = best;
   return CHEMORA_OK;
@@ -519,6 +554,8 @@ void destroy_amr(chemora_amr* A) {
   cudaFree(A->dev_boxes);
   cudaFree(A->dev_pd);
   cudaFree(A->items);
+  for (FieldPlan& P : A->plan) field_plan_free(&P);
+  cudaFree(A->work);
   cudaFree(A->counters);
   cudaFree(A->err);
   A->type = 0;

@@ -12,6 +12,8 @@ namespace chemora {
 
 constexpr int CTX = 32, CTY = 4;
 
+// The constraints in one kernel without a workspace (a stream that is being
+// captured, no memory left).
 __global__ void __launch_bounds__(CTX * CTY, 2) bssn_constraints_kernel(Dims d, Scalars sc,
                                                                         const double* __restrict__ st,
                                                                         double* __restrict__ out) {
@@ -90,8 +92,15 @@ int chemora_constraints(chemora_system* sys, const double* state, double* out, v
   if (sys->kind != CHEMORA_BSSN) return set_error(CHEMORA_EINVAL, "chemora_constraints needs a CHEMORA_BSSN system");
   if (!state || !out) return set_error(CHEMORA_EINVAL, "NULL state or out");
   const Dims& d = sys->grid->d;
+  cudaStream_t s = (cudaStream_t)stream;
+  const FieldWork work = take_field_work(sys, s);
+  if (work.w) {
+    const int rc = launch_constraints_split(d, sys->sc, state, out, work, s);
+    give_field_work(work, s);
+    return rc;
+  }
   dim3 grid((d.nx + CTX - 1) / CTX, (d.ny + CTY - 1) / CTY, d.nz);
-  bssn_constraints_kernel<<<grid, dim3(CTX, CTY), 0, (cudaStream_t)stream>>>(d, sys->sc, state, out);
+  bssn_constraints_kernel<<<grid, dim3(CTX, CTY), 0, s>>>(d, sys->sc, state, out);
   return launched("bssn_constraints_kernel");
 }
 

@@ -90,11 +90,11 @@ int validate_system(int kind, int nvars, int nghost, int order) {
 }
 
 int launch_stage(int kind, const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s,
-                 int variant) {
+                 int variant, const FieldWork& work) {
   switch (kind) {
     case CHEMORA_WAVE: return launch_wave_stage(d, sc, a, s, variant);
     case CHEMORA_WAVE_VARC: return launch_varc_stage(d, sc, a, s, variant);
-    case CHEMORA_BSSN: return launch_bssn_stage(d, sc, a, s, variant);
+    case CHEMORA_BSSN: return launch_bssn_stage(d, sc, a, s, variant, work);
     case CHEMORA_WAVE1: return launch_wave1_stage(d, sc, a, s, variant);
     default: return set_error(CHEMORA_EINVAL, "unknown system kind %d", kind);
   }
@@ -166,12 +166,63 @@ int prof_end(chemora_system* sys, cudaStream_t s, cudaEvent_t e0) {
   return CHEMORA_OK;
 }
 
-static int run_stage(chemora_system* sys, const StageParams& a, cudaStream_t s) {
+FieldWork system_field_work(chemora_system* sys, bool alloc) {
+  FieldWork w;
+  if (sys->kind != CHEMORA_BSSN || !bssn_shape_splits(sys->grid->d, sys->variant)) return w;
+  if (!sys->field_work && alloc) {
+    const int64_t points = field_work_points(sys->grid->d);
+    if (cudaMalloc(&sys->field_work, field_work_bytes(points)) == cudaSuccess) {
+      sys->field_points = points;
+    } else {
+      sys->field_work = nullptr;
+      cudaGetLastError();
+    }
+  }
+  w.w = sys->field_work;
+  w.points = sys->field_points;
+  return w;
+}
+
+FieldWork take_field_work(chemora_system* sys, cudaStream_t s) {
+  FieldWork w;
+  cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cst) != cudaSuccess || cst != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return w;
+  }
+  if (!sys->pool) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    if (cudaGetDevice(&props.location.id) != cudaSuccess || cudaMemPoolCreate(&sys->pool, &props) != cudaSuccess) {
+      sys->pool = nullptr;
+      cudaGetLastError();
+      return w;
+    }
+    uint64_t keep = UINT64_MAX;  // memory stays with the pool between calls, until the system is destroyed
+    cudaMemPoolSetAttribute(sys->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  }
+  const int64_t points = field_work_points(sys->grid->d);
+  void* p = nullptr;
+  if (cudaMallocFromPoolAsync(&p, field_work_bytes(points), sys->pool, s) != cudaSuccess) {
+    cudaGetLastError();
+    return w;
+  }
+  w.w = static_cast<double*>(p);
+  w.points = points;
+  return w;
+}
+
+void give_field_work(const FieldWork& w, cudaStream_t s) {
+  if (w.w) cudaFreeAsync(w.w, s);
+}
+
+static int run_stage(chemora_system* sys, const StageParams& a, const FieldWork& work, cudaStream_t s) {
   cudaEvent_t e0;
   int rc = prof_begin(sys, s, &e0);
   if (rc) return rc;
-  rc = jit_active(sys) ? jit_launch(sys, a, s)
-                       : launch_stage(sys->kind, sys->grid->d, sys->sc, a, s, sys->variant);
+  rc = jit_active(sys, work) ? jit_launch(sys, a, work, s)
+                             : launch_stage(sys->kind, sys->grid->d, sys->sc, a, s, sys->variant, work);
   if (rc) return rc;
   return prof_end(sys, s, e0);
 }
@@ -179,7 +230,7 @@ static int run_stage(chemora_system* sys, const StageParams& a, cudaStream_t s) 
 // One RK4 step: four fused stages, each preceded by a ghost fill of the
 // buffer its stencils read.  Buffers: Y (caller's state), A (accumulator),
 // Sa/Sb (stage states, alternating so no stage reads what it writes).
-static int rk4_one(chemora_system* sys, double* Y, double dt, cudaStream_t s) {
+static int rk4_one(chemora_system* sys, double* Y, double dt, const FieldWork& work, cudaStream_t s) {
   const Dims& d = sys->grid->d;
   const int nv = sys->nvars;
   const size_t n = (size_t)nv * sys->grid->fsize;
@@ -191,16 +242,16 @@ static int rk4_one(chemora_system* sys, double* Y, double dt, cudaStream_t s) {
   p.coef = sys->coef;
   if ((rc = fill_ghosts(d, nv, Y, s))) return rc;
   p.src = Y; p.yn = Y; p.acc = A; p.dst = Sa; p.c1 = 0.0; p.c2 = 0.5 * dt; p.mode = 1;
-  if ((rc = run_stage(sys, p, s))) return rc;
+  if ((rc = run_stage(sys, p, work, s))) return rc;
   if ((rc = fill_ghosts(d, nv, Sa, s))) return rc;
   p.src = Sa; p.dst = Sb; p.c2 = 0.5 * dt; p.mode = 2;
-  if ((rc = run_stage(sys, p, s))) return rc;
+  if ((rc = run_stage(sys, p, work, s))) return rc;
   if ((rc = fill_ghosts(d, nv, Sb, s))) return rc;
   p.src = Sb; p.dst = Sa; p.c2 = dt; p.mode = 3;
-  if ((rc = run_stage(sys, p, s))) return rc;
+  if ((rc = run_stage(sys, p, work, s))) return rc;
   if ((rc = fill_ghosts(d, nv, Sa, s))) return rc;
   p.src = Sa; p.dst = Y; p.c1 = dt / 6.0; p.c2 = 0.0; p.mode = 4;
-  return run_stage(sys, p, s);
+  return run_stage(sys, p, work, s);
 }
 
 void free_step_graph(chemora_system* sys) {
@@ -211,16 +262,26 @@ void free_step_graph(chemora_system* sys) {
   sys->graph_state = nullptr;
 }
 
+// One right-hand side or stage of a call that shares no scratch with others:
+// its derivative fields come from the system's pool, in stream order.
+static int run_single_stage(chemora_system* sys, const StageParams& p, cudaStream_t s) {
+  FieldWork work;
+  if (sys->kind == CHEMORA_BSSN && bssn_shape_splits(sys->grid->d, sys->variant)) work = take_field_work(sys, s);
+  const int rc = run_stage(sys, p, work, s);
+  give_field_work(work, s);
+  return rc;
+}
+
 // One RK4 step captured into a CUDA graph (on a private stream: the legacy
 // default stream cannot be captured), cached per (state, dt, variant).
-static int step_graph(chemora_system* sys, double* state, double dt) {
+static int step_graph(chemora_system* sys, double* state, double dt, const FieldWork& work) {
   if (sys->graph_exec && sys->graph_state == state && sys->graph_dt == dt &&
       sys->graph_variant == sys->variant)
     return CHEMORA_OK;
   free_step_graph(sys);
   if (!sys->cap_stream) CHEMORA_CUDA(cudaStreamCreateWithFlags(&sys->cap_stream, cudaStreamNonBlocking));
   CHEMORA_CUDA(cudaStreamBeginCapture(sys->cap_stream, cudaStreamCaptureModeThreadLocal));
-  int rc = rk4_one(sys, state, dt, sys->cap_stream);
+  int rc = rk4_one(sys, state, dt, work, sys->cap_stream);
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(sys->cap_stream, &g);
   if (rc) {
@@ -314,7 +375,7 @@ int chemora_rhs(chemora_system* sys, const double* state, double* rhs, void* str
     return set_error(CHEMORA_EINVAL, "variable-speed system without a speed (chemora_system_set_speed)");
   StageParams p{};
   p.src = state; p.dst = rhs; p.coef = sys->coef; p.mode = 0;
-  return run_stage(sys, p, (cudaStream_t)stream);
+  return run_single_stage(sys, p, (cudaStream_t)stream);
 }
 
 int chemora_rk4_step(chemora_system* sys, double* state, double dt, int nsteps, void* stream) {
@@ -332,14 +393,15 @@ int chemora_rk4_step(chemora_system* sys, double* state, double dt, int nsteps, 
   // The scalar wave's launch-chained path (small grids, chosen by the autotuner).
   if (sys->chain_on && chain_available(sys) && !sys->profile_on && cst == cudaStreamCaptureStatusNone)
     return chain_rk4(sys, state, dt, nsteps, s);
+  const FieldWork work = system_field_work(sys, cst == cudaStreamCaptureStatusNone);
   // Plain launches while profiling (events bracket each stage) or when the
   // caller is capturing the stream itself; otherwise replay a captured step.
   if (sys->profile_on || cst != cudaStreamCaptureStatusNone || nsteps < 2) {
     for (int n = 0; n < nsteps; ++n)
-      if ((rc = rk4_one(sys, state, dt, s))) return rc;
+      if ((rc = rk4_one(sys, state, dt, work, s))) return rc;
     return fill_ghosts(sys->grid->d, sys->nvars, state, s);
   }
-  if ((rc = step_graph(sys, state, dt))) return rc;
+  if ((rc = step_graph(sys, state, dt, work))) return rc;
   for (int n = 0; n < nsteps; ++n) {
     CHEMORA_CUDA(cudaGraphLaunch(sys->graph_exec, s));
     if ((rc = launched("cudaGraphLaunch(RK4 step)", 8))) return rc;
@@ -390,7 +452,7 @@ int chemora_stage(chemora_system* sys, int mode, const double* src, const double
   StageParams p{};
   p.src = src; p.yn = yn; p.acc = acc; p.dst = dst; p.coef = sys->coef;
   p.c1 = c1; p.c2 = c2; p.mode = mode;
-  return run_stage(sys, p, (cudaStream_t)stream);
+  return run_single_stage(sys, p, (cudaStream_t)stream);
 }
 
 int chemora_profile_enable(chemora_system* sys, int on) {

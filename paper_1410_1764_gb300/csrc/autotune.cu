@@ -36,7 +36,8 @@ static double model_cost(int kind, const Dims& d, const LaunchVariant& v, int sm
   // lane-sharing shapes need whole warps of x points
   if ((v.xshare == 1 || v.xshare == 2) && d.nx % v.tx != 0) return 1e300;
   const double nbx = ceil((double)d.nx / v.tx), nby = ceil((double)d.ny / v.ty);
-  const double blocks = nbx * nby * d.nz;
+  const bool split = kind == CHEMORA_BSSN && !v.xshare;  // blocks of consecutive points: no edge threads
+  const double blocks = split ? ceil((double)d.nx * d.ny * d.nz / (v.tx * v.ty)) : nbx * nby * d.nz;
   const double threads = blocks * v.tx * v.ty;  // launched, including idle edge threads
   // resident blocks per SM: register-bound for BSSN (255 regs), thread-bound otherwise
   const int per_block = v.tx * v.ty;
@@ -45,14 +46,15 @@ static double model_cost(int kind, const Dims& d, const LaunchVariant& v, int sm
   if (bps < 1) bps = 1;
   const double waves = blocks / (double)(sms * bps);
   const double quant = waves < 1.0 ? 1.0 / std::max(waves, 1e-9) : ceil(waves) / waves;
-  // x-sharing bodies issue about 11 % fewer FP64 instructions per point
+  // the split kernels issue less than half the direct body's FP64
+  // instructions, x-sharing bodies about 11 % fewer
   // (the marching wave shapes: fewer loads and integer operations)
-  const double work = v.xshare == 2 ? 0.81 : (v.xshare == 1 ? 0.89 : (v.xshare == 4 ? 0.8 : 1.0));
+  const double work = split ? 0.5 : (v.xshare == 2 ? 0.81 : (v.xshare == 1 ? 0.89 : (v.xshare == 4 ? 0.8 : 1.0)));
   return work * threads * (waves < 8.0 ? quant : 1.0 + 0.5 / waves);
 }
 
 int autotune_stage(int kind, const Dims& d, const Scalars& sc, const StageParams& p, cudaStream_t s, int* best,
-                   float* best_ms) {
+                   float* best_ms, const FieldWork& work) {
   int dev = 0, sms = 152;
   CHEMORA_CUDA(cudaGetDevice(&dev));
   CHEMORA_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -70,11 +72,11 @@ int autotune_stage(int kind, const Dims& d, const Scalars& sc, const StageParams
   float best_t = 1e30f;
   for (int v = 0; v < nv && rc == CHEMORA_OK; ++v) {
     if (cost[v] > 1.5 * cmin) continue;
-    if ((rc = launch_stage(kind, d, sc, p, s, v))) break;  // warm-up
+    if ((rc = launch_stage(kind, d, sc, p, s, v, work))) break;  // warm-up
     float tmin = 1e30f;
     for (int rep = 0; rep < 2; ++rep) {
       cudaEventRecord(e0, s);
-      if ((rc = launch_stage(kind, d, sc, p, s, v))) break;
+      if ((rc = launch_stage(kind, d, sc, p, s, v, work))) break;
       cudaEventRecord(e1, s);
       cudaEventSynchronize(e1);
       float ms = 0.f;
@@ -131,6 +133,13 @@ int chemora_system_opcount(chemora_system* sys, int64_t* fp64_instructions, int6
     if (flops) *flops = CHEMORA_OPS_BSSN_X_FLOPS;
     return CHEMORA_OK;
   }
+  if (sys->kind == CHEMORA_BSSN) {
+    // the split kernels: the algebra, and three fmas per mixed derivative
+    // (the other differences run on the integer units)
+    if (fp64_instructions) *fp64_instructions = CHEMORA_OPS_BSSN_ALG_INSTR + 3 * 33;
+    if (flops) *flops = CHEMORA_OPS_BSSN_FLOPS;
+    return CHEMORA_OK;
+  }
   return chemora_opcount(sys->kind, fp64_instructions, flops);
 }
 
@@ -166,7 +175,14 @@ int chemora_autotune(chemora_system* sys, double* state, int* variant, double* b
   p.coef = sys->coef; p.c1 = 0.0; p.c2 = 0.0; p.mode = 2;
   int best = sys->variant;
   float best_t = 1e30f;
-  rc = autotune_stage(sys->kind, d, sys->sc, p, s, &best, &best_t);
+  FieldWork work;  // every shape of a split right-hand side uses the same workspace
+  if (sys->kind == CHEMORA_BSSN) {
+    const int keep = sys->variant;
+    sys->variant = 0;
+    work = system_field_work(sys, true);
+    sys->variant = keep;
+  }
+  rc = autotune_stage(sys->kind, d, sys->sc, p, s, &best, &best_t, work);
   cudaEvent_t e0, e1;
   CHEMORA_CUDA(cudaEventCreate(&e0));
   CHEMORA_CUDA(cudaEventCreate(&e1));

@@ -12,15 +12,16 @@
 
 namespace chemora {
 
-template <int TX, int TY, int MINB>
-__global__ void __launch_bounds__(TX * TY, MINB) bssn_stage_kernel(Dims d, Scalars sc, StageParams a) {
-  bssn_direct_body<TX, TY>(d, sc, a);
+// The direct body in one kernel without a workspace: for callers that may not
+// allocate one (chemora_rk4_step_noalloc, a first call on a stream that is
+// being captured, no memory left).
+__global__ void __launch_bounds__(128, 2) bssn_stage_kernel(Dims d, Scalars sc, StageParams a) {
+  bssn_direct_body<32, 4>(d, sc, a);
 }
 
-template <int TX, int TY, int MINB>
-static int launch_bssn_variant(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s) {
-  dim3 grid((d.nx + TX - 1) / TX, (d.ny + TY - 1) / TY, d.nz);
-  bssn_stage_kernel<TX, TY, MINB><<<grid, dim3(TX, TY), 0, s>>>(d, sc, a);
+static int launch_bssn_direct(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s) {
+  dim3 grid((d.nx + 31) / 32, (d.ny + 3) / 4, d.nz);
+  bssn_stage_kernel<<<grid, dim3(32, 4), 0, s>>>(d, sc, a);
   return launched("bssn_stage_kernel");
 }
 
@@ -66,15 +67,16 @@ static int launch_bssn_xyvariant(const Dims& d, const Scalars& sc, const StagePa
 }
 
 // Launch shapes the autotuner chooses from (variant 0 is the default).
+// Sharing 0: the split kernels, tx x ty the algebra kernel's block.
 const LaunchVariant kBssnVariants[] = {
-    {32, 4, 2, launch_bssn_variant<32, 4, 2>},
-    {32, 2, 4, launch_bssn_variant<32, 2, 4>},
-    {64, 2, 2, launch_bssn_variant<64, 2, 2>},
-    {16, 8, 2, launch_bssn_variant<16, 8, 2>},
-    {32, 8, 1, launch_bssn_variant<32, 8, 1>},
-    {32, 4, 3, launch_bssn_variant<32, 4, 3>},
-    {32, 4, 4, launch_bssn_variant<32, 4, 4>},
-    {64, 2, 3, launch_bssn_variant<64, 2, 3>},
+    {32, 4, 3, launch_bssn_direct},
+    {32, 4, 2, launch_bssn_direct},
+    {32, 4, 4, launch_bssn_direct},
+    {32, 2, 5, launch_bssn_direct},
+    {32, 2, 8, launch_bssn_direct},
+    {64, 2, 3, launch_bssn_direct},
+    {64, 2, 2, launch_bssn_direct},
+    {64, 1, 5, launch_bssn_direct},
     {32, 2, 4, launch_bssn_xvariant<32, 2, 4>, 1},
     {32, 4, 2, launch_bssn_xvariant<32, 4, 2>, 1},
     {64, 2, 2, launch_bssn_xvariant<64, 2, 2>, 1},
@@ -92,12 +94,20 @@ const LaunchVariant kBssnVariants[] = {
 };
 const int kNumBssnVariants = sizeof(kBssnVariants) / sizeof(kBssnVariants[0]);
 
-int launch_bssn_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s, int variant) {
+static bool shape_shares(const Dims& d, const LaunchVariant& v) { return v.xshare && d.nx % v.tx == 0 && d.g >= 3; }
+
+bool bssn_shape_splits(const Dims& d, int variant) {
   if (variant < 0 || variant >= kNumBssnVariants) variant = 0;
-  const LaunchVariant& v = kBssnVariants[variant];
-  if (v.xshare && (d.nx % v.tx != 0 || d.g < 3))
-    return kBssnVariants[0].launch(d, sc, a, s);
-  return v.launch(d, sc, a, s);
+  return !shape_shares(d, kBssnVariants[variant]);
+}
+
+int launch_bssn_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s, int variant,
+                      const FieldWork& work) {
+  if (variant < 0 || variant >= kNumBssnVariants) variant = 0;
+  const LaunchVariant* v = &kBssnVariants[variant];
+  if (shape_shares(d, *v)) return v->launch(d, sc, a, s);
+  if (v->xshare) v = &kBssnVariants[0];
+  return work.w ? launch_bssn_split(d, sc, a, work, v->tx * v->ty, v->minb, s) : v->launch(d, sc, a, s);
 }
 
 }  // namespace chemora

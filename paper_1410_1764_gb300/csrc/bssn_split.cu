@@ -1,0 +1,358 @@
+// The split BSSN right-hand side (bssn_fields.cuh): the derivative-field
+// kernel, the algebra kernels for one grid and for work-lists over many
+// regions (batched patches, refined boxes), and the constraints.
+#include <algorithm>
+
+#include "internal.h"
+#include "bssn_algebra.cuh"
+#include "bssn_split.h"
+#include "generated/gen_bssn_constraints_alg.cuh"
+
+namespace chemora {
+
+// ---------------------------------------------------------------------------
+// derivative fields
+// ---------------------------------------------------------------------------
+constexpr int kTileThreads = 256, kTileRows = 32;
+constexpr int kRowMax = 448;  // doubles of a row array: (tw + 4) x (th + 4) for every tile shape tile_shape() returns
+
+// One block: one variable (blockIdx.y) on one tile of one plane, a point per
+// thread.  The mixed derivatives are first-derivative stencils of the
+// neighbours' first-derivative rows, in FP64 (3 fmas each: fewer cycles than
+// their 16 points in integers, on a pipe this kernel leaves idle); the rows
+// pass through shared memory, those past the tile's edge are computed by the
+// block again.
+__global__ void __launch_bounds__(kTileThreads)
+bssn_fields_kernel(const FieldRegion* __restrict__ regions, FieldRegion one_region, const int2* __restrict__ tiles,
+                   const double* __restrict__ base, double* __restrict__ work, double one, double eight) {
+  __shared__ double row_y[kRowMax], row_z[kRowMax];
+  int tile = blockIdx.x, region = 0;
+  if (tiles) {
+    const int2 q = tiles[blockIdx.x];
+    region = q.x;
+    tile = q.y;
+  }
+  const FieldRegion R = regions ? regions[region] : one_region;
+  const Dims& d = R.d;
+  const int v = blockIdx.y, ddi = dd_index(v);
+  const int txy = tile % (R.tnx * R.tny), k = tile / (R.tnx * R.tny);
+  const int x0 = (txy % R.tnx) * R.tw, y0 = (txy / R.tnx) * R.th;
+  const int w = min(R.tw, d.nx - x0), h = min(R.th, d.ny - y0);
+  const int t = threadIdx.x, ly = t / R.tw, lx = t - ly * R.tw;
+  const bool active = lx < w && ly < h;
+  const double* org = base + R.offset + v * d.sv + (int64_t)(k + d.g) * d.sz + (int64_t)(y0 + d.g) * d.sy + x0 + d.g;
+  double* out = nullptr;
+  if (active)
+    out = work + field_base(R.w0 + ((int64_t)k * d.ny + y0 + ly) * d.nx + x0 + lx);
+  double d1[3], d2[3], ko;
+  Star3 s;
+  if (ddi < 0) {
+    if (!active) return;
+    s.load(org + (int64_t)ly * d.sy + lx, d.sy, d.sz);
+    star3_differences<false>(s, d1, d2, ko);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) out[(kFieldD1 + 3 * v + a) * kFieldBlock] = d1[a];
+    out[(kFieldKo + v) * kFieldBlock] = ko;
+    return;
+  }
+  const int pw = R.tw + 4;  // row pitch; the tile's point (0, 0) sits at [2][2] of row_z, [0][2] of row_y
+  if (active) {
+    s.load(org + (int64_t)ly * d.sy + lx, d.sy, d.sz);
+    star3_differences<true>(s, d1, d2, ko);
+    row_y[ly * pw + lx + 2] = d1[1];
+    row_z[(ly + 2) * pw + lx + 2] = d1[2];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      out[(kFieldD1 + 3 * v + a) * kFieldBlock] = d1[a];
+      out[(kFieldD2 + 6 * ddi + a) * kFieldBlock] = d2[a];
+    }
+    out[(kFieldKo + v) * kFieldBlock] = ko;
+  }
+  // rows past the edge: columns -2, -1, w, w+1 (y and z rows), then rows
+  // -2, -1, h, h+1 (z rows)
+  for (int q = t; q < 4 * h + 4 * h + 4 * w; q += kTileThreads) {
+    if (q < 8 * h) {
+      const int r = q % h, e = (q / h) & 3, x = e < 2 ? e - 2 : w + e - 2;
+      const double* p = org + (int64_t)r * d.sy + x;
+      if (q < 4 * h)
+        row_y[r * pw + x + 2] = d1_row_fp64(p, d.sy, one, eight);
+      else
+        row_z[(r + 2) * pw + x + 2] = d1_row_fp64(p, d.sz, one, eight);
+    } else {
+      const int r = (q - 8 * h) / w, x = (q - 8 * h) % w, y = r < 2 ? r - 2 : h + r - 2;
+      row_z[(y + 2) * pw + x + 2] = d1_row_fp64(org + (int64_t)y * d.sy + x, d.sz, one, eight);
+    }
+  }
+  __syncthreads();
+  if (!active) return;
+  auto mixed = [&](const double* r, int st) {
+    const double q1 = fma(r[-st], -one, r[st]), q2 = fma(r[-2 * st], -one, r[2 * st]);
+    return fma(eight, q1, -q2);
+  };
+  const double* ry = row_y + ly * pw + lx + 2;
+  const double* rz = row_z + (ly + 2) * pw + lx + 2;
+  out[(kFieldD2 + 6 * ddi + 3) * kFieldBlock] = mixed(ry, 1);
+  out[(kFieldD2 + 6 * ddi + 4) * kFieldBlock] = mixed(rz, 1);
+  out[(kFieldD2 + 6 * ddi + 5) * kFieldBlock] = mixed(rz, pw);
+}
+
+// Tiles of nearly equal shape, at most 32 wide, at most 256 points, so that
+// ragged grids leave few threads idle.
+static void tile_shape(FieldRegion* R) {
+  const Dims& d = R->d;
+  R->tnx = (d.nx + 31) / 32;
+  R->tw = (d.nx + R->tnx - 1) / R->tnx;
+  const int rows = std::min(kTileRows, kTileThreads / R->tw);
+  R->tny = (d.ny + rows - 1) / rows;
+  R->th = (d.ny + R->tny - 1) / R->tny;
+}
+
+FieldRegion field_region(const Dims& d, int64_t offset, int64_t w0) {
+  FieldRegion R;
+  R.d = d;
+  R.offset = offset;
+  R.npts = (int64_t)d.nx * d.ny * d.nz;
+  R.w0 = w0;
+  tile_shape(&R);
+  return R;
+}
+
+// Planes of d that fit in `cap` workspace points (at least one).
+static int chunk_planes(const Dims& d, int64_t cap) {
+  const int64_t plane = (int64_t)d.nx * d.ny;
+  return (int)std::min<int64_t>(d.nz, std::max<int64_t>(1, cap / plane));
+}
+
+int64_t field_work_points(const Dims& d) {
+  return (int64_t)d.nx * d.ny * chunk_planes(d, kFieldWorkPoints);
+}
+
+int field_chunk_planes(const Dims& d, const FieldWork& work) {
+  const int planes = chunk_planes(d, work.points);
+  return (int64_t)d.nx * d.ny * planes <= work.points ? planes : 0;
+}
+
+size_t field_work_bytes(int64_t points) {
+  return (size_t)((points + kFieldBlock - 1) / kFieldBlock) * kFields * kFieldBlock * sizeof(double);
+}
+
+int launch_fields(const FieldRegion& R, int nvars, const double* src, double* work, const Scalars& sc,
+                         cudaStream_t s) {
+  const dim3 grid((unsigned)(R.tnx * R.tny * R.d.nz), (unsigned)nvars);
+  bssn_fields_kernel<<<grid, kTileThreads, 0, s>>>(nullptr, R, nullptr, src, work, sc.k[CHEMORA_K_ONE],
+                                                   sc.k[CHEMORA_K_EIGHT]);
+  return launched("bssn_fields_kernel");
+}
+
+// ---------------------------------------------------------------------------
+// algebra, one region
+// ---------------------------------------------------------------------------
+// MODE: the RK stage mode, compiled in (modes 2 and 3 are the same update).
+template <int BLK, int MINB, int MODE>
+__global__ void __launch_bounds__(BLK, MINB)
+bssn_algebra_kernel(FieldRegion R, Scalars sc, StageParams a_in, const double* __restrict__ work) {
+  StageParams a = a_in;
+  a.mode = MODE;
+  bssn_algebra<BLK>(R.d, R, sc, a, work);
+}
+
+template <int BLK, int MINB, int MODE>
+static void launch_algebra_mode(const FieldRegion& R, const Scalars& sc, const StageParams& a, const double* work,
+                                cudaStream_t s) {
+  bssn_algebra_kernel<BLK, MINB, MODE><<<(unsigned)((R.npts + BLK - 1) / BLK), BLK, 0, s>>>(R, sc, a, work);
+}
+
+template <int BLK, int MINB>
+static int launch_algebra(const FieldRegion& R, const Scalars& sc, const StageParams& a, const double* work,
+                          cudaStream_t s) {
+  switch (a.mode) {
+    case 0: launch_algebra_mode<BLK, MINB, 0>(R, sc, a, work, s); break;
+    case 1: launch_algebra_mode<BLK, MINB, 1>(R, sc, a, work, s); break;
+    case 2:
+    case 3: launch_algebra_mode<BLK, MINB, 2>(R, sc, a, work, s); break;
+    default: launch_algebra_mode<BLK, MINB, 4>(R, sc, a, work, s); break;
+  }
+  return launched("bssn_algebra_kernel");
+}
+
+int launch_bssn_split(const Dims& d, const Scalars& sc, const StageParams& a, const FieldWork& work, int block,
+                      int minb, cudaStream_t s) {
+  return for_field_chunks(d, sc, a.src, 24, work, s, [&](const FieldRegion& R) {
+    if (block == 64) return minb >= 8 ? launch_algebra<64, 8>(R, sc, a, work.w, s) : launch_algebra<64, 5>(R, sc, a, work.w, s);
+    if (minb == 2) return launch_algebra<128, 2>(R, sc, a, work.w, s);
+    return minb == 4 ? launch_algebra<128, 4>(R, sc, a, work.w, s) : launch_algebra<128, 3>(R, sc, a, work.w, s);
+  });
+}
+
+// ---------------------------------------------------------------------------
+// algebra over many regions
+// ---------------------------------------------------------------------------
+// Persistent blocks pull work items -- 128 consecutive interior points of one
+// region -- from the list with an atomic counter, so uneven regions keep every
+// SM busy.  The loop is bounded by the item count (the counter only grows), an
+// item naming a region outside the table sets bit 0 of the error word instead
+// of touching memory, and a block past the time limit takes no more items and
+// sets bit 1.
+template <int MODE>
+__global__ void __launch_bounds__(kItemPoints, 3)
+batch_algebra_kernel(const FieldRegion* __restrict__ regions, int nregions, const WorkItem* __restrict__ items,
+                     int nitems, unsigned int* counter, int* err, long long limit, Scalars sc, StageParams a_in,
+                     const double* __restrict__ work) {
+  StageParams a = a_in;
+  a.mode = MODE;
+  __shared__ unsigned int s_item;
+  const long long t0 = clock64();
+  for (int iter = 0; iter <= nitems; ++iter) {
+    if (threadIdx.x == 0) {
+      if (limit > 0 && clock64() - t0 > limit) {
+        atomicOr(err, 2);
+        s_item = (unsigned)nitems;
+      } else {
+        s_item = atomicAdd(counter, 1u);
+      }
+    }
+    __syncthreads();
+    const unsigned int it = s_item;
+    __syncthreads();
+    if (it >= (unsigned)nitems) break;
+    const WorkItem q = items[it];
+    if (q.patch < 0 || q.patch >= nregions) {
+      if (threadIdx.x == 0) atomicOr(err, 1);
+      continue;
+    }
+    const FieldRegion& R = regions[q.patch];
+    const int64_t lin = (int64_t)q.start + threadIdx.x;
+    if (q.start < 0 || lin >= R.npts) continue;
+    bssn_algebra_point(R.d, R, lin, sc, a, work);
+  }
+}
+
+int field_plan_create(const std::vector<PatchDesc>& patches, FieldPlan* plan) {
+  // chunks of nearly equal size, each at most kFieldWorkPoints points (or one plane)
+  int64_t total = 0;
+  for (const PatchDesc& P : patches) total += P.npts;
+  const int64_t nchunks = (total + kFieldWorkPoints - 1) / kFieldWorkPoints;
+  const int64_t target = std::max<int64_t>(1, (total + nchunks - 1) / std::max<int64_t>(1, nchunks));
+  std::vector<FieldRegion> regions;
+  std::vector<WorkItem> items;
+  std::vector<int2> tiles;
+  plan->chunks.clear();
+  plan->points = 0;
+  int64_t cur = 0;
+  FieldPlan::Chunk ch{0, 0, 0, 0};
+  auto close = [&]() {
+    if (cur == 0) return;
+    ch.item1 = (int)items.size();
+    ch.tile1 = (int)tiles.size();
+    plan->chunks.push_back(ch);
+    plan->points = std::max(plan->points, cur);
+    ch = FieldPlan::Chunk{ch.item1, 0, ch.tile1, 0};
+    cur = 0;
+  };
+  for (const PatchDesc& P : patches) {
+    const int64_t plane = (int64_t)P.d.nx * P.d.ny;
+    for (int k0 = 0; k0 < P.d.nz;) {
+      if (cur > 0 && cur + plane > target) close();
+      Dims dk = P.d;
+      dk.nz = (int)std::min<int64_t>(P.d.nz - k0, std::max<int64_t>(1, (target - cur) / plane));
+      const FieldRegion R = field_region(dk, P.offset + (int64_t)k0 * P.d.sz, cur);
+      const int q = (int)regions.size();
+      regions.push_back(R);
+      append_items(items, q, R.npts);
+      const int64_t nt = (int64_t)R.tnx * R.tny * dk.nz;
+      for (int64_t t = 0; t < nt; ++t) tiles.push_back(int2{q, (int)t});
+      cur += R.npts;
+      k0 += dk.nz;
+    }
+  }
+  close();
+  if (items.size() > (size_t)0x7fffffff || tiles.size() > (size_t)0x7fffffff)
+    return set_error(CHEMORA_EINVAL, "too many work items");
+  plan->nregions = (int)regions.size();
+  plan->nitems = (int)items.size();
+  cudaError_t e = cudaMalloc(&plan->regions, regions.size() * sizeof(FieldRegion));
+  if (e == cudaSuccess) e = cudaMalloc(&plan->items, items.size() * sizeof(WorkItem));
+  if (e == cudaSuccess) e = cudaMalloc(&plan->tiles, tiles.size() * sizeof(int2));
+  if (e == cudaSuccess)
+    e = cudaMemcpy(plan->regions, regions.data(), regions.size() * sizeof(FieldRegion), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(plan->items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess)
+    e = cudaMemcpy(plan->tiles, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    field_plan_free(plan);
+    return set_error(e == cudaErrorMemoryAllocation ? CHEMORA_ENOMEM : CHEMORA_ECUDA, "work-list storage: %s",
+                     cudaGetErrorString(e));
+  }
+  return CHEMORA_OK;
+}
+
+void field_plan_free(FieldPlan* plan) {
+  cudaFree(plan->regions);
+  cudaFree(plan->items);
+  cudaFree(plan->tiles);
+  plan->regions = nullptr;
+  plan->items = nullptr;
+  plan->tiles = nullptr;
+}
+
+static int persistent_algebra_blocks() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+    sms = 152;
+  return 3 * sms;
+}
+
+int launch_field_plan(const FieldPlan& plan, unsigned int* counters, int* err, long long limit, const Scalars& sc,
+                      const StageParams& p, double* work, cudaStream_t s) {
+  const int blocks = persistent_algebra_blocks();
+  int rc;
+  for (size_t q = 0; q < plan.chunks.size(); ++q) {
+    const FieldPlan::Chunk& c = plan.chunks[q];
+    bssn_fields_kernel<<<dim3((unsigned)(c.tile1 - c.tile0), 24), kTileThreads, 0, s>>>(
+        plan.regions, FieldRegion{}, plan.tiles + c.tile0, p.src, work, sc.k[CHEMORA_K_ONE], sc.k[CHEMORA_K_EIGHT]);
+    if ((rc = launched("bssn_fields_kernel"))) return rc;
+    const WorkItem* items = plan.items + c.item0;
+    const int n = c.item1 - c.item0;
+    switch (p.mode) {
+#define CHEMORA_BATCH_ALGEBRA(MODE)                                                                             \
+  batch_algebra_kernel<MODE><<<blocks, kItemPoints, 0, s>>>(plan.regions, plan.nregions, items, n, counters + q, \
+                                                            err, limit, sc, p, work)
+      case 1: CHEMORA_BATCH_ALGEBRA(1); break;
+      case 2:
+      case 3: CHEMORA_BATCH_ALGEBRA(2); break;
+      case 4: CHEMORA_BATCH_ALGEBRA(4); break;
+      default: return set_error(CHEMORA_EINVAL, "batched stage mode %d", p.mode);
+#undef CHEMORA_BATCH_ALGEBRA
+    }
+    if ((rc = launched("batch_algebra_kernel"))) return rc;
+  }
+  return CHEMORA_OK;
+}
+
+// ---------------------------------------------------------------------------
+// constraints
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(128, 3)
+bssn_constraints_algebra_kernel(FieldRegion R, Scalars sc, const double* __restrict__ st, double* __restrict__ out,
+                                const double* __restrict__ work) {
+  const int64_t lin = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  if (lin >= R.npts) return;
+  const int64_t c = R.offset + region_point(R.d, lin);
+  const FieldLoader ld{st + c, R.d.sv, work + field_base(R.w0 + lin)};
+  auto o = [&](int v, double x) { out[c + v * R.d.sv] = x; };
+  chemora_bssn_constraints_alg_point(ld, sc, o);
+}
+
+int launch_constraints_split(const Dims& d, const Scalars& sc, const double* state, double* out,
+                             const FieldWork& work, cudaStream_t s) {
+  // the constraints read no derivative of the lapse, the shift and B
+  return for_field_chunks(d, sc, state, 17, work, s, [&](const FieldRegion& R) {
+    bssn_constraints_algebra_kernel<<<(unsigned)((R.npts + 127) / 128), 128, 0, s>>>(R, sc, state, out, work.w);
+    return launched("bssn_constraints_algebra_kernel");
+  });
+}
+
+}  // namespace chemora

@@ -62,6 +62,12 @@ struct chemora_system {
   double* coef;
   // device copy of a host state for chemora_rk4_step_host (library-owned)
   double* dev_state;
+  // derivative fields of the split BSSN right-hand side: a workspace for the
+  // RK4 driver (allocated on first use), and a pool for calls that may run on
+  // several streams at once (chemora_rhs, chemora_stage, chemora_constraints)
+  double* field_work;
+  int64_t field_points;
+  cudaMemPool_t pool;
   // launch shape chosen by the autotuner (index into the kind's variants)
   int variant;
   // CUDA graph of one RK4 step (captured on cap_stream, replayed on the
@@ -97,14 +103,37 @@ int effective_order(int kind, const chemora_params& p);
 int fill_ghosts(const Dims& d, int nvars, double* state, cudaStream_t s);
 int fill_ghosts_axes(const Dims& d, int nvars, double* state, int mask, cudaStream_t s);
 
+// Workspace of the split BSSN right-hand side (bssn_split.cu): derivative
+// fields of up to `points` grid points; w NULL: none, the direct kernel runs.
+struct FieldWork {
+  double* w = nullptr;
+  int64_t points = 0;
+};
+constexpr int64_t kFieldWorkPoints = 1 << 20;  // points whose fields are held at once (1.36 GB)
+int64_t field_work_points(const Dims& d);      // workspace points a stage on d uses
+size_t field_work_bytes(int64_t points);
+int launch_bssn_split(const Dims& d, const Scalars& sc, const StageParams& a, const FieldWork& work, int block,
+                      int minb, cudaStream_t s);
+int launch_constraints_split(const Dims& d, const Scalars& sc, const double* state, double* out,
+                             const FieldWork& work, cudaStream_t s);
+// Does launch shape `variant` run the split kernels on d when it has a workspace?
+bool bssn_shape_splits(const Dims& d, int variant);
+// The RK4 driver's workspace (no workspace if there is no memory for one or
+// alloc is false and there is none yet), and one taken from and given back to
+// the system's pool in stream order.
+FieldWork system_field_work(chemora_system* sys, bool alloc);
+FieldWork take_field_work(chemora_system* sys, cudaStream_t s);
+void give_field_work(const FieldWork& w, cudaStream_t s);
+
 int launch_stage(int kind, const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s,
-                 int variant = 0);
+                 int variant = 0, const FieldWork& work = FieldWork());
 int launch_wave_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s, int variant);
 int launch_varc_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s, int variant);
 // G_d = D_d s (4th-order centred) on the interior of 3 grid functions at G,
 // svar apart; s with valid ghosts.
 int launch_varc_grad(const Dims& d, double i12h, const double* s, double* G, cudaStream_t st);
-int launch_bssn_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s, int variant);
+int launch_bssn_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s, int variant,
+                      const FieldWork& work);
 int launch_wave_order_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s,
                             int variant);
 int launch_wave1_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s, int variant);
@@ -134,7 +163,7 @@ const LaunchVariant* variant_info(int kind, int v);
 // arguments p, written into p.acc / p.dst) and return the fastest in *best
 // (left alone if none ran) and its time.  Synchronous.
 int autotune_stage(int kind, const Dims& d, const Scalars& sc, const StageParams& p, cudaStream_t s, int* best,
-                   float* best_ms);
+                   float* best_ms, const FieldWork& work = FieldWork());
 
 // timing helpers for systems with profiling enabled
 int prof_begin(chemora_system* sys, cudaStream_t s, cudaEvent_t* e0);
@@ -149,8 +178,8 @@ int chain_rk4(chemora_system* sys, double* state, double dt, int nsteps, cudaStr
 void chain_free(chemora_system* sys);
 
 // run-time specialisation (jit.cu)
-bool jit_active(const chemora_system* sys);
-int jit_launch(chemora_system* sys, const StageParams& a, cudaStream_t s);
+bool jit_active(const chemora_system* sys, const FieldWork& work);
+int jit_launch(chemora_system* sys, const StageParams& a, const FieldWork& work, cudaStream_t s);
 void jit_free(chemora_system* sys);
 
 // Batched work-lists (patches.cu): a table of patches (grids inside one
@@ -169,15 +198,35 @@ struct WorkItem {
 constexpr int kItemPoints = 128;
 // Append the work items of patch q (npts interior points) to `items`.
 void append_items(std::vector<WorkItem>& items, int q, int64_t npts);
-// One persistent batched stage launch of a system of nvars variables (24:
-// BSSN, 2: wave) over the device work-list `items` of the device patch table
-// `pd`; `counter` (device, zero before the launch) hands out the items; bit
+// One persistent batched stage launch of the scalar wave over the device
+// work-list `items` of the device patch table `pd`; `counter` (device, zero before the launch) hands out the items; bit
 // 0 of *err is set for an item naming a patch outside the table, bit 1 when
 // a block passed `limit` SM cycles (0: no limit).  src, yn, acc and dst of
 // `p` are the storage bases; each patch's offset is added per item.
-int launch_batch_stage(int nvars, const PatchDesc* pd, int npatch, const WorkItem* items, int nitems,
+int launch_batch_stage(const PatchDesc* pd, int npatch, const WorkItem* items, int nitems,
                        unsigned int* counter, int* err, long long limit, const Scalars& sc,
                        const StageParams& p, cudaStream_t s);
+
+// The split BSSN right-hand side over many regions: their z ranges, grouped
+// into chunks whose derivative fields fit in one workspace.  Per chunk one
+// field launch and one persistent algebra launch over a work-list.
+struct FieldRegion;
+struct FieldPlan {
+  struct Chunk {
+    int item0, item1, tile0, tile1;
+  };
+  std::vector<Chunk> chunks;
+  int nregions = 0, nitems = 0;
+  int64_t points = 0;  // workspace points
+  FieldRegion* regions = nullptr;  // device
+  WorkItem* items = nullptr;       // device: region and first point
+  int2* tiles = nullptr;           // device: region and tile
+};
+int field_plan_create(const std::vector<PatchDesc>& patches, FieldPlan* plan);
+void field_plan_free(FieldPlan* plan);
+// One stage; counters: one per chunk, zero before the launch.
+int launch_field_plan(const FieldPlan& plan, unsigned int* counters, int* err, long long limit, const Scalars& sc,
+                      const StageParams& p, double* work, cudaStream_t s);
 
 inline bool is_handle(const void* h, uint32_t t) {
   return h != nullptr && *reinterpret_cast<const uint32_t*>(h) == t;

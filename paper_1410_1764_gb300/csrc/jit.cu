@@ -31,6 +31,7 @@
 #include <thread>
 #include <vector>
 
+#include "bssn_split.h"
 #include "internal.h"
 
 namespace chemora {
@@ -118,22 +119,23 @@ std::string hexf(double v) {
 // The launch shape's body and geometry, after the same fall-backs the
 // ahead-of-time dispatch applies.
 struct Shape {
-  const char* body;  // device function in bssn_kernels.cuh
+  const char* body;  // device function in bssn_kernels.cuh (xshare 1, 2)
   int tx, ty, minb;
-  int xshare;        // 0 direct, 1 x lanes, 2 x lanes + y through shared memory
+  int xshare;        // 0 split (the algebra kernel), 1 x lanes, 2 x lanes + y through shared memory
 };
 
 Shape shape_of(const Dims& d, int variant) {
   const LaunchVariant* v = variant_info(CHEMORA_BSSN, variant);
   if (!v || (v->xshare && (d.nx % v->tx != 0 || d.g < 3)))
     v = variant_info(CHEMORA_BSSN, 0);
-  static const char* const bodies[] = {"bssn_direct_body", "bssn_x_body", "bssn_xy_body"};
+  static const char* const bodies[] = {"bssn_algebra", "bssn_x_body", "bssn_xy_body"};
   return Shape{bodies[v->xshare], v->tx, v->ty, v->minb, v->xshare};
 }
 
 std::string kernel_source(const Dims& d, const Scalars& sc, const Shape& sh, int mode) {
   char b[4096];
-  std::string src = "// run-time specialised BSSN stage kernel\n#include \"bssn_kernels.cuh\"\n";
+  std::string src = "// run-time specialised BSSN stage kernel\n";
+  src += sh.xshare ? "#include \"bssn_kernels.cuh\"\n" : "#include \"bssn_algebra.cuh\"\n";
   snprintf(b, sizeof b,
            "struct JitScalars {\n"
            "  static constexpr double i12h = %s, i12h2 = %s, i144h2 = %s, ko_scale = %s, eta = %s;\n"
@@ -145,6 +147,23 @@ std::string kernel_source(const Dims& d, const Scalars& sc, const Shape& sh, int
            hexf(sc.ko_scale).c_str(), hexf(sc.eta).c_str(), hexf(sc.ih).c_str(), hexf(sc.ih2).c_str(),
            sc.slicing, sc.shift, sc.order);
   src += b;
+  if (sh.xshare == 0) {
+    snprintf(b, sizeof b,
+             "extern \"C\" __global__ void __launch_bounds__(%d, %d)\n"
+             "chemora_jit_stage(chemora::StageParams a0, chemora::KTable kt, chemora::FieldSlab R,\n"
+             "                  const double* __restrict__ work) {\n"
+             "  const chemora::Dims d = {%d, %d, %d, %d, %lldLL, %lldLL, %lldLL};\n"
+             "  chemora::StageParams a = a0;\n"
+             "  a.mode = %d;\n"
+             "  JitScalars sc;\n"
+             "#pragma unroll\n"
+             "  for (int q = 0; q < CHEMORA_NK; ++q) sc.k[q] = kt.k[q];\n"
+             "  chemora::bssn_algebra<%d>(d, R, sc, a, work);\n}\n",
+             sh.tx * sh.ty, sh.minb, d.nx, d.ny, d.nz, d.g, (long long)d.sy, (long long)d.sz, (long long)d.sv, mode,
+             sh.tx * sh.ty);
+    src += b;
+    return src;
+  }
   snprintf(b, sizeof b,
            "extern \"C\" __global__ void __launch_bounds__(%d, %d)\n"
            "chemora_jit_stage(chemora::StageParams a0, chemora::KTable kt) {\n"
@@ -163,7 +182,7 @@ std::string kernel_source(const Dims& d, const Scalars& sc, const Shape& sh, int
              "  chemora::%s<%d, %d>(d, sc, a, smem);\n}\n",
              sh.body, sh.tx, sh.ty);
   } else {
-    snprintf(b, sizeof b, "  chemora::%s<%d, %d>(d, sc, a);\n}\n", sh.body, sh.tx, sh.ty);
+    snprintf(b, sizeof b, "  chemora::%s<%d, %d>(d, sc, a);\n}\n", sh.body, sh.tx, sh.ty);  // x lanes
   }
   src += b;
   return src;
@@ -279,6 +298,7 @@ void compile_one(const Nvrtc& n, const std::vector<std::string>& opts, CompileJo
 
 struct JitModule {
   int variant = -1;
+  bool split = false;  // specialised algebra kernels: they need a field workspace
   dim3 grid, block;
   unsigned smem = 0;
   cudaLibrary_t lib[kModes] = {};
@@ -296,16 +316,27 @@ void jit_free(chemora_system* sys) {
   sys->jit_on = 0;
 }
 
-bool jit_active(const chemora_system* sys) {
-  return sys->jit_on && sys->jit && sys->jit->variant == sys->variant;
+bool jit_active(const chemora_system* sys, const FieldWork& work) {
+  return sys->jit_on && sys->jit && sys->jit->variant == sys->variant && (work.w || !sys->jit->split);
 }
 
-int jit_launch(chemora_system* sys, const StageParams& a, cudaStream_t s) {
+int jit_launch(chemora_system* sys, const StageParams& a, const FieldWork& work, cudaStream_t s) {
   const JitModule* J = sys->jit;
   if (a.mode < 0 || a.mode >= kModes) return set_error(CHEMORA_EINVAL, "stage mode %d", a.mode);
   StageParams p = a;
   KTable kt;
   for (int i = 0; i < CHEMORA_NK; ++i) kt.k[i] = sys->sc.k[i];
+  if (J->split) {
+    const unsigned block = J->block.x;
+    return for_field_chunks(sys->grid->d, sys->sc, a.src, 24, work, s, [&](const FieldRegion& R) -> int {
+      FieldSlab slab{R.offset, R.npts, R.w0};
+      const double* w = work.w;
+      void* args[] = {&p, &kt, &slab, &w};
+      CHEMORA_CUDA(cudaLaunchKernel((const void*)J->k[a.mode], dim3((unsigned)((R.npts + block - 1) / block)),
+                                    J->block, args, 0, s));
+      return launched("chemora_jit_stage");
+    });
+  }
   void* args[] = {&p, &kt};
   CHEMORA_CUDA(cudaLaunchKernel((const void*)J->k[a.mode], J->grid, J->block, args, J->smem, s));
   return launched("chemora_jit_stage");
@@ -361,9 +392,10 @@ static int jit_build(chemora_system* sys, const char* cache_dir) {
   JitModule* J = new (std::nothrow) JitModule();
   if (!J) return set_error(CHEMORA_ENOMEM, "host allocation");
   J->variant = sys->variant;
-  J->block = dim3(sh.tx, sh.ty, 1);
+  J->split = sh.xshare == 0;
+  J->block = J->split ? dim3(sh.tx * sh.ty) : dim3(sh.tx, sh.ty, 1);
   // the grids of the ahead-of-time launchers in bssn.cu
-  J->grid = dim3(sh.xshare == 0 ? (d.nx + sh.tx - 1) / sh.tx : d.nx / sh.tx, (d.ny + sh.ty - 1) / sh.ty, d.nz);
+  J->grid = dim3(d.nx / sh.tx, (d.ny + sh.ty - 1) / sh.ty, d.nz);
   J->smem = sh.xshare == 2 ? bssn_xy_smem_bytes(sh.tx, sh.ty) : 0u;
   J->compile_s = secs;
   J->cached = 1;

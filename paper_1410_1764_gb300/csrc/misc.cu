@@ -114,6 +114,8 @@ void chemora_destroy(void* handle) {
     chain_free(s);
     if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
     if (s->scratch) cudaFree(s->scratch);
+    if (s->field_work) cudaFree(s->field_work);
+    if (s->pool) cudaMemPoolDestroy(s->pool);
     if (s->coef) cudaFree(s->coef);
     if (s->dev_state) cudaFree(s->dev_state);
     for (cudaEvent_t e : s->ev_pool) cudaEventDestroy(e);

@@ -2,13 +2,15 @@
 // patches of an AMR or multi-block driver, Sec. 4) advanced together.
 //
 // mode 0 (batched): per RK stage one ghost-fill launch over every patch and
-// one persistent stage launch.  The persistent kernel's blocks pull work
-// items -- 128 consecutive interior points of one patch, x fastest -- from a
-// work-list with an atomic counter, so uneven patches keep every SM busy and
-// no thread idles on a partial x-tile.  The loop is bounded by the item count (the
-// counter only grows), and an item naming a patch outside the table sets a
-// device error word instead of touching memory.  The whole RK4 step is
-// captured once in a CUDA graph and replayed.
+// one persistent stage launch (BSSN: per chunk of the derivative workspace
+// one field launch and one persistent algebra launch, bssn_split.cu).  The
+// persistent kernel's blocks pull work items -- 128 consecutive interior
+// points of one patch, x fastest -- from a work-list with an atomic counter,
+// so uneven patches keep every SM busy and no thread idles on a partial
+// x-tile.  The loop is bounded by the item count (the counter only grows),
+// and an item naming a patch outside the table sets a device error word
+// instead of touching memory.  The whole RK4 step is captured once in a CUDA
+// graph and replayed.
 // mode 1 (per patch): the single-grid kernels launched patch by patch, stage
 // by stage (the schedule a driver without batching would use).
 #include <math.h>
@@ -19,7 +21,6 @@
 
 #include "internal.h"
 #include "stage.cuh"
-#include "generated/gen_bssn.cuh"
 #include "wave_point.cuh"
 
 struct chemora_batch {
@@ -34,7 +35,10 @@ struct chemora_batch {
   chemora::PatchDesc* dev_pd;
   chemora::WorkItem* items;
   int nitems;
-  unsigned int* counters;  // one per stage of a step
+  chemora::FieldPlan plan;  // BSSN: regions, work-list and chunks
+  double* work;             // BSSN: derivative fields of a chunk
+  int ncounters;            // per stage
+  unsigned int* counters;   // 4 x ncounters: one per stage and chunk of a step
   int* err;                // device error word: bit 0 bad work item, bit 1 time limit
   long long limit_cycles;  // time limit of a persistent stage launch in SM cycles (0: none)
   cudaStream_t cap_stream;  // private stream the step graph is captured on
@@ -46,36 +50,16 @@ struct chemora_batch {
 
 namespace chemora {
 
-// one block of 128 threads (kItemPoints) per work item
-
-template <int NV>
-struct BatchBody;
-
-template <>
-struct BatchBody<24> {
-  template <class LD, class OUT>
-  __device__ __forceinline__ static void eval(const LD& ld, const Scalars& sc, OUT& out) {
-    chemora_bssn_point(ld, sc, out);
-  }
-};
-
-template <>
-struct BatchBody<2> {
-  template <class LD, class OUT>
-  __device__ __forceinline__ static void eval(const LD& ld, const Scalars& sc, OUT& out) {
-    wave_point(ld, sc, out);
-  }
-};
-
-// MODE: the RK stage mode compiled in (its update's branches fold), or -1
-// for the mode of the stage arguments.
-template <int NV, int MODE>
+// The scalar wave's persistent stage kernel, one block of 128 threads
+// (kItemPoints) per work item.  MODE: the RK stage mode, compiled in (modes 2
+// and 3 are the same update).
+template <int MODE>
 __global__ void __launch_bounds__(128, 3)
 batch_stage_kernel(const PatchDesc* __restrict__ pd, int npatch, const WorkItem* __restrict__ items,
                    int nitems, unsigned int* counter, int* err, long long limit, Scalars sc,
                    StageParams base_in) {
   StageParams base = base_in;
-  if (MODE >= 0) base.mode = MODE;
+  base.mode = MODE;
   __shared__ unsigned int s_item;
   const long long t0 = clock64();
   for (int iter = 0; iter <= nitems; ++iter) {  // bounded: one counter value per pass
@@ -106,14 +90,9 @@ batch_stage_kernel(const PatchDesc* __restrict__ pd, int npatch, const WorkItem*
     const int j = (int)(r / P.d.nx);
     const int i = (int)(r - (int64_t)j * P.d.nx);
     const int64_t c = P.offset + (int64_t)(k + P.d.g) * P.d.sz + (int64_t)(j + P.d.g) * P.d.sy + (i + P.d.g);
-    Loader<NV> ld{base.src + c, nullptr, P.d.sy, P.d.sz, P.d.sv};
-    if (NV == 2) {  // the scalar wave's update (StageOutFma), as in its single-grid kernels
-      StageOutFma out = CHEMORA_STAGE_OUT_FMA(base, c, P.d.sv, sc);
-      BatchBody<NV>::eval(ld, sc, out);
-    } else {
-      StageOut out = CHEMORA_STAGE_OUT(base, c, P.d.sv, sc);
-      BatchBody<NV>::eval(ld, sc, out);
-    }
+    Loader<2> ld{base.src + c, nullptr, P.d.sy, P.d.sz, P.d.sv};
+    StageOutFma out = CHEMORA_STAGE_OUT_FMA(base, c, P.d.sv, sc);
+    wave_point(ld, sc, out);
   }
 }
 
@@ -173,47 +152,24 @@ static int persistent_blocks() {
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     sms = 152;
-  cached = 3 * sms;  // three 128-thread blocks per SM (168 registers; measured best of 2-4)
+  cached = 3 * sms;  // three 128-thread blocks per SM
   return cached;
 }
 
-struct BatchLaunch {
-  const PatchDesc* pd;
-  int npatch;
-  const WorkItem* items;
-  int nitems;
-  unsigned int* counter;
-  int* err;
-  long long limit;
-};
-
-template <int NV, int MODE>
-static void launch_batch_mode(const BatchLaunch& L, const Scalars& sc, const StageParams& p, cudaStream_t s) {
-  batch_stage_kernel<NV, MODE><<<persistent_blocks(), kItemPoints, 0, s>>>(L.pd, L.npatch, L.items, L.nitems,
-                                                                          L.counter, L.err, L.limit, sc, p);
-}
-
-template <int NV>
-static void launch_batch_nv(const BatchLaunch& L, const Scalars& sc, const StageParams& p, cudaStream_t s) {
-  switch (p.mode) {
-    case 1: launch_batch_mode<NV, 1>(L, sc, p, s); break;
-    case 2: launch_batch_mode<NV, 2>(L, sc, p, s); break;
-    case 3: launch_batch_mode<NV, 3>(L, sc, p, s); break;
-    case 4: launch_batch_mode<NV, 4>(L, sc, p, s); break;
-    default: launch_batch_mode<NV, -1>(L, sc, p, s); break;
-  }
-}
-
-int launch_batch_stage(int nvars, const PatchDesc* pd, int npatch, const WorkItem* items, int nitems,
+int launch_batch_stage(const PatchDesc* pd, int npatch, const WorkItem* items, int nitems,
                        unsigned int* counter, int* err, long long limit, const Scalars& sc,
                        const StageParams& p, cudaStream_t s) {
-  const BatchLaunch L{pd, npatch, items, nitems, counter, err, limit};
-  if (nvars == 24)
-    launch_batch_nv<24>(L, sc, p, s);
-  else if (nvars == 2)
-    launch_batch_nv<2>(L, sc, p, s);
-  else
-    return set_error(CHEMORA_EINVAL, "batched stage kernels exist for 24 (BSSN) and 2 (wave) variables");
+#define CHEMORA_BATCH_STAGE(MODE)                                                                               \
+  batch_stage_kernel<MODE><<<persistent_blocks(), kItemPoints, 0, s>>>(pd, npatch, items, nitems, counter, err, \
+                                                                       limit, sc, p)
+  switch (p.mode) {
+    case 1: CHEMORA_BATCH_STAGE(1); break;
+    case 2:
+    case 3: CHEMORA_BATCH_STAGE(2); break;
+    case 4: CHEMORA_BATCH_STAGE(4); break;
+    default: return set_error(CHEMORA_EINVAL, "batched stage mode %d", p.mode);
+  }
+#undef CHEMORA_BATCH_STAGE
   return launched("batch_stage_kernel");
 }
 
@@ -222,8 +178,10 @@ void append_items(std::vector<WorkItem>& items, int q, int64_t npts) {
 }
 
 static int batch_stage(chemora_batch* b, const StageParams& p, int stage, cudaStream_t s) {
-  return launch_batch_stage(b->nvars, b->dev_pd, b->npatch, b->items, b->nitems, b->counters + stage, b->err,
-                            b->limit_cycles, b->sc, p, s);
+  unsigned int* counters = b->counters + stage * b->ncounters;
+  if (b->kind == CHEMORA_BSSN)
+    return launch_field_plan(b->plan, counters, b->err, b->limit_cycles, b->sc, p, b->work, s);
+  return launch_batch_stage(b->dev_pd, b->npatch, b->items, b->nitems, counters, b->err, b->limit_cycles, b->sc, p, s);
 }
 
 // One RK4 step of every patch, batched: 4 x (ghost fill + persistent stage).
@@ -234,7 +192,7 @@ static int batch_rk4_one(chemora_batch* b, double dt, cudaStream_t s) {
   double* Sa = b->scratch + n;
   double* Sb = b->scratch + 2 * n;
   int rc;
-  CHEMORA_CUDA(cudaMemsetAsync(b->counters, 0, 4 * sizeof(unsigned int), s));
+  CHEMORA_CUDA(cudaMemsetAsync(b->counters, 0, 4 * b->ncounters * sizeof(unsigned int), s));
   StageParams p{};
   if ((rc = batch_ghosts(b, Y, s))) return rc;
   p.src = Y; p.yn = Y; p.acc = A; p.dst = Sa; p.c2 = 0.5 * dt; p.mode = 1;
@@ -259,20 +217,23 @@ static int patch_rk4_one(chemora_batch* b, int q, double dt, cudaStream_t s) {
   double* Sa = b->scratch + n + P.offset;
   double* Sb = b->scratch + 2 * n + P.offset;
   const int kind = b->kind;
+  FieldWork work;
+  work.w = b->work;
+  work.points = b->plan.points;
   int rc;
   StageParams p{};
   if ((rc = fill_ghosts(P.d, b->nvars, Y, s))) return rc;
   p.src = Y; p.yn = Y; p.acc = A; p.dst = Sa; p.c2 = 0.5 * dt; p.mode = 1;
-  if ((rc = launch_stage(kind, P.d, b->sc, p, s))) return rc;
+  if ((rc = launch_stage(kind, P.d, b->sc, p, s, 0, work))) return rc;
   if ((rc = fill_ghosts(P.d, b->nvars, Sa, s))) return rc;
   p.src = Sa; p.dst = Sb; p.c2 = 0.5 * dt; p.mode = 2;
-  if ((rc = launch_stage(kind, P.d, b->sc, p, s))) return rc;
+  if ((rc = launch_stage(kind, P.d, b->sc, p, s, 0, work))) return rc;
   if ((rc = fill_ghosts(P.d, b->nvars, Sb, s))) return rc;
   p.src = Sb; p.dst = Sa; p.c2 = dt; p.mode = 3;
-  if ((rc = launch_stage(kind, P.d, b->sc, p, s))) return rc;
+  if ((rc = launch_stage(kind, P.d, b->sc, p, s, 0, work))) return rc;
   if ((rc = fill_ghosts(P.d, b->nvars, Sa, s))) return rc;
   p.src = Sa; p.dst = Y; p.c1 = dt / 6.0; p.c2 = 0.0; p.mode = 4;
-  return launch_stage(kind, P.d, b->sc, p, s);
+  return launch_stage(kind, P.d, b->sc, p, s, 0, work);
 }
 
 static void free_graph(chemora_batch* b) {
@@ -288,7 +249,11 @@ void destroy_batch(chemora_batch* b) {
   cudaFree(b->state);
   cudaFree(b->scratch);
   cudaFree(b->dev_pd);
-  cudaFree(b->items);
+  if (b->kind == CHEMORA_BSSN)
+    field_plan_free(&b->plan);  // items is the plan's
+  else
+    cudaFree(b->items);
+  cudaFree(b->work);
   cudaFree(b->counters);
   cudaFree(b->err);
   b->type = 0;
@@ -314,7 +279,7 @@ static int capture_step(chemora_batch* b, double dt) {
   b->graph = g;
   CHEMORA_CUDA(cudaGraphInstantiate(&b->exec, g, 0));
   b->graph_dt = dt;
-  b->graph_kernels = 8;
+  b->graph_kernels = b->kind == CHEMORA_BSSN ? 4 + 8 * (int)b->plan.chunks.size() : 8;
   return CHEMORA_OK;
 }
 
@@ -356,7 +321,7 @@ int chemora_patches_create(int npatch, const int* dims, int nghost, double dx, i
     P.offset = off;
     P.npts = (int64_t)nx * ny * nz;
     off += (P.d.sv * nvars + 31) / 32 * 32;  // 256-byte aligned patch states
-    append_items(items, q, P.npts);
+    if (kind == CHEMORA_WAVE) append_items(items, q, P.npts);
   }
   if (items.size() > (size_t)0x7fffffff) return set_error(CHEMORA_EINVAL, "too many work items");
   chemora_batch* b = new (std::nothrow) chemora_batch();
@@ -367,19 +332,30 @@ int chemora_patches_create(int npatch, const int* dims, int nghost, double dx, i
   b->host_pd = pd;
   b->total = off;
   b->nitems = (int)items.size();
+  b->ncounters = 1;
   cudaError_t e = cudaSuccess;
+  if (kind == CHEMORA_BSSN) {
+    if ((rc = field_plan_create(pd, &b->plan))) {
+      destroy_batch(b);
+      return rc;
+    }
+    b->items = b->plan.items;
+    b->nitems = b->plan.nitems;
+    b->ncounters = (int)b->plan.chunks.size();
+    e = cudaMalloc(&b->work, field_work_bytes(b->plan.points));
+  }
   if (e == cudaSuccess) e = cudaMalloc(&b->state, off * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&b->scratch, 3 * off * sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&b->dev_pd, npatch * sizeof(PatchDesc));
-  if (e == cudaSuccess) e = cudaMalloc(&b->items, items.size() * sizeof(WorkItem));
-  if (e == cudaSuccess) e = cudaMalloc(&b->counters, 4 * sizeof(unsigned int));
+  if (e == cudaSuccess && kind == CHEMORA_WAVE) e = cudaMalloc(&b->items, items.size() * sizeof(WorkItem));
+  if (e == cudaSuccess) e = cudaMalloc(&b->counters, 4 * b->ncounters * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMalloc(&b->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(b->state, 0, off * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(b->scratch, 0, 3 * off * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(b->err, 0, sizeof(int));
   if (e == cudaSuccess)
     e = cudaMemcpy(b->dev_pd, pd.data(), npatch * sizeof(PatchDesc), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && kind == CHEMORA_WAVE)
     e = cudaMemcpy(b->items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -395,7 +371,8 @@ int chemora_patches_inject_fault(chemora_batch* batch, int item) {
   if (!is_handle(batch, H_BATCH)) return set_error(CHEMORA_EINVAL, "not a batch handle");
   if (item < 0 || item >= batch->nitems)
     return set_error(CHEMORA_EINVAL, "work item %d outside [0, %d)", item, batch->nitems);
-  const WorkItem bad{batch->npatch + 7, 0};  // names a patch outside the table
+  const int table = batch->kind == CHEMORA_BSSN ? batch->plan.nregions : batch->npatch;
+  const WorkItem bad{table + 7, 0};  // names a patch outside the table
   CHEMORA_CUDA(cudaMemcpy(batch->items + item, &bad, sizeof bad, cudaMemcpyHostToDevice));
   return CHEMORA_OK;
 }

@@ -31,6 +31,12 @@ def _sym_expr(name):
     m = re.match(r"sdz_(\d+)_(-?\d+)$", name)
     if m:
         return "ld.sdz(%d, %s)" % (stencil.ZROW_VARS.index(int(m.group(1))), m.group(2)), True
+    m = re.match(r"g(1|2|11)_(\d+)_(\d+)$", name)
+    if m:
+        return "ld.g%s(%s, %s)" % m.groups(), True
+    m = re.match(r"gko_(\d+)$", name)
+    if m:
+        return "ld.gko(%s)" % m.group(1), True
     return "sc." + name, False
 
 
@@ -81,6 +87,16 @@ def _bssn_xshare():
 def _bssn_xyshare():
     with stencil.xshare(), stencil.yshare():
         return systems.bssn()
+
+
+def _bssn_fields():
+    with stencil.fields():
+        return systems.bssn()
+
+
+def _bssn_constraints_fields():
+    with stencil.fields():
+        return systems.bssn_constraints()
 
 
 def _read(name):
@@ -155,6 +171,12 @@ def _render():
     specs.append(("wave_varc", "chemora_varc_point", systems.wave_varc,
                   "variable-speed wave: u_t = rho, rho_t = s Lap u + G . grad u, with s = c^2 "
                   "and G = grad s read from grid functions 2 and 3-5"))
+    specs.append(("bssn_alg", "chemora_bssn_alg_point", _bssn_fields,
+                  "BSSN as chemora_bssn_point, every derivative read from precomputed fields: "
+                  "the algebra of one point"))
+    specs.append(("bssn_constraints_alg", "chemora_bssn_constraints_alg_point", _bssn_constraints_fields,
+                  "BSSN constraints as chemora_bssn_constraints_point, every derivative read from "
+                  "precomputed fields"))
     for key, fname, build, comment in specs:
         outs = build()
         nout = len(outs)
@@ -172,7 +194,8 @@ def _render():
     files["opcounts.json"] = json.dumps(counts, indent=1, sort_keys=True) + "\n"
     inc = [HEADER.rstrip("\n") + "\n", "// per interior point and RHS evaluation\n"]
     for key, tag in (("wave", "WAVE"), ("wave_varc", "VARC"), ("bssn", "BSSN"), ("wave1_o4", "WAVE1"),
-                     ("bssn_x", "BSSN_X"), ("bssn_xy", "BSSN_XY"), ("wave_xz", "WAVE_XZ")):
+                     ("bssn_x", "BSSN_X"), ("bssn_xy", "BSSN_XY"), ("wave_xz", "WAVE_XZ"),
+                     ("bssn_alg", "BSSN_ALG"), ("bssn_constraints_alg", "CONSTRAINTS_ALG")):
         inc.append("#define CHEMORA_OPS_%s_INSTR %d\n" % (tag, counts[key]["fp64_instructions"]))
         inc.append("#define CHEMORA_OPS_%s_FLOPS %d\n" % (tag, counts[key]["flops"]))
     files["opcounts.inc"] = "".join(inc)

@@ -87,6 +87,23 @@ class zqueue:
         _ZQUEUE[0] = self.prev
 
 
+_FIELDS = [False]
+
+
+class fields:
+    """Context manager: every derivative is read from precomputed fields
+    (symbols g1_<v>_<a>: 12h D_a f, g2_<v>_<a>: 12h^2 D_aa f, g11_<v>_<ab>:
+    144h^2 D_ab f, gko_<v>: 64h/eps KO f), so the body holds the algebra alone
+    and reads the state at the point only."""
+
+    def __enter__(self):
+        self.prev = _FIELDS[0]
+        _FIELDS[0] = True
+
+    def __exit__(self, *exc):
+        _FIELDS[0] = self.prev
+
+
 def _zq(what, v):
     return E.sym("zq%s_%d" % (what, v))
 
@@ -124,6 +141,8 @@ def _xabc(v):
 
 def d1_raw(v, a, base=(0, 0, 0)):
     """12h * D1_a at base: 8 (f+1 - f-1) - (f+2 - f-2)."""
+    if _FIELDS[0]:
+        return E.sym("g1_%d_%d" % (v, a))
     if _YSHARE[0] and base == (0, 0, 0):
         if a == 1:
             s1 = E.box(_dy(v, 0) + _dy(v, -1))
@@ -152,6 +171,8 @@ def d1(v, a):
 
 def d2_raw(v, a):
     """12h^2 * pure second derivative: 16 d1 - d2, d_k = (f+k - f0) + (f-k - f0)."""
+    if _FIELDS[0]:
+        return E.sym("g2_%d_%d" % (v, a))
     if _XSHARE[0] and a == 0:
         xa, xb, _ = _xabc(v)
         return E.box(15 * xa - xb)  # 16 a - (a + b)
@@ -171,6 +192,8 @@ def d2(v, a):
 def d11_raw(v, a, b):
     """144h^2 * mixed derivative D_a D_b: the first-derivative stencil along
     b applied to first-derivative rows along a."""
+    if _FIELDS[0]:
+        return E.sym("g11_%d_%d" % (v, a + b - 1))
     if _YSHARE[0] and a == 1 and b == 2 and v in ZROW_VARS:
         # the y stencil applied to the z-derivative rows of the rows y +- m
         Z = {m: _zrow(v, m) for m in (-2, -1, 1, 2)}
@@ -206,6 +229,8 @@ def ko_raw(v, a):
 
 def ko(v):
     """Kreiss-Oliger dissipation summed over the three directions."""
+    if _FIELDS[0]:
+        return E.box(E.sym("gko_%d" % v) * KO_SCALE)
     return E.box(E.box(ko_raw(v, 0) + ko_raw(v, 1) + ko_raw(v, 2)) * KO_SCALE)
 
 
