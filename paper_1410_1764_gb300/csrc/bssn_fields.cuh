@@ -40,10 +40,11 @@ struct FieldSlab {
   int64_t w0;      // its first point in the workspace
 };
 
-// A slab with its extents and strides, and its tiles of tw x th points of one plane.
+// A slab with its extents and strides, and its tiles: columns of tw x th
+// points and zb planes.
 struct FieldRegion : FieldSlab {
   Dims d;
-  int tw, th, tnx, tny;
+  int tw, th, zb, tnx, tny;
 };
 
 // Loader of the algebra bodies: the state at the point and its fields.
@@ -65,77 +66,6 @@ struct FieldLoader {
 };
 
 #if defined(__CUDACC__) && !defined(__CUDACC_RTC__)
-// The radius-3 star around a point: centre and n[6 a + {+1, -1, +2, -2, +3, -3}].
-struct Star3 {
-  double c, n[18];
-  __device__ __forceinline__ void load(const double* __restrict__ p, int64_t sy, int64_t sz) {
-    const int64_t st[3] = {1, sy, sz};
-    c = __ldg(p);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        n[6 * a + 2 * m] = __ldg(p + (m + 1) * st[a]);
-        n[6 * a + 2 * m + 1] = __ldg(p - (m + 1) * st[a]);
-      }
-  }
-  __device__ __forceinline__ unsigned exponent() const {
-    unsigned e = fx::ebits(c);
-#pragma unroll
-    for (int q = 0; q < 18; ++q) e = fx::emax(e, fx::ebits(n[q]));
-    return e;
-  }
-  __device__ __forceinline__ bool all_zero() const {
-    bool z = c == 0.0;
-#pragma unroll
-    for (int q = 0; q < 18; ++q) z = z && n[q] == 0.0;
-    return z;
-  }
-};
-
-// Raw differences of a star: d1[a] = 12h D_a, d2[a] = 12h^2 D_aa (when DD)
-// and ko = 64h/eps KO.  Four guard bits: the weights of each axis add up to 64
-// in magnitude at most, so every axis sum fits in 64 bits; the dissipation's
-// three axis sums are added a quarter each (their truncation is 2^-55 of the
-// largest value, on a term of weight eps/64).
-template <bool DD>
-__device__ __forceinline__ void star3_differences(const Star3& s, double* d1, double* d2, double& ko) {
-  const unsigned e = s.exponent();
-  if (fx::in_range(e)) {
-    const long long c = fx::align<4>(s.c, e);
-    long long k = 0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const long long p1 = fx::align<4>(s.n[6 * a], e), m1 = fx::align<4>(s.n[6 * a + 1], e);
-      const long long p2 = fx::align<4>(s.n[6 * a + 2], e), m2 = fx::align<4>(s.n[6 * a + 3], e);
-      const long long p3 = fx::align<4>(s.n[6 * a + 4], e), m3 = fx::align<4>(s.n[6 * a + 5], e);
-      const long long s1 = p1 + m1, s2 = p2 + m2;
-      d1[a] = fx::to_double<4>(8 * (p1 - m1) - (p2 - m2), e);
-      if (DD) d2[a] = fx::to_double<4>(16 * s1 - s2 - 30 * c, e);
-      k += (15 * s1 - 6 * s2 + (p3 + m3) - 20 * c) >> 2;
-    }
-    ko = fx::to_double<2>(k, e);
-  } else if (s.all_zero()) {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      d1[a] = 0.0;
-      if (DD) d2[a] = 0.0;
-    }
-    ko = 0.0;
-  } else {  // the ends of the FP64 range, Inf, NaN: FP64 differences
-    ko = 0.0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const double* n = s.n + 6 * a;
-      const double c1 = (n[0] - s.c) + (n[1] - s.c), c2 = (n[2] - s.c) + (n[3] - s.c);
-      const double c3 = (n[4] - s.c) + (n[5] - s.c);
-      d1[a] = fma(8.0, n[0] - n[1], -(n[2] - n[3]));
-      if (DD) d2[a] = fma(16.0, c1, -c2);
-      ko += fma(15.0, c1, fma(-6.0, c2, c3));
-    }
-  }
-}
-
 // 8 (f+1 - f-1) - (f+2 - f-2) along stride st, in FP64 (rows of the mixed
 // derivatives past a tile's edge).
 __device__ __forceinline__ double d1_row_fp64(const double* __restrict__ p, int64_t st, double one, double eight) {

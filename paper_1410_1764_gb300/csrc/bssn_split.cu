@@ -14,17 +14,35 @@ namespace chemora {
 // derivative fields
 // ---------------------------------------------------------------------------
 constexpr int kTileThreads = 256, kTileRows = 32;
-constexpr int kRowMax = 448;  // doubles of a row array: (tw + 4) x (th + 4) for every tile shape tile_shape() returns
+constexpr int kRowMax = 448;    // (tw + 4) x (th + 4) of every tile shape tile_shape() returns
+constexpr int kPlaneMax = 532;  // (tw + 6) x (th + 6)
+constexpr int kGuard = 4;       // guard bits: an axis' weights add up to 64 in magnitude, 64 x 2^57 fits
 
-// One block: one variable (blockIdx.y) on one tile of one plane, a point per
-// thread.  The mixed derivatives are first-derivative stencils of the
-// neighbours' first-derivative rows, in FP64 (3 fmas each: fewer cycles than
-// their 16 points in integers, on a pipe this kernel leaves idle); the rows
-// pass through shared memory, those past the tile's edge are computed by the
-// block again.
-__global__ void __launch_bounds__(kTileThreads)
+// One block: one variable (blockIdx.y) on a tile of tw x th columns, marching
+// through zb planes, a point per thread and plane.  Each value is taken apart
+// into integers once: a thread keeps its column's seven values in registers,
+// the plane in hand lies in shared memory (significands and exponents) with
+// its halo, so a tap costs a shift to the star's largest exponent and an
+// addition.  First differences go back to doubles through the conversion
+// instruction, the others by integer operations, which shares the work
+// between the two pipes.  The mixed derivatives are first-derivative stencils
+// of the neighbours' first-derivative rows, in FP64 (three fmas each: fewer
+// cycles than their 16 points in integers); the rows pass through shared
+// memory, those past the tile's edge are computed by the block again.
+//
+// GB300, all 24 variables of 128 x 128 x 64 points: 546 us (the field writes
+// alone take 200 us of HBM time); each value taken apart by each of its 19
+// readers, no march: 846 us; conversion instruction for every difference 603,
+// for none 572 us; two or four blocks per SM 637, 708 us; significand and
+// exponent in one 16-byte cell 621 us; one kernel for both sorts of variable
+// 580 us.  Bound by the latency of its integer chains at 24 warps per SM
+// (2.2 instructions per clock; FP64 pipe 45 % busy).
+template <bool DD>
+__global__ void __launch_bounds__(kTileThreads, 3)
 bssn_fields_kernel(const FieldRegion* __restrict__ regions, FieldRegion one_region, const int2* __restrict__ tiles,
                    const double* __restrict__ base, double* __restrict__ work, double one, double eight) {
+  __shared__ long long pm[2][kPlaneMax];
+  __shared__ int pe[2][kPlaneMax];
   __shared__ double row_y[kRowMax], row_z[kRowMax];
   int tile = blockIdx.x, region = 0;
   if (tiles) {
@@ -34,70 +52,166 @@ bssn_fields_kernel(const FieldRegion* __restrict__ regions, FieldRegion one_regi
   }
   const FieldRegion R = regions ? regions[region] : one_region;
   const Dims& d = R.d;
-  const int v = blockIdx.y, ddi = dd_index(v);
-  const int txy = tile % (R.tnx * R.tny), k = tile / (R.tnx * R.tny);
+  // the DD kernel takes the variables with second derivatives, the other the rest
+  const int v = DD ? (blockIdx.y < 7 ? blockIdx.y : blockIdx.y + 10)
+                   : (blockIdx.y < 10 ? blockIdx.y + 7 : blockIdx.y + 11);
+  const int ddi = blockIdx.y;
+  const int txy = tile % (R.tnx * R.tny), k0 = (tile / (R.tnx * R.tny)) * R.zb;
   const int x0 = (txy % R.tnx) * R.tw, y0 = (txy / R.tnx) * R.th;
-  const int w = min(R.tw, d.nx - x0), h = min(R.th, d.ny - y0);
+  const int w = min(R.tw, d.nx - x0), h = min(R.th, d.ny - y0), nz = min(R.zb, d.nz - k0);
   const int t = threadIdx.x, ly = t / R.tw, lx = t - ly * R.tw;
   const bool active = lx < w && ly < h;
-  const double* org = base + R.offset + v * d.sv + (int64_t)(k + d.g) * d.sz + (int64_t)(y0 + d.g) * d.sy + x0 + d.g;
-  double* out = nullptr;
-  if (active)
-    out = work + field_base(R.w0 + ((int64_t)k * d.ny + y0 + ly) * d.nx + x0 + lx);
-  double d1[3], d2[3], ko;
-  Star3 s;
-  if (ddi < 0) {
-    if (!active) return;
-    s.load(org + (int64_t)ly * d.sy + lx, d.sy, d.sz);
-    star3_differences<false>(s, d1, d2, ko);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) out[(kFieldD1 + 3 * v + a) * kFieldBlock] = d1[a];
-    out[(kFieldKo + v) * kFieldBlock] = ko;
-    return;
+  const double* org = base + R.offset + v * d.sv + (int64_t)(k0 + d.g) * d.sz + (int64_t)(y0 + d.g) * d.sy + x0 + d.g;
+  const double* col = org + (int64_t)ly * d.sy + lx;
+  const int pp = R.tw + 6, pc = (ly + 3) * pp + lx + 3;  // plane pitch, this point
+  const int rp = R.tw + 4;                               // row pitch
+  // this thread's halo cell: columns -3..-1, w..w+2 of the tile's rows, then
+  // rows -3..-1, h..h+2
+  const bool halo = t < 6 * (w + h);
+  int hx = 0, hy = 0;
+  if (t < 6 * h) {
+    const int e = t / h;
+    hy = t - e * h;
+    hx = e < 3 ? e - 3 : w + e - 3;
+  } else if (halo) {
+    const int e = (t - 6 * h) / w;
+    hx = t - 6 * h - e * w;
+    hy = e < 3 ? e - 3 : h + e - 3;
   }
-  const int pw = R.tw + 4;  // row pitch; the tile's point (0, 0) sits at [2][2] of row_z, [0][2] of row_y
+  const double* hp = org + (int64_t)hy * d.sy + hx;
+  const int hc = (hy + 3) * pp + hx + 3;
+  fx::Parts z[7];
+  double znext = 0.0, hnext = 0.0;
+#pragma unroll
+  for (int m = 0; m < 7; ++m) z[m] = fx::Parts{0, 0};
   if (active) {
-    s.load(org + (int64_t)ly * d.sy + lx, d.sy, d.sz);
-    star3_differences<true>(s, d1, d2, ko);
-    row_y[ly * pw + lx + 2] = d1[1];
-    row_z[(ly + 2) * pw + lx + 2] = d1[2];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      out[(kFieldD1 + 3 * v + a) * kFieldBlock] = d1[a];
-      out[(kFieldD2 + 6 * ddi + a) * kFieldBlock] = d2[a];
-    }
-    out[(kFieldKo + v) * kFieldBlock] = ko;
+    for (int m = 1; m < 7; ++m) z[m] = fx::parts<kGuard>(__ldg(col + (int64_t)(m - 4) * d.sz));
+    znext = __ldg(col + 3 * d.sz);
   }
-  // rows past the edge: columns -2, -1, w, w+1 (y and z rows), then rows
-  // -2, -1, h, h+1 (z rows)
-  for (int q = t; q < 4 * h + 4 * h + 4 * w; q += kTileThreads) {
-    if (q < 8 * h) {
-      const int r = q % h, e = (q / h) & 3, x = e < 2 ? e - 2 : w + e - 2;
-      const double* p = org + (int64_t)r * d.sy + x;
-      if (q < 4 * h)
-        row_y[r * pw + x + 2] = d1_row_fp64(p, d.sy, one, eight);
-      else
-        row_z[(r + 2) * pw + x + 2] = d1_row_fp64(p, d.sz, one, eight);
-    } else {
-      const int r = (q - 8 * h) / w, x = (q - 8 * h) % w, y = r < 2 ? r - 2 : h + r - 2;
-      row_z[(y + 2) * pw + x + 2] = d1_row_fp64(org + (int64_t)y * d.sy + x, d.sz, one, eight);
+  if (halo) hnext = __ldg(hp);
+  int64_t point = R.w0 + ((int64_t)k0 * d.ny + y0 + ly) * d.nx + x0 + lx;
+#pragma unroll 1
+  for (int k = 0; k < nz; ++k) {
+    long long* const M = pm[k & 1];
+    int* const E = pe[k & 1];
+#pragma unroll
+    for (int m = 0; m < 6; ++m) z[m] = z[m + 1];
+    z[6] = fx::parts<kGuard>(znext);
+    if (active) {
+      M[pc] = z[3].m;
+      E[pc] = z[3].e;
+    }
+    if (halo) {
+      const fx::Parts q = fx::parts<kGuard>(hnext);
+      M[hc] = q.m;
+      E[hc] = q.e;
+      if (k + 1 < nz) hnext = __ldg(hp + (int64_t)(k + 1) * d.sz);
+    }
+    if (active && k + 1 < nz) znext = __ldg(col + (int64_t)(k + 4) * d.sz);
+    __syncthreads();
+    double* out = work + field_base(point);
+    point += (int64_t)d.nx * d.ny;
+    if (active) {
+      int ex[6], ey[6], e = z[3].e;
+#pragma unroll
+      for (int m = 0; m < 6; ++m) {
+        const int o = m < 3 ? m - 3 : m - 2;
+        ex[m] = E[pc + o];
+        ey[m] = E[pc + o * pp];
+        e = fx::emax(e, fx::emax(fx::emax(ex[m], ey[m]), z[m < 3 ? m : m + 1].e));
+      }
+      double d1[3], d2[3], ko = 0.0;
+      if (fx::in_range(e)) {
+        const long long c = fx::align(z[3], e);
+        const long long c30 = 30 * c;
+        long long s1t = 0, s2t = 0, s3t = 0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          long long f[6];
+#pragma unroll
+          for (int m = 0; m < 6; ++m) {
+            const int o = m < 3 ? m - 3 : m - 2;
+            f[m] = a == 0 ? fx::sar(M[pc + o], (unsigned)(e - ex[m]))
+                          : (a == 1 ? fx::sar(M[pc + o * pp], (unsigned)(e - ey[m]))
+                                    : fx::align(z[m < 3 ? m : m + 1], e));
+          }
+          const long long s1 = f[3] + f[2], s2 = f[4] + f[1], s3 = f[5] + f[0];
+          d1[a] = fx::to_double_cvt<kGuard>(8 * (f[3] - f[2]) - (f[4] - f[1]), e);
+          if (DD) d2[a] = fx::to_double<kGuard>(16 * s1 - s2 - c30, e);
+          s1t += s1;
+          s2t += s2;
+          s3t += s3;
+        }
+        // the dissipation's weights add up to 192: a quarter of the sum fits,
+        // formed from the quarters and the remainders of its parts
+        const int r = (15 * ((int)s1t & 3) - 6 * ((int)s2t & 3) + ((int)s3t & 3)) >> 2;
+        ko = fx::to_double<kGuard - 2>(15 * (s1t >> 2) - 6 * (s2t >> 2) + (s3t >> 2) - 15 * c + r, e);
+      } else {
+        // zeros (all differences zero), the ends of the FP64 range, Inf, NaN
+        const int64_t st[3] = {1, d.sy, d.sz};
+        const double* p = col + (int64_t)k * d.sz;
+        const double c = __ldg(p);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          double n[6];
+#pragma unroll
+          for (int m = 0; m < 3; ++m) {
+            n[2 * m] = __ldg(p + (m + 1) * st[a]);
+            n[2 * m + 1] = __ldg(p - (m + 1) * st[a]);
+          }
+          const double c1 = (n[0] - c) + (n[1] - c), c2 = (n[2] - c) + (n[3] - c), c3 = (n[4] - c) + (n[5] - c);
+          d1[a] = fma(8.0, n[0] - n[1], -(n[2] - n[3]));
+          d2[a] = fma(16.0, c1, -c2);
+          ko += fma(15.0, c1, fma(-6.0, c2, c3));
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a) out[(kFieldD1 + 3 * v + a) * kFieldBlock] = d1[a];
+      out[(kFieldKo + v) * kFieldBlock] = ko;
+      if (DD) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) out[(kFieldD2 + 6 * ddi + a) * kFieldBlock] = d2[a];
+        row_y[ly * rp + lx + 2] = d1[1];
+        row_z[(ly + 2) * rp + lx + 2] = d1[2];
+      }
+    }
+    if constexpr (DD) {
+      // rows past the edge: columns -2, -1, w, w+1 (y and z rows), then rows
+      // -2, -1, h, h+1 (z rows)
+      for (int q = t; q < 8 * h + 4 * w; q += kTileThreads) {
+        const double* src = org + (int64_t)k * d.sz;
+        if (q < 8 * h) {
+          const int e = q / h, r = q - e * h, x = (e & 3) < 2 ? (e & 3) - 2 : w + (e & 3) - 2;
+          const double* p = src + (int64_t)r * d.sy + x;
+          if (e < 4)
+            row_y[r * rp + x + 2] = d1_row_fp64(p, d.sy, one, eight);
+          else
+            row_z[(r + 2) * rp + x + 2] = d1_row_fp64(p, d.sz, one, eight);
+        } else {
+          const int e = (q - 8 * h) / w, x = q - 8 * h - e * w, y = e < 2 ? e - 2 : h + e - 2;
+          row_z[(y + 2) * rp + x + 2] = d1_row_fp64(src + (int64_t)y * d.sy + x, d.sz, one, eight);
+        }
+      }
+      __syncthreads();
+      if (active) {
+        auto mixed = [&](const double* r, int st) {
+          const double q1 = fma(r[-st], -one, r[st]), q2 = fma(r[-2 * st], -one, r[2 * st]);
+          return fma(eight, q1, -q2);
+        };
+        const double* ry = row_y + ly * rp + lx + 2;
+        const double* rz = row_z + (ly + 2) * rp + lx + 2;
+        out[(kFieldD2 + 6 * ddi + 3) * kFieldBlock] = mixed(ry, 1);
+        out[(kFieldD2 + 6 * ddi + 4) * kFieldBlock] = mixed(rz, 1);
+        out[(kFieldD2 + 6 * ddi + 5) * kFieldBlock] = mixed(rz, rp);
+      }
     }
   }
-  __syncthreads();
-  if (!active) return;
-  auto mixed = [&](const double* r, int st) {
-    const double q1 = fma(r[-st], -one, r[st]), q2 = fma(r[-2 * st], -one, r[2 * st]);
-    return fma(eight, q1, -q2);
-  };
-  const double* ry = row_y + ly * pw + lx + 2;
-  const double* rz = row_z + (ly + 2) * pw + lx + 2;
-  out[(kFieldD2 + 6 * ddi + 3) * kFieldBlock] = mixed(ry, 1);
-  out[(kFieldD2 + 6 * ddi + 4) * kFieldBlock] = mixed(rz, 1);
-  out[(kFieldD2 + 6 * ddi + 5) * kFieldBlock] = mixed(rz, pw);
 }
 
 // Tiles of nearly equal shape, at most 32 wide, at most 256 points, so that
-// ragged grids leave few threads idle.
+// ragged grids leave few threads idle; 16 planes deep where that leaves enough
+// blocks to fill the GPU, else fewer.
 static void tile_shape(FieldRegion* R) {
   const Dims& d = R->d;
   R->tnx = (d.nx + 31) / 32;
@@ -105,7 +219,13 @@ static void tile_shape(FieldRegion* R) {
   const int rows = std::min(kTileRows, kTileThreads / R->tw);
   R->tny = (d.ny + rows - 1) / rows;
   R->th = (d.ny + R->tny - 1) / R->tny;
+  int zb = 16;
+  while (zb > 4 && (int64_t)R->tnx * R->tny * ((d.nz + zb - 1) / zb) * 24 < 4 * 152) zb /= 2;
+  const int nseg = (d.nz + zb - 1) / zb;
+  R->zb = (d.nz + nseg - 1) / nseg;
 }
+
+static int64_t region_tiles(const FieldRegion& R) { return (int64_t)R.tnx * R.tny * ((R.d.nz + R.zb - 1) / R.zb); }
 
 FieldRegion field_region(const Dims& d, int64_t offset, int64_t w0) {
   FieldRegion R;
@@ -136,12 +256,21 @@ size_t field_work_bytes(int64_t points) {
   return (size_t)((points + kFieldBlock - 1) / kFieldBlock) * kFields * kFieldBlock * sizeof(double);
 }
 
+static int launch_field_kernels(const FieldRegion* regions, const FieldRegion& R, const int2* tiles, unsigned ntiles,
+                                int nvars, const double* src, double* work, const Scalars& sc, cudaStream_t s) {
+  // 24 variables: 11 with second derivatives, 13 without; the constraints' 17: 7 and 10
+  const unsigned ndd = nvars == 24 ? 11 : 7, nd = nvars - ndd;
+  bssn_fields_kernel<true><<<dim3(ntiles, ndd), kTileThreads, 0, s>>>(regions, R, tiles, src, work,
+                                                                     sc.k[CHEMORA_K_ONE], sc.k[CHEMORA_K_EIGHT]);
+  bssn_fields_kernel<false><<<dim3(ntiles, nd), kTileThreads, 0, s>>>(regions, R, tiles, src, work,
+                                                                     sc.k[CHEMORA_K_ONE], sc.k[CHEMORA_K_EIGHT]);
+  return launched("bssn_fields_kernel", 2);
+}
+
 int launch_fields(const FieldRegion& R, int nvars, const double* src, double* work, const Scalars& sc,
                          cudaStream_t s) {
-  const dim3 grid((unsigned)(R.tnx * R.tny * R.d.nz), (unsigned)nvars);
-  bssn_fields_kernel<<<grid, kTileThreads, 0, s>>>(nullptr, R, nullptr, src, work, sc.k[CHEMORA_K_ONE],
-                                                   sc.k[CHEMORA_K_EIGHT]);
-  return launched("bssn_fields_kernel");
+  const unsigned n = (unsigned)region_tiles(R);
+  return launch_field_kernels(nullptr, R, nullptr, n, nvars, src, work, sc, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -259,7 +388,7 @@ int field_plan_create(const std::vector<PatchDesc>& patches, FieldPlan* plan) {
       const int q = (int)regions.size();
       regions.push_back(R);
       append_items(items, q, R.npts);
-      const int64_t nt = (int64_t)R.tnx * R.tny * dk.nz;
+      const int64_t nt = region_tiles(R);
       for (int64_t t = 0; t < nt; ++t) tiles.push_back(int2{q, (int)t});
       cur += R.npts;
       k0 += dk.nz;
@@ -311,9 +440,9 @@ int launch_field_plan(const FieldPlan& plan, unsigned int* counters, int* err, l
   int rc;
   for (size_t q = 0; q < plan.chunks.size(); ++q) {
     const FieldPlan::Chunk& c = plan.chunks[q];
-    bssn_fields_kernel<<<dim3((unsigned)(c.tile1 - c.tile0), 24), kTileThreads, 0, s>>>(
-        plan.regions, FieldRegion{}, plan.tiles + c.tile0, p.src, work, sc.k[CHEMORA_K_ONE], sc.k[CHEMORA_K_EIGHT]);
-    if ((rc = launched("bssn_fields_kernel"))) return rc;
+    if ((rc = launch_field_kernels(plan.regions, FieldRegion{}, plan.tiles + c.tile0,
+                                   (unsigned)(c.tile1 - c.tile0), 24, p.src, work, sc, s)))
+      return rc;
     const WorkItem* items = plan.items + c.item0;
     const int n = c.item1 - c.item0;
     switch (p.mode) {

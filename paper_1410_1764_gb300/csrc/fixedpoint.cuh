@@ -6,10 +6,10 @@
 // per fma, or a load, do not slow a saturated fma stream).  A stencil is a
 // sum of values times small integers, so it is evaluated in integers: the
 // values it reads are written as multiples of one power of two, taken from
-// the largest of them (align), added exactly in 64 or 96 bits, and the sum is
+// the largest of them (align), added exactly in 64 bits, and the sum is
 // rounded once to a double (to_double).  With K guard bits every value down
 // to 2^-K of the largest is represented exactly and a smaller one is
-// truncated at 2^(-52-K) of the largest value's power of two, so the result
+// rounded down at 2^(-52-K) of the largest value's power of two, so the result
 // is at least as close to the exact sum as that of a chain of FP64
 // additions.  It depends on the values alone, not on the order of the sum or
 // on the launch shape that evaluates it.
@@ -31,15 +31,15 @@ namespace fx {
 CHEMORA_FX unsigned hiword(double v) { return (unsigned)__double2hiint(v); }
 CHEMORA_FX unsigned loword(double v) { return (unsigned)__double2loint(v); }
 CHEMORA_FX double from_bits(unsigned long long b) { return __longlong_as_double((long long)b); }
-// PTX shifts clamp: an amount of 64 or more gives 0
-CHEMORA_FX unsigned long long shr(unsigned long long a, unsigned s) {
-  unsigned long long r;
-  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(s));
-  return r;
-}
+// PTX shifts clamp: an amount of 64 or more gives 0 (or the sign)
 CHEMORA_FX unsigned long long shl(unsigned long long a, unsigned s) {
   unsigned long long r;
   asm("shl.b64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(s));
+  return r;
+}
+CHEMORA_FX long long sar(long long a, unsigned s) {
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(s));
   return r;
 }
 CHEMORA_FX int clz64(unsigned long long a) { return __clzll((long long)a); }
@@ -57,41 +57,61 @@ CHEMORA_FX double from_bits(unsigned long long b) {
   memcpy(&v, &b, 8);
   return v;
 }
-CHEMORA_FX unsigned long long shr(unsigned long long a, unsigned s) { return s > 63 ? 0 : a >> s; }
 CHEMORA_FX unsigned long long shl(unsigned long long a, unsigned s) { return s > 63 ? 0 : a << s; }
+CHEMORA_FX long long sar(long long a, unsigned s) { return a >> (s > 63 ? 63 : s); }
 CHEMORA_FX int clz64(unsigned long long a) { return a ? __builtin_clzll(a) : 64; }
 #endif
 
-// The exponent field of v, in place (bits 20-30 of the high word).
-CHEMORA_FX unsigned ebits(double v) { return hiword(v) & 0x7ff00000u; }
-CHEMORA_FX unsigned emax(unsigned a, unsigned b) { return a > b ? a : b; }
-constexpr unsigned kExpMin = 128u << 20, kExpMax = 2030u << 20;
-CHEMORA_FX bool in_range(unsigned e) { return e - kExpMin <= kExpMax - kExpMin; }
+constexpr int kExpMin = 128, kExpMax = 2030;
+CHEMORA_FX bool in_range(int e) { return (unsigned)(e - kExpMin) <= (unsigned)(kExpMax - kExpMin); }
+CHEMORA_FX int exponent(double v) { return (int)(hiword(v) >> 20) & 0x7ff; }
+CHEMORA_FX int emax(int a, int b) { return a > b ? a : b; }
 
-// v in units of 2^(E - 1075 - K), E the exponent field e of the largest value:
-// |result| < 2^(53 + K).  Zeros and subnormals carry a false leading bit that
-// the shift (at least 128) removes.
+// A double taken apart: its exponent field e and its signed significand in
+// units of 2^(e - 1075 - K).  Zeros and subnormals have e = 0 and a small
+// non-negative m, which every shift to an exponent in range removes.
+struct Parts {
+  long long m;
+  int e;
+};
 template <int K>
-CHEMORA_FX long long align(double v, unsigned e) {
-  const unsigned h = hiword(v), d = (e - (h & 0x7ff00000u)) >> 20;
-  unsigned long long m = (unsigned long long)((h & 0xfffffu) | 0x100000u) << 32 | loword(v);
-  m = shr(m << K, d);
-  const unsigned long long s = (unsigned long long)(long long)((int)h >> 31);
-  return (long long)((m ^ s) - s);
+CHEMORA_FX Parts parts(double v) {
+  const unsigned h = hiword(v);
+  const unsigned long long m = ((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32 | loword(v)) << K;
+  const unsigned long long s = h >= 0x80100000u ? ~0ull : 0ull;
+  return Parts{(long long)((m ^ s) - s), exponent(v)};
 }
+
+// In units of 2^(E - 1075 - K), E the exponent of the largest value: |result|
+// <= 2^(53 + K).
+CHEMORA_FX long long align(const Parts& p, int e) { return sar(p.m, (unsigned)(e - p.e)); }
+template <int K>
+CHEMORA_FX long long align(double v, int e) { return align(parts<K>(v), e); }
 
 // v units of 2^(E - 1075 - K) as a double (nearest, ties away from zero).
 template <int K>
-CHEMORA_FX double to_double(long long v, unsigned e) {
+CHEMORA_FX double to_double(long long v, int e) {
   const unsigned long long s = (unsigned long long)(v >> 63);
   const unsigned long long a = ((unsigned long long)v ^ s) - s;
   const int lz = clz64(a);
   const unsigned long long m = shl(a, (unsigned)lz);
   unsigned long long r = (m >> 11) + ((m >> 10) & 1);
-  r += (unsigned long long)((e >> 20) + (unsigned)(10 - K) - (unsigned)lz) << 52;
+  r += (unsigned long long)(unsigned)(e + 10 - K - lz) << 52;
   r |= s & 0x8000000000000000ull;
   return a == 0 ? 0.0 : from_bits(r);
 }
+
+#if defined(__CUDACC__)
+// The same through the conversion instruction (nearest, ties to even), which
+// takes a slot of the FP64 pipe and a few integer operations instead of some
+// thirty of these.
+template <int K>
+CHEMORA_FX double to_double_cvt(long long v, int e) {
+  const double d = __ll2double_rn(v);
+  const int h = __double2hiint(d);
+  return __hiloint2double(h == 0 ? 0 : h + ((e - 1075 - K) << 20), __double2loint(d));
+}
+#endif
 
 }  // namespace fx
 }  // namespace chemora

@@ -32,17 +32,17 @@ struct Star2 {
     n[10] = ld(0, 0, 0, 2);
     n[11] = ld(0, 0, 0, -2);
   }
-  CHEMORA_FX unsigned exponent() const {
-    unsigned e = fx::ebits(c);
+  CHEMORA_FX int exponent() const {
+    int e = fx::exponent(c);
 #pragma unroll
-    for (int q = 0; q < 12; ++q) e = fx::emax(e, fx::ebits(n[q]));
+    for (int q = 0; q < 12; ++q) e = fx::emax(e, fx::exponent(n[q]));
     return e;
   }
 };
 
 // 12 h^2 times the order-4 Laplacian: 16 sum (u+-1) - sum (u+-2) - 90 u.  The
 // weights' magnitudes add up to 192, so two guard bits fit in 64 bits.
-CHEMORA_FX double star2_lap(const Star2& s, unsigned e) {
+CHEMORA_FX double star2_lap(const Star2& s, int e) {
   long long s1 = 0, s2 = 0;
 #pragma unroll
   for (int q = 0; q < 12; q += 4) {
@@ -70,7 +70,7 @@ template <class LD, class OUT>
 CHEMORA_FX void wave_point(const LD& ld, const Scalars& sc, OUT& out) {
   Star2 s;
   s.load(ld);
-  const unsigned e = s.exponent();
+  const int e = s.exponent();
   if (fx::in_range(e)) {
     out(0, ld(1, 0, 0, 0));
     out(1, fma(star2_lap(s, e), sc.i12h2, sc.k[CHEMORA_K_MZERO]));

@@ -17,8 +17,8 @@ HARNESS = r"""
 #include "fixedpoint.cuh"
 using namespace chemora;
 extern "C" int lap(const double* n, double c, double* out) {
-  unsigned e = fx::ebits(c);
-  for (int q = 0; q < 12; ++q) e = fx::emax(e, fx::ebits(n[q]));
+  int e = fx::exponent(c);
+  for (int q = 0; q < 12; ++q) e = fx::emax(e, fx::exponent(n[q]));
   if (!fx::in_range(e)) return 0;
   long long s1 = 0, s2 = 0;
   for (int q = 0; q < 12; q += 4) {
@@ -79,6 +79,7 @@ def test_special_values(lap):
     assert lap([3.0] * 12, 3.0) == 0.0
     assert lap([0.0] * 12, -2.0) == 180.0
     assert lap([5e-324] * 12, 1.0) == -90.0
+    assert lap([-0.0, -5e-324] * 6, 1.0) == -90.0
     assert lap([0.0] * 12, 0.0) is None
     assert lap([1.0] * 12, float("nan")) is None
     assert lap([float("inf")] + [1.0] * 11, 1.0) is None
