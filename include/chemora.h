@@ -351,9 +351,9 @@ int chemora_variant_count(int kind);
  * and algebra in two kernels, tx x ty the algebra kernel's block), 1 x-direction work shared across warp lanes (needs
  * nx % tx == 0 and 3 ghost layers), 2 in addition y-direction differences
  * and z-derivative rows shared through shared memory (any ny), 4 (scalar
- * wave, order 4) x-direction work shared across warp lanes and each thread
- * marching along z with a register queue of z first differences (needs
- * nx % tx == 0).  A shape whose condition fails on a grid runs as shape 0.  Outputs may be NULL;
+ * wave, order 4) each thread marching along z with its column's values in
+ * registers and the plane in hand in shared memory.  A shape whose condition
+ * fails on a grid runs as shape 0.  Outputs may be NULL;
  * CHEMORA_EINVAL for an unknown kind or index. */
 int chemora_variant_info(int kind, int variant, int* tx, int* ty, int* min_blocks, int* sharing);
 

@@ -115,11 +115,14 @@ int chemora_variant_info(int kind, int variant, int* tx, int* ty, int* min_block
 int chemora_system_opcount(chemora_system* sys, int64_t* fp64_instructions, int64_t* flops) {
   if (!is_handle(sys, H_SYSTEM)) return set_error(CHEMORA_EINVAL, "not a system handle");
   const LaunchVariant* v = variant_info(sys->kind, sys->variant);
-  if (sys->kind == CHEMORA_WAVE && sys->sc.order == 4) {
-    // the stencil runs on the integer units: one FP64 multiply is left
-    if (fp64_instructions) *fp64_instructions = 1;
-    if (flops) *flops = CHEMORA_OPS_WAVE_FLOPS;
-    return CHEMORA_OK;
+  if (sys->kind == CHEMORA_WAVE || sys->kind == CHEMORA_WAVE1) {
+    // the stencils run on the integer units: one FP64 multiply per evolved
+    // derivative is left
+    int64_t f = 0;
+    const int rc = chemora_opcount(sys->kind, nullptr, &f);
+    if (fp64_instructions) *fp64_instructions = sys->nvars - 1;
+    if (flops) *flops = f;
+    return rc;
   }
   const bool xs = v && v->xshare && sys->grid->d.nx % v->tx == 0 && sys->grid->d.g >= 3;
   if (sys->kind == CHEMORA_BSSN && xs && v->xshare == 2) {

@@ -42,6 +42,11 @@ CHEMORA_FX long long sar(long long a, unsigned s) {
   asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(s));
   return r;
 }
+CHEMORA_FX unsigned long long shr(unsigned long long a, unsigned s) {
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(s));
+  return r;
+}
 CHEMORA_FX int clz64(unsigned long long a) { return __clzll((long long)a); }
 #else
 #define CHEMORA_FX inline
@@ -59,6 +64,7 @@ CHEMORA_FX double from_bits(unsigned long long b) {
 }
 CHEMORA_FX unsigned long long shl(unsigned long long a, unsigned s) { return s > 63 ? 0 : a << s; }
 CHEMORA_FX long long sar(long long a, unsigned s) { return a >> (s > 63 ? 63 : s); }
+CHEMORA_FX unsigned long long shr(unsigned long long a, unsigned s) { return s > 63 ? 0 : a >> s; }
 CHEMORA_FX int clz64(unsigned long long a) { return a ? __builtin_clzll(a) : 64; }
 #endif
 
@@ -82,6 +88,16 @@ CHEMORA_FX Parts parts(double v) {
   return Parts{(long long)((m ^ s) - s), exponent(v)};
 }
 
+// The same, with the exponent of zeros far below every other: a set of values
+// whose largest exponent is kZeroExp is all zeros.
+constexpr int kZeroExp = -4096;
+template <int K>
+CHEMORA_FX Parts parts_or_zero(double v) {
+  Parts p = parts<K>(v);
+  if (((hiword(v) << 1) | loword(v)) == 0) p.e = kZeroExp;
+  return p;
+}
+
 // In units of 2^(E - 1075 - K), E the exponent of the largest value: |result|
 // <= 2^(53 + K).
 CHEMORA_FX long long align(const Parts& p, int e) { return sar(p.m, (unsigned)(e - p.e)); }
@@ -101,8 +117,38 @@ CHEMORA_FX double to_double(long long v, int e) {
   return a == 0 ? 0.0 : from_bits(r);
 }
 
+// A sum of 64-bit integers with constant weights, exact in 96 bits: hi 2^32 + lo.
+struct Sum96 {
+  long long hi = 0, lo = 0;
+  template <int W>
+  CHEMORA_FX void add(long long v) {
+    hi += (long long)W * (int)(v >> 32);
+    if (W > 0)
+      lo += (long long)((unsigned long long)(unsigned)W * (unsigned)v);
+    else
+      lo -= (long long)((unsigned long long)(unsigned)-W * (unsigned)v);
+  }
+};
+template <int K>
+CHEMORA_FX double to_double(const Sum96& v, int e) {
+  const long long h = v.hi + (v.lo >> 32);
+  const unsigned s = (unsigned)(h >> 63);
+  unsigned long long a = (unsigned long long)(h ^ (h >> 63));
+  unsigned b = ((unsigned)v.lo ^ s) - s;
+  a += (s & 1u) & (unsigned)(b == 0);
+  const bool small = a == 0;
+  a = small ? b : a;
+  b = small ? 0u : b;
+  const int lz = clz64(a);
+  const unsigned long long m = shl(a, (unsigned)lz) | shr((unsigned long long)b << 32, (unsigned)(64 - lz));
+  unsigned long long r = (m >> 11) + ((m >> 10) & 1);
+  r += (unsigned long long)(unsigned)(e + (small ? 10 : 42) - K - lz) << 52;
+  r |= (unsigned long long)(s & 0x80000000u) << 32;
+  return a == 0 ? 0.0 : from_bits(r);
+}
+
 #if defined(__CUDACC__)
-// The same through the conversion instruction (nearest, ties to even), which
+// to_double through the conversion instruction (nearest, ties to even), which
 // takes a slot of the FP64 pipe and a few integer operations instead of some
 // thirty of these.
 template <int K>

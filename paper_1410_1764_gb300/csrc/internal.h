@@ -136,6 +136,9 @@ int launch_bssn_stage(const Dims& d, const Scalars& sc, const StageParams& a, cu
                       const FieldWork& work);
 int launch_wave_order_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s,
                             int variant);
+// Order-4 wave on planes in shared memory (wave_orders.cu).
+template <int TX, int TY>
+int launch_wave_planes(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s);
 int launch_wave1_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s, int variant);
 
 // A compiled launch shape of a stage kernel (tx x ty threads, min blocks/SM).
@@ -144,9 +147,8 @@ struct LaunchVariant {
   int tx, ty, minb;
   StageLaunchFn launch;
   int xshare;  // 1: lanes share x-direction work (nx % tx == 0); 2: and y via
-               // shared memory; 4: z-march with the column's values in
-               // registers (order-4 wave); 8: the one-point body on
-               // a cp.async-staged tile with halos (order-4 wave; any nx)
+               // shared memory; 4: z-march, the column in registers,
+               // the plane in hand in shared memory (order-4 wave)
 };
 extern const LaunchVariant kBssnVariants[];
 extern const int kNumBssnVariants;
