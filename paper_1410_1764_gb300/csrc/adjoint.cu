@@ -19,59 +19,23 @@
 // derivatives of u; the newest segment's tape is written by the forward
 // pass itself.
 //
-// Every product is formed at the neighbour points and then differenced, the
-// same order as the oracle's definition; a point is written by one thread,
-// so results are deterministic.
+// Every product is formed at the neighbour points and then differenced, as the
+// oracle's definition does; a point is written by one thread, so results are
+// deterministic.
 #include <math.h>
 #include <string.h>
 
 #include <vector>
 
 #include "internal.h"
+#include "varc_march.cuh"
 
 namespace chemora {
 
 constexpr int ATX = 32, ATY = 8;
 
-// FP64 constants of the stage kernels, passed as a kernel parameter.  Every
-// add is issued as fma(b, one, a) and every product as fma(a, b, mzero)
-// (mzero = -0.0): both give exactly the add's or the product's result, and
-// no operand is an immediate.  On GB300 an fma with register or
-// constant-bank operands issues faster than DADD, DMUL or an fma with an
-// immediate operand.
-struct FmaK {
-  double one, mzero, eight, sixteen, two;
-};
-
-static FmaK fma_k() { return FmaK{1.0, -0.0, 8.0, 16.0, 2.0}; }
-
 __device__ __forceinline__ int64_t at_(const Dims& d, int i, int j, int k) {
   return (int64_t)(k + d.g) * d.sz + (int64_t)(j + d.g) * d.sy + (i + d.g);
-}
-
-// Store v at interior point (i, j, k) (offset c) of a grid function and, when
-// `imaged`, also at each of its periodic images in the ghost zones (points
-// within g of a face have one image per near face, and edge and corner
-// images): the ghost zones are then valid without a fill pass.  Needs
-// n >= g on every axis (each ghost point then has exactly one interior
-// source), which the host checks before passing imaged = 1.
-__device__ __forceinline__ void store_imaged(double* f, const Dims& d, int i, int j, int k, int64_t c, double v,
-                                             int imaged) {
-  f[c] = v;
-  if (!imaged) return;
-  const int g = d.g;
-  int64_t xs[3] = {0, 0, 0}, ys[3] = {0, 0, 0}, zs[3] = {0, 0, 0};
-  int nx = 1, ny = 1, nz = 1;
-  if (i < g) xs[nx++] = d.nx;
-  if (i >= d.nx - g) xs[nx++] = -d.nx;
-  if (j < g) ys[ny++] = (int64_t)d.ny * d.sy;
-  if (j >= d.ny - g) ys[ny++] = -(int64_t)d.ny * d.sy;
-  if (k < g) zs[nz++] = (int64_t)d.nz * d.sz;
-  if (k >= d.nz - g) zs[nz++] = -(int64_t)d.nz * d.sz;
-  for (int a = 0; a < nx; ++a)
-    for (int b = 0; b < ny; ++b)
-      for (int e = 0; e < nz; ++e)
-        if (a | b | e) f[c + xs[a] + ys[b] + zs[e]] = v;
 }
 
 // G_d = D_d s on the interior (3 grid functions).
@@ -91,112 +55,196 @@ __global__ void __launch_bounds__(ATX * ATY) varc_grad_s_kernel(Dims d, double i
   }
 }
 
-// Forward RK stage of the variable-speed wave equation (modes as in the
-// stage kernels), optionally writing the tape: Lap u and D_d u of the stage
-// state src.
-__global__ void __launch_bounds__(ATX * ATY)
-varc_fwd_stage_kernel(Dims d, double i12h, double i12h2, const double* __restrict__ s,
-                      const double* __restrict__ G, StageParams a, double* __restrict__ tape, FmaK K,
-                      int imaged) {
-  const int i = blockIdx.x * ATX + threadIdx.x, j = blockIdx.y * ATY + threadIdx.y, k = blockIdx.z;
-  if (i >= d.nx || j >= d.ny) return;
-  const int64_t c = at_(d, i, j, k);
-  const int64_t st[3] = {1, d.sy, d.sz};
-  const double* u = a.src + c;
-  const double f0 = u[0];
-  double lap = K.mzero, adv = K.mzero, du[3];
+// One transposed stage (see the file comment) on the tile's columns, marching
+// through z.  The stencils act on the products s w, G_d w and w D_d u_q, formed
+// once per point (and once more per halo cell) and differenced on the integer
+// units (star_march.cuh): x and y neighbours come from the plane in shared
+// memory, z neighbours from the thread's registers.  Six guard bits for the
+// Laplacian and products rounded to nearest: values cut off downwards leave an
+// error that adds up over the steps (with two, and products cut off, grad_u0
+// of 24 steps on 64^3 was 18 % further from exact values than FP64 sums).
+//
+// GB300, 128^3: 118 us, against 320 us when each point formed the 37 products
+// of its stencils itself in FP64 (72 instructions of 17.8 cycles).  Products in
+// FP64 here: 123 us.  640 threads per SM (20 bytes spilled): 7 % more.  Bound by
+// the latency of its integer chains at 16 warps per SM; ten FP64 instructions
+// per point are left (36 us), HBM alone takes 47 us.
+// kb: 2 grid functions with valid ghosts; coef: s and G_d (ghosts valid); tape:
+// Lap u_q (interior) and 12 h D_d u_q (ghosts valid).  first: yacc = yp + yhat
+// (else yacc += yhat).  kbn (if non-NULL): kbn = cq yp + aq yhat, or, after the
+// step's last stage, cq yacc.
+constexpr int kAdjThreads = 512;  // resident threads per SM
+template <int TX, int TY>
+__global__ void __launch_bounds__(TX * TY, kAdjThreads / (TX * TY))
+varc_adj_march_kernel(Dims d, double i12h, double i12h2, double i144h2, const double* __restrict__ kb,
+                      const double* __restrict__ coef, const double* __restrict__ tape,
+                      const double* __restrict__ yp, double* __restrict__ yacc, double* __restrict__ kbn,
+                      double* __restrict__ sbar, double cq, double aq, int first, int last, int zb,
+                      double one, double mzero, int imaged) {
+  constexpr int R = 2, P = TX + 2 * R;
+  constexpr int KA = 6, KD = Guard<R>::d1;
+  // s w with both halos; G_x w and w D_x u with the x halo; G_y w and w D_y u with the y halo
+  constexpr int NA = P * (TY + 2 * R), NX = P * TY, NY = TX * (TY + 2 * R);
+  __shared__ long long pm[2][NA + 2 * NX + 2 * NY];
+  __shared__ int pe[2][NA + 2 * NX + 2 * NY];
+  const MarchPlace<TX, TY> p(d, zb);
+  const MarchHalo<R, TX, TY> hl(p);
+  const int64_t own = (int64_t)p.ly * d.sy + p.lx;
+  const int oa = (p.ly + R) * P + p.lx + R;
+  const int ox = NA + p.ly * P + p.lx + R;                 // G_x w, then w D_x u NX further
+  const int oy = NA + 2 * NX + (p.ly + R) * TX + p.lx;     // G_y w, then w D_y u NY further
+  const double* w = kb + d.sv;                             // kb_rho
+  const double* cz = coef + 3 * d.sv;                      // G_z
+  const double* tz = tape + 3 * d.sv;
+  auto mul = [&](double x, double y) { return __fma_rn(x, y, mzero); };
+  fx::Parts za[5], zg[5], zt[5];  // s w, G_z w, w D_z u of the column
 #pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    const int64_t o = st[q];
-    const double up1 = u[o], um1 = u[-o], up2 = u[2 * o], um2 = u[-2 * o];
-    // (u+1 - f0) + (u-1 - f0), (u+2 - f0) + (u-2 - f0)
-    const double d1 = fma(fma(f0, -K.one, um1), K.one, fma(f0, -K.one, up1));
-    const double d2 = fma(fma(f0, -K.one, um2), K.one, fma(f0, -K.one, up2));
-    lap = fma(fma(K.sixteen, d1, -d2), i12h2, lap);
-    // (8 (u+1 - u-1) - (u+2 - u-2)) / (12 h)
-    const double t = fma(K.eight, fma(um1, -K.one, up1), -fma(um2, -K.one, up2));
-    du[q] = fma(t, i12h, K.mzero);
-    adv = fma(G[q * d.sv + c], du[q], adv);
-  }
-  const double krho = fma(s[c], lap, adv);
-  const double ku = a.src[d.sv + c];
-  const double kk[2] = {ku, krho};
+  for (int m = 0; m < 5; ++m) za[m] = zg[m] = zt[m] = fx::Parts{0, 0};
+  int64_t c = p.org + own;
+  if (p.active) {
 #pragma unroll
-  for (int v = 0; v < 2; ++v) {
-    const int64_t cv = c + v * d.sv;
-    const double k_ = kk[v];
-    // the scalar-wave systems' RK update, each product contracted into its
-    // addition (as StageOutFma in the other wave kernels)
-    switch (a.mode) {
-      case 1:  // acc = k; dst = yn + c2 k
-        a.acc[cv] = k_;
-        store_imaged(a.dst, d, i, j, k, cv, fma(a.c2, k_, a.yn[cv]), imaged);
-        break;
-      case 2:
-      case 3:  // acc += 2 k; dst = yn + c2 k
-        a.acc[cv] = fma(K.two, k_, a.acc[cv]);
-        store_imaged(a.dst, d, i, j, k, cv, fma(a.c2, k_, a.yn[cv]), imaged);
-        break;
-      default:  // dst = yn + c1 (acc + k)
-        store_imaged(a.dst, d, i, j, k, cv, fma(a.c1, fma(a.acc[cv], K.one, k_), a.yn[cv]), imaged);
-        break;
+    for (int m = 1; m < 5; ++m) {
+      const int64_t o = c + (int64_t)(m - 3) * d.sz;
+      const fx::Factor<11> wv = fx::factor<11>(__ldg(w + o));
+      za[m] = fx::product<KA>(wv, fx::factor<KA + 1>(__ldg(coef + o)));
+      zg[m] = fx::product<KD>(wv, fx::factor<KD + 1>(__ldg(cz + o)));
+      zt[m] = fx::product<KD>(wv, fx::factor<KD + 1>(__ldg(tz + o)));
     }
   }
-  if (tape) {
-    tape[c] = lap;  // read at the point only
-    // D_d u_q is read at stencil neighbours by the transposed stage
-    store_imaged(tape, d, i, j, k, d.sv + c, du[0], imaged);
-    store_imaged(tape, d, i, j, k, 2 * d.sv + c, du[1], imaged);
-    store_imaged(tape, d, i, j, k, 3 * d.sv + c, du[2], imaged);
-  }
-}
-
-// One transposed stage (see the file comment).  kb: 2 grid functions with
-// valid ghosts; tape: Lap u_q (interior) and D_d u_q (ghosts valid).
-// first: yacc = yp + yhat (else yacc += yhat).  kbn (if non-NULL):
-// kbn = cq yp + aq yhat.
-__global__ void __launch_bounds__(ATX * ATY)
-varc_adj_stage_kernel(Dims d, double i12h, double i12h2, const double* __restrict__ kb,
-                      const double* __restrict__ s, const double* __restrict__ G,
-                      const double* __restrict__ tape, const double* __restrict__ yp,
-                      double* __restrict__ yacc, double* __restrict__ kbn, double* __restrict__ sbar,
-                      double cq, double aq, int first, FmaK K, int imaged) {
-  const int i = blockIdx.x * ATX + threadIdx.x, j = blockIdx.y * ATY + threadIdx.y, k = blockIdx.z;
-  if (i >= d.nx || j >= d.ny) return;
-  const int64_t c = at_(d, i, j, k);
-  const int64_t st[3] = {1, d.sy, d.sz};
-  const double* w = kb + d.sv + c;  // kb_rho
-  const double* sp = s + c;
-  const double t0 = fma(sp[0], w[0], K.mzero);
-  double lap_sw = K.mzero, div1 = K.mzero, div2 = K.mzero;
+#pragma unroll 1
+  for (int k = 0; k < p.nz; ++k, c += d.sz) {
+    long long* const M = pm[k & 1];
+    int* const E = pe[k & 1];
+    double wc = 0.0, kbu = 0.0, lapu = 0.0, y0 = 0.0, y1 = 0.0, a0 = 0.0, a1 = 0.0, sb = 0.0;
 #pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    const int64_t o = st[q];
-    const double wp1 = w[o], wm1 = w[-o], wp2 = w[2 * o], wm2 = w[-2 * o];
-    // Lap(s w): second differences of the product s w from the centre, each
-    // neighbour's product minus the centre's in one fma
-    const double d1 = fma(fma(sp[-o], wm1, -t0), K.one, fma(sp[o], wp1, -t0));
-    const double d2 = fma(fma(sp[-2 * o], wm2, -t0), K.one, fma(sp[2 * o], wp2, -t0));
-    lap_sw = fma(fma(K.sixteen, d1, -d2), i12h2, lap_sw);
-    // D_d(G_d w): (8 (p+1 - p-1) - (p+2 - p-2)) / (12 h), p = G_d w
-    const double* g = G + q * d.sv + c;
-    const double g1 = fma(g[o], wp1, -fma(g[-o], wm1, K.mzero));
-    const double g2 = fma(g[2 * o], wp2, -fma(g[-2 * o], wm2, K.mzero));
-    div1 = fma(fma(K.eight, g1, -g2), i12h, div1);
-    // D_d(w D_d u_q), the same with p = w D_d u_q
-    const double* pu = tape + (1 + q) * d.sv + c;
-    const double h1 = fma(wp1, pu[o], -fma(wm1, pu[-o], K.mzero));
-    const double h2 = fma(wp2, pu[2 * o], -fma(wm2, pu[-2 * o], K.mzero));
-    div2 = fma(fma(K.eight, h1, -h2), i12h, div2);
-  }
-  const double yh[2] = {fma(div1, -K.one, lap_sw), kb[c]};
-  sbar[c] = fma(fma(w[0], tape[c], -div2), K.one, sbar[c]);
+    for (int m = 0; m < 4; ++m) {
+      za[m] = za[m + 1];
+      zg[m] = zg[m + 1];
+      zt[m] = zt[m + 1];
+    }
+    auto put = [&](int o, const fx::Parts& v) {
+      M[o] = v.m;
+      E[o] = v.e;
+    };
+    if (p.active) {
+      const int64_t o = c + 2 * d.sz;
+      const double wz = __ldg(w + o), sz = __ldg(coef + o), gz = __ldg(cz + o), uz = __ldg(tz + o);
+      wc = __ldg(w + c);
+      const double gx = __ldg(coef + d.sv + c), gy = __ldg(coef + 2 * d.sv + c);
+      const double ux = __ldg(tape + d.sv + c), uy = __ldg(tape + 2 * d.sv + c);
+      kbu = __ldg(kb + c);
+      lapu = __ldg(tape + c);
+      y0 = __ldg(yp + c);
+      y1 = __ldg(yp + d.sv + c);
+      a0 = first ? y0 : yacc[c];
+      a1 = first ? y1 : yacc[d.sv + c];
+      sb = sbar[c];
+      const fx::Factor<11> fz = fx::factor<11>(wz), fc = fx::factor<11>(wc);
+      za[4] = fx::product<KA>(fz, fx::factor<KA + 1>(sz));
+      zg[4] = fx::product<KD>(fz, fx::factor<KD + 1>(gz));
+      zt[4] = fx::product<KD>(fz, fx::factor<KD + 1>(uz));
+      put(oa, za[2]);
+      put(ox, fx::product<KD>(fc, fx::factor<KD + 1>(gx)));
+      put(ox + NX, fx::product<KD>(fc, fx::factor<KD + 1>(ux)));
+      put(oy, fx::product<KD>(fc, fx::factor<KD + 1>(gy)));
+      put(oy + NY, fx::product<KD>(fc, fx::factor<KD + 1>(uy)));
+    }
 #pragma unroll
-  for (int v = 0; v < 2; ++v) {
-    const int64_t cv = c + v * d.sv;
-    yacc[cv] = fma(yh[v], K.one, first ? yp[cv] : yacc[cv]);
-    if (kbn)  // the next transposed stage reads kb at stencil neighbours
-      store_imaged(kbn, d, i, j, k, cv, fma(fma(aq, yh[v], K.mzero), K.one, fma(cq, yp[cv], K.mzero)), imaged);
+    for (int q = 0; q < hl.n; ++q)
+      if (hl.live[q]) {
+        const int64_t o = p.org + k * d.sz + (int64_t)hl.y[q] * d.sy + hl.x[q];
+        const int64_t ax = (hl.along_x[q] ? 1 : 2) * d.sv;
+        const fx::Factor<11> wv = fx::factor<11>(__ldg(w + o));
+        put((hl.y[q] + R) * P + hl.x[q] + R, fx::product<KA>(wv, fx::factor<KA + 1>(__ldg(coef + o))));
+        const int b = hl.along_x[q] ? NA + hl.y[q] * P + hl.x[q] + R : NA + 2 * NX + (hl.y[q] + R) * TX + hl.x[q];
+        put(b, fx::product<KD>(wv, fx::factor<KD + 1>(__ldg(coef + ax + o))));
+        put(b + (hl.along_x[q] ? NX : NY), fx::product<KD>(wv, fx::factor<KD + 1>(__ldg(tape + ax + o))));
+      }
+    __syncthreads();
+    if (!p.active) continue;
+    double lap = 0.0, div[2] = {0.0, 0.0};  // of s w; of G_d w and of w D_d u
+    {
+      int ex[4], ey[4], e = za[2].e;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        ex[m] = E[oa + tap<R>(m)];
+        ey[m] = E[oa + tap<R>(m) * P];
+        e = fx::emax(e, fx::emax(fx::emax(ex[m], ey[m]), za[2 + tap<R>(m)].e));
+      }
+      if (!star_ok<R>(e)) {
+        const int64_t st[3] = {1, d.sy, d.sz};
+        const double t0 = mul(coef[c], w[c]);
+#pragma unroll 1
+        for (int q = 0; q < 3; ++q)
+          for (int m = 1; m <= 2; ++m) {
+            const int64_t o = m * st[q];
+            const double v = (coef[c + o] * w[c + o] - t0) + (coef[c - o] * w[c - o] - t0);
+            lap = __fma_rn(m == 1 ? 16.0 : -1.0, v, lap);
+          }
+      } else if (e != fx::kZeroExp) {
+        long long s2[R] = {0, 0};
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const int o = tap<R>(m), q = o < 0 ? -o - 1 : o - 1;
+          s2[q] += fx::sar(M[oa + o], (unsigned)(e - ex[m])) + fx::sar(M[oa + o * P], (unsigned)(e - ey[m])) +
+                   fx::align(za[2 + o], e);
+        }
+        lap = star_lap<R, KA>(s2, fx::align(za[2], e), e);
+      }
+    }
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+      const int bx = ox + f * NX, by = oy + f * NY;
+      int ex[4], ey[4], e = fx::kZeroExp;
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        ex[m] = E[bx + tap<R>(m)];
+        ey[m] = E[by + tap<R>(m) * TX];
+        e = fx::emax(e, fx::emax(fx::emax(ex[m], ey[m]), (f ? zt : zg)[2 + tap<R>(m)].e));
+      }
+      if (!star_ok<R>(e)) {
+        const int64_t st[3] = {1, d.sy, d.sz};
+        double v = 0.0;
+#pragma unroll 1
+        for (int q = 0; q < 3; ++q) {
+          const double* g = (f ? tape : coef) + (1 + q) * d.sv + c;
+          const double* wv = w + c;
+          for (int m = 1; m <= 2; ++m) {
+            const int64_t o = m * st[q];
+            v = __fma_rn(m == 1 ? 8.0 : -1.0, g[o] * wv[o] - g[-o] * wv[-o], v);
+          }
+        }
+        div[f] = v;
+      } else if (e != fx::kZeroExp) {
+        long long t[R];
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          const int u1 = R + q, dn = R - 1 - q, o = q + 1;
+          const fx::Parts& zu = (f ? zt : zg)[2 + o];
+          const fx::Parts& zd = (f ? zt : zg)[2 - o];
+          t[q] = (fx::sar(M[bx + o], (unsigned)(e - ex[u1])) - fx::sar(M[bx - o], (unsigned)(e - ex[dn]))) +
+                 (fx::sar(M[by + o * TX], (unsigned)(e - ey[u1])) - fx::sar(M[by - o * TX], (unsigned)(e - ey[dn]))) +
+                 (fx::align(zu, e) - fx::align(zd, e));
+        }
+        div[f] = star_d1<R>(t, e);
+      }
+    }
+    const double yh = __fma_rn(div[0], -i12h, mul(lap, i12h2));
+    sbar[c] = __fma_rn(wc, lapu, __fma_rn(div[1], -i144h2, sb));
+    a0 = __fma_rn(yh, one, a0);
+    a1 = __fma_rn(kbu, one, a1);
+    yacc[c] = a0;
+    yacc[d.sv + c] = a1;
+    if (kbn) {  // the next transposed stage reads kb at stencil neighbours
+      const int i = p.x0 + p.lx, j = p.y0 + p.ly, kz = p.k0 + k;
+      double n0 = mul(cq, last ? a0 : y0), n1 = mul(cq, last ? a1 : y1);
+      if (!last) {
+        n0 = __fma_rn(aq, yh, n0);
+        n1 = __fma_rn(aq, kbu, n1);
+      }
+      store_imaged(kbn, d, i, j, kz, c, n0, imaged);
+      store_imaged(kbn, d, i, j, kz, d.sv + c, n1, imaged);
+    }
   }
 }
 
@@ -264,18 +312,20 @@ int launch_varc_grad(const Dims& d, double i12h, const double* s, double* G, cud
 }
 
 struct AdjBufs {
-  double *s, *G, *Y, *ck, *seg, *tape, *yp, *yacc, *kb, *kbn, *sbar, *loss;
+  double *s, *G,  // G right behind s
+       *Y, *ck, *tape, *yp, *yacc, *kb, *kbn, *sbar, *loss;
   int64_t* recv;
   double* data;
 };
 
-// One forward RK4 step of the variable-speed wave (in place on Y), tape of
-// the 4 stages written at tape (16 grid functions) when non-NULL.
-// Stage outputs written with their ghost images (no fill passes) when every
+// Stage outputs are written with their ghost images (no fill passes) when every
 // axis has at least g points.
 static int imaged_ok(const Dims& d) { return d.nx >= d.g && d.ny >= d.g && d.nz >= d.g ? 1 : 0; }
 
-static int fwd_step(chemora_system* sys, const AdjBufs& B, double* Y, double dt, double* tape,
+// One forward RK4 step of the variable-speed wave from Y to Ynext (which may
+// be Y), tape of the 4 stages written at tape (16 grid functions) when
+// non-NULL.
+static int fwd_step(chemora_system* sys, const AdjBufs& B, double* Y, double* Ynext, double dt, double* tape,
                     cudaStream_t s) {
   const Dims& d = sys->grid->d;
   const int im = imaged_ok(d);
@@ -283,42 +333,45 @@ static int fwd_step(chemora_system* sys, const AdjBufs& B, double* Y, double dt,
   double* A = sys->scratch;
   double* Sa = sys->scratch + 2 * fs;
   double* Sb = sys->scratch + 4 * fs;
-  const double i12h = sys->sc.i12h, i12h2 = sys->sc.i12h2;
   StageParams p{};
   int rc;
   double* srcs[4] = {Y, Sa, Sb, Sa};
-  double* dsts[4] = {Sa, Sb, Sa, Y};
+  double* dsts[4] = {Sa, Sb, Sa, Ynext};
   const double c2[4] = {0.5 * dt, 0.5 * dt, dt, 0.0};
   for (int q = 0; q < 4; ++q) {
     if (!im && (rc = fill_ghosts(d, 2, srcs[q], s))) return rc;
     p.src = srcs[q]; p.yn = Y; p.acc = A; p.dst = dsts[q]; p.c1 = dt / 6.0; p.c2 = c2[q]; p.mode = q + 1;
-    varc_fwd_stage_kernel<<<agrid(d), dim3(ATX, ATY), 0, s>>>(d, i12h, i12h2, B.s, B.G, p,
-                                                                tape ? tape + (size_t)q * 4 * fs : nullptr,
-                                                                fma_k(), im);
-    if ((rc = launched("varc_fwd_stage_kernel"))) return rc;
+    p.coef = B.s;
+    if ((rc = launch_varc_march<32, 4>(d, sys->sc, p, tape ? tape + (size_t)q * 4 * fs : nullptr, im, s))) return rc;
   }
-  return im ? CHEMORA_OK : fill_ghosts(d, 2, Y, s);
+  return im ? CHEMORA_OK : fill_ghosts(d, 2, Ynext, s);
 }
 
-// One reverse RK4 step: on entry B.yp holds ybar'; on exit B.yacc holds ybar_n.
-static int rev_step(chemora_system* sys, const AdjBufs& B, const double* tape, double dt, cudaStream_t s) {
+// One reverse RK4 step: on entry B.yp holds ybar' and, unless it is the first,
+// B.kb dt/6 ybar'; on exit B.yacc holds ybar_n and, unless it is the last, B.kb
+// dt/6 ybar_n.
+static int rev_step(chemora_system* sys, const AdjBufs& B, const double* tape, double dt, bool first_step,
+                    bool last_step, cudaStream_t s) {
   const Dims& d = sys->grid->d;
   const size_t fs = sys->grid->fsize;
   const double i12h = sys->sc.i12h, i12h2 = sys->sc.i12h2;
-  const int im = imaged_ok(d);
+  constexpr int ADJX = 32, ADJY = 4;
+  const int im = imaged_ok(d), zb = march_depth(d, ADJX, ADJY, kAdjThreads / (ADJX * ADJY));
   int rc;
-  scale_state_kernel<<<agrid(d), dim3(ATX, ATY), 0, s>>>(d, dt / 6.0, B.yp, B.kb, im);
-  if ((rc = launched("scale_state_kernel"))) return rc;
-  const double cq[4] = {0.0, dt / 6.0, dt / 3.0, dt / 3.0};  // weight of ybar' in kb_{q-1}
+  if (first_step) {
+    scale_state_kernel<<<agrid(d), dim3(ATX, ATY), 0, s>>>(d, dt / 6.0, B.yp, B.kb, im);
+    if ((rc = launched("scale_state_kernel"))) return rc;
+  }
+  const double cq[4] = {dt / 6.0, dt / 6.0, dt / 3.0, dt / 3.0};  // weight of ybar' in kb_{q-1} (of ybar_n: q = 0)
   const double aq[4] = {0.0, 0.5 * dt, 0.5 * dt, dt};        // a_q dt
   double* kb = B.kb;
   double* kbn = B.kbn;
   for (int q = 3; q >= 0; --q) {
     if (!im && (rc = fill_ghosts(d, 2, kb, s))) return rc;
-    varc_adj_stage_kernel<<<agrid(d), dim3(ATX, ATY), 0, s>>>(
-        d, i12h, i12h2, kb, B.s, B.G, tape + (size_t)q * 4 * fs, B.yp, B.yacc, q > 0 ? kbn : nullptr,
-        B.sbar, cq[q], aq[q], q == 3 ? 1 : 0, fma_k(), im);
-    if ((rc = launched("varc_adj_stage_kernel"))) return rc;
+    varc_adj_march_kernel<ADJX, ADJY><<<march_grid(d, ADJX, ADJY, zb), ADJX * ADJY, 0, s>>>(
+        d, i12h, i12h2, sys->sc.i144h2, kb, B.s, tape + (size_t)q * 4 * fs, B.yp, B.yacc,
+        q > 0 || !last_step ? kbn : nullptr, B.sbar, cq[q], aq[q], q == 3 ? 1 : 0, q == 0 ? 1 : 0, zb, sys->sc.k[CHEMORA_K_ONE], sys->sc.k[CHEMORA_K_MZERO], im);
+    if ((rc = launched("varc_adj_march_kernel"))) return rc;
     double* t = kb;
     kb = kbn;
     kbn = t;
@@ -356,11 +409,18 @@ extern "C" int chemora_adjoint_rk4(chemora_system* sys, const double* state0, co
   cudaStream_t s = (cudaStream_t)stream;
   const int K = ckpt_every < nsteps ? ckpt_every : nsteps;
   const int nck = (nsteps + K - 1) / K;
-  // fields: s 1, G 3, Y 2, ck 2 nck, seg 2 K, tape 16 K, yp 2, yacc 2, kb 2, kbn 2, sbar 1, loss
-  const size_t nfields = 1 + 3 + 2 + 2 * (size_t)nck + 2 * (size_t)K + 16 * (size_t)K + 2 + 2 + 2 + 2 + 1;
+  // fields: s 1, G 3, Y 2, ck 2 nck, tape 16 K, yp 2, yacc 2, kb 2, kbn 2, sbar 1, loss
+  const size_t nfields = 1 + 3 + 2 + 2 * (size_t)nck + 16 * (size_t)K + 2 + 2 + 2 + 2 + 1;
   const size_t bytes = (nfields * fs + 32) * sizeof(double) + (size_t)nrecv * (sizeof(int64_t) + sizeof(double));
   char* buf = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&buf, bytes, s);
+  // kept by the system's pool: from the device's own pool, which gives freed
+  // memory back at each synchronisation, 3.4 GB cost about 10 ms a call
+  const cudaMemPool_t pool = system_pool(sys);
+  cudaError_t e = pool ? cudaMallocFromPoolAsync((void**)&buf, bytes, pool, s) : cudaErrorMemoryAllocation;
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    e = cudaMallocAsync((void**)&buf, bytes, s);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     return set_error(CHEMORA_ENOMEM, "adjoint work space of %zu bytes: %s", bytes, cudaGetErrorString(e));
@@ -371,7 +431,6 @@ extern "C" int chemora_adjoint_rk4(chemora_system* sys, const double* state0, co
   B.G = q; q += 3 * fs;
   B.Y = q; q += 2 * fs;
   B.ck = q; q += 2 * (size_t)nck * fs;
-  B.seg = q; q += 2 * (size_t)K * fs;
   B.tape = q; q += 16 * (size_t)K * fs;
   B.yp = q; q += 2 * fs;
   B.yacc = q; q += 2 * fs;
@@ -398,41 +457,34 @@ extern "C" int chemora_adjoint_rk4(chemora_system* sys, const double* state0, co
     // tape here (the same kernel on the same states as a recomputation), so
     // the reverse sweep recomputes only the older segments
     const int nlast = (nck - 1) * K;
-    CHEMORA_CUDA(cudaMemcpyAsync(B.Y, state0, 2 * fs * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    if ((r = fill_ghosts(d, 2, B.Y, s))) return r;
+    auto ckpt = [&](int q) { return B.ck + (size_t)q * 2 * fs; };
+    double* y = ckpt(0);
+    CHEMORA_CUDA(cudaMemcpyAsync(y, state0, 2 * fs * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    if ((r = fill_ghosts(d, 2, y, s))) return r;
     for (int n = 0; n < nsteps; ++n) {
-      if (n % K == 0)
-        CHEMORA_CUDA(cudaMemcpyAsync(B.ck + (size_t)(n / K) * 2 * fs, B.Y, 2 * fs * sizeof(double),
-                                     cudaMemcpyDeviceToDevice, s));
       double* tp = n >= nlast ? B.tape + (size_t)(n - nlast) * 16 * fs : nullptr;
-      if ((r = fwd_step(sys, B, B.Y, dt, tp, s))) return r;
+      double* next = (n + 1) % K == 0 && n + 1 < nsteps ? ckpt((n + 1) / K) : B.Y;
+      if ((r = fwd_step(sys, B, y, next, dt, tp, s))) return r;
+      y = next;
     }
     // loss and seed
-    receivers_kernel<<<1, 1024, 0, s>>>(B.Y, B.recv, B.data, nrecv, B.yp, B.loss);
+    receivers_kernel<<<1, 1024, 0, s>>>(y, B.recv, B.data, nrecv, B.yp, B.loss);
     if ((r = launched("receivers_kernel"))) return r;
     // reverse sweep, newest segment first
     for (int sg = nck - 1; sg >= 0; --sg) {
       const int n0 = sg * K, n1 = (n0 + K < nsteps) ? n0 + K : nsteps;
-      if (sg < nck - 1)
-        CHEMORA_CUDA(cudaMemcpyAsync(B.seg, B.ck + (size_t)sg * 2 * fs, 2 * fs * sizeof(double),
-                                     cudaMemcpyDeviceToDevice, s));
-      for (int n = n0; n < n1 && sg < nck - 1; ++n) {
-        double* yn = B.seg + (size_t)(n - n0) * 2 * fs;
-        if (n + 1 < n1) {
-          double* y1 = yn + 2 * fs;
-          CHEMORA_CUDA(cudaMemcpyAsync(y1, yn, 2 * fs * sizeof(double), cudaMemcpyDeviceToDevice, s));
-          if ((r = fwd_step(sys, B, y1, dt, B.tape + (size_t)(n - n0) * 16 * fs, s))) return r;
-        } else {
-          // last step of the segment: only its tape is needed
-          CHEMORA_CUDA(cudaMemcpyAsync(B.Y, yn, 2 * fs * sizeof(double), cudaMemcpyDeviceToDevice, s));
-          if ((r = fwd_step(sys, B, B.Y, dt, B.tape + (size_t)(n - n0) * 16 * fs, s))) return r;
+      if (sg < nck - 1) {
+        y = ckpt(sg);
+        for (int n = n0; n < n1; ++n) {
+          if ((r = fwd_step(sys, B, y, B.Y, dt, B.tape + (size_t)(n - n0) * 16 * fs, s))) return r;
+          y = B.Y;
         }
       }
       // the tape's D_d u fields are read at stencil neighbours: periodic
       // ghosts (written with their images by the forward kernel when it can)
       if (!imaged_ok(d) && (r = fill_ghosts(d, 16 * (n1 - n0), B.tape, s))) return r;
       for (int n = n1 - 1; n >= n0; --n) {
-        if ((r = rev_step(sys, B, B.tape + (size_t)(n - n0) * 16 * fs, dt, s))) return r;
+        if ((r = rev_step(sys, B, B.tape + (size_t)(n - n0) * 16 * fs, dt, n == nsteps - 1, n == 0, s))) return r;
         double* t = B.yp;
         B.yp = B.yacc;
         B.yacc = t;

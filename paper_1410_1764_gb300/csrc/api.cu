@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <atomic>
+#include <mutex>
 #include <new>
 
 #include "internal.h"
@@ -183,6 +184,23 @@ FieldWork system_field_work(chemora_system* sys, bool alloc) {
   return w;
 }
 
+cudaMemPool_t system_pool(chemora_system* sys) {
+  static std::mutex m;  // right-hand sides of one system may run in several threads
+  const std::lock_guard<std::mutex> lock(m);
+  if (sys->pool) return sys->pool;
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  if (cudaGetDevice(&props.location.id) != cudaSuccess || cudaMemPoolCreate(&sys->pool, &props) != cudaSuccess) {
+    sys->pool = nullptr;
+    cudaGetLastError();
+    return nullptr;
+  }
+  uint64_t keep = (uint64_t)8 << 30;  // memory kept between calls, until the system is destroyed
+  cudaMemPoolSetAttribute(sys->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  return sys->pool;
+}
+
 FieldWork take_field_work(chemora_system* sys, cudaStream_t s) {
   FieldWork w;
   cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
@@ -190,21 +208,11 @@ FieldWork take_field_work(chemora_system* sys, cudaStream_t s) {
     cudaGetLastError();
     return w;
   }
-  if (!sys->pool) {
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    if (cudaGetDevice(&props.location.id) != cudaSuccess || cudaMemPoolCreate(&sys->pool, &props) != cudaSuccess) {
-      sys->pool = nullptr;
-      cudaGetLastError();
-      return w;
-    }
-    uint64_t keep = UINT64_MAX;  // memory stays with the pool between calls, until the system is destroyed
-    cudaMemPoolSetAttribute(sys->pool, cudaMemPoolAttrReleaseThreshold, &keep);
-  }
+  const cudaMemPool_t pool = system_pool(sys);
+  if (!pool) return w;
   const int64_t points = field_work_points(sys->grid->d);
   void* p = nullptr;
-  if (cudaMallocFromPoolAsync(&p, field_work_bytes(points), sys->pool, s) != cudaSuccess) {
+  if (cudaMallocFromPoolAsync(&p, field_work_bytes(points), pool, s) != cudaSuccess) {
     cudaGetLastError();
     return w;
   }

@@ -48,6 +48,7 @@ CHEMORA_FX unsigned long long shr(unsigned long long a, unsigned s) {
   return r;
 }
 CHEMORA_FX int clz64(unsigned long long a) { return __clzll((long long)a); }
+CHEMORA_FX unsigned long long mulhi64(unsigned long long a, unsigned long long b) { return __umul64hi(a, b); }
 #else
 #define CHEMORA_FX inline
 CHEMORA_FX unsigned long long bits(double v) {
@@ -66,6 +67,9 @@ CHEMORA_FX unsigned long long shl(unsigned long long a, unsigned s) { return s >
 CHEMORA_FX long long sar(long long a, unsigned s) { return a >> (s > 63 ? 63 : s); }
 CHEMORA_FX unsigned long long shr(unsigned long long a, unsigned s) { return s > 63 ? 0 : a >> s; }
 CHEMORA_FX int clz64(unsigned long long a) { return a ? __builtin_clzll(a) : 64; }
+CHEMORA_FX unsigned long long mulhi64(unsigned long long a, unsigned long long b) {
+  return (unsigned long long)((unsigned __int128)a * b >> 64);
+}
 #endif
 
 constexpr int kExpMin = 128, kExpMax = 2030;
@@ -96,6 +100,32 @@ CHEMORA_FX Parts parts_or_zero(double v) {
   Parts p = parts<K>(v);
   if (((hiword(v) << 1) | loword(v)) == 0) p.e = kZeroExp;
   return p;
+}
+
+// A factor of a product: its significand 2^S times, its sign, its exponent
+// (very low for zero, very high for subnormals, Inf and NaN, so that the
+// products are zero and out of every range).
+template <int S>
+struct Factor {
+  unsigned long long m;
+  unsigned s;
+  int e;
+};
+template <int S>
+CHEMORA_FX Factor<S> factor(double v) {
+  const unsigned h = hiword(v);
+  const unsigned long long m = ((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32 | loword(v)) << S;
+  int e = exponent(v);
+  if ((unsigned)(e - 1) >= 2046u) e = ((h << 1) | loword(v)) == 0 ? -8192 : 16384;
+  return Factor<S>{m, h, e};
+}
+// a b in units of 2^(e - 1075 - K), rounded to nearest: a unit is at most
+// 2^(1 - K) ulps of the product.
+template <int K>
+CHEMORA_FX Parts product(const Factor<11>& a, const Factor<K + 1>& b) {
+  const unsigned long long m = (mulhi64(a.m, b.m) + 1) >> 1;
+  const unsigned long long s = (unsigned long long)((long long)(int)(a.s ^ b.s) >> 63);
+  return Parts{(long long)((m ^ s) - s), emax(a.e + b.e - 1022, kZeroExp)};
 }
 
 // In units of 2^(E - 1075 - K), E the exponent of the largest value: |result|

@@ -65,6 +65,7 @@ struct chemora_system {
   // derivative fields of the split BSSN right-hand side: a workspace for the
   // RK4 driver (allocated on first use), and a pool for calls that may run on
   // several streams at once (chemora_rhs, chemora_stage, chemora_constraints)
+  // and for the adjoint's work space
   double* field_work;
   int64_t field_points;
   cudaMemPool_t pool;
@@ -122,6 +123,7 @@ bool bssn_shape_splits(const Dims& d, int variant);
 // alloc is false and there is none yet), and one taken from and given back to
 // the system's pool in stream order.
 FieldWork system_field_work(chemora_system* sys, bool alloc);
+cudaMemPool_t system_pool(chemora_system* sys);  // NULL: none could be made
 FieldWork take_field_work(chemora_system* sys, cudaStream_t s);
 void give_field_work(const FieldWork& w, cudaStream_t s);
 

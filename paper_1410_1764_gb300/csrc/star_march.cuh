@@ -34,11 +34,13 @@ struct Central<4> {
   static constexpr int d2[4] = {8064, -1008, 128, -9}, den2 = 5040, d1[4] = {672, -168, 32, -3}, den1 = 840;
 };
 
-// Guard bits: with two, the order-4 Laplacian (weights 192 in all) fits in 64
-// bits; with six, sums of twelve values do, and the weighted sums take 96.
+// Guard bits: with six, sums of twelve values fit in 64 bits, and the weighted
+// sums of such sums take 96; with two, the order-4 Laplacian (weights 192 in
+// all) stays in 64, which saves 3 to 5 % of its kernels' time and moves the
+// error against exact values by less than its spread over inputs (3 %).
 template <int R>
 struct Guard {
-  static constexpr int lap = R == 2 ? 2 : 6, d1 = R <= 2 ? 4 : (R == 3 ? 3 : 6);
+  static constexpr int lap = R == 2 ? 2 : 6, d1 = R <= 2 ? 4 : 6;
 };
 
 // Exponents from which no weighted sum (orders 6 and 8: below 2^18 times the
@@ -51,26 +53,26 @@ CHEMORA_FX bool star_ok(int e) {
 
 // den2 h^2 times the Laplacian from the sums s[k] of the six values at
 // distance k + 1 and the centre c, aligned to exponent e.
-template <int R>
+template <int R, int K = Guard<R>::lap>
 CHEMORA_FX double star_lap(const long long (&s)[R], long long c, int e) {
   typedef Central<R> W;
   if constexpr (R == 1) {
-    return fx::to_double<Guard<R>::lap>(s[0] - 6 * c, e);
-  } else if constexpr (R == 2) {
-    return fx::to_double<Guard<R>::lap>(16 * s[0] - s[1] - 90 * c, e);
+    return fx::to_double<K>(s[0] - 6 * c, e);
+  } else if constexpr (R == 2 && K <= 2) {
+    return fx::to_double<K>(16 * s[0] - s[1] - 90 * c, e);
   } else {
     fx::Sum96 v;
     v.add<W::d2[0]>(s[0] - 6 * c);
     v.add<W::d2[1]>(s[1] - 6 * c);
-    v.add<W::d2[2]>(s[2] - 6 * c);
+    if constexpr (R >= 3) v.add<W::d2[2]>(s[R < 3 ? 0 : 2] - 6 * c);
     if constexpr (R == 4) v.add<W::d2[3]>(s[R - 1] - 6 * c);
-    return fx::to_double<Guard<R>::lap>(v, e);
+    return fx::to_double<K>(v, e);
   }
 }
 
-// den1 h times a sum of NS first differences from the sums t[k] of their
+// den1 h times a sum of up to three first differences from the sums t[k] of their
 // differences f(k + 1) - f(-k - 1), aligned to exponent e.
-template <int R, int NS>
+template <int R>
 CHEMORA_FX double star_d1(const long long (&t)[R], int e) {
   typedef Central<R> W;
   constexpr int K = Guard<R>::d1;
@@ -78,8 +80,6 @@ CHEMORA_FX double star_d1(const long long (&t)[R], int e) {
     return fx::to_double<K>(t[0], e);
   } else if constexpr (R == 2) {
     return fx::to_double<K>(8 * t[0] - t[1], e);
-  } else if constexpr (R == 3 && NS == 1) {
-    return fx::to_double<K>(45 * t[0] - 9 * t[1] + t[2], e);
   } else {
     fx::Sum96 v;
     v.add<W::d1[0]>(t[0]);
@@ -182,17 +182,19 @@ struct MarchUpdate {
   }
 };
 
-// Planes a block marches through: the depth with the least work in whole
-// waves of resident blocks, a block's start counted as `start` planes.
-inline int march_depth(const Dims& d, int tx, int ty, int resident, int start) {
+// Planes a block marches through.  An SM (of 152) works through the planes of
+// its blocks, a block's start costing about one and a half, and drains over
+// about three quarters of its resident blocks.  us per stage at depths 4, 8, 16
+// and 32: variable speed, 128^3 58, 60, 69, 70; order 4, 256^3 264, 253, 249,
+// 256; first-order form of order 6, 117 x 90 x 131 92, 97, 114, 115.
+inline int march_depth(const Dims& d, int tx, int ty, int resident) {
   const int64_t tiles = (int64_t)((d.nx + tx - 1) / tx) * ((d.ny + ty - 1) / ty);
-  const int64_t slots = 152 * (int64_t)resident;
   int best = 1;
   double cost = 1e300;
   for (int zb = 1; zb <= 64 && zb <= d.nz; ++zb) {
     const int64_t blocks = tiles * ((d.nz + zb - 1) / zb);
-    const double waves = (double)blocks / (double)slots;
-    const double c = (waves < 8.0 ? (double)((blocks + slots - 1) / slots) : waves + 0.5) * (zb + start);
+    const int64_t per_sm = (blocks + 151) / 152;
+    const double c = ((double)per_sm + 0.75 * resident) * (zb + 1.5);
     if (c < cost) {
       cost = c;
       best = zb;

@@ -4,8 +4,8 @@
 #include "internal.h"
 #include "stage.cuh"
 #include "star_march.cuh"
+#include "varc_march.cuh"
 #include "wave_point.cuh"
-#include "generated/gen_wave_varc.cuh"
 
 namespace chemora {
 
@@ -27,31 +27,6 @@ __global__ void __launch_bounds__(TX * TY) wave_stage_kernel(Dims d, Scalars sc,
   up.apply(a, c, d.sv, kk, sc.k[CHEMORA_K_ONE], sc.k[CHEMORA_K_TWO], [&](int64_t o, double x) { a.dst[o] = x; });
 }
 
-// Loader of the variable-speed body: state variables 0-1, then the
-// coefficient fields s, D_x s, D_y s, D_z s (svar apart) as variables 2-5.
-struct VarcLoader {
-  const double* __restrict__ p;  // centre point of variable 0
-  const double* __restrict__ q;  // centre point of s
-  int64_t sy, sz, sv;
-  __device__ __forceinline__ double operator()(int v, int dx, int dy, int dz) const {
-    const int64_t off = dx + dy * sy + dz * sz;
-    if (v < 2) return __ldg(p + v * sv + off);
-    return __ldg(q + (v - 2) * sv + off);
-  }
-};
-
-template <int TX, int TY>
-__global__ void __launch_bounds__(TX * TY) varc_stage_kernel(Dims d, Scalars sc, StageParams a) {
-  const int i = blockIdx.x * TX + threadIdx.x;
-  const int j = blockIdx.y * TY + threadIdx.y;
-  const int k = blockIdx.z;
-  if (i >= d.nx || j >= d.ny) return;
-  const int64_t c = (int64_t)(k + d.g) * d.sz + (int64_t)(j + d.g) * d.sy + (i + d.g);
-  VarcLoader ld{a.src + c, a.coef + c, d.sy, d.sz, d.sv};
-  StageOutFma out = CHEMORA_STAGE_OUT_FMA(a, c, d.sv, sc);
-  chemora_varc_point(ld, sc, out);
-}
-
 template <int TX, int TY>
 static int launch_wave_variant(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s) {
   dim3 grid((d.nx + TX - 1) / TX, (d.ny + TY - 1) / TY, d.nz);
@@ -61,9 +36,7 @@ static int launch_wave_variant(const Dims& d, const Scalars& sc, const StagePara
 
 template <int TX, int TY>
 static int launch_varc_variant(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s) {
-  dim3 grid((d.nx + TX - 1) / TX, (d.ny + TY - 1) / TY, d.nz);
-  varc_stage_kernel<TX, TY><<<grid, dim3(TX, TY), 0, s>>>(d, sc, a);
-  return launched("varc_stage_kernel");
+  return launch_varc_march<TX, TY>(d, sc, a, nullptr, 0, s);
 }
 
 // Planes in shared memory (wave_orders.cu) win where blocks marching through
@@ -80,9 +53,9 @@ const LaunchVariant kWaveVariants[] = {
 const int kNumWaveVariants = sizeof(kWaveVariants) / sizeof(kWaveVariants[0]);
 
 const LaunchVariant kVarcVariants[] = {
-    {32, 8, 0, launch_varc_variant<32, 8>},  {32, 4, 0, launch_varc_variant<32, 4>},
-    {64, 4, 0, launch_varc_variant<64, 4>},  {128, 2, 0, launch_varc_variant<128, 2>},
-    {32, 16, 0, launch_varc_variant<32, 16>}, {16, 16, 0, launch_varc_variant<16, 16>},
+    {32, 8, 0, launch_varc_variant<32, 8>},   {32, 4, 0, launch_varc_variant<32, 4>},
+    {64, 4, 0, launch_varc_variant<64, 4>},   {16, 16, 0, launch_varc_variant<16, 16>},
+    {16, 8, 0, launch_varc_variant<16, 8>},
 };
 const int kNumVarcVariants = sizeof(kVarcVariants) / sizeof(kVarcVariants[0]);
 

@@ -239,7 +239,7 @@ wave1_march_kernel(Dims d, Scalars sc, StageParams a, int zb, double scale) {
             const long long f0 = x < 2 ? M[pr - (q + 1) * st[x & 1]] : z[R - q - 1].m;
             t[q] = fx::sar(f1, (unsigned)(e - te[up1])) - fx::sar(f0, (unsigned)(e - te[dn]));
           }
-          kk[2 + x] = e == fx::kZeroExp ? 0.0 : star_d1<R, 1>(t, e);
+          kk[2 + x] = e == fx::kZeroExp ? 0.0 : star_d1<R>(t, e);
         }
       }
       {  // the divergence of v, one sum
@@ -260,7 +260,7 @@ wave1_march_kernel(Dims d, Scalars sc, StageParams a, int zb, double scale) {
                   fx::sar(M[py - (q + 1) * TX], (unsigned)(e - ey[dn]))) +
                  (fx::align(vz[R + q + 1], e) - fx::align(vz[R - q - 1], e));
         }
-        kk[1] = e == fx::kZeroExp ? 0.0 : star_d1<R, 3>(t, e);
+        kk[1] = e == fx::kZeroExp ? 0.0 : star_d1<R>(t, e);
       }
       if (ok) {
         kk[0] = rho;
@@ -278,7 +278,7 @@ wave1_march_kernel(Dims d, Scalars sc, StageParams a, int zb, double scale) {
 
 template <class BODY, int R, int TX, int TY>
 static int launch_order(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s) {
-  const int zb = march_depth(d, TX, TY, march_threads<BODY::nv, R>() / (TX * TY), R + 1);
+  const int zb = march_depth(d, TX, TY, march_threads<BODY::nv, R>() / (TX * TY));
   const dim3 grid = march_grid(d, TX, TY, zb);
   if constexpr (BODY::nv == 2)
     wave_march_order_kernel<BODY, R, TX, TY><<<grid, TX * TY, 0, s>>>(
