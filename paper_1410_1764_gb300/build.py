@@ -23,7 +23,8 @@ NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompil
 
 
 # device headers the run-time specialised stage kernel includes (NVRTC)
-JIT_HEADERS = ("device_types.cuh", "stage.cuh", "bssn_kernels.cuh", "bssn_fields.cuh", "bssn_algebra.cuh",
+JIT_HEADERS = ("device_types.cuh", "stage.cuh", "bssn_kernels.cuh", "fixedpoint.cuh", "bssn_fields.cuh",
+               "bssn_prologue.cuh", "bssn_algebra.cuh",
                "generated/gen_constants.cuh", "generated/gen_bssn.cuh", "generated/gen_bssn_x.cuh",
                "generated/gen_bssn_xy.cuh", "generated/gen_bssn_alg.cuh")
 JIT_INC = os.path.join(CSRC, "generated", "jit_sources.inc")

@@ -69,9 +69,9 @@ static int launch_bssn_xyvariant(const Dims& d, const Scalars& sc, const StagePa
 // Launch shapes the autotuner chooses from (variant 0 is the default).
 // Sharing 0: the split kernels, tx x ty the algebra kernel's block.
 const LaunchVariant kBssnVariants[] = {
-    {32, 4, 3, launch_bssn_direct},
-    {32, 4, 2, launch_bssn_direct},
     {32, 4, 4, launch_bssn_direct},
+    {32, 4, 2, launch_bssn_direct},
+    {32, 4, 3, launch_bssn_direct},
     {32, 2, 5, launch_bssn_direct},
     {32, 2, 8, launch_bssn_direct},
     {64, 2, 3, launch_bssn_direct},

@@ -5,16 +5,14 @@
 // the Kreiss-Oliger term, 162 numbers per point -- almost entirely on the
 // integer units (fixedpoint.cuh) and writes them to a workspace; the second
 // reads them back, one number per load, and does the algebra: 1058 FP64
-// instructions per point where the fused bodies issue 2039 (x/y sharing) to
-// 2642 (direct).  FP64 issue is what bounds these equations on GB300, so the
+// operations per point, 272 of them on the integer units (bssn_prologue.cuh),
+// where the fused bodies issue 2039 (x/y sharing) to 2642 (direct).  FP64 issue is what bounds these equations on GB300, so the
 // 2.6 KB per point that the workspace costs in memory traffic is the cheaper
 // side.  Neither kernel needs a particular grid shape, so small and ragged
 // grids, patches and refined boxes run the same code at the same rate.
 #pragma once
 #include "device_types.cuh"
-#if !defined(__CUDACC_RTC__)
 #include "fixedpoint.cuh"
-#endif
 
 namespace chemora {
 
@@ -47,11 +45,22 @@ struct FieldRegion : FieldSlab {
   int tw, th, zb, tnx, tny;
 };
 
-// Loader of the algebra bodies: the state at the point and its fields.
+// What the integer prologue of the algebra kernels (bssn_prologue.cuh) leaves
+// in shared memory for the point's thread, kPre columns of BLK threads: sums
+// adv of the variables but gt_ij, traces tr of the variables with second
+// derivatives but phi, the inverse metric, the shift's derivatives.
+constexpr int kPreAdv = 0, kPreTr = 18, kPreGu = 28, kPreDb = 34, kPre = 43;
+__host__ __device__ constexpr int adv_index(int v) { return kPreAdv + (v == 0 ? 0 : v - 6); }
+__host__ __device__ constexpr int tr_index(int v) { return kPreTr + (v < 7 ? v - 1 : v - 11); }
+
+// Loader of the algebra bodies: the state at the point, its fields, and the
+// prologue's results (unused, s NULL, by the constraints).
+template <int BLK>
 struct FieldLoader {
   const double* __restrict__ p;  // variable 0 at the point
   int64_t sv;
   const double* __restrict__ w;  // field 0 at the point
+  double* s;                     // the thread's column of the prologue's results
   __device__ __forceinline__ double operator()(int v, int, int, int) const { return __ldg(p + v * sv); }
   __device__ __forceinline__ double g1(int v, int a) const {
     return __ldg(w + (kFieldD1 + 3 * v + a) * kFieldBlock);
@@ -63,6 +72,10 @@ struct FieldLoader {
     return __ldg(w + (kFieldD2 + 6 * dd_index(v) + 3 + ab) * kFieldBlock);
   }
   __device__ __forceinline__ double gko(int v) const { return __ldg(w + (kFieldKo + v) * kFieldBlock); }
+  __device__ __forceinline__ double adv(int v) const { return s[adv_index(v) * BLK]; }
+  __device__ __forceinline__ double tr(int v) const { return s[tr_index(v) * BLK]; }
+  __device__ __forceinline__ double gu(int ab) const { return s[(kPreGu + ab) * BLK]; }
+  __device__ __forceinline__ double db(int i, int a) const { return s[(kPreDb + 3 * i + a) * BLK]; }
 };
 
 #if defined(__CUDACC__) && !defined(__CUDACC_RTC__)

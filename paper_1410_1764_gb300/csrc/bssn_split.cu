@@ -306,6 +306,10 @@ static int launch_algebra(const FieldRegion& R, const Scalars& sc, const StagePa
 
 int launch_bssn_split(const Dims& d, const Scalars& sc, const StageParams& a, const FieldWork& work, int block,
                       int minb, cudaStream_t s) {
+  // Fewer than two waves of 128-thread blocks (four per SM): half the block
+  // evens out the SMs' shares (37 x 29 x 23, field and algebra kernels: 122 us
+  // with 128 threads, 106 with 64; 128^3: 4.73 and 4.83 ms).
+  if ((int64_t)d.nx * d.ny * d.nz < 2 * 152 * 4 * 128) block = 64, minb = 8;
   return for_field_chunks(d, sc, a.src, 24, work, s, [&](const FieldRegion& R) {
     if (block == 64) return minb >= 8 ? launch_algebra<64, 8>(R, sc, a, work.w, s) : launch_algebra<64, 5>(R, sc, a, work.w, s);
     if (minb == 2) return launch_algebra<128, 2>(R, sc, a, work.w, s);
@@ -323,13 +327,14 @@ int launch_bssn_split(const Dims& d, const Scalars& sc, const StageParams& a, co
 // of touching memory, and a block past the time limit takes no more items and
 // sets bit 1.
 template <int MODE>
-__global__ void __launch_bounds__(kItemPoints, 3)
+__global__ void __launch_bounds__(kItemPoints, 4)
 batch_algebra_kernel(const FieldRegion* __restrict__ regions, int nregions, const WorkItem* __restrict__ items,
                      int nitems, unsigned int* counter, int* err, long long limit, Scalars sc, StageParams a_in,
                      const double* __restrict__ work) {
   StageParams a = a_in;
   a.mode = MODE;
   __shared__ unsigned int s_item;
+  __shared__ double pre[kPre * kItemPoints];
   const long long t0 = clock64();
   for (int iter = 0; iter <= nitems; ++iter) {
     if (threadIdx.x == 0) {
@@ -352,7 +357,7 @@ batch_algebra_kernel(const FieldRegion* __restrict__ regions, int nregions, cons
     const FieldRegion& R = regions[q.patch];
     const int64_t lin = (int64_t)q.start + threadIdx.x;
     if (q.start < 0 || lin >= R.npts) continue;
-    bssn_algebra_point(R.d, R, lin, sc, a, work);
+    bssn_algebra_point<kItemPoints>(R.d, R, lin, sc, a, work, pre);
   }
 }
 
@@ -431,7 +436,7 @@ static int persistent_algebra_blocks() {
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
     sms = 152;
-  return 3 * sms;
+  return 4 * sms;
 }
 
 int launch_field_plan(const FieldPlan& plan, unsigned int* counters, int* err, long long limit, const Scalars& sc,
@@ -470,7 +475,7 @@ bssn_constraints_algebra_kernel(FieldRegion R, Scalars sc, const double* __restr
   const int64_t lin = (int64_t)blockIdx.x * 128 + threadIdx.x;
   if (lin >= R.npts) return;
   const int64_t c = R.offset + region_point(R.d, lin);
-  const FieldLoader ld{st + c, R.d.sv, work + field_base(R.w0 + lin)};
+  const FieldLoader<128> ld{st + c, R.d.sv, work + field_base(R.w0 + lin), nullptr};
   auto o = [&](int v, double x) { out[c + v * R.d.sv] = x; };
   chemora_bssn_constraints_alg_point(ld, sc, o);
 }

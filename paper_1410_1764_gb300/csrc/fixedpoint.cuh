@@ -18,7 +18,9 @@
 // numbers near the ends of the FP64 range, Inf, NaN) is left to the caller's
 // FP64 body (in_range).  Compiles for the host too (tests).
 #pragma once
+#if !defined(__CUDACC_RTC__)
 #include <stdint.h>
+#endif
 #if !defined(__CUDACC__)
 #include <string.h>
 #endif
@@ -49,6 +51,12 @@ CHEMORA_FX unsigned long long shr(unsigned long long a, unsigned s) {
 }
 CHEMORA_FX int clz64(unsigned long long a) { return __clzll((long long)a); }
 CHEMORA_FX unsigned long long mulhi64(unsigned long long a, unsigned long long b) { return __umul64hi(a, b); }
+CHEMORA_FX int mulhi32(int a, int b) { return __mulhi(a, b); }
+CHEMORA_FX long long mad_wide(int a, int b, long long c) {
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+}
 #else
 #define CHEMORA_FX inline
 CHEMORA_FX unsigned long long bits(double v) {
@@ -70,6 +78,8 @@ CHEMORA_FX int clz64(unsigned long long a) { return a ? __builtin_clzll(a) : 64;
 CHEMORA_FX unsigned long long mulhi64(unsigned long long a, unsigned long long b) {
   return (unsigned long long)((unsigned __int128)a * b >> 64);
 }
+CHEMORA_FX int mulhi32(int a, int b) { return (int)((long long)a * b >> 32); }
+CHEMORA_FX long long mad_wide(int a, int b, long long c) { return (long long)a * b + c; }
 #endif
 
 constexpr int kExpMin = 128, kExpMax = 2030;
@@ -128,6 +138,40 @@ CHEMORA_FX Parts product(const Factor<11>& a, const Factor<K + 1>& b) {
   return Parts{(long long)((m ^ s) - s), emax(a.e + b.e - 1022, kZeroExp)};
 }
 
+// The same in four multiplications, for sums with guard bits to spare: a signed
+// significand 2^S times as its high word and 31 bits of its low word.
+template <int S>
+struct Term {
+  int hi, lo;
+  int e;
+};
+template <int S>
+CHEMORA_FX Term<S> term(double v) {
+  const unsigned h = hiword(v);
+  unsigned long long m = ((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32 | loword(v)) << S;
+  const unsigned long long s = (unsigned long long)(long long)((int)h >> 31);
+  m = (m ^ s) - s;
+  int e = exponent(v);
+  if ((unsigned)(e - 1) >= 2046u) e = ((h << 1) | loword(v)) == 0 ? -8192 : 16384;
+  return Term<S>{(int)(m >> 32), (int)((unsigned)m >> 1), e};
+}
+// a b in units of 2^(e - 1075 - K), within six units: the product of the low
+// words is left out.
+template <int K>
+CHEMORA_FX Parts term_product(const Term<10>& a, const Term<K + 1>& b) {
+  const int x = mulhi32(a.hi, b.lo) + mulhi32(a.lo, b.hi);
+  return Parts{mad_wide(x, 2, mad_wide(a.hi, b.hi, 0)), emax(a.e + b.e - 1022, kZeroExp)};
+}
+// The sum of N products as a double, at the guard bits with which N of them fit
+// in 64 bits (N 2^(53 + k) < 2^63): within 6 N units, a sixteenth of an ulp of
+// the largest product each; false if their exponents leave the range to FP64.
+template <int N>
+struct DotGuard {
+  static constexpr int k = N <= 7 ? 7 : 6;
+};
+template <int N>
+CHEMORA_FX bool dot(const Parts (&p)[N], double* sum);
+
 // In units of 2^(E - 1075 - K), E the exponent of the largest value: |result|
 // <= 2^(53 + K).
 CHEMORA_FX long long align(const Parts& p, int e) { return sar(p.m, (unsigned)(e - p.e)); }
@@ -145,6 +189,25 @@ CHEMORA_FX double to_double(long long v, int e) {
   r += (unsigned long long)(unsigned)(e + 10 - K - lz) << 52;
   r |= s & 0x8000000000000000ull;
   return a == 0 ? 0.0 : from_bits(r);
+}
+
+template <int N>
+CHEMORA_FX bool dot(const Parts (&p)[N], double* sum) {
+  int e = kZeroExp;
+#if defined(__CUDACC__)
+#pragma unroll
+#endif
+  for (int q = 0; q < N; ++q) e = emax(e, p[q].e);
+  *sum = 0.0;
+  if (e == kZeroExp) return true;
+  if (!in_range(e)) return false;
+  long long m = 0;
+#if defined(__CUDACC__)
+#pragma unroll
+#endif
+  for (int q = 0; q < N; ++q) m += align(p[q], e);
+  *sum = to_double<DotGuard<N>::k>(m, e);
+  return true;
 }
 
 // A sum of 64-bit integers with constant weights, exact in 96 bits: hi 2^32 + lo.

@@ -34,9 +34,12 @@ def _sym_expr(name):
     m = re.match(r"g(1|2|11)_(\d+)_(\d+)$", name)
     if m:
         return "ld.g%s(%s, %s)" % m.groups(), True
-    m = re.match(r"gko_(\d+)$", name)
+    m = re.match(r"(gko|adv|tr|gu)_(\d+)$", name)
     if m:
-        return "ld.gko(%s)" % m.group(1), True
+        return "ld.%s(%s)" % m.groups(), True
+    m = re.match(r"db_(\d+)_(\d+)$", name)
+    if m:
+        return "ld.db(%s, %s)" % m.groups(), True
     return "sc." + name, False
 
 
@@ -89,8 +92,13 @@ def _bssn_xyshare():
         return systems.bssn()
 
 
-def _bssn_fields():
+def _bssn_fields_alone():
     with stencil.fields():
+        return systems.bssn()
+
+
+def _bssn_fields():
+    with stencil.fields(sums=True):
         return systems.bssn()
 
 
@@ -172,8 +180,11 @@ def _render():
                   "variable-speed wave: u_t = rho, rho_t = s Lap u + G . grad u, with s = c^2 "
                   "and G = grad s read from grid functions 2 and 3-5"))
     specs.append(("bssn_alg", "chemora_bssn_alg_point", _bssn_fields,
-                  "BSSN as chemora_bssn_point, every derivative read from precomputed fields: "
-                  "the algebra of one point"))
+                  "BSSN as chemora_bssn_point, derivatives read from precomputed fields, sums of products "
+                  "of the integer prologue through ld.adv, ld.tr, ld.gu, ld.db: the rest of the algebra "
+                  "of one point (gt_ij: all of it is in the prologue)"))
+    # numbering pass: the constraints' body keeps the term order it was measured with
+    specs.append(("", "chemora_bssn_fields_point", _bssn_fields_alone, ""))
     specs.append(("bssn_constraints_alg", "chemora_bssn_constraints_alg_point", _bssn_constraints_fields,
                   "BSSN constraints as chemora_bssn_constraints_point, every derivative read from "
                   "precomputed fields"))
@@ -185,7 +196,7 @@ def _render():
             continue
         if key in NUMBERING_ORDER:
             emit.emit_function(fname, [(v, outs[v]) for v in NUMBERING_ORDER[key]], _sym_expr, nout, comment)
-        order = EMIT_ORDER.get(key, list(range(nout)))
+        order = [v for v in EMIT_ORDER.get(key, list(range(nout))) if outs[v] is not None]
         src, L = emit.emit_function(fname, [(v, outs[v]) for v in order],
                                     _sym_expr, nout, comment)
         files["gen_%s.cuh" % key] = HEADER + src

@@ -88,20 +88,26 @@ class zqueue:
 
 
 _FIELDS = [False]
+_SUMS = [False]
 
 
 class fields:
     """Context manager: every derivative is read from precomputed fields
     (symbols g1_<v>_<a>: 12h D_a f, g2_<v>_<a>: 12h^2 D_aa f, g11_<v>_<ab>:
     144h^2 D_ab f, gko_<v>: 64h/eps KO f), so the body holds the algebra alone
-    and reads the state at the point only."""
+    and reads the state at the point only.  With `sums` the inverse metric, the
+    shift's derivatives and some sums of products are symbols too (gu_<ab>,
+    db_<i>_<a>, tr_<v>: gt^ab D_ab f, adv_<v>)."""
+
+    def __init__(self, sums=False):
+        self.sums = sums
 
     def __enter__(self):
-        self.prev = _FIELDS[0]
-        _FIELDS[0] = True
+        self.prev = _FIELDS[0], _SUMS[0]
+        _FIELDS[0], _SUMS[0] = True, self.sums
 
     def __exit__(self, *exc):
-        _FIELDS[0] = self.prev
+        _FIELDS[0], _SUMS[0] = self.prev
 
 
 def _zq(what, v):

@@ -16,6 +16,7 @@ identical components are the same DAG node.
 from fractions import Fraction
 
 from . import expr as E
+from . import stencil
 from .stencil import (val, d1, dd, ko, d1_raw, d2_raw, d11_raw, d1o_raw, d2o_raw, _centre_diffs, I12H,
                       I12H2, IH, IH2,
                       KO_SCALE)
@@ -78,9 +79,12 @@ def _bssn_geometry():
 
     # advection beta^k D_k f with the stencil scale folded into the shift:
     # sum_k (beta^k / 12h) (12h D_k f)
+    sums = stencil._SUMS[0]
     bs = [E.box(be[k] * I12H) for k in R3]
 
     def advect(df, v=None):
+        if sums and v is not None:  # with the dissipation, and for At all terms in the shift
+            return E.sym("adv_%d" % v)
         if v is not None:
             return E.box(sum((bs[k] * d1_raw(v, k) for k in R3), E.const(0)))
         return E.box(sum((be[k] * df[k] for k in R3), E.const(0)))
@@ -90,6 +94,8 @@ def _bssn_geometry():
     gtu6 = [[None] * 3 for _ in R3]
 
     def gtu_dd(v):
+        if sums:
+            return E.sym("tr_%d" % v)
         acc = E.const(0)
         for l in R3:
             for m in R3:
@@ -101,6 +107,9 @@ def _bssn_geometry():
                     acc = acc + gtu6[l][m] * d11_raw(v, l, m)
         return E.box(E.box(acc) * I12H2)
 
+    if sums:
+        dbe = [[E.sym("db_%d_%d" % (i, k)) for k in R3] for i in R3]
+
     # inverse conformal metric (adjugate / determinant, one reciprocal)
     c00 = E.box(gt[1][1] * gt[2][2] - gt[1][2] * gt[1][2])
     c01 = E.box(gt[1][2] * gt[0][2] - gt[0][1] * gt[2][2])
@@ -111,7 +120,7 @@ def _bssn_geometry():
     det = E.box(gt[0][0] * c00 + gt[0][1] * c01 + gt[0][2] * c02)
     idet = E.rcp(det)
     cof = [[c00, c01, c02], [c01, c11, c12], [c02, c12, c22]]
-    gtu = [[E.box(cof[i][j] * idet) for j in R3] for i in R3]
+    gtu = [[E.sym("gu_%d" % SYM[i][j]) if sums else E.box(cof[i][j] * idet) for j in R3] for i in R3]
 
     # Christoffel symbols: first kind Gl[k][i][j], second kind Gu[k][i][j]
     Gl = [[[E.box(E.const(0.5) * (dgt[j][k][i] + dgt[i][k][j] - dgt[i][j][k]))
@@ -162,7 +171,7 @@ def _bssn_geometry():
             DDal[i][j] = DDal[j][i] = E.box(
                 ddal[i][j] - sum((Gu[k][i][j] * dal[k] for k in R3), E.const(0))
                 - 2 * (dphi[i] * dal[j] + dphi[j] * dal[i]) + 2 * gt[i][j] * dphidal)
-    tr_ddal = sum((gtu[i][j] * ddal[i][j] for i in R3 for j in R3), E.const(0))
+    tr_ddal = gtu_dd(ALPHA) if sums else sum((gtu[i][j] * ddal[i][j] for i in R3 for j in R3), E.const(0))
     Xdal = sum((Xtn[k] * dal[k] for k in R3), E.const(0))
     trDDal = E.box(e4 * E.box(tr_ddal - Xdal + 2 * dphidal))
 
@@ -174,7 +183,10 @@ def bssn(eta_sym="eta"):
     variable.  The gauge is chosen at run time: sc.slicing 0 1+log,
     1 harmonic, 2 frozen lapse; sc.shift 0 Gamma-driver, 1 frozen shift and B
     (frozen variables have a zero right-hand side and no dissipation).
-    An output is a node or a list of (condition, node) alternatives."""
+    An output is a node or a list of (condition, node) alternatives.  On
+    precomputed fields with sums (stencil.fields) the advection and dissipation
+    terms, all of gt_ij's right-hand side and At_ij's terms in the shift are
+    read as one number (adv_<v>), and gt_ij has no output here."""
     eta = E.sym(eta_sym)
     G = _bssn_geometry()
     (phi, K, al, gt, At, Xt, be, B) = (G["phi"], G["K"], G["al"], G["gt"], G["At"], G["Xt"], G["be"], G["B"])
@@ -185,9 +197,12 @@ def bssn(eta_sym="eta"):
         G["DDal"], G["trDDal"], G["advect"], G["gtu_dd"])
     divbe = E.box(dbe[0][0] + dbe[1][1] + dbe[2][2])
     out = [None] * 24
+    sums = G["sums"]
     out[PHI] = advect(dphi, PHI) + E.const(1) / 6 * (divbe - al * K)
     for i in R3:
         for j in range(i, 3):
+            if sums:
+                break
             s = advect(dgt[i][j], GT + SYM[i][j])
             s = s + sum((gt[i][k] * dbe[k][j] + gt[j][k] * dbe[k][i] for k in R3), E.const(0))
             s = s - E.const(2) / 3 * gt[i][j] * divbe - 2 * al * At[i][j]
@@ -198,8 +213,9 @@ def bssn(eta_sym="eta"):
     for i in R3:
         for j in range(i, 3):
             s = advect(dAt[i][j], AT + SYM[i][j])
-            s = s + sum((At[i][k] * dbe[k][j] + At[j][k] * dbe[k][i] for k in R3), E.const(0))
-            s = s - E.const(2) / 3 * At[i][j] * divbe
+            if not (sums):
+                s = s + sum((At[i][k] * dbe[k][j] + At[j][k] * dbe[k][i] for k in R3), E.const(0))
+                s = s - E.const(2) / 3 * At[i][j] * divbe
             s = s + e4 * E.box(X[i][j] - E.const(1) / 3 * gt[i][j] * trX)
             AtAt = sum((At[i][k] * Atm[k][j] for k in R3), E.const(0))
             s = s + al * E.box(K * At[i][j] - 2 * AtAt)
@@ -210,7 +226,7 @@ def bssn(eta_sym="eta"):
                                    for k in R3 if k != j), E.const(0))) * I12H2) for j in R3]
     rXt = [None] * 3
     for i in R3:
-        s = advect(dXt[i], XT + i)
+        s = E.const(0) if sums else advect(dXt[i], XT + i)
         s = s - sum((Xtn[j] * dbe[i][j] for j in R3), E.const(0))
         s = s + E.const(2) / 3 * Xtn[i] * divbe
         s = s + gtu_dd(BETA + i)
@@ -221,18 +237,19 @@ def bssn(eta_sym="eta"):
              - E.const(2) / 3 * sum((gtu[i][j] * dK[j] for j in R3), E.const(0)))
         s = s + 2 * al * E.box(t)
         rXt[i] = E.box(s)
-        out[XT + i] = rXt[i]
+        out[XT + i] = rXt[i] + advect(dXt[i], XT + i) if sums else rXt[i]
     # gauge: alternatives selected at run time by the uniform flags
-    kov = {v: ko(v) for v in (ALPHA,) + tuple(range(BETA, BB + 3))}
+    kov = {v: E.const(0) if sums else ko(v) for v in (ALPHA,) + tuple(range(BETA, BB + 3))}
     out[ALPHA] = [("sc.slicing == 0", E.box(advect(dal, ALPHA) - 2 * al * K) + kov[ALPHA]),
                   ("sc.slicing == 1", E.box(advect(dal, ALPHA) - al * al * K) + kov[ALPHA]),
                   (None, E.const(0))]
     for i in R3:
         out[BETA + i] = [("sc.shift == 0", E.box(advect(dbe[i], BETA + i) + E.const(3) / 4 * B[i]) + kov[BETA + i]),
                          (None, E.const(0))]
-        out[BB + i] = [("sc.shift == 0", E.box(advect(dB[i], BB + i) + (rXt[i] - advect(dXt[i], XT + i)) - eta * B[i])
+        out[BB + i] = [("sc.shift == 0", E.box(advect(dB[i], BB + i) + (rXt[i] if sums else rXt[i] - advect(dXt[i], XT + i)) - eta * B[i])
                         + kov[BB + i]), (None, E.const(0))]
-    return [out[v] if isinstance(out[v], list) else E.box(out[v]) + ko(v) for v in range(24)]
+    return [out[v] if out[v] is None or isinstance(out[v], list) else
+            (E.box(out[v]) if sums else E.box(out[v]) + ko(v)) for v in range(24)]
 
 
 def bssn_constraints():
