@@ -60,11 +60,11 @@ __global__ void __launch_bounds__(ATX * ATY) varc_grad_s_kernel(Dims d, double i
 // once per point (and once more per halo cell) and differenced on the integer
 // units (star_march.cuh): x and y neighbours come from the plane in shared
 // memory, z neighbours from the thread's registers.  Six guard bits for the
-// Laplacian and products rounded to nearest: values cut off downwards leave an
-// error that adds up over the steps (with two, and products cut off, grad_u0
-// of 24 steps on 64^3 was 18 % further from exact values than FP64 sums).
+// Laplacian: values cut off leave an error that adds up over the steps (with
+// two bits grad_u0 of 24 steps on 64^3 was 18 % further from exact values than
+// FP64 sums, with six 2 %, and grad_c 3 % closer).
 //
-// GB300, 128^3: 118 us, against 320 us when each point formed the 37 products
+// GB300, 128^3: 116 us, against 320 us when each point formed the 37 products
 // of its stencils itself in FP64 (72 instructions of 17.8 cycles).  Products in
 // FP64 here: 123 us.  640 threads per SM (20 bytes spilled): 7 % more.  Bound by
 // the latency of its integer chains at 16 warps per SM; ten FP64 instructions
@@ -105,10 +105,10 @@ varc_adj_march_kernel(Dims d, double i12h, double i12h2, double i144h2, const do
 #pragma unroll
     for (int m = 1; m < 5; ++m) {
       const int64_t o = c + (int64_t)(m - 3) * d.sz;
-      const fx::Factor<11> wv = fx::factor<11>(__ldg(w + o));
-      za[m] = fx::product<KA>(wv, fx::factor<KA + 1>(__ldg(coef + o)));
-      zg[m] = fx::product<KD>(wv, fx::factor<KD + 1>(__ldg(cz + o)));
-      zt[m] = fx::product<KD>(wv, fx::factor<KD + 1>(__ldg(tz + o)));
+      const fx::Term<10> wv = fx::term<10>(__ldg(w + o));
+      za[m] = fx::term_product<KA>(wv, fx::term<KA + 1>(__ldg(coef + o)));
+      zg[m] = fx::term_product<KD>(wv, fx::term<KD + 1>(__ldg(cz + o)));
+      zt[m] = fx::term_product<KD>(wv, fx::term<KD + 1>(__ldg(tz + o)));
     }
   }
 #pragma unroll 1
@@ -139,26 +139,26 @@ varc_adj_march_kernel(Dims d, double i12h, double i12h2, double i144h2, const do
       a0 = first ? y0 : yacc[c];
       a1 = first ? y1 : yacc[d.sv + c];
       sb = sbar[c];
-      const fx::Factor<11> fz = fx::factor<11>(wz), fc = fx::factor<11>(wc);
-      za[4] = fx::product<KA>(fz, fx::factor<KA + 1>(sz));
-      zg[4] = fx::product<KD>(fz, fx::factor<KD + 1>(gz));
-      zt[4] = fx::product<KD>(fz, fx::factor<KD + 1>(uz));
+      const fx::Term<10> fz = fx::term<10>(wz), fc = fx::term<10>(wc);
+      za[4] = fx::term_product<KA>(fz, fx::term<KA + 1>(sz));
+      zg[4] = fx::term_product<KD>(fz, fx::term<KD + 1>(gz));
+      zt[4] = fx::term_product<KD>(fz, fx::term<KD + 1>(uz));
       put(oa, za[2]);
-      put(ox, fx::product<KD>(fc, fx::factor<KD + 1>(gx)));
-      put(ox + NX, fx::product<KD>(fc, fx::factor<KD + 1>(ux)));
-      put(oy, fx::product<KD>(fc, fx::factor<KD + 1>(gy)));
-      put(oy + NY, fx::product<KD>(fc, fx::factor<KD + 1>(uy)));
+      put(ox, fx::term_product<KD>(fc, fx::term<KD + 1>(gx)));
+      put(ox + NX, fx::term_product<KD>(fc, fx::term<KD + 1>(ux)));
+      put(oy, fx::term_product<KD>(fc, fx::term<KD + 1>(gy)));
+      put(oy + NY, fx::term_product<KD>(fc, fx::term<KD + 1>(uy)));
     }
 #pragma unroll
     for (int q = 0; q < hl.n; ++q)
       if (hl.live[q]) {
         const int64_t o = p.org + k * d.sz + (int64_t)hl.y[q] * d.sy + hl.x[q];
         const int64_t ax = (hl.along_x[q] ? 1 : 2) * d.sv;
-        const fx::Factor<11> wv = fx::factor<11>(__ldg(w + o));
-        put((hl.y[q] + R) * P + hl.x[q] + R, fx::product<KA>(wv, fx::factor<KA + 1>(__ldg(coef + o))));
+        const fx::Term<10> wv = fx::term<10>(__ldg(w + o));
+        put((hl.y[q] + R) * P + hl.x[q] + R, fx::term_product<KA>(wv, fx::term<KA + 1>(__ldg(coef + o))));
         const int b = hl.along_x[q] ? NA + hl.y[q] * P + hl.x[q] + R : NA + 2 * NX + (hl.y[q] + R) * TX + hl.x[q];
-        put(b, fx::product<KD>(wv, fx::factor<KD + 1>(__ldg(coef + ax + o))));
-        put(b + (hl.along_x[q] ? NX : NY), fx::product<KD>(wv, fx::factor<KD + 1>(__ldg(tape + ax + o))));
+        put(b, fx::term_product<KD>(wv, fx::term<KD + 1>(__ldg(coef + ax + o))));
+        put(b + (hl.along_x[q] ? NX : NY), fx::term_product<KD>(wv, fx::term<KD + 1>(__ldg(tape + ax + o))));
       }
     __syncthreads();
     if (!p.active) continue;

@@ -50,7 +50,6 @@ CHEMORA_FX unsigned long long shr(unsigned long long a, unsigned s) {
   return r;
 }
 CHEMORA_FX int clz64(unsigned long long a) { return __clzll((long long)a); }
-CHEMORA_FX unsigned long long mulhi64(unsigned long long a, unsigned long long b) { return __umul64hi(a, b); }
 CHEMORA_FX int mulhi32(int a, int b) { return __mulhi(a, b); }
 CHEMORA_FX long long mad_wide(int a, int b, long long c) {
   long long r;
@@ -75,9 +74,6 @@ CHEMORA_FX unsigned long long shl(unsigned long long a, unsigned s) { return s >
 CHEMORA_FX long long sar(long long a, unsigned s) { return a >> (s > 63 ? 63 : s); }
 CHEMORA_FX unsigned long long shr(unsigned long long a, unsigned s) { return s > 63 ? 0 : a >> s; }
 CHEMORA_FX int clz64(unsigned long long a) { return a ? __builtin_clzll(a) : 64; }
-CHEMORA_FX unsigned long long mulhi64(unsigned long long a, unsigned long long b) {
-  return (unsigned long long)((unsigned __int128)a * b >> 64);
-}
 CHEMORA_FX int mulhi32(int a, int b) { return (int)((long long)a * b >> 32); }
 CHEMORA_FX long long mad_wide(int a, int b, long long c) { return (long long)a * b + c; }
 #endif
@@ -112,34 +108,10 @@ CHEMORA_FX Parts parts_or_zero(double v) {
   return p;
 }
 
-// A factor of a product: its significand 2^S times, its sign, its exponent
-// (very low for zero, very high for subnormals, Inf and NaN, so that the
-// products are zero and out of every range).
-template <int S>
-struct Factor {
-  unsigned long long m;
-  unsigned s;
-  int e;
-};
-template <int S>
-CHEMORA_FX Factor<S> factor(double v) {
-  const unsigned h = hiword(v);
-  const unsigned long long m = ((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32 | loword(v)) << S;
-  int e = exponent(v);
-  if ((unsigned)(e - 1) >= 2046u) e = ((h << 1) | loword(v)) == 0 ? -8192 : 16384;
-  return Factor<S>{m, h, e};
-}
-// a b in units of 2^(e - 1075 - K), rounded to nearest: a unit is at most
-// 2^(1 - K) ulps of the product.
-template <int K>
-CHEMORA_FX Parts product(const Factor<11>& a, const Factor<K + 1>& b) {
-  const unsigned long long m = (mulhi64(a.m, b.m) + 1) >> 1;
-  const unsigned long long s = (unsigned long long)((long long)(int)(a.s ^ b.s) >> 63);
-  return Parts{(long long)((m ^ s) - s), emax(a.e + b.e - 1022, kZeroExp)};
-}
-
-// The same in four multiplications, for sums with guard bits to spare: a signed
-// significand 2^S times as its high word and 31 bits of its low word.
+// A factor of a product: its signed significand 2^S times, as the high word and
+// 31 bits of the low word, and its exponent (very low for zero, very high for
+// subnormals, Inf and NaN, so that the products are zero and out of every
+// range).
 template <int S>
 struct Term {
   int hi, lo;
@@ -155,8 +127,8 @@ CHEMORA_FX Term<S> term(double v) {
   if ((unsigned)(e - 1) >= 2046u) e = ((h << 1) | loword(v)) == 0 ? -8192 : 16384;
   return Term<S>{(int)(m >> 32), (int)((unsigned)m >> 1), e};
 }
-// a b in units of 2^(e - 1075 - K), within six units: the product of the low
-// words is left out.
+// a b in units of 2^(e - 1075 - K), within six units, in four multiplications:
+// the product of the low words is left out.
 template <int K>
 CHEMORA_FX Parts term_product(const Term<10>& a, const Term<K + 1>& b) {
   const int x = mulhi32(a.hi, b.lo) + mulhi32(a.lo, b.hi);

@@ -38,11 +38,6 @@ template <int R, int NS> static int star(const double* n, double c, double* out)
 template <int R> static int order(int ns, const double* n, double c, double* out) {
   return ns == 0 ? star<R, 0>(n, c, out) : (ns == 1 ? star<R, 1>(n, c, out) : star<R, 3>(n, c, out));
 }
-extern "C" int mul(double a, double b, long long* m) {
-  const fx::Parts p = fx::product<2>(fx::factor<11>(a), fx::factor<3>(b));
-  *m = p.m;
-  return p.e;
-}
 extern "C" int run(int R, int ns, const double* n, double c, double* out) {
   return R == 1 ? order<1>(ns, n, c, out) : R == 2 ? order<2>(ns, n, c, out)
        : R == 3 ? order<3>(ns, n, c, out) : order<4>(ns, n, c, out);
@@ -62,12 +57,9 @@ def star(tmp_path_factory):
     L.run.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_double), ctypes.c_double,
                       ctypes.POINTER(ctypes.c_double)]
 
-    L.mul.argtypes = [ctypes.c_double, ctypes.c_double, ctypes.POINTER(ctypes.c_longlong)]
-
     def f(R, ns, n, c=0.0):
         o = ctypes.c_double()
         return o.value if L.run(R, ns, (ctypes.c_double * len(n))(*n), c, ctypes.byref(o)) else None
-    f.mul = L.mul
     return f
 
 
@@ -127,19 +119,3 @@ def test_special_values(star, R):
     assert star(R, 0, [1.7e308] * n3, 0.0) is None
     big = 2.0 ** ((2030 if R <= 2 else 2020) - 1023)         # the largest exponent taken
     assert star(R, 0, [big] * n3, -big) == 12 * sum(_weights(R, 0)) * big
-
-
-def test_products_against_rationals(star):
-    """A product of two doubles rounded at two guard bits: within half a unit of
-    the exact product, its size at most 2^55; zeros, and operands it leaves to FP64."""
-    rng, m = np.random.default_rng(0), ctypes.c_longlong()
-    for _ in range(2000):
-        a, b = (float(q) for q in rng.standard_normal(2) * np.exp2(rng.integers(-400, 400, 2)))
-        e = star.mul(a, b, ctypes.byref(m))
-        unit = Fraction(2) ** (e - 1075 - 2)
-        assert abs(m.value * unit - Fraction(a) * Fraction(b)) <= unit / 2 and 2 ** 53 <= abs(m.value) <= 2 ** 55
-    assert star.mul(1.0, 1.0, ctypes.byref(m)) == 1024 and m.value == 2 ** 53
-    assert star.mul(0.0, 3.0, ctypes.byref(m)) == star.mul(-3.0, -0.0, ctypes.byref(m)) == -4096
-    for a, b in ((math.inf, 1.0), (0.0, math.nan), (5e-324, 1e300), (-math.inf, 0.0), (1e300, 1e300)):
-        assert star.mul(a, b, ctypes.byref(m)) > 2030
-    assert star.mul(1e-300, 1e-300, ctypes.byref(m)) < 128
