@@ -318,10 +318,6 @@ struct AdjBufs {
   double* data;
 };
 
-// Stage outputs are written with their ghost images (no fill passes) when every
-// axis has at least g points.
-static int imaged_ok(const Dims& d) { return d.nx >= d.g && d.ny >= d.g && d.nz >= d.g ? 1 : 0; }
-
 // One forward RK4 step of the variable-speed wave from Y to Ynext (which may
 // be Y), tape of the 4 stages written at tape (16 grid functions) when
 // non-NULL.
@@ -342,7 +338,8 @@ static int fwd_step(chemora_system* sys, const AdjBufs& B, double* Y, double* Yn
     if (!im && (rc = fill_ghosts(d, 2, srcs[q], s))) return rc;
     p.src = srcs[q]; p.yn = Y; p.acc = A; p.dst = dsts[q]; p.c1 = dt / 6.0; p.c2 = c2[q]; p.mode = q + 1;
     p.coef = B.s;
-    if ((rc = launch_varc_march<32, 4>(d, sys->sc, p, tape ? tape + (size_t)q * 4 * fs : nullptr, im, s))) return rc;
+    p.imaged = im;
+    if ((rc = launch_varc_march<32, 4>(d, sys->sc, p, tape ? tape + (size_t)q * 4 * fs : nullptr, s))) return rc;
   }
   return im ? CHEMORA_OK : fill_ghosts(d, 2, Ynext, s);
 }

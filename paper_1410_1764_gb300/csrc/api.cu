@@ -235,9 +235,19 @@ static int run_stage(chemora_system* sys, const StageParams& a, const FieldWork&
   return prof_end(sys, s, e0);
 }
 
-// One RK4 step: four fused stages, each preceded by a ghost fill of the
-// buffer its stencils read.  Buffers: Y (caller's state), A (accumulator),
-// Sa/Sb (stage states, alternating so no stage reads what it writes).
+// Do the system's stages write their ghost images?  Variable-speed wave, 128^3
+// x 20 steps: 4373 us with fill passes, 4095 with images.  The other wave
+// systems lose by it (order 8, 128^3 x 10: 2266 and 2374; first-order form of
+// order 6, 117 x 90 x 131: 3605 and 4059): wider ghost zones and more variables
+// leave more of a warp's stores to a few lanes.
+static int stage_images(const chemora_system* sys) {
+  return sys->kind == CHEMORA_WAVE_VARC && imaged_ok(sys->grid->d);
+}
+
+// One RK4 step: four fused stages, the buffer each reads with valid ghosts: a
+// fill before the stage, or, where stages write their images, those (the
+// caller fills Y's once).  Buffers: Y (caller's state), A (accumulator), Sa/Sb
+// (stage states, alternating so no stage reads what it writes).
 static int rk4_one(chemora_system* sys, double* Y, double dt, const FieldWork& work, cudaStream_t s) {
   const Dims& d = sys->grid->d;
   const int nv = sys->nvars;
@@ -245,21 +255,20 @@ static int rk4_one(chemora_system* sys, double* Y, double dt, const FieldWork& w
   double* A = sys->scratch;
   double* Sa = sys->scratch + n;
   double* Sb = sys->scratch + 2 * n;
+  double* const src[4] = {Y, Sa, Sb, Sa};
+  double* const dst[4] = {Sa, Sb, Sa, Y};
+  const double c2[4] = {0.5 * dt, 0.5 * dt, dt, 0.0};
   int rc;
-  StageParams p{};
-  p.coef = sys->coef;
-  if ((rc = fill_ghosts(d, nv, Y, s))) return rc;
-  p.src = Y; p.yn = Y; p.acc = A; p.dst = Sa; p.c1 = 0.0; p.c2 = 0.5 * dt; p.mode = 1;
-  if ((rc = run_stage(sys, p, work, s))) return rc;
-  if ((rc = fill_ghosts(d, nv, Sa, s))) return rc;
-  p.src = Sa; p.dst = Sb; p.c2 = 0.5 * dt; p.mode = 2;
-  if ((rc = run_stage(sys, p, work, s))) return rc;
-  if ((rc = fill_ghosts(d, nv, Sb, s))) return rc;
-  p.src = Sb; p.dst = Sa; p.c2 = dt; p.mode = 3;
-  if ((rc = run_stage(sys, p, work, s))) return rc;
-  if ((rc = fill_ghosts(d, nv, Sa, s))) return rc;
-  p.src = Sa; p.dst = Y; p.c1 = dt / 6.0; p.c2 = 0.0; p.mode = 4;
-  return run_stage(sys, p, work, s);
+  for (int q = 0; q < 4; ++q) {
+    StageParams p{};
+    p.coef = sys->coef;
+    p.imaged = stage_images(sys);
+    p.src = src[q]; p.yn = Y; p.acc = A; p.dst = dst[q];
+    p.c1 = q == 3 ? dt / 6.0 : 0.0; p.c2 = c2[q]; p.mode = q + 1;
+    if (!p.imaged && (rc = fill_ghosts(d, nv, src[q], s))) return rc;
+    if ((rc = run_stage(sys, p, work, s))) return rc;
+  }
+  return CHEMORA_OK;
 }
 
 void free_step_graph(chemora_system* sys) {
@@ -404,17 +413,19 @@ int chemora_rk4_step(chemora_system* sys, double* state, double dt, int nsteps, 
   const FieldWork work = system_field_work(sys, cst == cudaStreamCaptureStatusNone);
   // Plain launches while profiling (events bracket each stage) or when the
   // caller is capturing the stream itself; otherwise replay a captured step.
+  const int images = stage_images(sys);
+  if (images && (rc = fill_ghosts(sys->grid->d, sys->nvars, state, s))) return rc;
   if (sys->profile_on || cst != cudaStreamCaptureStatusNone || nsteps < 2) {
     for (int n = 0; n < nsteps; ++n)
       if ((rc = rk4_one(sys, state, dt, work, s))) return rc;
-    return fill_ghosts(sys->grid->d, sys->nvars, state, s);
+    return images ? CHEMORA_OK : fill_ghosts(sys->grid->d, sys->nvars, state, s);
   }
   if ((rc = step_graph(sys, state, dt, work))) return rc;
   for (int n = 0; n < nsteps; ++n) {
     CHEMORA_CUDA(cudaGraphLaunch(sys->graph_exec, s));
-    if ((rc = launched("cudaGraphLaunch(RK4 step)", 8))) return rc;
+    if ((rc = launched("cudaGraphLaunch(RK4 step)", images ? 4 : 8))) return rc;
   }
-  return fill_ghosts(sys->grid->d, sys->nvars, state, s);
+  return images ? CHEMORA_OK : fill_ghosts(sys->grid->d, sys->nvars, state, s);
 }
 
 int chemora_rk4_step_host(chemora_system* sys, double* host_state, double dt, int nsteps,

@@ -52,6 +52,7 @@ struct StageParams {
   const double* coef;  // coefficient grid functions (variable-speed wave: s, D_x s, D_y s, D_z s), else NULL
   double c1, c2;
   int mode;
+  int imaged;  // variable-speed wave: dst is written with its periodic ghost images (needs n >= g on every axis)
 };
 
 // Bytes of dynamic shared memory of the BSSN x/y-sharing stage body for

@@ -52,14 +52,13 @@ __device__ __forceinline__ void star2_fp64(const double* p, const Dims& d, doubl
   }
 }
 
-// One stage of the tile's columns.  coef: s and G_d, svar apart; imaged: dst
-// and tape are written with their ghost images; tape (or NULL): Lap u and
+// One stage of the tile's columns.  coef: s and G_d, svar apart; tape (or NULL): Lap u and
 // 12 h D_d u of the stage state, svar apart.
 constexpr int kVarcThreads = 768;  // resident threads per SM
 template <int TX, int TY>
 __global__ void __launch_bounds__(TX * TY, kVarcThreads / (TX * TY))
 varc_march_kernel(Dims d, double i12h, double i12h2, double one, double two, double mzero, StageParams a, int zb,
-                  double* __restrict__ tape, int imaged) {
+                  double* __restrict__ tape) {
   constexpr int R = 2, P = TX + 2 * R, K = 5;  // 18 x 2^58, the first differences, fits in 64 bits
   __shared__ long long pm[2][P * (TY + 2 * R)];
   __shared__ int pe[2][P * (TY + 2 * R)];
@@ -144,22 +143,21 @@ varc_march_kernel(Dims d, double i12h, double i12h2, double one, double two, dou
     const double kk[2] = {rho, __fma_rn(s, lap, __fma_rn(adv, i12h, mzero))};
     const int i = p.x0 + p.lx, j = p.y0 + p.ly, kz = p.k0 + k;
     up.apply(a, c, d.sv, kk, one, two,
-             [&](int64_t o, double x) { store_imaged(a.dst, d, i, j, kz, o, x, imaged); });
+             [&](int64_t o, double x) { store_imaged(a.dst, d, i, j, kz, o, x, a.imaged); });
     if (tape) {
       tape[c] = lap;  // read at the point only
       // D_d u is read at stencil neighbours by the transposed stage
 #pragma unroll
-      for (int q = 0; q < 3; ++q) store_imaged(tape, d, i, j, kz, (1 + q) * d.sv + c, t[q], imaged);
+      for (int q = 0; q < 3; ++q) store_imaged(tape, d, i, j, kz, (1 + q) * d.sv + c, t[q], a.imaged);
     }
   }
 }
 
 template <int TX, int TY>
-int launch_varc_march(const Dims& d, const Scalars& sc, const StageParams& a, double* tape, int imaged,
-                      cudaStream_t s) {
+int launch_varc_march(const Dims& d, const Scalars& sc, const StageParams& a, double* tape, cudaStream_t s) {
   const int zb = march_depth(d, TX, TY, kVarcThreads / (TX * TY));
   varc_march_kernel<TX, TY><<<march_grid(d, TX, TY, zb), TX * TY, 0, s>>>(
-      d, sc.i12h, sc.i12h2, sc.k[CHEMORA_K_ONE], sc.k[CHEMORA_K_TWO], sc.k[CHEMORA_K_MZERO], a, zb, tape, imaged);
+      d, sc.i12h, sc.i12h2, sc.k[CHEMORA_K_ONE], sc.k[CHEMORA_K_TWO], sc.k[CHEMORA_K_MZERO], a, zb, tape);
   return launched("varc_march_kernel");
 }
 

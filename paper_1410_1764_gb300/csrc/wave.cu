@@ -36,7 +36,7 @@ static int launch_wave_variant(const Dims& d, const Scalars& sc, const StagePara
 
 template <int TX, int TY>
 static int launch_varc_variant(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s) {
-  return launch_varc_march<TX, TY>(d, sc, a, nullptr, 0, s);
+  return launch_varc_march<TX, TY>(d, sc, a, nullptr, s);
 }
 
 // Planes in shared memory (wave_orders.cu) win where blocks marching through
