@@ -102,9 +102,9 @@ int effective_order(int kind, const chemora_params& p);
 
 // ghost fill of nvars grid functions (periodic image of the interior)
 int fill_ghosts(const Dims& d, int nvars, double* state, cudaStream_t s);
-// Stages of the variable-speed wave write their outputs' ghost images
-// themselves, with no fill passes between them, when every axis has at least g
-// points.
+// Every axis has at least g points: each ghost point lies within one period of
+// the interior, and stages of the variable-speed wave write their outputs'
+// ghost images themselves, with no fill passes between them.
 inline int imaged_ok(const Dims& d) { return d.nx >= d.g && d.ny >= d.g && d.nz >= d.g ? 1 : 0; }
 int fill_ghosts_axes(const Dims& d, int nvars, double* state, int mask, cudaStream_t s);
 
