@@ -137,9 +137,9 @@ int chemora_system_opcount(chemora_system* sys, int64_t* fp64_instructions, int6
     return CHEMORA_OK;
   }
   if (sys->kind == CHEMORA_BSSN) {
-    // the split kernels: the algebra, and three fmas per mixed derivative
-    // (the other differences run on the integer units)
-    if (fp64_instructions) *fp64_instructions = CHEMORA_OPS_BSSN_ALG_INSTR + 3 * 33;
+    // the split kernels: the algebra's body and prologue, and three fmas per
+    // mixed derivative (the other differences run on the integer units)
+    if (fp64_instructions) *fp64_instructions = CHEMORA_OPS_BSSN_ALG_INSTR + 44 + 3 * 33;
     if (flops) *flops = CHEMORA_OPS_BSSN_FLOPS;
     return CHEMORA_OK;
   }
