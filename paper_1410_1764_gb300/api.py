@@ -226,8 +226,10 @@ def opcount(kind):
 
 
 def variant_info(kind, variant):
-    """(tx, ty, min_blocks, sharing) of a compiled launch shape; sharing 0 =
-    direct body, 1 = x lanes, 2 = x lanes + y through shared memory."""
+    """(tx, ty, min_blocks, sharing) of a compiled launch shape; sharing 0 = a
+    point per thread (BSSN: field and algebra kernels; other wave orders and
+    systems: marching tiles), 1 = x lanes, 2 = x lanes + y through shared
+    memory, 4 = order-4 wave on marching tiles."""
     o = [ctypes.c_int() for _ in range(4)]
     check(lib().chemora_variant_info(int(kind), int(variant), *[ctypes.byref(x) for x in o]),
           "chemora_variant_info")

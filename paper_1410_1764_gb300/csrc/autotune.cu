@@ -3,8 +3,8 @@
 //
 // Candidates are the compiled block shapes of the system's stage kernel.  A
 // model ranks them by the threads they launch (x/y tile waste on ragged
-// grids), by wave quantisation (blocks per SM slot count) and by the FP64
-// instruction count of their body; candidates the model predicts more than
+// grids), by wave quantisation (blocks per SM slot count) and by their body's
+// relative work; candidates the model predicts more than
 // 1.5x slower than its best are skipped, the rest are timed with CUDA
 // events on the caller's grid (a middle RK stage, two repetitions after a
 // warm-up) and the fastest is kept by the system.  Shapes of one body

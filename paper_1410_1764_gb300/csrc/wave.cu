@@ -1,6 +1,6 @@
 // Scalar wave (Sec. 3, Eq. 1, two-variable form) and variable-speed wave
-// stage kernels.  Bodies generated from gen/systems.py; a few block shapes
-// are compiled for the autotuner.
+// stage kernels, stencils on the integer units; a few block shapes are compiled
+// for the autotuner.
 #include "internal.h"
 #include "stage.cuh"
 #include "star_march.cuh"
