@@ -23,16 +23,16 @@
 
 namespace chemora {
 
-// Neighbours at their periodic images: offsets of the wrapped x, y and z
-// indices (d = -2..2) in the padded layout, read through L2 (the grid may
-// start while its predecessor still runs, so nothing is read before the
-// dependency wait and nothing is served from the SM's L1).
+// The star's points of u at their periodic images, in Star2's order and the
+// centre, read through L2 (the grid may start while its predecessor still runs,
+// so nothing is read before the dependency wait and nothing is served from the
+// SM's L1).
 struct WrapLoader {
-  const double* p;  // variable 0 at the padded origin
+  const double* q[13];
   int64_t sv;
-  int ox[5], oy[5], oz[5];
   __device__ __forceinline__ double operator()(int v, int dx, int dy, int dz) const {
-    return __ldcg(p + v * sv + (int64_t)ox[dx + 2] + oy[dy + 2] + oz[dz + 2]);
+    const int a = dx != 0 ? 0 : (dy != 0 ? 4 : 8), m = dx + dy + dz;
+    return __ldcg(q[m == 0 ? 12 : a + (m == 1 ? 0 : (m == -1 ? 1 : (m == 2 ? 2 : 3)))] + v * sv);
   }
 };
 
@@ -70,21 +70,29 @@ __device__ __forceinline__ int wrap_index(int i, int n) { return i < 0 ? i + n :
 // fastest).
 __global__ void __launch_bounds__(128) wave_chain_stage_kernel(Dims d, Scalars sc, StageParams a) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int64_t t = (int64_t)blockIdx.x * 128 + threadIdx.x;
-  const int64_t npts = (int64_t)d.nx * d.ny * d.nz;
-  const int i = (int)(t % d.nx);
-  const int j = (int)((t / d.nx) % d.ny);
-  const int k = (int)(t / ((int64_t)d.nx * d.ny));
-  WrapLoader ld;
-  ld.p = a.src;
-  ld.sv = d.sv;
-#pragma unroll
-  for (int m = -2; m <= 2; ++m) {
-    ld.ox[m + 2] = wrap_index(i + m, d.nx) + d.g;
-    ld.oy[m + 2] = (wrap_index(j + m, d.ny) + d.g) * (int)d.sy;
-    ld.oz[m + 2] = (wrap_index(k + m, d.nz) + d.g) * (int)d.sz;
-  }
+  // 32-bit indices (chain_available): 64-bit divisions for the point's place
+  // took a third of the instructions.  The addresses are pinned here, before the
+  // wait, where they cost nothing: left to the compiler, 32-bit ones are formed
+  // after it (61 x 75 x 53 x 20 steps 525 us, 32^3 x 100 steps 1247; pinned 491
+  // and 1162; with 64-bit indices 530 and 1205).
+  const unsigned t = blockIdx.x * 128 + threadIdx.x;
+  const unsigned npts = (unsigned)d.nx * d.ny * d.nz;
+  const unsigned row = t / (unsigned)d.nx;
+  const int k = (int)(row / (unsigned)d.ny);
+  const int j = (int)(row - (unsigned)k * d.ny), i = (int)(t - row * d.nx);
   const int64_t c = (int64_t)(k + d.g) * d.sz + (int64_t)(j + d.g) * d.sy + (i + d.g);
+  WrapLoader ld;
+  ld.sv = d.sv;
+  ld.q[12] = a.src + c;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const int o = m == 0 ? 1 : (m == 1 ? -1 : (m == 2 ? 2 : -2));
+    ld.q[m] = ld.q[12] + (wrap_index(i + o, d.nx) - i);
+    ld.q[4 + m] = ld.q[12] + (wrap_index(j + o, d.ny) - j) * (int)d.sy;
+    ld.q[8 + m] = ld.q[12] + (wrap_index(k + o, d.nz) - k) * (int)d.sz;
+  }
+#pragma unroll
+  for (int m = 0; m < 13; ++m) asm volatile("" : "+l"(ld.q[m]));
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (t >= npts) return;
   ChainStageOut out{a, c, d.sv, sc.k[CHEMORA_K_ONE], sc.k[CHEMORA_K_TWO], {0.0, 0.0}, {0.0, 0.0}};
