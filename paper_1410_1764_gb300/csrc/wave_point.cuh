@@ -3,12 +3,12 @@
 // with x lanes and a z queue sharing differences) become one multiply and
 // about 200 integer operations, which run beside the FP64 update.  GB300, one
 // RK4 step: 256^3 3.21 -> 1.20 ms (0.97 on planes in shared memory,
-// wave_orders.cu); 61 x 75 x 53, launch-chained: 58.5 -> 24.5 us; 32^3, the
+// wave_orders.cu); 61 x 75 x 53, launch-chained: 58.5 -> 25.1 us; 32^3, the
 // same: 18.7 -> 11.6 us.  Bound by the integer pipes and the latency of its
 // loads (HBM alone would take 0.63 ms at 256^3).
 #pragma once
 #include "device_types.cuh"
-#include "fixedpoint.cuh"
+#include "star_march.cuh"
 #include "generated/gen_wave.cuh"
 
 namespace chemora {
@@ -41,16 +41,16 @@ struct Star2 {
   }
 };
 
-// 12 h^2 times the order-4 Laplacian: 16 sum (u+-1) - sum (u+-2) - 90 u.  The
-// weights' magnitudes add up to 192, so two guard bits fit in 64 bits.
+// 12 h^2 times the order-4 Laplacian: 16 sum (u+-1) - sum (u+-2) - 90 u.
 CHEMORA_FX double star2_lap(const Star2& s, int e) {
-  long long s1 = 0, s2 = 0;
+  constexpr int K = Guard<2>::lap;
+  long long t[2] = {0, 0};
 #pragma unroll
   for (int q = 0; q < 12; q += 4) {
-    s1 += fx::align<2>(s.n[q], e) + fx::align<2>(s.n[q + 1], e);
-    s2 += fx::align<2>(s.n[q + 2], e) + fx::align<2>(s.n[q + 3], e);
+    t[0] += fx::align<K>(s.n[q], e) + fx::align<K>(s.n[q + 1], e);
+    t[1] += fx::align<K>(s.n[q + 2], e) + fx::align<K>(s.n[q + 3], e);
   }
-  return fx::to_double<2>(16 * s1 - s2 - 90 * fx::align<2>(s.c, e), e);
+  return star_lap<2>(t, fx::align<K>(s.c, e), e);
 }
 
 // Loader of a point whose star is at hand, for the FP64 body.

@@ -73,7 +73,7 @@ def _weights(R, ns):
     return [int(w * den) for w in out]
 
 
-GUARD = {ns: {1: 4 if ns else 6, 2: 4 if ns else 2, 3: 6, 4: 6} for ns in (0, 1, 3)}
+GUARD = {ns: {1: 6, 2: 4 if ns else 6, 3: 6, 4: 6} for ns in (0, 1, 3)}
 
 
 @pytest.mark.parametrize("R", [1, 2, 3, 4])
