@@ -86,7 +86,7 @@ bssn_fields_kernel(const FieldRegion* __restrict__ regions, FieldRegion one_regi
   for (int m = 0; m < 7; ++m) z[m] = fx::Parts{0, 0};
   if (active) {
 #pragma unroll
-    for (int m = 1; m < 7; ++m) z[m] = fx::parts<kGuard>(__ldg(col + (int64_t)(m - 4) * d.sz));
+    for (int m = 1; m < 7; ++m) z[m] = fx::parts_or_zero<kGuard>(__ldg(col + (int64_t)(m - 4) * d.sz));
     znext = __ldg(col + 3 * d.sz);
   }
   if (halo) hnext = __ldg(hp);
@@ -97,13 +97,13 @@ bssn_fields_kernel(const FieldRegion* __restrict__ regions, FieldRegion one_regi
     int* const E = pe[k & 1];
 #pragma unroll
     for (int m = 0; m < 6; ++m) z[m] = z[m + 1];
-    z[6] = fx::parts<kGuard>(znext);
+    z[6] = fx::parts_or_zero<kGuard>(znext);
     if (active) {
       M[pc] = z[3].m;
       E[pc] = z[3].e;
     }
     if (halo) {
-      const fx::Parts q = fx::parts<kGuard>(hnext);
+      const fx::Parts q = fx::parts_or_zero<kGuard>(hnext);
       M[hc] = q.m;
       E[hc] = q.e;
       if (k + 1 < nz) hnext = __ldg(hp + (int64_t)(k + 1) * d.sz);
@@ -122,7 +122,7 @@ bssn_fields_kernel(const FieldRegion* __restrict__ regions, FieldRegion one_regi
         e = fx::emax(e, fx::emax(fx::emax(ex[m], ey[m]), z[m < 3 ? m : m + 1].e));
       }
       double d1[3], d2[3], ko = 0.0;
-      if (fx::in_range(e)) {
+      if (e == fx::kZeroExp || fx::in_range(e)) {  // (of zeros alone, all differences are exactly zero)
         const long long c = fx::align(z[3], e);
         const long long c30 = 30 * c;
         long long s1t = 0, s2t = 0, s3t = 0;
@@ -148,7 +148,7 @@ bssn_fields_kernel(const FieldRegion* __restrict__ regions, FieldRegion one_regi
         const int r = (15 * ((int)s1t & 3) - 6 * ((int)s2t & 3) + ((int)s3t & 3)) >> 2;
         ko = fx::to_double<kGuard - 2>(15 * (s1t >> 2) - 6 * (s2t >> 2) + (s3t >> 2) - 15 * c + r, e);
       } else {
-        // zeros (all differences zero), the ends of the FP64 range, Inf, NaN
+        // the ends of the FP64 range, Inf, NaN
         const int64_t st[3] = {1, d.sy, d.sz};
         const double* p = col + (int64_t)k * d.sz;
         const double c = __ldg(p);
