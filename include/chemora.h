@@ -120,8 +120,9 @@ int chemora_fill_ghosts_axes(chemora_system* sys, double* state, int axes, void*
 /* rhs <- RHS(state) on the interior (Sec. 3.2: the "RHS" calculation).  The
  * ghosts of state must be valid; the ghosts of rhs are left untouched.
  * state and rhs must not overlap.  A BSSN system takes a workspace of
- * derivative fields from a pool of its own in stream order (also in
- * chemora_stage and chemora_constraints), so calls on several streams do not
+ * derivative fields from the device's pool in stream order (also in
+ * chemora_stage and chemora_constraints; the pool is shared by all systems,
+ * keeps up to 4 GB while one exists and 64 MB when none does), so calls on several streams do not
  * share one; without a workspace (a stream that is being captured, no memory
  * left) it runs a slower kernel that agrees to rounding. */
 int chemora_rhs(chemora_system* sys, const double* state, double* rhs, void* stream);

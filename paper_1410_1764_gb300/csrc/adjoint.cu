@@ -410,18 +410,11 @@ extern "C" int chemora_adjoint_rk4(chemora_system* sys, const double* state0, co
   const size_t nfields = 1 + 3 + 2 + 2 * (size_t)nck + 16 * (size_t)K + 2 + 2 + 2 + 2 + 1;
   const size_t bytes = (nfields * fs + 32) * sizeof(double) + (size_t)nrecv * (sizeof(int64_t) + sizeof(double));
   char* buf = nullptr;
-  // kept by the system's pool: from the device's own pool, which gives freed
-  // memory back at each synchronisation, 3.4 GB cost about 10 ms a call
-  const cudaMemPool_t pool = system_pool(sys);
-  cudaError_t e = pool ? cudaMallocFromPoolAsync((void**)&buf, bytes, pool, s) : cudaErrorMemoryAllocation;
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    e = cudaMallocAsync((void**)&buf, bytes, s);
-  }
-  if (e != cudaSuccess) {
-    cudaGetLastError();
+  // from the device's pool: from CUDA's default one, which gives freed memory
+  // back at each synchronisation, 3.4 GB cost about 10 ms a call
+  const cudaError_t e = pool_alloc((void**)&buf, bytes, s);
+  if (e != cudaSuccess)
     return set_error(CHEMORA_ENOMEM, "adjoint work space of %zu bytes: %s", bytes, cudaGetErrorString(e));
-  }
   AdjBufs B;
   double* q = (double*)buf;
   B.s = q; q += fs;
@@ -498,7 +491,7 @@ extern "C" int chemora_adjoint_rk4(chemora_system* sys, const double* state0, co
     return CHEMORA_OK;
   };
   rc = run();
-  cudaFreeAsync(buf, s);
+  pool_free(buf, s);
   cudaError_t e2 = cudaStreamSynchronize(s);
   if (rc) return rc;
   if (e2 != cudaSuccess) return cuda_error(e2, "cudaStreamSynchronize(adjoint)");

@@ -401,14 +401,14 @@ static int create_amr(int kind, const int* nc, int nbox, const int* lo, const in
   const size_t cs = (size_t)nv * A->dc.sv;
   const size_t total = cs * (1 + 3 + 3) + (size_t)foff * (1 + 3) + (size_t)woff;
   double* buf = nullptr;
-  cudaError_t e = cudaMalloc(&buf, total * sizeof(double));
+  cudaError_t e = device_alloc(&buf, total * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(buf, 0, total * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&A->dev_boxes, nbox * sizeof(AmrBox));
-  if (e == cudaSuccess) e = cudaMalloc(&A->dev_pd, 4 * nbox * sizeof(PatchDesc));
-  if (e == cudaSuccess && kind == CHEMORA_WAVE) e = cudaMalloc(&A->items, items.size() * sizeof(WorkItem));
-  if (e == cudaSuccess && kind == CHEMORA_BSSN) e = cudaMalloc(&A->work, field_work_bytes(A->work_points));
-  if (e == cudaSuccess) e = cudaMalloc(&A->counters, 2 * A->counter_off[4] * sizeof(unsigned int));
-  if (e == cudaSuccess) e = cudaMalloc(&A->err, sizeof(int));
+  if (e == cudaSuccess) e = device_alloc(&A->dev_boxes, nbox * sizeof(AmrBox));
+  if (e == cudaSuccess) e = device_alloc(&A->dev_pd, 4 * nbox * sizeof(PatchDesc));
+  if (e == cudaSuccess && kind == CHEMORA_WAVE) e = device_alloc(&A->items, items.size() * sizeof(WorkItem));
+  if (e == cudaSuccess && kind == CHEMORA_BSSN) e = device_alloc(&A->work, field_work_bytes(A->work_points));
+  if (e == cudaSuccess) e = device_alloc(&A->counters, 2 * A->counter_off[4] * sizeof(unsigned int));
+  if (e == cudaSuccess) e = device_alloc(&A->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(A->err, 0, sizeof(int));
   if (e == cudaSuccess)
     e = cudaMemcpy(A->dev_boxes, A->boxes.data(), nbox * sizeof(AmrBox), cudaMemcpyHostToDevice);

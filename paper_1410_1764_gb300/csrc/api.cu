@@ -8,7 +8,6 @@
 #include <string.h>
 
 #include <atomic>
-#include <mutex>
 #include <new>
 
 #include "internal.h"
@@ -124,7 +123,7 @@ const LaunchVariant* variant_info(int kind, int v) {
 int ensure_scratch(chemora_system* sys) {
   if (sys->scratch) return CHEMORA_OK;
   const size_t n = (size_t)sys->nvars * sys->grid->fsize;
-  cudaError_t e = cudaMalloc(&sys->scratch, 3 * n * sizeof(double));
+  cudaError_t e = device_alloc(&sys->scratch, 3 * n * sizeof(double));
   if (e != cudaSuccess) {
     sys->scratch = nullptr;
     cudaGetLastError();
@@ -172,7 +171,7 @@ FieldWork system_field_work(chemora_system* sys, bool alloc) {
   if (sys->kind != CHEMORA_BSSN || !bssn_shape_splits(sys->grid->d, sys->variant)) return w;
   if (!sys->field_work && alloc) {
     const int64_t points = field_work_points(sys->grid->d);
-    if (cudaMalloc(&sys->field_work, field_work_bytes(points)) == cudaSuccess) {
+    if (device_alloc(&sys->field_work, field_work_bytes(points)) == cudaSuccess) {
       sys->field_points = points;
     } else {
       sys->field_work = nullptr;
@@ -184,23 +183,6 @@ FieldWork system_field_work(chemora_system* sys, bool alloc) {
   return w;
 }
 
-cudaMemPool_t system_pool(chemora_system* sys) {
-  static std::mutex m;  // right-hand sides of one system may run in several threads
-  const std::lock_guard<std::mutex> lock(m);
-  if (sys->pool) return sys->pool;
-  cudaMemPoolProps props = {};
-  props.allocType = cudaMemAllocationTypePinned;
-  props.location.type = cudaMemLocationTypeDevice;
-  if (cudaGetDevice(&props.location.id) != cudaSuccess || cudaMemPoolCreate(&sys->pool, &props) != cudaSuccess) {
-    sys->pool = nullptr;
-    cudaGetLastError();
-    return nullptr;
-  }
-  uint64_t keep = (uint64_t)8 << 30;  // memory kept between calls, until the system is destroyed
-  cudaMemPoolSetAttribute(sys->pool, cudaMemPoolAttrReleaseThreshold, &keep);
-  return sys->pool;
-}
-
 FieldWork take_field_work(chemora_system* sys, cudaStream_t s) {
   FieldWork w;
   cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
@@ -208,21 +190,16 @@ FieldWork take_field_work(chemora_system* sys, cudaStream_t s) {
     cudaGetLastError();
     return w;
   }
-  const cudaMemPool_t pool = system_pool(sys);
-  if (!pool) return w;
   const int64_t points = field_work_points(sys->grid->d);
   void* p = nullptr;
-  if (cudaMallocFromPoolAsync(&p, field_work_bytes(points), pool, s) != cudaSuccess) {
-    cudaGetLastError();
-    return w;
-  }
+  if (pool_alloc(&p, field_work_bytes(points), s) != cudaSuccess) return w;
   w.w = static_cast<double*>(p);
   w.points = points;
   return w;
 }
 
 void give_field_work(const FieldWork& w, cudaStream_t s) {
-  if (w.w) cudaFreeAsync(w.w, s);
+  if (w.w) pool_free(w.w, s);
 }
 
 static int run_stage(chemora_system* sys, const StageParams& a, const FieldWork& work, cudaStream_t s) {
@@ -280,7 +257,7 @@ void free_step_graph(chemora_system* sys) {
 }
 
 // One right-hand side or stage of a call that shares no scratch with others:
-// its derivative fields come from the system's pool, in stream order.
+// its derivative fields come from the device's pool, in stream order.
 static int run_single_stage(chemora_system* sys, const StageParams& p, cudaStream_t s) {
   FieldWork work;
   if (sys->kind == CHEMORA_BSSN && bssn_shape_splits(sys->grid->d, sys->variant)) work = take_field_work(sys, s);
@@ -374,6 +351,7 @@ int chemora_system_create(chemora_grid* grid, int kind, const chemora_params* pa
   s->nvars = grid->nvars;
   s->params = p;
   s->sc = make_scalars(grid->dx, p);
+  pool_count_systems(1);
   *out = s;
   return CHEMORA_OK;
 }
@@ -434,7 +412,7 @@ int chemora_rk4_step_host(chemora_system* sys, double* host_state, double dt, in
   if (!host_state) return set_error(CHEMORA_EINVAL, "host_state is NULL");
   const size_t bytes = (size_t)sys->nvars * sys->grid->fsize * sizeof(double);
   if (!sys->dev_state) {
-    cudaError_t e = cudaMalloc(&sys->dev_state, bytes);
+    cudaError_t e = device_alloc(&sys->dev_state, bytes);
     if (e != cudaSuccess) {
       sys->dev_state = nullptr;
       cudaGetLastError();

@@ -197,7 +197,7 @@ int chemora_autotune(chemora_system* sys, double* state, int* variant, double* b
   if (rc == CHEMORA_OK && chain_available(sys)) {
     const size_t bytes = n * sizeof(double);
     double* tmp = nullptr;
-    if (cudaMalloc(&tmp, bytes) == cudaSuccess) {
+    if (device_alloc(&tmp, bytes) == cudaSuccess) {
       const double dt = 0.25 * sys->grid->dx;
       float tm[2] = {1e30f, 1e30f};
       for (int m = 0; m < 2 && rc == CHEMORA_OK; ++m) {

@@ -404,9 +404,9 @@ int field_plan_create(const std::vector<PatchDesc>& patches, FieldPlan* plan) {
     return set_error(CHEMORA_EINVAL, "too many work items");
   plan->nregions = (int)regions.size();
   plan->nitems = (int)items.size();
-  cudaError_t e = cudaMalloc(&plan->regions, regions.size() * sizeof(FieldRegion));
-  if (e == cudaSuccess) e = cudaMalloc(&plan->items, items.size() * sizeof(WorkItem));
-  if (e == cudaSuccess) e = cudaMalloc(&plan->tiles, tiles.size() * sizeof(int2));
+  cudaError_t e = device_alloc(&plan->regions, regions.size() * sizeof(FieldRegion));
+  if (e == cudaSuccess) e = device_alloc(&plan->items, items.size() * sizeof(WorkItem));
+  if (e == cudaSuccess) e = device_alloc(&plan->tiles, tiles.size() * sizeof(int2));
   if (e == cudaSuccess)
     e = cudaMemcpy(plan->regions, regions.data(), regions.size() * sizeof(FieldRegion), cudaMemcpyHostToDevice);
   if (e == cudaSuccess)

@@ -62,13 +62,12 @@ struct chemora_system {
   double* coef;
   // device copy of a host state for chemora_rk4_step_host (library-owned)
   double* dev_state;
-  // derivative fields of the split BSSN right-hand side: a workspace for the
-  // RK4 driver (allocated on first use), and a pool for calls that may run on
-  // several streams at once (chemora_rhs, chemora_stage, chemora_constraints)
-  // and for the adjoint's work space
+  // derivative fields of the split BSSN right-hand side for the RK4 driver
+  // (allocated on first use); calls that may run on several streams at once
+  // (chemora_rhs, chemora_stage, chemora_constraints) take theirs from the
+  // device's pool
   double* field_work;
   int64_t field_points;
-  cudaMemPool_t pool;
   // launch shape chosen by the autotuner (index into the kind's variants)
   int variant;
   // CUDA graph of one RK4 step (captured on cap_stream, replayed on the
@@ -125,11 +124,21 @@ int launch_constraints_split(const Dims& d, const Scalars& sc, const double* sta
 bool bssn_shape_splits(const Dims& d, int variant);
 // The RK4 driver's workspace (no workspace if there is no memory for one or
 // alloc is false and there is none yet), and one taken from and given back to
-// the system's pool in stream order.
+// the device's pool in stream order.
 FieldWork system_field_work(chemora_system* sys, bool alloc);
-cudaMemPool_t system_pool(chemora_system* sys);  // NULL: none could be made
 FieldWork take_field_work(chemora_system* sys, cudaStream_t s);
 void give_field_work(const FieldWork& w, cudaStream_t s);
+
+// device memory in stream order from the device's pool (pool.cu), and for good
+// (cudaMalloc; the pool's unused memory makes room)
+cudaError_t pool_alloc(void** p, size_t bytes, cudaStream_t s);
+void pool_free(void* p, cudaStream_t s);
+void pool_count_systems(int by);  // a system was made (+1) or destroyed (-1)
+cudaError_t device_alloc(void** p, size_t bytes);
+template <class T>
+cudaError_t device_alloc(T** p, size_t bytes) {
+  return device_alloc(reinterpret_cast<void**>(p), bytes);
+}
 
 int launch_stage(int kind, const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s,
                  int variant = 0, const FieldWork& work = FieldWork());

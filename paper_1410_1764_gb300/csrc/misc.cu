@@ -115,12 +115,12 @@ void chemora_destroy(void* handle) {
     if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
     if (s->scratch) cudaFree(s->scratch);
     if (s->field_work) cudaFree(s->field_work);
-    if (s->pool) cudaMemPoolDestroy(s->pool);
     if (s->coef) cudaFree(s->coef);
     if (s->dev_state) cudaFree(s->dev_state);
     for (cudaEvent_t e : s->ev_pool) cudaEventDestroy(e);
     s->type = 0;
     delete s;
+    pool_count_systems(-1);
   } else if (is_handle(handle, H_BATCH)) {
     destroy_batch((chemora_batch*)handle);
   } else if (is_handle(handle, H_AMR)) {

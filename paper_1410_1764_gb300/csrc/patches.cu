@@ -342,14 +342,14 @@ int chemora_patches_create(int npatch, const int* dims, int nghost, double dx, i
     b->items = b->plan.items;
     b->nitems = b->plan.nitems;
     b->ncounters = (int)b->plan.chunks.size();
-    e = cudaMalloc(&b->work, field_work_bytes(b->plan.points));
+    e = device_alloc(&b->work, field_work_bytes(b->plan.points));
   }
-  if (e == cudaSuccess) e = cudaMalloc(&b->state, off * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&b->scratch, 3 * off * sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&b->dev_pd, npatch * sizeof(PatchDesc));
-  if (e == cudaSuccess && kind == CHEMORA_WAVE) e = cudaMalloc(&b->items, items.size() * sizeof(WorkItem));
-  if (e == cudaSuccess) e = cudaMalloc(&b->counters, 4 * b->ncounters * sizeof(unsigned int));
-  if (e == cudaSuccess) e = cudaMalloc(&b->err, sizeof(int));
+  if (e == cudaSuccess) e = device_alloc(&b->state, off * sizeof(double));
+  if (e == cudaSuccess) e = device_alloc(&b->scratch, 3 * off * sizeof(double));
+  if (e == cudaSuccess) e = device_alloc(&b->dev_pd, npatch * sizeof(PatchDesc));
+  if (e == cudaSuccess && kind == CHEMORA_WAVE) e = device_alloc(&b->items, items.size() * sizeof(WorkItem));
+  if (e == cudaSuccess) e = device_alloc(&b->counters, 4 * b->ncounters * sizeof(unsigned int));
+  if (e == cudaSuccess) e = device_alloc(&b->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(b->state, 0, off * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(b->scratch, 0, 3 * off * sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(b->err, 0, sizeof(int));

@@ -1,0 +1,84 @@
+"""The pool that single BSSN calls take their derivative fields from: systems
+destroyed with a call in flight, the first call of a new system, memory held by
+idle systems, and memory given back once none is left.  In a process of its own:
+a crash ends that process alone, and no other test's systems count."""
+import subprocess
+import sys
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+SCRIPT = r"""
+import gc, time
+import torch
+from paper_1410_1764_gb300 import api, synth
+
+def state(n):
+    p = torch.randn(24, n + 6, n + 6, n + 6, device="cuda", dtype=torch.float64) * 1e-2
+    return p + torch.from_numpy(synth.BSSN_FLAT).cuda()[:, None, None, None]
+
+def system(n):
+    return api.make_system(api.BSSN, n, n, n, 1.0 / n)
+
+def free():
+    gc.collect()
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+def wall(f):
+    torch.cuda.synchronize()
+    t = time.perf_counter()
+    f()
+    torch.cuda.synchronize()
+    return time.perf_counter() - t
+
+y16, y64 = state(16), state(64)
+outs = [torch.empty_like(y64) for _ in range(2)]
+con = torch.empty(7, *y64.shape[1:], device="cuda", dtype=torch.float64)
+torch.cuda.synchronize()
+start = free()
+
+# destroyed with a right-hand side or the constraints in flight
+for _ in range(10):
+    system(64).rhs(y64, outs[0])
+    system(64).constraints(y64, con)
+torch.cuda.synchronize()
+a = system(64)
+a.rhs(y64, outs[1])
+assert torch.equal(outs[0][:, 3:-3, 3:-3, 3:-3], outs[1][:, 3:-3, 3:-3, 3:-3])
+
+# eight idle systems hold no more than one
+one = free()
+more = [system(64) for _ in range(8)]
+for s in more:
+    s.rhs(y64, outs[0])
+assert one - free() < 32 << 20, (one, free())
+
+# a new system's first right-hand side: 2.6 times its second's time with a pool of its own
+out16 = torch.empty_like(y16)
+steady = min(wall(lambda: more[0].rhs(y64, outs[0])) for _ in range(3))
+small = system(16)
+small.rhs(y16, out16)
+second = min(wall(lambda: small.rhs(y16, out16)) for _ in range(20))
+first = []
+for _ in range(5):
+    s = system(16)
+    first.append(wall(lambda: s.rhs(y16, out16)))
+    more.append(s)
+assert min(first) < 1.5 * second + 2e-5, (first, second)
+
+# with no system left the memory goes back
+del a, s, small
+more.clear()
+assert start - free() < 192 << 20, (start, free())
+print("ok")
+"""
+
+
+def test_pool():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    r = subprocess.run([sys.executable, "-c", SCRIPT], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip().endswith("ok"), (r.returncode, r.stderr[-2000:])
