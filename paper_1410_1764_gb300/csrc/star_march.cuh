@@ -98,6 +98,22 @@ CHEMORA_FX double star_d1(const long long (&t)[R], int e) {
   }
 }
 
+// One axis of an order-4 star from its values' significands and exponents at
+// offsets -2, -1, 1, 2, aligned to the largest exponent e of the four, so that a
+// first difference is as close as in FP64 however large the values along the
+// other axes are.
+struct Axis4 {
+  long long near, far;  // sums of the pairs at distance 1 and 2
+  long long diff;       // 12 h D f: 8 (f(+1) - f(-1)) - (f(+2) - f(-2)), at most 18 2^(53 + K)
+  CHEMORA_FX Axis4(const long long (&m)[4], const int (&x)[4], int e) {
+    const long long a = fx::sar(m[0], (unsigned)(e - x[0])), b = fx::sar(m[1], (unsigned)(e - x[1]));
+    const long long c = fx::sar(m[2], (unsigned)(e - x[2])), d = fx::sar(m[3], (unsigned)(e - x[3]));
+    near = c + b;
+    far = d + a;
+    diff = 8 * (c - b) - (d - a);
+  }
+};
+
 // Offset m of 2R taken in the order -R .. -1, 1 .. R.
 template <int R>
 CHEMORA_FX constexpr int tap(int m) { return m < R ? m - R : m - R + 1; }

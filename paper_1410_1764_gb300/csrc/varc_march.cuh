@@ -1,8 +1,12 @@
 // Stage kernel of the variable-speed wave equation (u_t = rho, rho_t = s Lap u
 // + sum_d G_d D_d u, s = c^2, G_d = D_d s) with its stencils on the integer
 // units (star_march.cuh), shared by the Runge-Kutta driver and the adjoint's
-// forward pass.  GB300, 128^3: 55 us per stage against 180 us in FP64 (45
+// forward pass.  GB300, 128^3: 52 us per stage against 180 us in FP64 (45
 // instructions); ten FP64 instructions are left (36 us), HBM alone takes 30.
+// Each axis' values are aligned to their own largest exponent (to the star's, a
+// first difference beside larger values along another axis lost digits: 51 us);
+// one, two or three of the first differences through the conversion instruction:
+// 55, 57, 59 us.
 #pragma once
 #include "internal.h"
 #include "star_march.cuh"
@@ -84,7 +88,7 @@ varc_march_kernel(Dims d, double i12h, double i12h2, double one, double two, dou
     long long* const M = pm[k & 1];
     int* const E = pe[k & 1];
     MarchUpdate<2> up;
-    double rho = 0.0, s = 0.0, G[3] = {0.0, 0.0, 0.0};
+    double rho = 0.0, speed2 = 0.0, G[3] = {0.0, 0.0, 0.0};
 #pragma unroll
     for (int m = 0; m < 4; ++m) z[m] = z[m + 1];
     z[4] = fx::parts_or_zero<K>(znext);
@@ -92,7 +96,7 @@ varc_march_kernel(Dims d, double i12h, double i12h2, double one, double two, dou
       M[pc] = z[2].m;
       E[pc] = z[2].e;
       rho = __ldg(a.src + d.sv + c);
-      s = __ldg(a.coef + c);
+      speed2 = __ldg(a.coef + c);
 #pragma unroll
       for (int q = 0; q < 3; ++q) G[q] = __ldg(a.coef + (1 + q) * d.sv + c);
       up.load(a, c, d.sv);
@@ -109,38 +113,37 @@ varc_march_kernel(Dims d, double i12h, double i12h2, double one, double two, dou
       }
     __syncthreads();
     if (!p.active) continue;
-    int ex[4], ey[4], e = z[2].e;
+    int x[3][4], ea[3], e = z[2].e;
+    unsigned low = ~0u;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      ex[m] = E[pc + tap<R>(m)];
-      ey[m] = E[pc + tap<R>(m) * P];
-      e = fx::emax(e, fx::emax(fx::emax(ex[m], ey[m]), z[2 + tap<R>(m)].e));
+    for (int ax = 0; ax < 3; ++ax) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) x[ax][q] = ax == 2 ? z[2 + tap<R>(q)].e : E[pc + tap<R>(q) * (ax == 0 ? 1 : P)];
+      ea[ax] = fx::emax(fx::emax(x[ax][0], x[ax][1]), fx::emax(x[ax][2], x[ax][3]));
+      low = min(low, (unsigned)ea[ax]);  // (an axis of zeros, kZeroExp, is a large number)
+      e = fx::emax(e, ea[ax]);
     }
     double lap = 0.0, t[3] = {0.0, 0.0, 0.0};
-    if (star_ok<R>(e)) {
-      if (e != fx::kZeroExp) {
-        long long s2[R] = {0, 0};
+    if (low >= (unsigned)fx::kExpMin && star_ok<R>(e)) {
+      // each axis' values to their own largest exponent, the pairs' sums then to the star's
+      long long s[R] = {0, 0};
 #pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
-          long long f[4];
+      for (int ax = 0; ax < 3; ++ax) {
+        long long m[4];
 #pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            const int o = tap<R>(m);
-            f[m] = ax == 0 ? fx::sar(M[pc + o], (unsigned)(e - ex[m]))
-                           : (ax == 1 ? fx::sar(M[pc + o * P], (unsigned)(e - ey[m])) : fx::align(z[2 + o], e));
-          }
-          s2[0] += f[2] + f[1];
-          s2[1] += f[3] + f[0];
-          t[ax] = fx::to_double<K>(8 * (f[2] - f[1]) - (f[3] - f[0]), e);
-        }
-        lap = star_lap<R, K>(s2, fx::align(z[2], e), e);
+        for (int q = 0; q < 4; ++q) m[q] = ax == 2 ? z[2 + tap<R>(q)].m : M[pc + tap<R>(q) * (ax == 0 ? 1 : P)];
+        const Axis4 f(m, x[ax], ea[ax]);
+        t[ax] = fx::to_double<K>(f.diff, ea[ax]);
+        s[0] += fx::sar(f.near, (unsigned)(e - ea[ax]));
+        s[1] += fx::sar(f.far, (unsigned)(e - ea[ax]));
       }
+      lap = star_lap<R, K>(s, fx::align(z[2], e), e);
     } else {
       star2_fp64(a.src + c, d, &lap, t);
     }
     lap = __fma_rn(lap, i12h2, mzero);
     const double adv = __fma_rn(G[2], t[2], __fma_rn(G[1], t[1], __fma_rn(G[0], t[0], mzero)));
-    const double kk[2] = {rho, __fma_rn(s, lap, __fma_rn(adv, i12h, mzero))};
+    const double kk[2] = {rho, __fma_rn(speed2, lap, __fma_rn(adv, i12h, mzero))};
     const int i = p.x0 + p.lx, j = p.y0 + p.ly, kz = p.k0 + k;
     up.apply(a, c, d.sv, kk, one, two,
              [&](int64_t o, double x) { store_imaged(a.dst, d, i, j, kz, o, x, a.imaged); });

@@ -4,7 +4,7 @@
 // about 200 integer operations, which run beside the FP64 update.  GB300, one
 // RK4 step: 256^3 3.21 -> 1.20 ms (0.97 on planes in shared memory,
 // wave_orders.cu); 61 x 75 x 53, launch-chained: 58.5 -> 25.1 us; 32^3, the
-// same: 18.7 -> 11.6 us.  Bound by the integer pipes and the latency of its
+// same: 18.7 -> 12.0 us.  Bound by the integer pipes and the latency of its
 // loads (HBM alone would take 0.63 ms at 256^3).
 #pragma once
 #include "device_types.cuh"

@@ -93,6 +93,23 @@ template <int R> static void star(const double* f, double c, double* out) {
     out[5 + 2 * a] = star_d1<R>(t, e) * (1.0 / Central<R>::den1);
   }
 }
+// order-4 first differences with an axis of its own exponent (the variable-speed wave's): FP64 and integers, over 12 h
+extern "C" void axes(const double* f, double* out) {
+  constexpr int K = 5;
+  for (int a = 0; a < 3; ++a) {
+    const double p1 = f[4 * a], m1 = f[4 * a + 1], p2 = f[4 * a + 2], m2 = f[4 * a + 3];
+    out[2 * a] = fma(8.0, p1 - m1, -(p2 - m2));
+    const double v[4] = {m2, m1, p1, p2};
+    long long m[4];
+    int x[4], e = fx::kZeroExp;
+    for (int q = 0; q < 4; ++q) {
+      m[q] = fx::parts_or_zero<K>(v[q]).m;
+      x[q] = fx::parts_or_zero<K>(v[q]).e;
+      e = fx::emax(e, x[q]);
+    }
+    out[2 * a + 1] = fx::to_double<K>(Axis4(m, x, e).diff, e);
+  }
+}
 extern "C" void run(int R, const double* f, double c, double* out) {
   R == 1 ? star<1>(f, c, out) : R == 2 ? star<2>(f, c, out) : R == 3 ? star<3>(f, c, out) : star<4>(f, c, out);
 }
@@ -168,3 +185,18 @@ def test_no_further_from_exact_than_fp64(L, R, field):
     rms = np.sqrt(np.stack([sq[0], sq[1], sq[2:].mean(0)]))  # the Laplacian, the divergence, the first differences
     # 1e-3: the scale of orders 6 and 8 is rounded
     assert (rms[:, 1] <= rms[:, 0] * 1.001 + 1e-3).all(), rms
+
+
+@pytest.mark.parametrize("field", FIELDS)
+def test_axis_differences(L, field):
+    """Relative to the largest value of the axis itself."""
+    err = []
+    for f, _ in stars(field, 2, 400, np.random.default_rng(7)):
+        out = (ctypes.c_double * 6)()
+        L.axes((ctypes.c_double * 12)(*f), out)
+        for a in range(3):
+            p1, m1, p2, m2 = (Fraction(q) for q in f[4 * a:4 * a + 4])
+            exact, top = 8 * (p1 - m1) - (p2 - m2), ulp(max(map(abs, f[4 * a:4 * a + 4])))
+            err.append([float(Fraction(out[2 * a + m]) - exact) / top for m in range(2)])
+    rms = np.sqrt((np.array(err) ** 2).mean(0))
+    assert rms[1] <= rms[0], rms
