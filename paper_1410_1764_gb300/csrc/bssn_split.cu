@@ -6,6 +6,7 @@
 #include "internal.h"
 #include "bssn_algebra.cuh"
 #include "bssn_split.h"
+#include "star_march.cuh"
 #include "generated/gen_bssn_constraints_alg.cuh"
 
 namespace chemora {
@@ -22,16 +23,18 @@ constexpr int kGuard = 4;       // guard bits: an axis' weights add up to 64 in 
 // through zb planes, a point per thread and plane.  Each value is taken apart
 // into integers once: a thread keeps its column's seven values in registers,
 // the plane in hand lies in shared memory (significands and exponents) with
-// its halo, so a tap costs a shift to the star's largest exponent and an
-// addition.  First differences go back to doubles through the conversion
+// its halo, so a tap costs a shift and an addition.  An axis' differences are
+// aligned to its own largest exponent (to the star's, they lost digits beside
+// larger values along another axis), the dissipation to the star's.  First differences go back to doubles through the conversion
 // instruction, the others by integer operations, which shares the work
 // between the two pipes.  The mixed derivatives are first-derivative stencils
 // of the neighbours' first-derivative rows, in FP64 (three fmas each: fewer
 // cycles than their 16 points in integers); the rows pass through shared
 // memory, those past the tile's edge are computed by the block again.
 //
-// GB300, all 24 variables of 128 x 128 x 64 points: 546 us (the field writes
-// alone take 200 us of HBM time); each value taken apart by each of its 19
+// GB300, all 24 variables of 128 x 128 x 64 points: 578 us (the field writes
+// alone take 200 us of HBM time).  With every value aligned to the star's
+// largest exponent 546 us, and then: each value taken apart by each of its 19
 // readers, no march: 846 us; conversion instruction for every difference 603,
 // for none 572 us; two or four blocks per SM 637, 708 us; significand and
 // exponent in one 16-byte cell 621 us; one kernel for both sorts of variable
@@ -113,40 +116,51 @@ bssn_fields_kernel(const FieldRegion* __restrict__ regions, FieldRegion one_regi
     double* out = work + field_base(point);
     point += (int64_t)d.nx * d.ny;
     if (active) {
-      int ex[6], ey[6], e = z[3].e;
+      // each axis' largest exponent over the offsets -2, -1, 1, 2, and the star's
+      int x[3][6], ea[3], e = z[3].e;
+      unsigned low = (unsigned)e;
 #pragma unroll
-      for (int m = 0; m < 6; ++m) {
-        const int o = m < 3 ? m - 3 : m - 2;
-        ex[m] = E[pc + o];
-        ey[m] = E[pc + o * pp];
-        e = fx::emax(e, fx::emax(fx::emax(ex[m], ey[m]), z[m < 3 ? m : m + 1].e));
+      for (int a = 0; a < 3; ++a) {
+#pragma unroll
+        for (int m = 0; m < 6; ++m) {
+          const int o = m < 3 ? m - 3 : m - 2;
+          x[a][m] = a == 2 ? z[3 + o].e : E[pc + o * (a == 0 ? 1 : pp)];
+        }
+        ea[a] = fx::emax(fx::emax(x[a][1], x[a][2]), fx::emax(x[a][3], x[a][4]));
+        e = fx::emax(e, fx::emax(ea[a], fx::emax(x[a][0], x[a][5])));
+        low = min(low, (unsigned)ea[a]);  // (zeros, kZeroExp, are a large number)
       }
       double d1[3], d2[3], ko = 0.0;
-      if (e == fx::kZeroExp || fx::in_range(e)) {  // (of zeros alone, all differences are exactly zero)
-        const long long c = fx::align(z[3], e);
-        const long long c30 = 30 * c;
-        long long s1t = 0, s2t = 0, s3t = 0;
+      if (low >= (unsigned)fx::kExpMin && (e == fx::kZeroExp || fx::in_range(e))) {
+        long long kq = 0;  // the dissipation's weights add up to 192: its sum in quarters and their remainders
+        int kr = 0;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
           long long f[6];
+          int xa[4];
 #pragma unroll
           for (int m = 0; m < 6; ++m) {
             const int o = m < 3 ? m - 3 : m - 2;
-            f[m] = a == 0 ? fx::sar(M[pc + o], (unsigned)(e - ex[m]))
-                          : (a == 1 ? fx::sar(M[pc + o * pp], (unsigned)(e - ey[m]))
-                                    : fx::align(z[m < 3 ? m : m + 1], e));
+            f[m] = a == 2 ? z[3 + o].m : M[pc + o * (a == 0 ? 1 : pp)];
           }
-          const long long s1 = f[3] + f[2], s2 = f[4] + f[1], s3 = f[5] + f[0];
-          d1[a] = fx::to_double_cvt<kGuard>(8 * (f[3] - f[2]) - (f[4] - f[1]), e);
-          if (DD) d2[a] = fx::to_double<kGuard>(16 * s1 - s2 - c30, e);
-          s1t += s1;
-          s2t += s2;
-          s3t += s3;
+          const long long g[4] = {f[1], f[2], f[3], f[4]};
+#pragma unroll
+          for (int m = 0; m < 4; ++m) xa[m] = x[a][m + 1];
+          const Axis4 s(g, xa, ea[a]);
+          d1[a] = fx::to_double_cvt<kGuard>(s.diff, ea[a]);
+          if (DD) {
+            const int ec = fx::emax(ea[a], z[3].e);
+            d2[a] = fx::to_double<kGuard>(
+                fx::sar(16 * s.near - s.far, (unsigned)(ec - ea[a])) - 30 * fx::align(z[3], ec), ec);
+          }
+          const long long k = fx::sar(15 * s.near - 6 * s.far, (unsigned)(e - ea[a])) +
+                              fx::sar(f[0], (unsigned)(e - x[a][0])) + fx::sar(f[5], (unsigned)(e - x[a][5]));
+          kq += k >> 2;
+          kr += (int)k & 3;
         }
-        // the dissipation's weights add up to 192: a quarter of the sum fits,
-        // formed from the quarters and the remainders of its parts
-        const int r = (15 * ((int)s1t & 3) - 6 * ((int)s2t & 3) + ((int)s3t & 3)) >> 2;
-        ko = fx::to_double<kGuard - 2>(15 * (s1t >> 2) - 6 * (s2t >> 2) + (s3t >> 2) - 15 * c + r, e);
+        kq += (kr >> 2) - 15 * fx::align(z[3], e);
+        const bool wide = (unsigned long long)(kq + (1ll << 59)) >> 60 != 0;
+        ko = fx::to_double<kGuard>(wide ? kq : 4 * kq + (kr & 3), wide ? e + 2 : e);
       } else {
         // the ends of the FP64 range, Inf, NaN
         const int64_t st[3] = {1, d.sy, d.sz};

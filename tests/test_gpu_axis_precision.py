@@ -58,3 +58,48 @@ def test_variable_speed(api, orc, axis, small):
         got = synth.interior(to_np(sysm.rhs(to_gpu(st))), g)[1]
         d = np.abs(got - want)[at][zero_speed]
         assert np.abs(want[at][zero_speed]).max() > 0 and d.max() <= bound, (v, d.max(), bound)
+
+
+def _flat(shape):
+    return synth.BSSN_FLAT[:, None, None, None] * np.ones((1,) + shape)
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("small", [2.0 ** -12, 2.0 ** -40])
+def test_bssn_first(api, orc, axis, small):
+    """Flat space with beta^a = 1 alone, no damping and dissipation: (B^x)_t = D_a B^x."""
+    dims, g, h = (19, 13, 12), 3, 1.0 / 16
+    shape = dims[::-1]
+    u, at = _row(shape, axis, np.random.default_rng(axis), small)
+    st = _flat(shape)
+    st[18 + axis], st[21] = 1.0, u
+    st = synth.pad(st, g)
+    orc.fill_ghosts(st, g)
+    want = synth.interior(orc.bssn_rhs(st, g, h, orc.Params(0.0, 0.0, 0, 0)), g)[21]
+    got = synth.interior(to_np(api.make_system(api.BSSN, *dims, h, params=api.default_params(0.0, 0.0, 0, 0))
+                               .rhs(to_gpu(st))), g)[21]
+    bound = 2.0 ** -52 * 20 * np.abs(u[at]).max() / (12 * h)  # some roundings of the row's values
+    assert np.abs(got - want)[at].max() <= bound
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+@pytest.mark.parametrize("small", [2.0 ** -12, 2.0 ** -40])
+def test_bssn_second(api, orc, axis, small):
+    """A constant metric of 1 along the axis and 2^60 across it: (Xt^a)_t is
+    4/3 D_aa beta^a and 2^-60 of the other second derivatives."""
+    dims, g, h = (19, 13, 12), 3, 1.0 / 16
+    shape = dims[::-1]
+    u, at = _row(shape, axis, np.random.default_rng(10 + axis), small)
+    st = _flat(shape)
+    for q, v in enumerate((1, 4, 6)):
+        st[v] = 1.0 if q == axis else 2.0 ** 60
+    st[18 + axis] = u
+    st = synth.pad(st, g)
+    orc.fill_ghosts(st, g)
+    want = synth.interior(orc.bssn_rhs(st, g, h, orc.Params(0.0, 0.0, 0, 0)), g)[14 + axis]
+    got = synth.interior(to_np(api.make_system(api.BSSN, *dims, h, params=api.default_params(0.0, 0.0, 0, 0))
+                               .rhs(to_gpu(st))), g)[14 + axis]
+    # the difference (weights 64), its scaling, the trace, the divergence's term and their sum, rounded on both
+    # sides: eight roundings of at most 4/3 of the largest second difference
+    bound = 8 * 2.0 ** -53 * 4 / 3 * 64 * np.abs(u[at]).max() / (12 * h * h)
+    assert np.abs(want[at]).max() > 0 and np.abs(got - want)[at].max() <= bound
