@@ -193,6 +193,12 @@ struct Sum96 {
     else
       lo -= (long long)((unsigned long long)(unsigned)-W * (unsigned)v);
   }
+  // rounded down to units 2^d larger
+  CHEMORA_FX void shift(unsigned d) {
+    const long long h = hi + (lo >> 32);
+    lo = (unsigned)(d < 32 ? shr((unsigned long long)h << 32 | (unsigned)lo, d) : (unsigned long long)sar(h, d - 32));
+    hi = sar(h, d);
+  }
 };
 template <int K>
 CHEMORA_FX double to_double(const Sum96& v, int e) {

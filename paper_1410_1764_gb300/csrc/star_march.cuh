@@ -55,47 +55,69 @@ CHEMORA_FX bool star_ok(int e) {
   return e == fx::kZeroExp || (unsigned)(e - fx::kExpMin) <= (unsigned)(top - fx::kExpMin);
 }
 
+// Values at distance 3 and 4 have weights 2^-7 and 2^-10 of the nearest ones'.
+// Those of distance 1 and 2 and the centre are aligned to their own largest
+// exponent, so that larger values far away do not cut them (order 8 on 33 x 40 x
+// 35, pulses: with one exponent for all, 12 times FP64's error where the right-hand
+// side is small).
+template <int R>
+constexpr bool is_near(int offset) {
+  return R <= 2 || (offset >= -2 && offset <= 2);
+}
+
 // den2 h^2 times the Laplacian from the sums s[k] of the six values at
-// distance k + 1 and the centre c, aligned to exponent e.
+// distance k + 1 and the centre: those near and cn aligned to exponent en, the
+// others and cf to e >= en.
 template <int R, int K = Guard<R>::lap>
-CHEMORA_FX double star_lap(const long long (&s)[R], long long c, int e) {
+CHEMORA_FX double star_lap(const long long (&s)[R], long long cn, int en, long long cf, int e) {
   typedef Central<R> W;
   if constexpr (R == 1) {
-    return fx::to_double<K>(s[0] - 6 * c, e);
+    return fx::to_double<K>(s[0] - 6 * cn, en);
   } else if constexpr (R == 2) {
     // 16 s1 - s2 - 90 c = 16 h - r, 0 <= r < 16: 68 bits, of which the low four
     // matter only where h is small.  Every part is at most 2^(57 + K) = 2^63.
-    const long long b = s[1] + 10 * c, h = s[0] - 5 * c - (b >> 4);
+    const long long b = s[1] + 10 * cn, h = s[0] - 5 * cn - (b >> 4);
     const bool wide = (unsigned long long)(h + (1ll << 57)) >> 58 != 0;
-    return fx::to_double<K>(wide ? h : 16 * h - (b & 15), wide ? e + 4 : e);
+    return fx::to_double<K>(wide ? h : 16 * h - (b & 15), wide ? en + 4 : en);
   } else {
     fx::Sum96 v;
-    v.add<W::d2[0]>(s[0] - 6 * c);
-    v.add<W::d2[1]>(s[1] - 6 * c);
-    if constexpr (R >= 3) v.add<W::d2[2]>(s[R < 3 ? 0 : 2] - 6 * c);
-    if constexpr (R == 4) v.add<W::d2[3]>(s[R - 1] - 6 * c);
+    v.add<W::d2[0]>(s[0] - 6 * cn);
+    v.add<W::d2[1]>(s[1] - 6 * cn);
+    v.shift((unsigned)(e - en));
+    v.add<W::d2[2]>(s[R < 3 ? 0 : 2] - 6 * cf);
+    if constexpr (R == 4) v.add<W::d2[3]>(s[R - 1] - 6 * cf);
     return fx::to_double<K>(v, e);
   }
 }
+template <int R, int K = Guard<R>::lap>
+CHEMORA_FX double star_lap(const long long (&s)[R], long long c, int e) {
+  return star_lap<R, K>(s, c, e, c, e);
+}
 
 // den1 h times a sum of up to three first differences from the sums t[k] of their
-// differences f(k + 1) - f(-k - 1), aligned to exponent e.
+// differences f(k + 1) - f(-k - 1), the near ones aligned to exponent en, the
+// others to e >= en.
 template <int R>
-CHEMORA_FX double star_d1(const long long (&t)[R], int e) {
+CHEMORA_FX double star_d1(const long long (&t)[R], int en, int e) {
   typedef Central<R> W;
   constexpr int K = Guard<R>::d1;
   if constexpr (R == 1) {
-    return fx::to_double<K>(t[0], e);
+    return fx::to_double<K>(t[0], en);
   } else if constexpr (R == 2) {
-    return fx::to_double<K>(8 * t[0] - t[1], e);
+    return fx::to_double<K>(8 * t[0] - t[1], en);
   } else {
     fx::Sum96 v;
     v.add<W::d1[0]>(t[0]);
     v.add<W::d1[1]>(t[1]);
+    v.shift((unsigned)(e - en));
     v.add<W::d1[2]>(t[2]);
     if constexpr (R == 4) v.add<W::d1[3]>(t[R - 1]);
     return fx::to_double<K>(v, e);
   }
+}
+template <int R>
+CHEMORA_FX double star_d1(const long long (&t)[R], int e) {
+  return star_d1<R>(t, e, e);
 }
 
 // One axis of an order-4 star from its values' significands and exponents at

@@ -46,10 +46,11 @@ CHEMORA_BODY(Wave1O8, 5, chemora_wave1_o8_point)
 
 // Threads per SM asked of the compiler, the most that leaves next to no spills
 // (order 4: 245 us per stage of 256^3 with 768 threads, 270 with 1024 and 20
-// bytes spilled; first-order form of order 6 on 117 x 90 x 131: 93 us with
-// 512, 141 with 640 and 160 bytes spilled).
+// bytes spilled; order 8: 10 steps on 128^3 2.01 ms with 640, 2.28 with 768 and
+// 48 bytes spilled; first-order form of order 6 on 117 x 90 x 131: 93 us per
+// stage with 512, 141 with 640 and 160 bytes spilled).
 template <int NV, int R>
-constexpr int march_threads() { return NV == 2 ? (R == 1 ? 1024 : 768) : (R == 1 ? 768 : 512); }
+constexpr int march_threads() { return NV == 2 ? (R == 1 ? 1024 : (R == 4 ? 640 : 768)) : (R == 1 ? 768 : 512); }
 
 // Two-variable form, order 2R: one Laplacian of u per point.
 template <class BODY, int R, int TX, int TY>
@@ -102,13 +103,15 @@ wave_march_order_kernel(Dims d, Scalars sc, StageParams a, int zb, double scale)
       }
     __syncthreads();
     if (p.active) {
-      int ex[2 * R], ey[2 * R], e = z[R].e;
+      int ex[2 * R], ey[2 * R], en = z[R].e, ef = fx::kZeroExp;
 #pragma unroll
       for (int m = 0; m < 2 * R; ++m) {
         ex[m] = E[pc + tap<R>(m)];
         ey[m] = E[pc + tap<R>(m) * P];
-        e = fx::emax(e, fx::emax(fx::emax(ex[m], ey[m]), z[R + tap<R>(m)].e));
+        int& t = is_near<R>(tap<R>(m)) ? en : ef;
+        t = fx::emax(t, fx::emax(fx::emax(ex[m], ey[m]), z[R + tap<R>(m)].e));
       }
+      const int e = fx::emax(en, ef);
       if (star_ok<R>(e)) {
         double lap = 0.0;
         if (e != fx::kZeroExp) {
@@ -117,11 +120,11 @@ wave_march_order_kernel(Dims d, Scalars sc, StageParams a, int zb, double scale)
           for (int q = 0; q < R; ++q) s[q] = 0;
 #pragma unroll
           for (int m = 0; m < 2 * R; ++m) {
-            const int o = tap<R>(m), q = o < 0 ? -o - 1 : o - 1;
-            s[q] += fx::sar(M[pc + o], (unsigned)(e - ex[m])) + fx::sar(M[pc + o * P], (unsigned)(e - ey[m])) +
-                    fx::align(z[R + o], e);
+            const int o = tap<R>(m), q = o < 0 ? -o - 1 : o - 1, to = is_near<R>(o) ? en : e;
+            s[q] += fx::sar(M[pc + o], (unsigned)(to - ex[m])) + fx::sar(M[pc + o * P], (unsigned)(to - ey[m])) +
+                    fx::align(z[R + o], to);
           }
-          lap = star_lap<R>(s, fx::align(z[R], e), e);
+          lap = star_lap<R>(s, fx::align(z[R], en), en, fx::align(z[R], e), e);
         }
         const double kk[2] = {rho, __fma_rn(lap, scale, sc.k[CHEMORA_K_MZERO])};
         up.apply(a, c, d.sv, kk, sc.k[CHEMORA_K_ONE], sc.k[CHEMORA_K_TWO], [&](int64_t o, double x) { a.dst[o] = x; });
@@ -224,10 +227,11 @@ wave1_march_kernel(Dims d, Scalars sc, StageParams a, int zb, double scale) {
         const int st[2] = {1, P};
 #pragma unroll
         for (int x = 0; x < 3; ++x) {
-          int te[2 * R], e = fx::kZeroExp;
+          int te[2 * R], en = fx::kZeroExp, e = fx::kZeroExp;
 #pragma unroll
           for (int m = 0; m < 2 * R; ++m) {
             te[m] = x < 2 ? E[pr + tap<R>(m) * st[x & 1]] : z[R + tap<R>(m)].e;
+            if (is_near<R>(tap<R>(m))) en = fx::emax(en, te[m]);
             e = fx::emax(e, te[m]);
           }
           ok = ok && star_ok<R>(e);
@@ -237,30 +241,33 @@ wave1_march_kernel(Dims d, Scalars sc, StageParams a, int zb, double scale) {
             const int up1 = R + q, dn = R - 1 - q;
             const long long f1 = x < 2 ? M[pr + (q + 1) * st[x & 1]] : z[R + q + 1].m;
             const long long f0 = x < 2 ? M[pr - (q + 1) * st[x & 1]] : z[R - q - 1].m;
-            t[q] = fx::sar(f1, (unsigned)(e - te[up1])) - fx::sar(f0, (unsigned)(e - te[dn]));
+            const int to = is_near<R>(q + 1) ? en : e;
+            t[q] = fx::sar(f1, (unsigned)(to - te[up1])) - fx::sar(f0, (unsigned)(to - te[dn]));
           }
-          kk[2 + x] = e == fx::kZeroExp ? 0.0 : star_d1<R>(t, e);
+          kk[2 + x] = e == fx::kZeroExp ? 0.0 : star_d1<R>(t, en, e);
         }
       }
       {  // the divergence of v, one sum
-        int ex[2 * R], ey[2 * R], e = fx::kZeroExp;
+        int ex[2 * R], ey[2 * R], en = fx::kZeroExp, ef = fx::kZeroExp;
 #pragma unroll
         for (int m = 0; m < 2 * R; ++m) {
           ex[m] = E[px + tap<R>(m)];
           ey[m] = E[py + tap<R>(m) * TX];
-          e = fx::emax(e, fx::emax(fx::emax(ex[m], ey[m]), vz[R + tap<R>(m)].e));
+          int& t = is_near<R>(tap<R>(m)) ? en : ef;
+          t = fx::emax(t, fx::emax(fx::emax(ex[m], ey[m]), vz[R + tap<R>(m)].e));
         }
+        const int e = fx::emax(en, ef);
         ok = ok && star_ok<R>(e);
         long long t[R];
 #pragma unroll
         for (int q = 0; q < R; ++q) {
-          const int u1 = R + q, dn = R - 1 - q;
-          t[q] = (fx::sar(M[px + q + 1], (unsigned)(e - ex[u1])) - fx::sar(M[px - q - 1], (unsigned)(e - ex[dn]))) +
-                 (fx::sar(M[py + (q + 1) * TX], (unsigned)(e - ey[u1])) -
-                  fx::sar(M[py - (q + 1) * TX], (unsigned)(e - ey[dn]))) +
-                 (fx::align(vz[R + q + 1], e) - fx::align(vz[R - q - 1], e));
+          const int u1 = R + q, dn = R - 1 - q, to = is_near<R>(q + 1) ? en : e;
+          t[q] = (fx::sar(M[px + q + 1], (unsigned)(to - ex[u1])) - fx::sar(M[px - q - 1], (unsigned)(to - ex[dn]))) +
+                 (fx::sar(M[py + (q + 1) * TX], (unsigned)(to - ey[u1])) -
+                  fx::sar(M[py - (q + 1) * TX], (unsigned)(to - ey[dn]))) +
+                 (fx::align(vz[R + q + 1], to) - fx::align(vz[R - q - 1], to));
         }
-        kk[1] = e == fx::kZeroExp ? 0.0 : star_d1<R>(t, e);
+        kk[1] = e == fx::kZeroExp ? 0.0 : star_d1<R>(t, en, e);
       }
       if (ok) {
         kk[0] = rho;

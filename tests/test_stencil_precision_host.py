@@ -1,6 +1,6 @@
 """Accuracy of the integer stencils (csrc/star_march.cuh) against FP64: compiled
 for the host with g++, each stencil's root mean square error against exact
-rational sums, in ulps of the largest value it reads, is no larger than that of
+rational sums, in ulps of its largest term (value times weight), is no larger than that of
 the generated FP64 body of the same system (gen_wave*.cuh) on pulses narrow and
 wide against the spacing, long waves, a small perturbation of one, and noise."""
 import ctypes
@@ -74,23 +74,35 @@ template <int R> static void star(const double* f, double c, double* out) {
   {
     constexpr int K = Guard<R>::lap;
     const fx::Parts pc = fx::parts_or_zero<K>(c);
-    int e = pc.e;
-    for (int q = 0; q < 6 * R; ++q) e = fx::emax(e, fx::parts_or_zero<K>(f[q]).e);
+    int en = pc.e, e = pc.e;
+    for (int q = 0; q < 6 * R; ++q) {
+      const int x = fx::parts_or_zero<K>(f[q]).e;
+      if (is_near<R>(1 + q % (2 * R) / 2)) en = fx::emax(en, x);
+      e = fx::emax(e, x);
+    }
     long long s[R] = {};
-    for (int q = 0; q < 6 * R; ++q) s[q % (2 * R) / 2] += fx::align(fx::parts_or_zero<K>(f[q]), e);
-    out[1] = star_lap<R>(s, fx::align(pc, e), e) * (R == 2 ? 1.0 : 1.0 / Central<R>::den2);
+    for (int q = 0; q < 6 * R; ++q) {
+      const int k = q % (2 * R) / 2;
+      s[k] += fx::align(fx::parts_or_zero<K>(f[q]), is_near<R>(k + 1) ? en : e);
+    }
+    out[1] = star_lap<R>(s, fx::align(pc, en), en, fx::align(pc, e), e) * (R == 2 ? 1.0 : 1.0 / Central<R>::den2);
   }
   constexpr int K = Guard<R>::d1;
   for (int a = -1; a < 3; ++a) {
     const int q0 = a < 0 ? 0 : 2 * R * a, q1 = a < 0 ? 6 * R : q0 + 2 * R;
-    int e = fx::kZeroExp;
-    for (int q = q0; q < q1; ++q) e = fx::emax(e, fx::parts_or_zero<K>(f[q]).e);
+    int en = fx::kZeroExp, e = fx::kZeroExp;
+    for (int q = q0; q < q1; ++q) {
+      const int x = fx::parts_or_zero<K>(f[q]).e;
+      if (is_near<R>(1 + q % (2 * R) / 2)) en = fx::emax(en, x);
+      e = fx::emax(e, x);
+    }
     long long t[R] = {};
     for (int q = q0; q < q1; ++q) {
-      const long long m = fx::align(fx::parts_or_zero<K>(f[q]), e);
-      t[q % (2 * R) / 2] += q & 1 ? -m : m;
+      const int k = q % (2 * R) / 2;
+      const long long m = fx::align(fx::parts_or_zero<K>(f[q]), is_near<R>(k + 1) ? en : e);
+      t[k] += q & 1 ? -m : m;
     }
-    out[5 + 2 * a] = star_d1<R>(t, e) * (1.0 / Central<R>::den1);
+    out[5 + 2 * a] = star_d1<R>(t, en, e) * (1.0 / Central<R>::den1);
   }
 }
 // order-4 first differences with an axis of its own exponent (the variable-speed wave's): FP64 and integers, over 12 h
@@ -160,7 +172,7 @@ def ulp(v):
     return 2.0 ** (math.frexp(v)[1] - 53)
 
 
-FIELDS = ["pulse/32", "pulse/128", "wave", "flat", "noise"]
+FIELDS = ["pulse/16", "pulse/32", "pulse/128", "wave", "flat", "noise"]
 
 
 @pytest.mark.parametrize("R", [1, 2, 3, 4])
@@ -169,22 +181,55 @@ def test_no_further_from_exact_than_fp64(L, R, field):
     w2, w1 = _weights(R, False), _weights(R, True)
     if R == 2:
         w2 = [12 * w for w in w2]  # the order-4 Laplacian is formed over 12 h^2
-    err = np.zeros((400, 5, 2))
+    err = np.zeros((400, 5, 3))  # FP64, integers, half an ulp of the result
     for i, (f, c) in enumerate(stars(field, R, len(err), np.random.default_rng(R))):
         out = (ctypes.c_double * 10)()
         L.run(R, (ctypes.c_double * len(f))(*f), ctypes.c_double(c), out)
         F = np.array([Fraction(q) for q in f], dtype=object).reshape(3, R, 2)
         d1 = [sum(w * (F[a, k, 0] - F[a, k, 1]) for k, w in enumerate(w1)) for a in range(3)]
         lap = sum(w * (F[a, k, 0] + F[a, k, 1] - 2 * Fraction(c)) for a in range(3) for k, w in enumerate(w2))
-        tops = [max(max(map(abs, f)), abs(c)), max(map(abs, f))] + [max(map(abs, f[2 * R * a:2 * R * a + 2 * R]))
-                                                                   for a in range(3)]
+        v = np.abs(np.array(f)).reshape(3, R, 2).max(2)  # per axis and distance
+        t1 = (v * np.abs(np.array(w1, float))).max(1)
+        tops = [max((v * np.abs(np.array(w2, float))).max(), abs(6 * c * float(sum(w2)))), t1.max()] + list(t1)
         for q, (exact, top) in enumerate(zip([lap, sum(d1)] + d1, tops)):
+            err[i, q, 2] = ulp(float(exact)) / ulp(top) / 2
             for m in range(2):
-                err[i, q, m] = float(Fraction(out[2 * q + m]) - exact) / ulp(top)
+                err[i, q, m] = float((Fraction(out[2 * q + m]) - exact) / Fraction(ulp(top)))
     sq = (err ** 2).mean(0)
     rms = np.sqrt(np.stack([sq[0], sq[1], sq[2:].mean(0)]))  # the Laplacian, the divergence, the first differences
-    # 1e-3: the scale of orders 6 and 8 is rounded
-    assert (rms[:, 1] <= rms[:, 0] * 1.001 + 1e-3).all(), rms
+    # 2 %: sampling (order 2's first differences are the same in both); orders 6 and 8 scale by a rounded constant
+    assert (rms[:, 1] ** 2 <= (rms[:, 0] * 1.02) ** 2 + (rms[:, 2] ** 2 if R >= 3 else 0)).all(), rms
+
+
+@pytest.mark.parametrize("R", [3, 4])
+@pytest.mark.parametrize("shift", [0, 5, 20, 31, 32, 40, 63, 64, 95, 96, 130, 600, -5, -40])
+def test_far_values(L, R, shift):
+    """Values at distance 3 and 4 a power of two larger (or smaller) than the
+    near ones, and near ones that are all zero: within half an ulp of the result,
+    a unit of the far values' 2^-58 for the near sum, and the cut of each group's
+    values below its own largest exponent."""
+    w2, w1 = _weights(R, False), _weights(R, True)
+    rng = np.random.default_rng(shift + 1000)
+    for trial in range(60):
+        v = rng.uniform(-1, 1, (3, R, 2))
+        v[:, 2:] *= 2.0 ** shift
+        c = float(rng.uniform(-1, 1))
+        if trial % 6 == 0:
+            v[:, :2], c = 0.0, 0.0
+        f = [float(q) for q in v.ravel()]
+        out = (ctypes.c_double * 10)()
+        L.run(R, (ctypes.c_double * len(f))(*f), ctypes.c_double(c), out)
+        F = np.array([Fraction(q) for q in f], dtype=object).reshape(3, R, 2)
+        for name, got, exact, w, centre in (
+                ("lap", out[1], sum(w * (F[a, k, 0] + F[a, k, 1] - 2 * Fraction(c)) for a in range(3)
+                                    for k, w in enumerate(w2)), w2, c),
+                ("div", out[3], sum(w * (F[a, k, 0] - F[a, k, 1]) for a in range(3) for k, w in enumerate(w1)), w1, 0.0)):
+            near = max(float(np.abs(v[:, :2]).max()), abs(centre))
+            top = max(near, float(np.abs(v[:, 2:]).max()))
+            cut = sum(6 * 2 * abs(q) * Fraction(ulp(near)) for q in w[:2]) if near else 0
+            cut += sum(6 * 2 * abs(q) * Fraction(ulp(top)) for q in w[2:]) + Fraction(ulp(top)) / 100
+            # three roundings: the sum, one over the weights' denominator, and their product
+            assert abs(Fraction(got) - exact) <= cut / 32 + abs(exact) * 3 / 2 ** 53 * (1 + Fraction(1, 2 ** 20)), (name, trial)
 
 
 @pytest.mark.parametrize("field", FIELDS)
