@@ -150,14 +150,17 @@ CHEMORA_FX long long align(const Parts& p, int e) { return sar(p.m, (unsigned)(e
 template <int K>
 CHEMORA_FX long long align(double v, int e) { return align(parts<K>(v), e); }
 
-// v units of 2^(E - 1075 - K) as a double (nearest, ties away from zero).
-template <int K>
+// v units of 2^(E - 1075 - K) as a double: nearest, ties away from zero, or to
+// even as FP64 rounds (a difference of two doubles is often a tie, and the even
+// one has a last bit less for the product with 1/h to round).
+template <int K, bool EVEN = false>
 CHEMORA_FX double to_double(long long v, int e) {
   const unsigned long long s = (unsigned long long)(v >> 63);
   const unsigned long long a = ((unsigned long long)v ^ s) - s;
   const int lz = clz64(a);
   const unsigned long long m = shl(a, (unsigned)lz);
-  unsigned long long r = (m >> 11) + ((m >> 10) & 1);
+  unsigned long long r = m >> 11;
+  r += EVEN ? ((unsigned)m & 0x7ffu) + ((unsigned)r & 1u) > 0x400u : (m >> 10) & 1;
   r += (unsigned long long)(unsigned)(e + 10 - K - lz) << 52;
   r |= s & 0x8000000000000000ull;
   return a == 0 ? 0.0 : from_bits(r);

@@ -102,7 +102,7 @@ CHEMORA_FX double star_d1(const long long (&t)[R], int en, int e) {
   typedef Central<R> W;
   constexpr int K = Guard<R>::d1;
   if constexpr (R == 1) {
-    return fx::to_double<K>(t[0], en);
+    return fx::to_double<K, true>(t[0], en);
   } else if constexpr (R == 2) {
     return fx::to_double<K>(8 * t[0] - t[1], en);
   } else {

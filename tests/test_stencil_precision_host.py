@@ -245,3 +245,19 @@ def test_axis_differences(L, field):
             err.append([float(Fraction(out[2 * a + m]) - exact) / top for m in range(2)])
     rms = np.sqrt((np.array(err) ** 2).mean(0))
     assert rms[1] <= rms[0], rms
+
+
+def test_order2_differences_round_as_fp64(L):
+    """A difference of two doubles within six binades, correctly rounded with
+    ties to even: the same bits as FP64 (differences are often ties)."""
+    rng = np.random.default_rng(9)
+    ties = 0
+    for _ in range(500):
+        f = rng.uniform(0.25, 1.0, 6) * rng.choice([-1.0, 1.0, 8.0], 6)
+        out = (ctypes.c_double * 10)()
+        L.run(1, (ctypes.c_double * 6)(*f), ctypes.c_double(0.5), out)
+        assert out[4:10:2] == out[5:10:2]
+        for a in range(3):
+            d = Fraction(f[2 * a]) - Fraction(f[2 * a + 1])
+            ties += 2 * abs(d - Fraction(float(d))) == Fraction(ulp(float(d)))
+    assert ties > 100
