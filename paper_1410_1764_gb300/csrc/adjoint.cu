@@ -68,8 +68,8 @@ __global__ void __launch_bounds__(ATX * ATY) varc_grad_s_kernel(Dims d, double i
 // GB300, 128^3: 116 us, against 320 us when each point formed the 37 products
 // of its stencils itself in FP64 (72 instructions of 17.8 cycles).  Products in
 // FP64 here: 123 us.  640 threads per SM (20 bytes spilled): 7 % more.  Bound by
-// the latency of its integer chains at 16 warps per SM; ten FP64 instructions
-// per point are left (36 us), HBM alone takes 47 us.
+// the latency of its integer chains at 16 warps per SM; eleven FP64 instructions
+// per point are left (40 us), HBM alone takes 47 us.
 // kb: 2 grid functions with valid ghosts; coef: s and G_d (ghosts valid); tape:
 // Lap u_q (interior) and 12 h D_d u_q (ghosts valid).  first: yacc = yp + yhat
 // (else yacc += yhat).  kbn (if non-NULL): kbn = cq yp + aq yhat, or, after the

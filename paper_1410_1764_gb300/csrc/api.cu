@@ -17,6 +17,7 @@ namespace chemora {
 
 static thread_local char g_err[512] = "";
 static std::atomic<int64_t> g_launches{0};
+static thread_local int64_t g_thread_launches = 0;
 
 int set_error(int code, const char* fmt, ...) {
   va_list ap;
@@ -32,9 +33,18 @@ int cuda_error(cudaError_t e, const char* what) {
 
 int launched(const char* name, int n) {
   g_launches.fetch_add(n, std::memory_order_relaxed);
+  g_thread_launches += n;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_error(e, name);
   return CHEMORA_OK;
+}
+
+CaptureTally::CaptureTally() : start_(g_thread_launches) {}
+
+int CaptureTally::take() const {
+  const int64_t n = g_thread_launches - start_;
+  g_launches.fetch_sub(n, std::memory_order_relaxed);
+  return (int)n;
 }
 
 Scalars make_scalars(double dx, const chemora_params& p) {
@@ -275,7 +285,9 @@ static int step_graph(chemora_system* sys, double* state, double dt, const Field
   free_step_graph(sys);
   if (!sys->cap_stream) CHEMORA_CUDA(cudaStreamCreateWithFlags(&sys->cap_stream, cudaStreamNonBlocking));
   CHEMORA_CUDA(cudaStreamBeginCapture(sys->cap_stream, cudaStreamCaptureModeThreadLocal));
+  const CaptureTally tally;
   int rc = rk4_one(sys, state, dt, work, sys->cap_stream);
+  sys->graph_launches = tally.take();
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(sys->cap_stream, &g);
   if (rc) {
@@ -401,7 +413,7 @@ int chemora_rk4_step(chemora_system* sys, double* state, double dt, int nsteps, 
   if ((rc = step_graph(sys, state, dt, work))) return rc;
   for (int n = 0; n < nsteps; ++n) {
     CHEMORA_CUDA(cudaGraphLaunch(sys->graph_exec, s));
-    if ((rc = launched("cudaGraphLaunch(RK4 step)", images ? 4 : 8))) return rc;
+    if ((rc = launched("cudaGraphLaunch(RK4 step)", sys->graph_launches))) return rc;
   }
   return images ? CHEMORA_OK : fill_ghosts(sys->grid->d, sys->nvars, state, s);
 }

@@ -24,6 +24,16 @@ int cuda_error(cudaError_t e, const char* what);
   } while (0)
 // after a kernel launch: count it and check the launch status
 int launched(const char* name, int n = 1);
+// Launches of this thread since the tally began, taken out of the count: they
+// were captured, and count when their graph is launched.
+class CaptureTally {
+ public:
+  CaptureTally();
+  int take() const;
+
+ private:
+  int64_t start_;
+};
 
 // ---------------------------------------------------------------------------
 // handles
@@ -78,6 +88,7 @@ struct chemora_system {
   double* graph_state;
   double graph_dt;
   int graph_variant;
+  int graph_launches;  // kernels of the step
   // run-time specialised stage kernels (NULL until chemora_system_specialize)
   chemora::JitModule* jit;
   int jit_on;

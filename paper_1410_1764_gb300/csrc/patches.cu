@@ -268,7 +268,9 @@ static int capture_step(chemora_batch* b, double dt) {
   if (!b->cap_stream) CHEMORA_CUDA(cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking));
   cudaStream_t s = b->cap_stream;
   CHEMORA_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+  const CaptureTally tally;
   int rc = batch_rk4_one(b, dt, s);
+  b->graph_kernels = tally.take();
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(s, &g);
   if (rc) {
@@ -279,7 +281,6 @@ static int capture_step(chemora_batch* b, double dt) {
   b->graph = g;
   CHEMORA_CUDA(cudaGraphInstantiate(&b->exec, g, 0));
   b->graph_dt = dt;
-  b->graph_kernels = b->kind == CHEMORA_BSSN ? 4 + 8 * (int)b->plan.chunks.size() : 8;
   return CHEMORA_OK;
 }
 

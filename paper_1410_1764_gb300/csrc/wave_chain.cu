@@ -109,6 +109,7 @@ struct ChainGraph {
   double* state = nullptr;
   double dt = 0.0;
   int steps = 0;
+  int launches = 0;
 };
 
 // Per-system state: graphs of K steps and of the remainder.
@@ -159,7 +160,9 @@ static int chain_graph(chemora_system* sys, ChainGraph& g, double* Y, double dt,
   g.exec = nullptr;
   if (!sys->cap_stream) CHEMORA_CUDA(cudaStreamCreateWithFlags(&sys->cap_stream, cudaStreamNonBlocking));
   CHEMORA_CUDA(cudaStreamBeginCapture(sys->cap_stream, cudaStreamCaptureModeThreadLocal));
+  const CaptureTally tally;
   int rc = chain_steps(sys, Y, dt, steps, sys->cap_stream);
+  g.launches = tally.take();
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamEndCapture(sys->cap_stream, &graph);
   if (rc) {
@@ -197,13 +200,13 @@ int chain_rk4(chemora_system* sys, double* state, double dt, int nsteps, cudaStr
     if ((rc = chain_graph(sys, cs->graph[0], state, dt, kChainGraphSteps))) return rc;
     for (int q = 0; q < full; ++q) {
       CHEMORA_CUDA(cudaGraphLaunch(cs->graph[0].exec, s));
-      if ((rc = launched("cudaGraphLaunch(chained RK4 steps)", 4 * kChainGraphSteps))) return rc;
+      if ((rc = launched("cudaGraphLaunch(chained RK4 steps)", cs->graph[0].launches))) return rc;
     }
   }
   if (rest) {
     if ((rc = chain_graph(sys, cs->graph[1], state, dt, rest))) return rc;
     CHEMORA_CUDA(cudaGraphLaunch(cs->graph[1].exec, s));
-    if ((rc = launched("cudaGraphLaunch(chained RK4 steps)", 4 * rest))) return rc;
+    if ((rc = launched("cudaGraphLaunch(chained RK4 steps)", cs->graph[1].launches))) return rc;
   }
   return fill_ghosts(sys->grid->d, sys->nvars, state, s);
 }
