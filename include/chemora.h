@@ -354,7 +354,8 @@ int chemora_variant_count(int kind);
  * and z-derivative rows shared through shared memory (any ny), 4 (scalar
  * wave, order 4) each thread marching along z with its column's values in
  * registers and the plane in hand in shared memory.  A shape whose condition
- * fails on a grid runs as shape 0.  Outputs may be NULL;
+ * fails on a grid runs as shape 0.  Shape 0 of BSSN runs blocks of 64 threads on
+ * grids below 155,648 points.  Outputs may be NULL;
  * CHEMORA_EINVAL for an unknown kind or index. */
 int chemora_variant_info(int kind, int variant, int* tx, int* ty, int* min_blocks, int* sharing);
 

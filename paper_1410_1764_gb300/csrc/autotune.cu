@@ -53,6 +53,19 @@ static double model_cost(int kind, const Dims& d, const LaunchVariant& v, int sm
   return work * threads * (waves < 8.0 ? quant : 1.0 + 0.5 / waves);
 }
 
+// Does shape v run what another one runs on d: one it falls back to, or an
+// earlier one of the same block?
+static bool same_kernel(int kind, const Dims& d, int v) {
+  if (kind != CHEMORA_BSSN) return false;
+  if (bssn_shape(d, v) != v) return true;
+  const LaunchVariant& a = *variant_info(kind, v);
+  for (int q = 0; q < v && !a.xshare; ++q) {
+    const LaunchVariant& b = *variant_info(kind, q);
+    if (bssn_shape(d, q) == q && !b.xshare && a.tx * a.ty == b.tx * b.ty && a.minb == b.minb) return true;
+  }
+  return false;
+}
+
 int autotune_stage(int kind, const Dims& d, const Scalars& sc, const StageParams& p, cudaStream_t s, int* best,
                    float* best_ms, const FieldWork& work) {
   int dev = 0, sms = 152;
@@ -62,7 +75,7 @@ int autotune_stage(int kind, const Dims& d, const Scalars& sc, const StageParams
   std::vector<double> cost(nv);
   double cmin = 1e300;
   for (int v = 0; v < nv; ++v) {
-    cost[v] = model_cost(kind, d, *variant_info(kind, v), sms);
+    cost[v] = same_kernel(kind, d, v) ? 1e300 : model_cost(kind, d, *variant_info(kind, v), sms);
     cmin = std::min(cmin, cost[v]);
   }
   cudaEvent_t e0, e1;
@@ -114,7 +127,6 @@ int chemora_variant_info(int kind, int variant, int* tx, int* ty, int* min_block
 
 int chemora_system_opcount(chemora_system* sys, int64_t* fp64_instructions, int64_t* flops) {
   if (!is_handle(sys, H_SYSTEM)) return set_error(CHEMORA_EINVAL, "not a system handle");
-  const LaunchVariant* v = variant_info(sys->kind, sys->variant);
   if (sys->kind == CHEMORA_WAVE || sys->kind == CHEMORA_WAVE1) {
     // the stencils run on the integer units: one FP64 multiply per evolved
     // derivative is left
@@ -124,19 +136,20 @@ int chemora_system_opcount(chemora_system* sys, int64_t* fp64_instructions, int6
     if (flops) *flops = f;
     return rc;
   }
-  const bool xs = v && v->xshare && sys->grid->d.nx % v->tx == 0 && sys->grid->d.g >= 3;
-  if (sys->kind == CHEMORA_BSSN && xs && v->xshare == 2) {
+  const LaunchVariant* v =
+      sys->kind == CHEMORA_BSSN ? variant_info(sys->kind, bssn_shape(sys->grid->d, sys->variant)) : nullptr;
+  if (v && v->xshare == 2) {
     // body plus the prologue's shared differences and z rows
     if (fp64_instructions) *fp64_instructions = CHEMORA_OPS_BSSN_XY_INSTR + xy_prologue_instr(v->ty);
     if (flops) *flops = CHEMORA_OPS_BSSN_XY_FLOPS + xy_prologue_flops(v->ty);
     return CHEMORA_OK;
   }
-  if (sys->kind == CHEMORA_BSSN && xs) {
+  if (v && v->xshare) {
     if (fp64_instructions) *fp64_instructions = CHEMORA_OPS_BSSN_X_INSTR;
     if (flops) *flops = CHEMORA_OPS_BSSN_X_FLOPS;
     return CHEMORA_OK;
   }
-  if (sys->kind == CHEMORA_BSSN) {
+  if (v) {
     // the split kernels: the algebra's body and prologue, and three fmas per
     // mixed derivative (the other differences run on the integer units)
     if (fp64_instructions) *fp64_instructions = CHEMORA_OPS_BSSN_ALG_INSTR + 44 + 3 * 33;

@@ -66,7 +66,8 @@ static int launch_bssn_xyvariant(const Dims& d, const Scalars& sc, const StagePa
   return launched("bssn_xystage_kernel");
 }
 
-// Launch shapes the autotuner chooses from (variant 0 is the default).
+// Launch shapes the autotuner chooses from (variant 0 is the default; bssn_shape
+// says which one runs on a grid).
 // Sharing 0: the split kernels, tx x ty the algebra kernel's block.
 const LaunchVariant kBssnVariants[] = {
     {32, 4, 4, launch_bssn_direct},
@@ -94,20 +95,26 @@ const LaunchVariant kBssnVariants[] = {
 };
 const int kNumBssnVariants = sizeof(kBssnVariants) / sizeof(kBssnVariants[0]);
 
-static bool shape_shares(const Dims& d, const LaunchVariant& v) { return v.xshare && d.nx % v.tx == 0 && d.g >= 3; }
-
-bool bssn_shape_splits(const Dims& d, int variant) {
+// The shape that runs for `variant` on d: the sharing shapes need whole warps of x
+// points and three ghost layers, else the default runs, which is half a block
+// (variant 4) below two waves of 128-thread blocks (four per SM), where it evens
+// out the SMs' shares (37 x 29 x 23, field and algebra kernels: 122 us with 128
+// threads, 106 with 64; 128^3: 4.73 and 4.83 ms).
+int bssn_shape(const Dims& d, int variant) {
   if (variant < 0 || variant >= kNumBssnVariants) variant = 0;
-  return !shape_shares(d, kBssnVariants[variant]);
+  const LaunchVariant& v = kBssnVariants[variant];
+  if (v.xshare && (d.nx % v.tx != 0 || d.g < 3)) variant = 0;
+  if (variant == 0 && (int64_t)d.nx * d.ny * d.nz < 2 * 152 * 4 * 128) variant = 4;
+  return variant;
 }
+
+bool bssn_shape_splits(const Dims& d, int variant) { return !kBssnVariants[bssn_shape(d, variant)].xshare; }
 
 int launch_bssn_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s, int variant,
                       const FieldWork& work) {
-  if (variant < 0 || variant >= kNumBssnVariants) variant = 0;
-  const LaunchVariant* v = &kBssnVariants[variant];
-  if (shape_shares(d, *v)) return v->launch(d, sc, a, s);
-  if (v->xshare) v = &kBssnVariants[0];
-  return work.w ? launch_bssn_split(d, sc, a, work, v->tx * v->ty, v->minb, s) : v->launch(d, sc, a, s);
+  const LaunchVariant& v = kBssnVariants[bssn_shape(d, variant)];
+  if (v.xshare || !work.w) return v.launch(d, sc, a, s);
+  return launch_bssn_split(d, sc, a, work, v.tx * v.ty, v.minb, s);
 }
 
 }  // namespace chemora

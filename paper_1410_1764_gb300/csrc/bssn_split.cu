@@ -320,10 +320,6 @@ static int launch_algebra(const FieldRegion& R, const Scalars& sc, const StagePa
 
 int launch_bssn_split(const Dims& d, const Scalars& sc, const StageParams& a, const FieldWork& work, int block,
                       int minb, cudaStream_t s) {
-  // Fewer than two waves of 128-thread blocks (four per SM): half the block
-  // evens out the SMs' shares (37 x 29 x 23, field and algebra kernels: 122 us
-  // with 128 threads, 106 with 64; 128^3: 4.73 and 4.83 ms).
-  if ((int64_t)d.nx * d.ny * d.nz < 2 * 152 * 4 * 128) block = 64, minb = 8;
   return for_field_chunks(d, sc, a.src, 24, work, s, [&](const FieldRegion& R) {
     if (block == 64) return minb >= 8 ? launch_algebra<64, 8>(R, sc, a, work.w, s) : launch_algebra<64, 5>(R, sc, a, work.w, s);
     if (minb == 2) return launch_algebra<128, 2>(R, sc, a, work.w, s);

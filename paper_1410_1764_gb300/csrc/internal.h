@@ -131,7 +131,9 @@ int launch_bssn_split(const Dims& d, const Scalars& sc, const StageParams& a, co
                       int minb, cudaStream_t s);
 int launch_constraints_split(const Dims& d, const Scalars& sc, const double* state, double* out,
                              const FieldWork& work, cudaStream_t s);
-// Does launch shape `variant` run the split kernels on d when it has a workspace?
+// The launch shape that runs for `variant` on d, and whether it runs the split
+// kernels when it has a workspace.
+int bssn_shape(const Dims& d, int variant);
 bool bssn_shape_splits(const Dims& d, int variant);
 // The RK4 driver's workspace (no workspace if there is no memory for one or
 // alloc is false and there is none yet), and one taken from and given back to

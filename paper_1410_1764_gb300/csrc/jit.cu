@@ -116,8 +116,8 @@ std::string hexf(double v) {
   return b;
 }
 
-// The launch shape's body and geometry, after the same fall-backs the
-// ahead-of-time dispatch applies.
+// The body and geometry of the shape that runs on d, the ahead-of-time
+// dispatch's choice.
 struct Shape {
   const char* body;  // device function in bssn_kernels.cuh (xshare 1, 2)
   int tx, ty, minb;
@@ -125,9 +125,7 @@ struct Shape {
 };
 
 Shape shape_of(const Dims& d, int variant) {
-  const LaunchVariant* v = variant_info(CHEMORA_BSSN, variant);
-  if (!v || (v->xshare && (d.nx % v->tx != 0 || d.g < 3)))
-    v = variant_info(CHEMORA_BSSN, 0);
+  const LaunchVariant* v = variant_info(CHEMORA_BSSN, bssn_shape(d, variant));
   static const char* const bodies[] = {"bssn_algebra", "bssn_x_body", "bssn_xy_body"};
   return Shape{bodies[v->xshare], v->tx, v->ty, v->minb, v->xshare};
 }

@@ -1,0 +1,75 @@
+"""The algebra kernel's blocks: every shape of its own in every Runge-Kutta mode
+on both sides of the rule for the default's block, with a partial last block; run-time
+specialisation compiles the block that runs without it."""
+import numpy as np
+import pytest
+
+from paper_1410_1764_gb300 import synth
+from helpers import scaled_err, to_gpu, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1410_1764_gb300 import api as A
+    A.lib()
+    return A
+
+
+def _state(orc, dims, seed=3):
+    nx, ny, nz = dims
+    st = synth.pad(synth.BSSN_FLAT[:, None, None, None]
+                   + 1e-2 * np.random.default_rng(seed).standard_normal((24, nz, ny, nx)), 3)
+    orc.fill_ghosts(st, 3)
+    return st
+
+
+@pytest.mark.parametrize("dims", [(13, 7, 5), (65, 44, 57)])  # 455 and 163,020 points: 7 and 76 of a block left
+def test_modes(api, orc, dims):
+    h = 0.05
+    st = _state(orc, dims)
+    want = orc.rk4(orc.BSSN, st, 3, h, 0.1 * h, 1)
+    rhs = orc.bssn_rhs(st, 3, h)
+    for v in range(8):
+        sysm = api.make_system(api.BSSN, *dims, h)
+        sysm.variant(v)
+        assert scaled_err(to_np(sysm.rhs(to_gpu(st))), rhs, 3) <= 1e-13, v
+        t = to_gpu(st)
+        sysm.rk4_step(t, 0.1 * h, 1)
+        assert scaled_err(to_np(t), want, 3) <= 1e-12, v
+
+
+def test_specialised_block(api, tmp_path):
+    """Tuned and specialised is no slower than the default on a small grid."""
+    import torch
+    dims = (37, 29, 23)
+    y = torch.from_numpy(synth.BSSN_FLAT).cuda()[:, None, None, None] + 1e-2 * torch.randn(
+        24, 29, 35, 43, dtype=torch.float64, device="cuda")
+    out = torch.empty_like(y)
+
+    def best(s):
+        times = []
+        for _ in range(15):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(20):
+                s.rhs(y, out)
+            e1.record()
+            torch.cuda.synchronize()
+            times.append(e0.elapsed_time(e1))
+        return min(times)
+
+    plain = api.make_system(api.BSSN, *dims, 0.05)
+    fast = []
+    for tune in (False, True):
+        s = api.make_system(api.BSSN, *dims, 0.05)
+        if tune:
+            s.autotune(y.clone())
+        s.specialize(True, cache_dir=tmp_path)
+        fast.append(best(s))
+    t = best(plain)
+    assert max(fast) <= 1.05 * t, (fast, t)  # 1.11 with the table's 128-thread block compiled

@@ -81,7 +81,7 @@ def test_bssn_field_tiles(api, orc, dims):
     orc.fill_ghosts(st, g)
     want = orc.bssn_rhs(st, g, h)
     sysm = api.make_system(api.BSSN, nx, ny, nz, h)
-    for v in range(8):                                       # every block of the algebra kernel
+    for v in range(8):                                       # the algebra kernel's five blocks
         sysm.variant(v)
         assert scaled_err(to_np(sysm.rhs(to_gpu(st))), want, g) <= 1e-13, v
 
