@@ -123,8 +123,10 @@ int chemora_fill_ghosts_axes(chemora_system* sys, double* state, int axes, void*
  * derivative fields from the device's pool in stream order (also in
  * chemora_stage and chemora_constraints; the pool is shared by all systems,
  * keeps up to 4 GB while one exists and 64 MB when none does), so calls on several streams do not
- * share one; without a workspace (a stream that is being captured, no memory
- * left) it runs a slower kernel that agrees to rounding. */
+ * share one; without a workspace (no memory left) it runs a slower kernel that
+ * agrees to rounding.  On a stream that is being captured the workspace belongs
+ * to the graph: it is freed at a later call once the graph and its instances
+ * are destroyed, and two instances of one graph must not run at once. */
 int chemora_rhs(chemora_system* sys, const double* state, double* rhs, void* stream);
 
 /* nsteps classic RK4 steps of size dt, in place (Sec. 2, time integrator).

@@ -12,8 +12,7 @@ namespace chemora {
 
 constexpr int CTX = 32, CTY = 4;
 
-// The constraints in one kernel without a workspace (a stream that is being
-// captured, no memory left).
+// The constraints in one kernel without a workspace (no memory left).
 __global__ void __launch_bounds__(CTX * CTY, 2) bssn_constraints_kernel(Dims d, Scalars sc,
                                                                         const double* __restrict__ st,
                                                                         double* __restrict__ out) {
@@ -96,7 +95,7 @@ int chemora_constraints(chemora_system* sys, const double* state, double* out, v
   const FieldWork work = take_field_work(sys, s);
   if (work.w) {
     const int rc = launch_constraints_split(d, sys->sc, state, out, work, s);
-    give_field_work(work, s);
+    give_field_work(sys, work, s);
     return rc;
   }
   dim3 grid((d.nx + CTX - 1) / CTX, (d.ny + CTY - 1) / CTY, d.nz);

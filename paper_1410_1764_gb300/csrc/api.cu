@@ -176,12 +176,12 @@ int prof_end(chemora_system* sys, cudaStream_t s, cudaEvent_t e0) {
   return CHEMORA_OK;
 }
 
-FieldWork system_field_work(chemora_system* sys, bool alloc) {
+FieldWork system_field_work(chemora_system* sys) {
   FieldWork w;
   if (sys->kind != CHEMORA_BSSN || !bssn_shape_splits(sys->grid->d, sys->variant)) return w;
-  if (!sys->field_work && alloc) {
+  if (!sys->field_work) {
     const int64_t points = field_work_points(sys->grid->d);
-    if (device_alloc(&sys->field_work, field_work_bytes(points)) == cudaSuccess) {
+    if (device_alloc_relaxed((void**)&sys->field_work, field_work_bytes(points)) == cudaSuccess) {
       sys->field_points = points;
     } else {
       sys->field_work = nullptr;
@@ -196,11 +196,13 @@ FieldWork system_field_work(chemora_system* sys, bool alloc) {
 FieldWork take_field_work(chemora_system* sys, cudaStream_t s) {
   FieldWork w;
   cudaStreamCaptureStatus cst = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cst) != cudaSuccess || cst != cudaStreamCaptureStatusNone) {
+  if (cudaStreamIsCapturing(s, &cst) != cudaSuccess) {
     cudaGetLastError();
     return w;
   }
   const int64_t points = field_work_points(sys->grid->d);
+  if (cst != cudaStreamCaptureStatusNone) return capture_field_work(sys, points, s);
+  free_orphans();
   void* p = nullptr;
   if (pool_alloc(&p, field_work_bytes(points), s) != cudaSuccess) return w;
   w.w = static_cast<double*>(p);
@@ -208,8 +210,11 @@ FieldWork take_field_work(chemora_system* sys, cudaStream_t s) {
   return w;
 }
 
-void give_field_work(const FieldWork& w, cudaStream_t s) {
-  if (w.w) pool_free(w.w, s);
+void give_field_work(chemora_system* sys, const FieldWork& w, cudaStream_t s) {
+  if (w.captured)
+    capture_work_used(sys, w, s);
+  else if (w.w)
+    pool_free(w.w, s);
 }
 
 static int run_stage(chemora_system* sys, const StageParams& a, const FieldWork& work, cudaStream_t s) {
@@ -267,12 +272,13 @@ void free_step_graph(chemora_system* sys) {
 }
 
 // One right-hand side or stage of a call that shares no scratch with others:
-// its derivative fields come from the device's pool, in stream order.
+// its derivative fields come from the device's pool, in stream order, or belong
+// to the graph it is captured into.
 static int run_single_stage(chemora_system* sys, const StageParams& p, cudaStream_t s) {
   FieldWork work;
   if (sys->kind == CHEMORA_BSSN && bssn_shape_splits(sys->grid->d, sys->variant)) work = take_field_work(sys, s);
   const int rc = run_stage(sys, p, work, s);
-  give_field_work(work, s);
+  give_field_work(sys, work, s);
   return rc;
 }
 
@@ -400,7 +406,7 @@ int chemora_rk4_step(chemora_system* sys, double* state, double dt, int nsteps, 
   // The scalar wave's launch-chained path (small grids, chosen by the autotuner).
   if (sys->chain_on && chain_available(sys) && !sys->profile_on && cst == cudaStreamCaptureStatusNone)
     return chain_rk4(sys, state, dt, nsteps, s);
-  const FieldWork work = system_field_work(sys, cst == cudaStreamCaptureStatusNone);
+  const FieldWork work = system_field_work(sys);
   // Plain launches while profiling (events bracket each stage) or when the
   // caller is capturing the stream itself; otherwise replay a captured step.
   const int images = stage_images(sys);

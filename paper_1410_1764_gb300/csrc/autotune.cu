@@ -195,7 +195,7 @@ int chemora_autotune(chemora_system* sys, double* state, int* variant, double* b
   if (sys->kind == CHEMORA_BSSN) {
     const int keep = sys->variant;
     sys->variant = 0;
-    work = system_field_work(sys, true);
+    work = system_field_work(sys);
     sys->variant = keep;
   }
   rc = autotune_stage(sys->kind, d, sys->sc, p, s, &best, &best_t, work);

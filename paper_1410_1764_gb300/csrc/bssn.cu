@@ -13,8 +13,7 @@
 namespace chemora {
 
 // The direct body in one kernel without a workspace: for callers that may not
-// allocate one (chemora_rk4_step_noalloc, a first call on a stream that is
-// being captured, no memory left).
+// allocate one (chemora_rk4_step_noalloc, no memory left).
 __global__ void __launch_bounds__(128, 2) bssn_stage_kernel(Dims d, Scalars sc, StageParams a) {
   bssn_direct_body<32, 4>(d, sc, a);
 }

@@ -58,6 +58,18 @@ struct chemora_grid {
   int64_t fsize;  // doubles per grid function
 };
 
+namespace chemora {
+// The workspace of a system's last call on a stream that is being captured
+// (capture.cu): capture, stream, last node of the call.
+struct CaptureWork {
+  double* w = nullptr;
+  int64_t points = 0;
+  unsigned long long id = 0;
+  cudaStream_t stream = nullptr;
+  cudaGraphNode_t last = nullptr;
+};
+}  // namespace chemora
+
 struct chemora_system {
   uint32_t type;
   chemora_grid* grid;
@@ -78,6 +90,7 @@ struct chemora_system {
   // device's pool
   double* field_work;
   int64_t field_points;
+  chemora::CaptureWork capture_work;
   // launch shape chosen by the autotuner (index into the kind's variants)
   int variant;
   // CUDA graph of one RK4 step (captured on cap_stream, replayed on the
@@ -123,6 +136,7 @@ int fill_ghosts_axes(const Dims& d, int nvars, double* state, int mask, cudaStre
 struct FieldWork {
   double* w = nullptr;
   int64_t points = 0;
+  bool captured = false;  // belongs to the graph the stream is captured into
 };
 constexpr int64_t kFieldWorkPoints = 1 << 20;  // points whose fields are held at once (1.36 GB)
 int64_t field_work_points(const Dims& d);      // workspace points a stage on d uses
@@ -135,12 +149,16 @@ int launch_constraints_split(const Dims& d, const Scalars& sc, const double* sta
 // kernels when it has a workspace.
 int bssn_shape(const Dims& d, int variant);
 bool bssn_shape_splits(const Dims& d, int variant);
-// The RK4 driver's workspace (no workspace if there is no memory for one or
-// alloc is false and there is none yet), and one taken from and given back to
-// the device's pool in stream order.
-FieldWork system_field_work(chemora_system* sys, bool alloc);
+// The RK4 driver's workspace (none if there is no memory for one), and one for a
+// call on s: taken from and given back to the device's pool in stream order, or,
+// while s is being captured, the graph's (capture.cu).
+FieldWork system_field_work(chemora_system* sys);
 FieldWork take_field_work(chemora_system* sys, cudaStream_t s);
-void give_field_work(const FieldWork& w, cudaStream_t s);
+void give_field_work(chemora_system* sys, const FieldWork& w, cudaStream_t s);
+FieldWork capture_field_work(chemora_system* sys, int64_t points, cudaStream_t s);
+void capture_work_used(chemora_system* sys, const FieldWork& w, cudaStream_t s);
+void free_orphans();  // workspaces of graphs that are gone
+cudaError_t device_alloc_relaxed(void** p, size_t bytes);  // also while a stream is being captured
 
 // device memory in stream order from the device's pool (pool.cu), and for good
 // (cudaMalloc; the pool's unused memory makes room)

@@ -121,6 +121,7 @@ void chemora_destroy(void* handle) {
     s->type = 0;
     delete s;
     pool_count_systems(-1);
+    free_orphans();
   } else if (is_handle(handle, H_BATCH)) {
     destroy_batch((chemora_batch*)handle);
   } else if (is_handle(handle, H_AMR)) {

@@ -1,0 +1,137 @@
+"""BSSN calls on a stream that is being captured: the bits and the speed of plain
+calls, workspaces shared by calls in a row and by no others, and given back with
+the graph."""
+import gc
+
+import numpy as np
+import pytest
+
+from paper_1410_1764_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def api():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1410_1764_gb300 import api as A
+    A.lib()
+    return A
+
+
+def _state(dims, seed=1):
+    import torch
+    nx, ny, nz = dims
+    p = 1e-2 * np.random.default_rng(seed).standard_normal((24, nz + 6, ny + 6, nx + 6))
+    return torch.from_numpy(synth.BSSN_FLAT[:, None, None, None] + p).cuda()
+
+
+def _capture(f):
+    import torch
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        f()
+    return graph
+
+
+def _inside(a):
+    return a[:, 3:-3, 3:-3, 3:-3]
+
+
+def _ms(f, n):
+    import torch
+    times = []
+    for _ in range(10):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        for _ in range(n):
+            f()
+        e1.record()
+        torch.cuda.synchronize()
+        times.append(e0.elapsed_time(e1) / n)
+    return min(times)
+
+
+@pytest.mark.parametrize("dims", [(37, 29, 23), (64, 64, 48)])
+@pytest.mark.parametrize("how", ["plain", "tuned", "specialised"])
+def test_same_as_plain(api, dims, how, tmp_path):
+    import torch
+    sysm, y = api.make_system(api.BSSN, *dims, 0.05), _state(dims)
+    if how != "plain":
+        sysm.autotune(y.clone())
+    if how == "specialised":
+        sysm.specialize(True, cache_dir=tmp_path)
+    out, con = torch.zeros_like(y), torch.zeros((7,) + y.shape[1:], dtype=torch.float64, device="cuda")
+    acc, dst, yn = torch.zeros_like(y), torch.zeros_like(y), y.clone()
+    rhs = _capture(lambda: sysm.rhs(y, out))
+    more = _capture(lambda: (sysm.constraints(y, con), sysm.stage(1, y, yn, acc, dst, c2=0.01)))
+    for _ in range(2):
+        rhs.replay()
+        more.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(_inside(out), _inside(sysm.rhs(y)))
+    assert torch.equal(_inside(con), _inside(sysm.constraints(y)))
+    a2, d2 = torch.zeros_like(y), torch.zeros_like(y)
+    sysm.stage(1, y, yn, a2, d2, c2=0.01)
+    assert torch.equal(_inside(acc), _inside(a2)) and torch.equal(_inside(dst), _inside(d2))
+    assert _ms(rhs.replay, 20) <= 1.1 * _ms(lambda: sysm.rhs(y, out), 20)
+
+
+def test_workspaces(api):
+    """Four calls in a row take one workspace; a call on a forked stream takes
+    its own, and the two run side by side."""
+    import torch
+    dims = (48, 48, 40)
+    sysm, ys = api.make_system(api.BSSN, *dims, 0.05), [_state(dims, q) for q in range(4)]
+    want = [sysm.rhs(y) for y in ys]
+    outs = [torch.zeros_like(y) for y in ys]
+    work = 1296 * 48 * 48 * 40
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    row = _capture(lambda: [sysm.rhs(y, o) for y, o in zip(ys, outs)])
+    assert before - torch.cuda.mem_get_info()[0] < 2 * work
+    row.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(_inside(o), _inside(w)) for o, w in zip(outs, want))
+    for o in outs:
+        o.zero_()
+    side = torch.cuda.Stream()
+
+    def fork():
+        main = torch.cuda.current_stream()
+        side.wait_stream(main)
+        for q in range(4):
+            with torch.cuda.stream(side if q % 2 else main):
+                sysm.rhs(ys[q], outs[q])
+        main.wait_stream(side)
+
+    both = _capture(fork)
+    for _ in range(5):
+        both.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(_inside(o), _inside(w)) for o, w in zip(outs, want))
+        for o in outs:
+            o.zero_()
+
+
+def test_given_back(api):
+    """Workspaces of graphs that are gone are freed at later calls."""
+    import torch
+    dims = (64, 64, 64)
+    sysm, y = api.make_system(api.BSSN, *dims, 0.05), _state(dims)
+    out = torch.zeros_like(y)
+    sysm.rhs(y, out)
+    held = []
+    for _ in range(6):
+        graph = _capture(lambda: sysm.rhs(y, out))
+        graph.replay()
+        torch.cuda.synchronize()
+        held.append(torch.cuda.mem_get_info()[0])
+        graph.reset()
+        del graph
+        gc.collect()
+        sysm.rhs(y, out)
+        torch.cuda.synchronize()
+    assert held[0] - min(held) < 2 * 1296 * 64 ** 3, held

@@ -102,8 +102,8 @@ def test_bssn_flat_and_nonfinite(api, orc):
 
 
 def test_bssn_rhs_without_a_workspace(api, orc):
-    """On a stream that is being captured the right-hand side allocates
-    nothing: the one-kernel body runs, and the graph replays it."""
+    """A first right-hand side on a stream that is being captured: it finds no
+    workspace of the system's, and the graph replays it."""
     import torch
     dims, g = (21, 10, 8), 3
     rng = np.random.default_rng(5)
