@@ -383,30 +383,26 @@ static int create_amr(int kind, const int* nc, int nbox, const int* lo, const in
     A->item_off[q + 1] = (int)items.size();
   }
   for (int q = 0; q <= 4; ++q) A->counter_off[q] = q;
-  if (kind == CHEMORA_BSSN) {
-    int rc = CHEMORA_OK;
-    A->work_points = field_work_points(A->dc);
-    for (int q = 0; q < 4 && !rc; ++q) {
-      const std::vector<PatchDesc> table(A->stage_pd.begin() + q * nbox, A->stage_pd.begin() + (q + 1) * nbox);
-      rc = field_plan_create(table, &A->plan[q]);
-      A->work_points = std::max(A->work_points, A->plan[q].points);
-      A->counter_off[q + 1] = A->counter_off[q] + (int)A->plan[q].chunks.size();
-    }
-    if (rc) {
-      for (FieldPlan& P : A->plan) field_plan_free(&P);
-      delete A;
-      return rc;
-    }
-  }
   const size_t cs = (size_t)nv * A->dc.sv;
   const size_t total = cs * (1 + 3 + 3) + (size_t)foff * (1 + 3) + (size_t)woff;
   double* buf = nullptr;
   cudaError_t e = device_alloc(&buf, total * sizeof(double));
+  if (e == cudaSuccess && kind == CHEMORA_BSSN) {
+    std::vector<PatchDesc> tables[4];
+    for (int q = 0; q < 4; ++q)
+      tables[q].assign(A->stage_pd.begin() + q * nbox, A->stage_pd.begin() + (q + 1) * nbox);
+    const int rc = field_plans_create(tables, 4, &A->dc, A->plan, &A->work, &A->work_points);
+    if (rc) {
+      cudaFree(buf);
+      delete A;
+      return rc;
+    }
+    for (int q = 0; q < 4; ++q) A->counter_off[q + 1] = A->counter_off[q] + (int)A->plan[q].chunks.size();
+  }
   if (e == cudaSuccess) e = cudaMemset(buf, 0, total * sizeof(double));
   if (e == cudaSuccess) e = device_alloc(&A->dev_boxes, nbox * sizeof(AmrBox));
   if (e == cudaSuccess) e = device_alloc(&A->dev_pd, 4 * nbox * sizeof(PatchDesc));
   if (e == cudaSuccess && kind == CHEMORA_WAVE) e = device_alloc(&A->items, items.size() * sizeof(WorkItem));
-  if (e == cudaSuccess && kind == CHEMORA_BSSN) e = device_alloc(&A->work, field_work_bytes(A->work_points));
   if (e == cudaSuccess) e = device_alloc(&A->counters, 2 * A->counter_off[4] * sizeof(unsigned int));
   if (e == cudaSuccess) e = device_alloc(&A->err, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(A->err, 0, sizeof(int));

@@ -257,9 +257,7 @@ static int chunk_planes(const Dims& d, int64_t cap) {
   return (int)std::min<int64_t>(d.nz, std::max<int64_t>(1, cap / plane));
 }
 
-int64_t field_work_points(const Dims& d) {
-  return (int64_t)d.nx * d.ny * chunk_planes(d, kFieldWorkPoints);
-}
+int64_t field_work_points(const Dims& d, int64_t cap) { return (int64_t)d.nx * d.ny * chunk_planes(d, cap); }
 
 int field_chunk_planes(const Dims& d, const FieldWork& work) {
   const int planes = chunk_planes(d, work.points);
@@ -371,11 +369,11 @@ batch_algebra_kernel(const FieldRegion* __restrict__ regions, int nregions, cons
   }
 }
 
-int field_plan_create(const std::vector<PatchDesc>& patches, FieldPlan* plan) {
-  // chunks of nearly equal size, each at most kFieldWorkPoints points (or one plane)
+// Chunks of nearly equal size, each at most `cap` points (or one plane).
+static int field_plan_create(const std::vector<PatchDesc>& patches, int64_t cap, FieldPlan* plan) {
   int64_t total = 0;
   for (const PatchDesc& P : patches) total += P.npts;
-  const int64_t nchunks = (total + kFieldWorkPoints - 1) / kFieldWorkPoints;
+  const int64_t nchunks = (total + cap - 1) / cap;
   const int64_t target = std::max<int64_t>(1, (total + nchunks - 1) / std::max<int64_t>(1, nchunks));
   std::vector<FieldRegion> regions;
   std::vector<WorkItem> items;
@@ -430,6 +428,32 @@ int field_plan_create(const std::vector<PatchDesc>& patches, FieldPlan* plan) {
                      cudaGetErrorString(e));
   }
   return CHEMORA_OK;
+}
+
+int field_plans_create(const std::vector<PatchDesc>* tables, int n, const Dims* grid, FieldPlan* plans, double** work,
+                       int64_t* points) {
+  int64_t cap = kFieldWorkPoints, tried = 0;
+  for (;;) {
+    int rc = CHEMORA_OK;
+    *points = grid ? field_work_points(*grid, cap) : 0;
+    for (int t = 0; t < n && !rc; ++t) {
+      rc = field_plan_create(tables[t], cap, &plans[t]);
+      *points = std::max(*points, plans[t].points);
+    }
+    if (!rc && *points == tried) {
+      rc = set_error(CHEMORA_ENOMEM, "derivative workspace of %zu bytes", field_work_bytes(*points));
+    } else if (!rc) {
+      const cudaError_t e = device_alloc(work, field_work_bytes(*points));
+      if (e == cudaSuccess) return CHEMORA_OK;
+      cudaGetLastError();
+      *work = nullptr;
+      if (e != cudaErrorMemoryAllocation) rc = cuda_error(e, "derivative workspace");
+    }
+    for (int t = 0; t < n; ++t) field_plan_free(&plans[t]);
+    if (rc) return rc;
+    tried = *points;
+    cap = std::max<int64_t>(1, std::min(cap, tried) / 2);
+  }
 }
 
 void field_plan_free(FieldPlan* plan) {

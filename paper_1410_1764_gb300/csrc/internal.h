@@ -139,7 +139,7 @@ struct FieldWork {
   bool captured = false;  // belongs to the graph the stream is captured into
 };
 constexpr int64_t kFieldWorkPoints = 1 << 20;  // points whose fields are held at once (1.36 GB)
-int64_t field_work_points(const Dims& d);      // workspace points a stage on d uses
+int64_t field_work_points(const Dims& d, int64_t cap = kFieldWorkPoints);  // workspace points a stage on d uses
 size_t field_work_bytes(int64_t points);
 int launch_bssn_split(const Dims& d, const Scalars& sc, const StageParams& a, const FieldWork& work, int block,
                       int minb, cudaStream_t s);
@@ -270,7 +270,11 @@ struct FieldPlan {
   WorkItem* items = nullptr;       // device: region and first point
   int2* tiles = nullptr;           // device: region and tile
 };
-int field_plan_create(const std::vector<PatchDesc>& patches, FieldPlan* plan);
+// The plans of n tables of regions and the workspace that they (and the stages of
+// *grid, if given) share: for kFieldWorkPoints points, or, where there is no memory
+// for it, for as many halvings fewer as it takes, down to a plane at a time.
+int field_plans_create(const std::vector<PatchDesc>* tables, int n, const Dims* grid, FieldPlan* plans, double** work,
+                       int64_t* points);
 void field_plan_free(FieldPlan* plan);
 // One stage; counters: one per chunk, zero before the launch.
 int launch_field_plan(const FieldPlan& plan, unsigned int* counters, int* err, long long limit, const Scalars& sc,

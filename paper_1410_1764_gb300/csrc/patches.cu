@@ -37,6 +37,7 @@ struct chemora_batch {
   int nitems;
   chemora::FieldPlan plan;  // BSSN: regions, work-list and chunks
   double* work;             // BSSN: derivative fields of a chunk
+  int64_t work_points;
   int ncounters;            // per stage
   unsigned int* counters;   // 4 x ncounters: one per stage and chunk of a step
   int* err;                // device error word: bit 0 bad work item, bit 1 time limit
@@ -219,7 +220,7 @@ static int patch_rk4_one(chemora_batch* b, int q, double dt, cudaStream_t s) {
   const int kind = b->kind;
   FieldWork work;
   work.w = b->work;
-  work.points = b->plan.points;
+  work.points = b->work_points;
   int rc;
   StageParams p{};
   if ((rc = fill_ghosts(P.d, b->nvars, Y, s))) return rc;
@@ -334,19 +335,17 @@ int chemora_patches_create(int npatch, const int* dims, int nghost, double dx, i
   b->total = off;
   b->nitems = (int)items.size();
   b->ncounters = 1;
-  cudaError_t e = cudaSuccess;
-  if (kind == CHEMORA_BSSN) {
-    if ((rc = field_plan_create(pd, &b->plan))) {
+  cudaError_t e = device_alloc(&b->state, off * sizeof(double));
+  if (e == cudaSuccess) e = device_alloc(&b->scratch, 3 * off * sizeof(double));
+  if (e == cudaSuccess && kind == CHEMORA_BSSN) {
+    if ((rc = field_plans_create(&pd, 1, nullptr, &b->plan, &b->work, &b->work_points))) {
       destroy_batch(b);
       return rc;
     }
     b->items = b->plan.items;
     b->nitems = b->plan.nitems;
     b->ncounters = (int)b->plan.chunks.size();
-    e = device_alloc(&b->work, field_work_bytes(b->plan.points));
   }
-  if (e == cudaSuccess) e = device_alloc(&b->state, off * sizeof(double));
-  if (e == cudaSuccess) e = device_alloc(&b->scratch, 3 * off * sizeof(double));
   if (e == cudaSuccess) e = device_alloc(&b->dev_pd, npatch * sizeof(PatchDesc));
   if (e == cudaSuccess && kind == CHEMORA_WAVE) e = device_alloc(&b->items, items.size() * sizeof(WorkItem));
   if (e == cudaSuccess) e = device_alloc(&b->counters, 4 * b->ncounters * sizeof(unsigned int));
