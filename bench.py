@@ -529,7 +529,9 @@ def bench_constraints(api, sysm, state, n, reps=10):
     torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / reps
     pps = n ** 3 / (ms * 1e-3)
-    instr = counts["fp64_instructions"] + 9 * 7  # the algebra; three fmas per mixed derivative
+    # the algebra; a conversion per first difference of 17 variables; for the 7 with second derivatives three
+    # fmas per mixed derivative and per row past the edges of 32 x 8 tiles
+    instr = counts["fp64_instructions"] + 17 * 3 + 7 * 9 + round(7 * 3 * (8 * 8 + 4 * 32) / 256.0)
     return {"workload": "bssn_constraints_%d^3" % n, "ms_per_launch": ms, "points_per_s": pps,
             "fp64_instr_per_point": instr,
             "fp64_issue_frac": instr * pps / ISSUE_PEAK[0] if ISSUE_PEAK[0] else None}

@@ -420,7 +420,7 @@ int chemora_opcount(int kind, int64_t* fp64_instructions, int64_t* flops);
  * shares x-direction work across warp lanes or y differences through shared
  * memory; the counts then include, per point, that sharing's own work).
  * Counts as chemora_opcount; a stencil evaluated on the integer units counts
- * its algorithmic flops and no FP64 instruction. */
+ * its algorithmic flops, and of FP64 instructions only conversions. */
 int chemora_system_opcount(chemora_system* sys, int64_t* fp64_instructions, int64_t* flops);
 
 /* Measure the device's FP64 fused-multiply-add throughput (flop/s, fma = 2)

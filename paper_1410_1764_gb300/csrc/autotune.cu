@@ -127,12 +127,12 @@ int chemora_variant_info(int kind, int variant, int* tx, int* ty, int* min_block
 
 int chemora_system_opcount(chemora_system* sys, int64_t* fp64_instructions, int64_t* flops) {
   if (!is_handle(sys, H_SYSTEM)) return set_error(CHEMORA_EINVAL, "not a system handle");
-  if (sys->kind == CHEMORA_WAVE || sys->kind == CHEMORA_WAVE1) {
+  if (sys->kind != CHEMORA_BSSN) {
     // the stencils run on the integer units: one FP64 multiply per evolved
-    // derivative is left
+    // derivative is left, for the variable speed the scales and products with s and G
     int64_t f = 0;
     const int rc = chemora_opcount(sys->kind, nullptr, &f);
-    if (fp64_instructions) *fp64_instructions = sys->nvars - 1;
+    if (fp64_instructions) *fp64_instructions = sys->kind == CHEMORA_WAVE_VARC ? 6 : sys->nvars - 1;
     if (flops) *flops = f;
     return rc;
   }
@@ -150,9 +150,9 @@ int chemora_system_opcount(chemora_system* sys, int64_t* fp64_instructions, int6
     return CHEMORA_OK;
   }
   if (v) {
-    // the split kernels: the algebra's body and prologue, and three fmas per
-    // mixed derivative (the other differences run on the integer units)
-    if (fp64_instructions) *fp64_instructions = CHEMORA_OPS_BSSN_ALG_INSTR + 44 + 3 * 33;
+    // the split kernels: the algebra's body and prologue, and the field kernels
+    if (fp64_instructions)
+      *fp64_instructions = CHEMORA_OPS_BSSN_ALG_INSTR + 44 + llround(field_fp64_instr(sys->grid->d));
     if (flops) *flops = CHEMORA_OPS_BSSN_FLOPS;
     return CHEMORA_OK;
   }

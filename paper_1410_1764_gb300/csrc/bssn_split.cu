@@ -268,6 +268,13 @@ size_t field_work_bytes(int64_t points) {
   return (size_t)((points + kFieldBlock - 1) / kFieldBlock) * kFields * kFieldBlock * sizeof(double);
 }
 
+// FP64 instructions of the field kernels per point of d: a conversion per first
+// difference, three fmas per mixed derivative and per row past a tile's edge.
+double field_fp64_instr(const Dims& d) {
+  const FieldRegion R = field_region(d, 0, 0);
+  return 24 * 3 + 11 * 3 * (3.0 + (8.0 * R.th + 4.0 * R.tw) / ((double)R.tw * R.th));
+}
+
 static int launch_field_kernels(const FieldRegion* regions, const FieldRegion& R, const int2* tiles, unsigned ntiles,
                                 int nvars, const double* src, double* work, const Scalars& sc, cudaStream_t s) {
   // 24 variables: 11 with second derivatives, 13 without; the constraints' 17: 7 and 10

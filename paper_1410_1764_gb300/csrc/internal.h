@@ -141,6 +141,7 @@ struct FieldWork {
 constexpr int64_t kFieldWorkPoints = 1 << 20;  // points whose fields are held at once (1.36 GB)
 int64_t field_work_points(const Dims& d, int64_t cap = kFieldWorkPoints);  // workspace points a stage on d uses
 size_t field_work_bytes(int64_t points);
+double field_fp64_instr(const Dims& d);
 int launch_bssn_split(const Dims& d, const Scalars& sc, const StageParams& a, const FieldWork& work, int block,
                       int minb, cudaStream_t s);
 int launch_constraints_split(const Dims& d, const Scalars& sc, const double* state, double* out,

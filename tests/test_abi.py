@@ -1,6 +1,7 @@
 """The C ABI library loads, exports every function include/chemora.h
 declares, and validates arguments on the host (no GPU needed)."""
 import ctypes
+import json
 import os
 import re
 
@@ -94,6 +95,25 @@ def test_generated_sources_up_to_date():
     for name, text in files.items():
         path = os.path.join(G.OUT, name)
         assert open(path).read() == text, "regenerate: python -m paper_1410_1764_gb300.gen"
+
+
+def test_system_opcounts(L):
+    """FP64 instructions of the kernels that run: the variable-speed wave's scales
+    and products; BSSN's algebra and prologue, 72 conversions, 33 mixed
+    derivatives, and on 128^3 (tiles of 32 x 8) the rows past the tiles' edges."""
+    with open(os.path.join(ROOT, "paper_1410_1764_gb300", "csrc", "generated", "opcounts.json")) as f:
+        counts = json.load(f)
+    for kind, nv, ng, n, want, flops in (
+            (N.WAVE, 2, 2, 16, 1, "wave"), (N.WAVE1, 5, 2, 16, 4, "wave1_o4"), (N.WAVE_VARC, 2, 2, 16, 6, "wave_varc"),
+            (N.BSSN, 24, 3, 128, counts["bssn_alg"]["fp64_instructions"] + 44 + 72 + 99 + 25, "bssn")):
+        g, s = ctypes.c_void_p(), ctypes.c_void_p()
+        assert L.chemora_grid_create(n, n, n, nv, ng, 0.1, ctypes.byref(g)) == N.OK
+        assert L.chemora_system_create(g, kind, None, ctypes.byref(s)) == N.OK
+        i, fl = ctypes.c_int64(), ctypes.c_int64()
+        assert L.chemora_system_opcount(s, ctypes.byref(i), ctypes.byref(fl)) == N.OK
+        assert (i.value, fl.value) == (want, counts[flops]["flops"]), kind
+        L.chemora_destroy(s)
+        L.chemora_destroy(g)
 
 
 def test_variant_queries(L):
