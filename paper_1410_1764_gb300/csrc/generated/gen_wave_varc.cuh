@@ -54,7 +54,7 @@ __device__ __forceinline__ void chemora_varc_point(const LD& ld, const SC& sc, O
   const double t126 = fma(sc.k[3], t121, (-t122));
   const double t128 = fma(sc.i12h, t126, sc.k[1]);
   const double v_f5_0_0_0 = ld(5, 0, 0, 0);
-  const double t13941 = fma(t128, v_f5_0_0_0, fma(t106, v_f4_0_0_0, fma(t85, v_f3_0_0_0, fma(t64, v_f2_0_0_0, sc.k[1]))));
+  const double t13930 = fma(t128, v_f5_0_0_0, fma(t106, v_f4_0_0_0, fma(t85, v_f3_0_0_0, fma(t64, v_f2_0_0_0, sc.k[1]))));
   out(0, v_f1_0_0_0);
-  out(1, t13941);
+  out(1, t13930);
 }

@@ -25,9 +25,6 @@ def _sym_expr(name):
     m = re.match(r"sdy_(\d+)_(-?\d+)$", name)
     if m:
         return "ld.sdy(%s, %s)" % m.groups(), True
-    m = re.match(r"zq([ab])_(\d+)$", name)
-    if m:
-        return "ld.q%s[%s]" % m.groups(), True
     m = re.match(r"sdz_(\d+)_(-?\d+)$", name)
     if m:
         return "ld.sdz(%d, %s)" % (stencil.ZROW_VARS.index(int(m.group(1))), m.group(2)), True
@@ -75,11 +72,6 @@ def _varc_numbering():
                         * stencil.I12H2)
     adv = sum((stencil.d1(S, a) * stencil.d1(U, a) for a in systems.R3), systems.E.const(0))
     return [systems.E.box(stencil.val(1)), systems.E.box(stencil.val(S) * lap + adv)]
-
-
-def _wave_xz():
-    with stencil.xshare(), stencil.zqueue():
-        return systems.wave()
 
 
 def _bssn_xshare():
@@ -172,10 +164,6 @@ def _render():
                       "scalar wave, first-order form of Eq. 1 (u, rho, v_i), order-%d D, "
                       "from gen/wave1.eqs" % p))
     # last, so that the constant table of the earlier bodies keeps its order
-    specs.append(("wave_xz", "chemora_wave_xz_point", _wave_xz,
-                  "scalar wave as chemora_wave_point, x-direction differences shared across warp "
-                  "lanes and the z-direction second difference from a register queue of z first "
-                  "differences kept by a thread marching along z"))
     specs.append(("wave_varc", "chemora_varc_point", systems.wave_varc,
                   "variable-speed wave: u_t = rho, rho_t = s Lap u + G . grad u, with s = c^2 "
                   "and G = grad s read from grid functions 2 and 3-5"))
@@ -205,8 +193,8 @@ def _render():
     files["opcounts.json"] = json.dumps(counts, indent=1, sort_keys=True) + "\n"
     inc = [HEADER.rstrip("\n") + "\n", "// per interior point and RHS evaluation\n"]
     for key, tag in (("wave", "WAVE"), ("wave_varc", "VARC"), ("bssn", "BSSN"), ("wave1_o4", "WAVE1"),
-                     ("bssn_x", "BSSN_X"), ("bssn_xy", "BSSN_XY"), ("wave_xz", "WAVE_XZ"),
-                     ("bssn_alg", "BSSN_ALG"), ("bssn_constraints_alg", "CONSTRAINTS_ALG")):
+                     ("bssn_x", "BSSN_X"), ("bssn_xy", "BSSN_XY"),
+                     ("bssn_alg", "BSSN_ALG")):
         inc.append("#define CHEMORA_OPS_%s_INSTR %d\n" % (tag, counts[key]["fp64_instructions"]))
         inc.append("#define CHEMORA_OPS_%s_FLOPS %d\n" % (tag, counts[key]["flops"]))
     files["opcounts.inc"] = "".join(inc)

@@ -1,11 +1,10 @@
-"""The lane-sharing point bodies (BSSN x/y-sharing, the bench's body, and the
-x-lane / z-queue scalar wave) run on the host: each statement of the
+"""The lane-sharing BSSN point bodies run on the host: each statement of the
 generated straight-line body is evaluated for the 32 lanes of a warp before
 the next (temporaries become arrays over lanes), so a warp shuffle reads the
 other lanes' values exactly as on the GPU.  The harness supplies what the
 kernels supply: neighbour loads, the halo lanes' x differences and derivative
 rows, the shared-memory y differences and z-derivative rows of the x/y
-prologue, and the z-difference queue; outputs are compared with the oracle.
+prologue; outputs are compared with the oracle.
 No GPU: a CPU check of the generated code the GPU kernels compile."""
 import ctypes
 import os
@@ -53,7 +52,6 @@ def _lanewise(header, fn):
         expr = expr.replace("ld(", "ld.at(l, ").replace("ld.ext_dx(", "ld.ext_dx(l, ")
         expr = expr.replace("ld.ext_d1y(", "ld.ext_d1y(l, ").replace("ld.ext_d1z(", "ld.ext_d1z(l, ")
         expr = expr.replace("ld.sdy(", "ld.sdy(l, ").replace("ld.sdz(", "ld.sdz(l, ")
-        expr = re.sub(r"ld\.q([ab])\[(\d+)\]", r"ld.q\1(l, \2)", expr)
         if m:
             body.append("  double %s[32];\n  for (int l = 0; l < 32; ++l) %s[l] = %s;" % (m.group(1), m.group(1), expr))
         else:
@@ -115,10 +113,6 @@ struct Warp {
     return val(v, x0 + l, y + m + 1, z) - val(v, x0 + l, y + m, z);
   }
   double sdz(int l, int vi, int m) const { return d1row(zrow[vi], x0 + l, y + m, z, 0); }
-  // the z queue of the x/z wave body: e_m = u(z+m+1) - u(z+m)
-  double e(int l, int m) const { return val(0, x0 + l, y, z + m + 1) - val(0, x0 + l, y, z + m); }
-  double qa(int l, int) const { return e(l, 0) - e(l, -1); }
-  double qb(int l, int) const { return e(l, 1) - e(l, -2); }
 };
 
 static double xshfl(const double* own, const double* ext, int m, int w, int l) {
@@ -191,7 +185,7 @@ def _run(lib, st, g, h):
 
 @pytest.mark.parametrize("amp", [3e-2, 1e-10])
 def test_xy_sharing_bssn_body(orc, tmp_path, amp):
-    """The bench's body (x lanes, y differences and z rows from the
+    """The x/y-sharing body (x lanes, y differences and z rows from the
     prologue) on two warps per row, 24 variables, against the oracle."""
     dims, g, h = (64, 6, 5), 3, 1.0 / 64
     rng = np.random.default_rng(41)
@@ -209,13 +203,4 @@ def test_x_sharing_bssn_body(orc, tmp_path):
     orc.fill_ghosts(st, g)
     want = orc.bssn_rhs(st, g, h)
     got = _run(_build(tmp_path, "gen_bssn_x.cuh", "chemora_bssn_x_point"), st, g, h)
-    assert scaled_err(got, want, g) <= 1e-12
-
-
-def test_xz_wave_body(orc, tmp_path):
-    dims, g, h = (64, 7, 9), 2, 1.0 / 64
-    st = synth.pad(np.random.default_rng(43).standard_normal((2, dims[2], dims[1], dims[0])), g)
-    orc.fill_ghosts(st, g)
-    want = orc.wave_rhs(st, g, h)
-    got = _run(_build(tmp_path, "gen_wave_xz.cuh", "chemora_wave_xz_point"), st, g, h)
     assert scaled_err(got, want, g) <= 1e-12
