@@ -4,8 +4,8 @@
 // warp instruction, and use little else.  Advection and dissipation of every
 // variable, gt_ij's whole right-hand side, At_ij's terms in the shift and the
 // traces gt^ab D_ab f are sums of products, 272 of the 1058 FP64 operations;
-// on the integer units, which run beside the FP64 pipe, such a sum is exact to
-// 2^-56 of its largest product and rounded once.  They are loops over
+// on the integer units, which run beside the FP64 pipe, such a sum is closer than
+// an FP64 chain (bounds and errors at fx::dot) and rounded once.  They are loops over
 // variables, not straight code, to keep the kernel in the instruction cache,
 // with the next variable's fields fetched an iteration ahead; results pass to
 // the generated body through the thread's column in shared memory.  Values

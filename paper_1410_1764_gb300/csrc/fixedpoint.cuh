@@ -127,16 +127,21 @@ CHEMORA_FX Term<S> term(double v) {
   if ((unsigned)(e - 1) >= 2046u) e = ((h << 1) | loword(v)) == 0 ? -8192 : 16384;
   return Term<S>{(int)(m >> 32), (int)((unsigned)m >> 1), e};
 }
-// a b in units of 2^(e - 1075 - K), within six units, in four multiplications:
-// the product of the low words is left out.
+// a b in units of 2^(e - 1075 - K) in four multiplications: the product of the low
+// words is left out, two halved low words and the high halves of two products are
+// cut, in all less than six units, of which two are added back (the mean).
 template <int K>
 CHEMORA_FX Parts term_product(const Term<10>& a, const Term<K + 1>& b) {
   const int x = mulhi32(a.hi, b.lo) + mulhi32(a.lo, b.hi);
-  return Parts{mad_wide(x, 2, mad_wide(a.hi, b.hi, 0)), emax(a.e + b.e - 1022, kZeroExp)};
+  return Parts{mad_wide(x, 2, mad_wide(a.hi, b.hi, 2)), emax(a.e + b.e - 1022, kZeroExp)};
 }
-// The sum of N products as a double, at the guard bits with which N of them fit
-// in 64 bits (N 2^(53 + k) < 2^63): within 6 N units, a sixteenth of an ulp of
-// the largest product each; false if their exponents leave the range to FP64.
+// The sum of N products as a double, at the guard bits k with which N of them fit
+// in 64 bits (N 2^(53 + k) < 2^63); false if their exponents leave the range to
+// FP64.  Within 7 N units of 2^(-52 - k) of the largest product's binade (a
+// product's cut and its alignment's) and half an ulp; N / 2 units, the
+// alignments' mean cut, are added back.  Root mean square errors in ulps of the
+// largest product, twelve terms: 0.3 to 1.2, an FP64 fma chain 0.6 to 2.5; mean
+// errors below 0.1 (0.3, all one way, with nothing added back).
 template <int N>
 struct DotGuard {
   static constexpr int k = N <= 7 ? 7 : 6;
@@ -176,7 +181,7 @@ CHEMORA_FX bool dot(const Parts (&p)[N], double* sum) {
   *sum = 0.0;
   if (e == kZeroExp) return true;
   if (!in_range(e)) return false;
-  long long m = 0;
+  long long m = N / 2;
 #if defined(__CUDACC__)
 #pragma unroll
 #endif

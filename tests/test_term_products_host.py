@@ -51,7 +51,8 @@ def L(tmp_path_factory):
 
 def test_products(L):
     """Within six units of the exact product: the low words' product, two
-    halved low words and three roundings down are at most one unit each."""
+    halved low words and three roundings down are at most one unit each (two
+    units, the mean, are added back)."""
     rng, m = np.random.default_rng(0), ctypes.c_longlong()
     ends = [1.0, -1.0, 2.0 - 2.0 ** -52, -2.0 + 2.0 ** -52, 1.0 + 2.0 ** -52]
     pairs = [(a, b) for a in ends for b in ends]
@@ -93,3 +94,35 @@ def test_sums(L, n, spread, cancel):
         x = [1.0] * n if not bad == 1e-300 else [bad] * n
         x[-1] = bad
         assert L.dot(n, D(*x), D(*([1e4 if bad == 1e308 else 1e-10] * n)), ctypes.byref(out)) == 0
+
+
+@pytest.mark.parametrize("n", [4, 6, 12])
+@pytest.mark.parametrize("field", ["normal", "spread", "sparse", "positive", "dominant"])
+def test_sums_against_fp64(L, n, field):
+    """No further from the exact sum than a chain of FP64 fmas, and without a
+    bias: in ulps of the largest product, over 3000 sums."""
+    rng = np.random.default_rng(n)
+    D = ctypes.c_double * n
+    err = np.zeros((3000, 2))
+    for i in range(len(err)):
+        a, b = rng.standard_normal((2, n))
+        if field == "spread":
+            a, b = a * np.exp2(-8 * rng.random(n)), b * np.exp2(-8 * rng.random(n))
+        elif field == "sparse":
+            a[max(2, n // 3):] = 0.0
+        elif field == "positive":
+            a, b = abs(a), abs(b)
+        elif field == "dominant":
+            a[1:] *= 1e-3
+        out = ctypes.c_double()
+        assert L.dot(n, D(*a), D(*b), ctypes.byref(out))
+        prods = [Fraction(float(x)) * Fraction(float(y)) for x, y in zip(a, b)]
+        chain = 0.0
+        for p in prods:  # a correctly rounded fma
+            chain = float(Fraction(chain) + p)
+        ulp = Fraction(2) ** (math.frexp(float(max(map(abs, prods))))[1] - 53)
+        err[i] = [float((Fraction(v) - sum(prods)) / ulp) for v in (chain, out.value)]
+    rms = np.sqrt((err ** 2).mean(0))
+    # a unit's share of the ulp (what is added back is whole units), and three standard errors of the mean
+    bias = 0.06 + 3 * rms[1] / len(err) ** 0.5
+    assert rms[1] <= rms[0] and abs(err[:, 1].mean()) <= bias, (rms, err.mean(0))
