@@ -123,10 +123,11 @@ RK_UPDATE_FLOPS = 3.25
 
 
 def _profile_traffic(kernel_key):
-    """DRAM traffic per launch of the timed stage kernel from the committed
-    machine-readable ncu figures (profiles/bssn_stage_kernel_128.json), or
-    None when they were taken on a different build of the kernel."""
-    path = os.path.join(ROOT, "profiles", "bssn_stage_kernel_128.json")
+    """DRAM traffic per RK stage of the timed kernels (derivative fields and
+    algebra) from the committed machine-readable ncu figures
+    (profiles/bssn_split_kernels.json), or None when they were taken on a
+    different build of the kernels."""
+    path = os.path.join(ROOT, "profiles", "bssn_split_kernels.json")
     try:
         with open(path) as f:
             vals = json.load(f)
@@ -140,18 +141,21 @@ def _profile_traffic(kernel_key):
 
 def kernel_source_hash():
     """Hash of the code (comments and blank lines removed) of the sources the
-    timed, run-time specialised BSSN stage kernel is built from: the device
-    headers NVRTC compiles (of the generated bodies, the x/y-sharing one the
-    profiled launch shape instantiates) and the part of the specialiser that
-    writes the kernel source and the compiler options."""
+    timed BSSN stage is built from: the derivative-field kernel, the algebra
+    body and what it includes, and the part of the specialiser that writes the
+    kernel source and the compiler options."""
     import hashlib
     import re
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1410_1764_gb300", "csrc")
-    for rel in ("bssn_kernels.cuh", "jit.cu", "stage.cuh", "device_types.cuh",
-                "generated/gen_constants.cuh", "generated/gen_bssn_xy.cuh"):
+    for rel in ("bssn_split.cu", "bssn_algebra.cuh", "bssn_prologue.cuh", "bssn_fields.cuh", "fixedpoint.cuh",
+                "jit.cu", "stage.cuh", "device_types.cuh", "generated/gen_constants.cuh",
+                "generated/gen_bssn_alg.cuh"):
         with open(os.path.join(csrc, rel)) as f:
             text = re.sub(r"/\*.*?\*/", "", f.read(), flags=re.S)
+        if rel == "bssn_split.cu":  # the field kernel
+            m = re.search(r"template <bool DD>.*?\n}\n", text, flags=re.S)
+            text = m.group(0) if m else text
         if rel == "jit.cu":  # only what shapes the kernel: its source text and the options
             m = re.search(r"std::string kernel_source\(.*?\n}\n", text, flags=re.S)
             opts = [ln for ln in text.splitlines() if "opts = {" in ln or "opts.push_back" in ln]
@@ -689,7 +693,8 @@ def run_chemora(args):
                            "frac_body_F: the executed body's own count; stencils and sums on the integer "
                            "units take no FP64 issue, so both may exceed 1: fp64_issue_frac is the share "
                            "of the FP64 pipe" % (FROZEN_RHS_FLOPS_BSSN, RK_UPDATE_FLOPS * NVARS),
-            "traffic": _profile_traffic(kernel_source_hash()),
+            "traffic": (_profile_traffic(kernel_source_hash())
+                        if api.variant_info(api.BSSN, variant)[3] == 0 else None),
             "kernel": _kernel_name(api, fp64_instr, variant, jit_s is not None),
             "specialised": jit_s is not None, "jit_compile_s": jit_s,
             "variant": variant, "block": list(block), "fp64_instr_per_point_rhs": fp64_instr, "kernel_ms_avg": kern_ms / kern_n if kern_n else None,

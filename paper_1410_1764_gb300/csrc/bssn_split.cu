@@ -38,8 +38,9 @@ constexpr int kGuard = 4;       // guard bits: an axis' weights add up to 64 in 
 // readers, no march: 846 us; conversion instruction for every difference 603,
 // for none 572 us; two or four blocks per SM 637, 708 us; significand and
 // exponent in one 16-byte cell 621 us; one kernel for both sorts of variable
-// 580 us.  Bound by the latency of its integer chains at 24 warps per SM
-// (2.2 instructions per clock; FP64 pipe 45 % busy).
+// 580 us.  Bound by its FP64 pipe (70 % busy for variables with second
+// derivatives) and the latency of its chains at 23 warps per SM (2.1 instructions
+// per clock).
 template <bool DD>
 __global__ void __launch_bounds__(kTileThreads, 3)
 bssn_fields_kernel(const FieldRegion* __restrict__ regions, FieldRegion one_region, const int2* __restrict__ tiles,

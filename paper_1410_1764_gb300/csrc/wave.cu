@@ -40,8 +40,8 @@ static int launch_varc_variant(const Dims& d, const Scalars& sc, const StagePara
 }
 
 // Planes in shared memory (wave_orders.cu) win where blocks marching through
-// many planes fill the GPU (256^3: 245 us per stage against 297), a point per
-// thread on small grids (61 x 75 x 53: 9.6 against 10.1); the autotuner times
+// many planes fill the GPU (256^3: 233 us per stage against 290), a point per
+// thread on small grids (61 x 75 x 53: 10.3 against 11.1); the autotuner times
 // both.
 const LaunchVariant kWaveVariants[] = {
     {32, 8, 0, launch_wave_variant<32, 8>},   {32, 4, 0, launch_wave_variant<32, 4>},

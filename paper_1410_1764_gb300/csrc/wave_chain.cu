@@ -74,7 +74,8 @@ __global__ void __launch_bounds__(128) wave_chain_stage_kernel(Dims d, Scalars s
   // took a third of the instructions.  The addresses are pinned here, before the
   // wait, where they cost nothing: left to the compiler, 32-bit ones are formed
   // after it (61 x 75 x 53 x 20 steps 525 us, 32^3 x 100 steps 1247; pinned 491
-  // and 1162; with 64-bit indices 530 and 1205).
+  // and 1162; with 64-bit indices 530 and 1205; order-4 Laplacian with two guard bits
+  // then, 503 and 1188 now).
   const unsigned t = blockIdx.x * 128 + threadIdx.x;
   const unsigned npts = (unsigned)d.nx * d.ny * d.nz;
   const unsigned row = t / (unsigned)d.nx;

@@ -6,13 +6,13 @@
 // run on the integer units (star_march.cuh); values those cannot take go to
 // the FP64 bodies generated from gen/systems.py.
 //
-// GB300, us per stage, bodies alone (FP64 issue: 49 and 42 instructions at
-// 17.8 cycles each) and now: two-variable form of order 8 on 128^3 222 and 57,
-// first-order form of order 6 on 117 x 90 x 131 174 and 93; order 4 on 256^3
-// with every point taking its 13 values apart itself (wave.cu) 297 and 245
-// here.  What bounds them now is the FP64 pipe (5 and 14 instructions per
-// point, half its time) and the latency of the integer chains at 24 and 16
-// warps per SM; HBM alone takes 158 us of the 245.
+// GB300, us per stage, FP64 bodies (49 and 42 instructions at 17.8 cycles each)
+// and now: two-variable form of order 8 on 128^3 222 and 48, first-order form of
+// order 6 on 117 x 90 x 131 174 and 84; order 4 on 256^3 with every point taking
+// its 13 values apart itself (wave.cu) 290 and 233 here.  What bounds them now is
+// the FP64 pipe (5 and 14 instructions per point, 40 to 54 % of its time) and the
+// latency of the integer chains at 20 and 15 warps per SM; HBM alone takes 158 us
+// of the 233.
 #include "internal.h"
 #include "stage.cuh"
 #include "star_march.cuh"
@@ -45,8 +45,8 @@ CHEMORA_BODY(Wave1O6, 5, chemora_wave1_o6_point)
 CHEMORA_BODY(Wave1O8, 5, chemora_wave1_o8_point)
 
 // Threads per SM asked of the compiler, the most that leaves next to no spills
-// (order 4: 245 us per stage of 256^3 with 768 threads, 270 with 1024 and 20
-// bytes spilled; order 8: 10 steps on 128^3 2.01 ms with 640, 2.28 with 768 and
+// (order 4, two guard bits: 245 us per stage of 256^3 with 768 threads, 270 with
+// 1024 and 20 bytes spilled; order 8: 10 steps on 128^3 2.01 ms with 640, 2.28 with 768 and
 // 48 bytes spilled; first-order form of order 6 on 117 x 90 x 131: 93 us per
 // stage with 512, 141 with 640 and 160 bytes spilled).
 template <int NV, int R>

@@ -249,9 +249,9 @@ def _shapes_with(api, kind, sharing):
 
 @pytest.mark.parametrize("dims", [(64, 12, 20), (32, 7, 37), (33, 9, 11)])
 def test_wave_xz_shapes(api, orc, dims):
-    """x-lane / z-queue wave shapes: every shape, ragged rows (ny = 7), nz not
-    a multiple of the march length, and nx % 32 != 0 (the shapes fall back to
-    the one-point kernel); one RHS and RK4 steps against the oracle."""
+    """The order-4 wave's marching shapes: every shape, ragged rows (ny = 7), nz
+    not a multiple of the march's depth, and nx % 32 != 0; one RHS and RK4 steps
+    against the oracle."""
     nx, ny, nz = dims
     g, h = 2, 1.0 / nx
     rng = np.random.default_rng(11)
@@ -271,7 +271,7 @@ def test_wave_xz_shapes(api, orc, dims):
 
 
 def test_wave_xz_plane_wave_100_steps(api, orc):
-    """The 32^3 plane-wave workload, 100 RK4 steps, on an x/z shape."""
+    """The 32^3 plane-wave workload, 100 RK4 steps, on a marching shape."""
     n, g = 32, 2
     y0, h = synth.plane_wave(n, g)
     want = orc.rk4(orc.WAVE, y0, g, h, 0.25 * h, 100)
