@@ -13,9 +13,11 @@
 
 namespace chemora {
 
+// Not held over a CUDA call: the destructors below run on a thread of CUDA's.
 static std::mutex g_capture_mu;
-// workspaces whose graphs are gone: their destructors may not call CUDA
-static std::vector<double*> g_orphans;
+// workspaces whose graphs are gone (a destructor may not free them: that is a CUDA
+// call); never destroyed, since graphs may outlive static objects
+static std::vector<double*>& g_orphans = *new std::vector<double*>();
 
 static void orphan(void* p) {
   const std::lock_guard<std::mutex> lock(g_capture_mu);
@@ -91,14 +93,15 @@ FieldWork capture_field_work(chemora_system* sys, int64_t points, cudaStream_t s
   w.captured = true;
   CaptureInfo c;
   if (!c.get(s)) return w;
-  CaptureWork& k = sys->capture_work;
+  CaptureWork k;
   {
     const std::lock_guard<std::mutex> lock(g_capture_mu);
-    if (k.w && k.id == c.id && k.stream == s && k.points == points && follows(c.ends, c.n, k.last)) {
-      w.w = k.w;
-      w.points = points;
-      return w;
-    }
+    k = sys->capture_work;
+  }
+  if (k.w && k.id == c.id && k.stream == s && k.points == points && follows(c.ends, c.n, k.last)) {
+    w.w = k.w;
+    w.points = points;
+    return w;
   }
   free_orphans();
   double* p = nullptr;
