@@ -48,14 +48,16 @@ const LaunchVariant kWaveVariants[] = {
     {64, 4, 0, launch_wave_variant<64, 4>},   {128, 2, 0, launch_wave_variant<128, 2>},
     {16, 16, 0, launch_wave_variant<16, 16>},
     {32, 8, 0, launch_wave_planes<32, 8>, 4}, {32, 4, 0, launch_wave_planes<32, 4>, 4},
-    {16, 16, 0, launch_wave_planes<16, 16>, 4},
+    {16, 16, 0, launch_wave_planes<16, 16>, 4}, {64, 4, 0, launch_wave_planes<64, 4>, 4},
+    {16, 8, 0, launch_wave_planes<16, 8>, 4},   {8, 16, 0, launch_wave_planes<8, 16>, 4},
+    {32, 16, 0, launch_wave_variant<32, 16>},   {16, 8, 0, launch_wave_variant<16, 8>},
 };
 const int kNumWaveVariants = sizeof(kWaveVariants) / sizeof(kWaveVariants[0]);
 
 const LaunchVariant kVarcVariants[] = {
     {32, 8, 0, launch_varc_variant<32, 8>},   {32, 4, 0, launch_varc_variant<32, 4>},
     {64, 4, 0, launch_varc_variant<64, 4>},   {16, 16, 0, launch_varc_variant<16, 16>},
-    {16, 8, 0, launch_varc_variant<16, 8>},
+    {16, 8, 0, launch_varc_variant<16, 8>},   {8, 16, 0, launch_varc_variant<8, 16>},
 };
 const int kNumVarcVariants = sizeof(kVarcVariants) / sizeof(kVarcVariants[0]);
 

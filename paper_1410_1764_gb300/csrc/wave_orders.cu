@@ -298,9 +298,9 @@ static int launch_order(const Dims& d, const Scalars& sc, const StageParams& a, 
 #define CHEMORA_SHAPES(BODY, R)                                                              \
   {{32, 8, 0, launch_order<BODY, R, 32, 8>},  {32, 4, 0, launch_order<BODY, R, 32, 4>},      \
    {64, 4, 0, launch_order<BODY, R, 64, 4>},  {16, 16, 0, launch_order<BODY, R, 16, 16>},    \
-   {16, 8, 0, launch_order<BODY, R, 16, 8>}}
+   {16, 8, 0, launch_order<BODY, R, 16, 8>},  {8, 16, 0, launch_order<BODY, R, 8, 16>}}
 
-constexpr int kOrderShapes = 5;
+constexpr int kOrderShapes = 6;
 static const LaunchVariant kWaveO2[kOrderShapes] = CHEMORA_SHAPES(WaveO2, 1);
 static const LaunchVariant kWaveO6[kOrderShapes] = CHEMORA_SHAPES(WaveO6, 3);
 static const LaunchVariant kWaveO8[kOrderShapes] = CHEMORA_SHAPES(WaveO8, 4);
@@ -319,6 +319,9 @@ int launch_wave_planes(const Dims& d, const Scalars& sc, const StageParams& a, c
 template int launch_wave_planes<32, 8>(const Dims&, const Scalars&, const StageParams&, cudaStream_t);
 template int launch_wave_planes<32, 4>(const Dims&, const Scalars&, const StageParams&, cudaStream_t);
 template int launch_wave_planes<16, 16>(const Dims&, const Scalars&, const StageParams&, cudaStream_t);
+template int launch_wave_planes<64, 4>(const Dims&, const Scalars&, const StageParams&, cudaStream_t);
+template int launch_wave_planes<16, 8>(const Dims&, const Scalars&, const StageParams&, cudaStream_t);
+template int launch_wave_planes<8, 16>(const Dims&, const Scalars&, const StageParams&, cudaStream_t);
 
 int launch_wave_order_stage(const Dims& d, const Scalars& sc, const StageParams& a, cudaStream_t s,
                             int variant) {

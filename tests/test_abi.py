@@ -116,6 +116,20 @@ def test_system_opcounts(L):
         L.chemora_destroy(g)
 
 
+def test_variant_numbers(L):
+    """A system accepts every number below its kind's count, no fewer than the
+    one-kernel bodies had: numbers that a program has written down stay valid."""
+    for kind, nv, ng, count in ((N.WAVE, 2, 2, 13), (N.WAVE_VARC, 2, 2, 6), (N.WAVE1, 5, 2, 6), (N.BSSN, 24, 3, 21)):
+        assert L.chemora_variant_count(kind) >= count
+        g, s = ctypes.c_void_p(), ctypes.c_void_p()
+        assert L.chemora_grid_create(8, 8, 8, nv, ng, 0.1, ctypes.byref(g)) == N.OK
+        assert L.chemora_system_create(g, kind, None, ctypes.byref(s)) == N.OK
+        for v in range(L.chemora_variant_count(kind)):
+            assert L.chemora_system_variant(s, v, None, None, None) == N.OK
+        L.chemora_destroy(s)
+        L.chemora_destroy(g)
+
+
 def test_variant_queries(L):
     for kind in (N.WAVE, N.WAVE_VARC, N.BSSN):
         assert L.chemora_variant_count(kind) >= 4
