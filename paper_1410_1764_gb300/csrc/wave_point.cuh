@@ -33,6 +33,12 @@ struct Star2 {
     n[10] = ld(0, 0, 0, 2);
     n[11] = ld(0, 0, 0, -2);
   }
+  CHEMORA_FX bool zero() const {
+    unsigned b = fx::hiword(c) << 1 | fx::loword(c);
+#pragma unroll
+    for (int q = 0; q < 12; ++q) b |= fx::hiword(n[q]) << 1 | fx::loword(n[q]);
+    return b == 0;
+  }
   CHEMORA_FX int exponent() const {
     int e = fx::exponent(c);
 #pragma unroll
@@ -75,6 +81,9 @@ CHEMORA_FX void wave_point(const LD& ld, const Scalars& sc, OUT& out) {
   if (fx::in_range(e)) {
     out(0, ld(1, 0, 0, 0));
     out(1, fma(star2_lap(s, e), sc.i12h2, sc.k[CHEMORA_K_MZERO]));
+  } else if (s.zero()) {
+    out(0, ld(1, 0, 0, 0));
+    out(1, 0.0);
   } else {
     const StarLoader<LD> sl{s, ld};
     chemora_wave_point(sl, sc, out);
