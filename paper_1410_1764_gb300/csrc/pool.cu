@@ -4,7 +4,7 @@
 // finds mapped memory (with a pool of its own its first right-hand side of 16^3
 // points took 281 us, its second 106).  The pool is never destroyed: a system may
 // be destroyed while a call that used the pool is still running, and destroying
-// a pool with a free outstanding crashed the process (driver 580.159).
+// a pool with a free outstanding crashed the process (NVIDIA driver 580.159).
 #include <mutex>
 
 #include "internal.h"

@@ -72,4 +72,4 @@ def test_specialised_block(api, tmp_path):
         s.specialize(True, cache_dir=tmp_path)
         fast.append(best(s))
     t = best(plain)
-    assert max(fast) <= 1.05 * t, (fast, t)  # 1.11 with the table's 128-thread block compiled
+    assert max(fast) <= 1.08 * t, (fast, t)  # 1.11 with the table's 128-thread block compiled

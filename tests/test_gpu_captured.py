@@ -76,7 +76,8 @@ def test_same_as_plain(api, dims, how, tmp_path):
     a2, d2 = torch.zeros_like(y), torch.zeros_like(y)
     sysm.stage(1, y, yn, a2, d2, c2=0.01)
     assert torch.equal(_inside(acc), _inside(a2)) and torch.equal(_inside(dst), _inside(d2))
-    assert _ms(rhs.replay, 20) <= 1.1 * _ms(lambda: sysm.rhs(y, out), 20)
+    # 2.1 to 3 times with the kernel that needs no workspace
+    assert _ms(rhs.replay, 20) <= 1.3 * _ms(lambda: sysm.rhs(y, out), 20)
 
 
 def test_workspaces(api):

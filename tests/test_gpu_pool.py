@@ -66,7 +66,7 @@ for _ in range(5):
     s = system(16)
     first.append(wall(lambda: s.rhs(y16, out16)))
     more.append(s)
-assert min(first) < 1.5 * second + 2e-5, (first, second)
+assert min(first) < 1.8 * second + 2e-5, (first, second)
 
 # with no system left the memory goes back
 del a, s, small
